@@ -367,3 +367,140 @@ def tolerance(case):
         return {"rel": 2e-6, "max": 1e-5, "differ": 2e-3}
     # bf16 outputs of sums whose weights are rounded to bf16: 2.3e-3 (largest 0.011) against 64 bits
     return {"rel": 1e-2, "max": 0.05, "differ": 2e-3}
+
+
+# ---- the same outputs in 64 bits, from the inputs alone
+def _prefix(pk, table, layer, length):
+    """Keys (or values) of the shared prefix, [length, hkv, dim]."""
+    x = pk[layer]
+    if table is None:
+        return x[:, :length].transpose(0, 1)
+    return x[table.long()].transpose(1, 2).flatten(0, 1)[:length]   # [pages, hkv, 64, dim] in the order of the table
+
+
+def _attention64(q, k, v, scale, causal_from):
+    """q [d, hq, dim] against k, v [keys, hkv, dim]; keys from causal_from on are visible up to the query's position."""
+    d, hq, dim = q.shape
+    hkv = k.shape[1]
+    qh = q.view(d, hkv, hq // hkv, dim).permute(1, 2, 0, 3).reshape(hkv, -1, dim)
+    sc = torch.matmul(qh, k.permute(1, 2, 0)) * scale
+    if causal_from is not None:
+        hidden = torch.ones((d, d), dtype=torch.bool, device=q.device).triu(1).repeat(hq // hkv, 1)
+        sc[:, :, causal_from:].masked_fill_(hidden, float("-inf"))
+    o = torch.matmul(torch.softmax(sc, -1), v.transpose(0, 1))
+    return o.view(hkv, hq // hkv, d, dim).permute(2, 0, 1, 3).reshape(-1)
+
+
+def _exact_attention(s):
+    c = s.case
+    hq, hkv, dim, causal = c["hq"], c["hkv"], c["dim"], c["causal"] or c["kind"] == "cycle"
+    before = c["blocks"] - 1 if c["kind"] == "block" else 0          # blocks that join the caches ahead of the last one
+    out = torch.zeros(s.out.shape, dtype=torch.float64, device="cuda")
+    for layer in range(c["layers"]):
+        at = 0
+        for (prefix, forks, d, _), (pk, pv, table) in zip(_scenes(c), s.keep):
+            shared = [_prefix(x, table, layer, prefix).double() for x in (pk, pv)]
+            for f in range(forks):
+                own = [x[layer].view(-1, hkv, dim)[at:at + d].double() for x in (s.k, s.v)]
+                kv = [[shared[i]] + [own[i]] * before for i in range(2)]
+                for e in s.keep[len(_scenes(c)):]:                   # blocks committed earlier (such cases have one scene and layer)
+                    for i in range(2):
+                        kv[i].append(e[i].view(forks, -1, hkv, dim)[f].double())
+                k, v = (torch.cat(kv[i] + [own[i]]) for i in range(2))
+                q = s.q[layer].view(-1, hq, dim)[at:at + d].double()
+                out[layer, at * hq * dim:(at + d) * hq * dim] = _attention64(q, k, v, s.scale, len(k) - d if causal else None)
+                at += d
+    return out
+
+
+def _exact_caches(s):
+    c = s.case
+    res, at = [], 0
+    for (prefix, forks, d, _), (sk, sv), (pk, pv, table) in zip(_scenes(c), s.suffixes, s.keep):
+        blocks = [x.view(c["layers"], -1, c["hkv"], c["dim"])[:, at:at + forks * d].view(c["layers"], forks, d, c["hkv"], c["dim"])
+                  for x in (s.k, s.v)]
+        at += forks * d
+        if not c["extend"]:
+            res += [b.transpose(2, 3).repeat(1, 1, 1, c["blocks"], 1).double() for b in blocks]
+            continue
+        pos = torch.arange(prefix, prefix + c["blocks"] * d, device="cuda")
+        for cache, b in zip((pk, pv), blocks):
+            x, rows = cache.double(), b[:, 0].repeat(1, c["blocks"], 1, 1).double()
+            if table is None:
+                x[:, :, pos] = rows.transpose(1, 2)
+            else:
+                x[:, table.long()[pos // c["page"]], :, pos % c["page"]] = rows.transpose(0, 1)
+            res.append(x)
+    return res
+
+
+def _exact_trajectory(s):
+    if not s.case["average"]:
+        return torch.zeros(s.traj_out.shape, dtype=torch.float64, device="cuda")
+    mean = s.traj.double().mean(0)
+    if s.case["average"] == "plain":
+        return mean
+    # least integral of squared jerk through the origin and the waypoints: sums of |t - knot|^5 and a parabola
+    n = WAYPOINTS + 1
+    kt = torch.arange(n, dtype=torch.float64)
+    par = torch.stack([kt ** e for e in range(3)], 1)
+    lhs = torch.zeros((n + 3, n + 3), dtype=torch.float64)
+    lhs[:n, :n], lhs[:n, n:], lhs[n:, :n] = (kt[:, None] - kt).abs() ** 5, par, par.T
+    rhs = torch.zeros((n + 3, 2), dtype=torch.float64)
+    rhs[1:n] = mean.cpu()
+    w = torch.linalg.solve(lhs, rhs)
+    t = (torch.arange(JMT_WAYPOINTS, dtype=torch.float64) + 1) * WAYPOINTS / JMT_WAYPOINTS
+    return (torch.cat([(t[:, None] - kt).abs() ** 5, torch.stack([t ** e for e in range(3)], 1)], 1) @ w).cuda()
+
+
+def _philox(c0, c1, key):
+    """Philox4x32-10 of the counters (c0, c1, 0, 0): int64 tensors holding 32-bit words; four words in the last dimension."""
+    low = 0xFFFFFFFF
+    c = [c0, c1, torch.zeros_like(c0), torch.zeros_like(c0)]
+    k = [key & low, key >> 32]
+    for _ in range(10):
+        p0, p1 = 0xD2511F53 * c[0], 0xCD9E8D57 * c[2]                # (wraps modulo 2^64: the same bits)
+        c = [((p1 >> 32) & low) ^ c[1] ^ k[0], p1 & low, ((p0 >> 32) & low) ^ c[3] ^ k[1], p0 & low]
+        k = [(k[0] + 0x9E3779B9) & low, (k[1] + 0xBB67AE85) & low]
+    return torch.stack(c, -1)
+
+
+def _gumbel(v, pos, keys):
+    """Draws of rows with positions pos and seeds keys (int64, one per row) at step 0 of block 0, [rows, v]: an
+    exponential race over groups of 16 ids whose leader the group's word names."""
+    groups = (v + 15) // 16
+    pos, keys = pos[:, None], keys[:, None]
+    r = _philox(torch.arange((groups + 3) // 4, device="cuda") + 0 * pos, 0 * keys + pos, keys).flatten(1)[:, :groups]
+    f = (_philox(torch.arange(groups * 4, device="cuda") + 0 * pos, 0 * keys + pos + 2 ** 31, keys) >> 9).view(len(pos), groups, 16)
+    fine = (f.double() + 0.5) * 2.0 ** -23
+    lead = (r & 15)[..., None]
+    e_lead = -torch.log(((r >> 4).double()[..., None] + fine.gather(2, lead)) * 2.0 ** -28) / 16
+    e = (e_lead - torch.log(fine)).scatter(2, lead, e_lead)
+    return -torch.log(e).flatten(1)[:, :v]
+
+
+def _exact_confidence(s, seed):
+    c = s.case
+    d, v = c["block"], c["vocab"]
+    scores = s.host.cuda() if c["kind"] == "host" else s.scores
+    conf = torch.full((c["forks"] * d,), float("nan"), dtype=torch.float64, device="cuda")
+    masked = torch.nonzero(s.template[4 * len(conf):] == fdd.FDD_MASKED).flatten()
+    for idx in masked.split(32):
+        x = scores[idx].double()
+        y = x if c["temperature"] == 0.0 else x + c["temperature"] * _gumbel(v, idx % d, seed * 1000003 + idx // d)
+        conf[idx] = torch.exp(x.gather(1, y.argmax(1, keepdim=True))[:, 0] - torch.logsumexp(x, 1))
+    return conf
+
+
+def exact(case, seed):
+    """What `run` returns, in 64 bits; whole numbers are left out."""
+    c = case
+    s = prepare(case, seed)
+    if c["kind"] == "attn":
+        return _exact_attention(s)
+    if c["kind"] == "cycle":
+        return {"tokens": None, "state": None, "accepted": None, "left": None, "out": _exact_attention(s)}
+    if c["kind"] in ("unmask", "host"):
+        return {"tokens": None, "state": None, "committed": None, "left": None, "conf": _exact_confidence(s, seed)}
+    return {"tokens": None, "state": None, "left": None, "out": _exact_attention(s), "caches": _exact_caches(s),
+            "trajectory": _exact_trajectory(s)}
