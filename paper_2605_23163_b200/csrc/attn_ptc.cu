@@ -26,6 +26,20 @@
 // Per key tile and query tile:
 //   S = Q K^T (smem x smem)  ->  soft-max warps: running max (rescaling O only when the max moved
 //   by more than 2^8), P = exp2(S * c - m) -> TMEM  ->  O += P V (TMEM x smem, V keys-major).
+//
+// Groups that are not a power of two.  A query tile then holds the group's rows at 128 / G positions (18
+// positions, 126 rows for G = 7; the last rows of the tile are never read), and P keeps 16 bits of every
+// probability, P = P_hi + P_lo with both halves bf16 (P_lo the rounding error of P_hi), as two products into
+// the same O: these shapes were computed in fp32 on the CUDA cores before, and with one bf16 P they would
+// lose precision (error against 64 bits: 1.66e-3 with both halves as before, the rounding of the output;
+// 2.3e-3 with P_hi alone).  TMEM is S0 | S1 | O0 | O1 for them: each query tile has scores of its own, and
+// the two halves of P overwrite them.  The chain of a query tile (scores, soft-max, output, the next scores)
+// is then a serial one, one issuing warp each; the other tile's chain fills the gaps.  Three products of a
+// tile step instead of two are 3072 clocks of the tensor pipe, what a step of the other layout takes with
+// two (its soft-max groups are the limit), so nothing is gained by overlapping more.  Measured: a block of
+// six rollouts, 28 / 4 heads, 27 positions, prefix 3001, two layers: 6180 us with the CUDA-core kernel that
+// served these shapes (32 rows a CTA, fp32 FMA), 530 us with this.
+//
 // The MMA warp issues QK(1, j), PV(1, j - 1), QK(0, j + 1), PV(0, j) in that order, which keeps the
 // tensor pipe fed while each soft-max group spends a whole period on one tile.
 // Items follow one another without a meeting of the whole CTA: Q of the next item is staged as soon as
@@ -63,7 +77,9 @@ struct SetParams {
     const int32_t* gate;       // per rollout, 0 = skip it; nullptr = every rollout takes part
     int fork_base;             // rollouts of the scenes before this one (index into the kernel's list)
     int units_per_fork;        // Hkv * row_pairs
-    int n_forks, d, n_q_heads, G, R;
+    int n_forks, d, n_q_heads, G;
+    int tile_pos, tile_rows;   // block positions of one query tile (128 / G) and the rows they make (tile_pos * G)
+    int q_tiles;               // query tiles of a (rollout, KV head)
     int prefix_len, page_tokens, n_phys_pages, suffix_len;
     int tiles_prefix, tiles_suffix, tiles_total;
     int row_pairs;
@@ -105,6 +121,9 @@ __device__ __forceinline__ TileInfo tile_info(const SetParams& p, int g) {
     }
     return t;
 }
+
+// How the scores and probabilities of the two query tiles share TMEM (see the top of the file).
+constexpr int kSharedScores = 0, kOwnScoresSplit = 1;
 
 template <int D>
 struct TcShape {
@@ -246,11 +265,12 @@ struct Deferred {
     long long unit_begin;
 };
 
-template <int D, int MAXSETS, int EMU>
+template <int D, int MAXSETS, int EMU, int MODE>
 __global__ void __launch_bounds__(kTcThreads, 1)
 attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
     using Shape = TcShape<D>;
     constexpr int kStages = Shape::kStages;
+    constexpr bool kOwn = MODE == kOwnScoresSplit;      // every query tile has a score buffer of its own, probabilities in two halves
     static_assert(EMU % 8 == 0 && EMU >= 0 && EMU <= 128, "EMU: emulated exponentials per 128-key tile");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -321,12 +341,12 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
         abort_s = 0;
         n_deferred_s = 0;
         tc::mbar_init(tc::smem_u32(&bar_q_full), 1);
-        tc::mbar_init(tc::smem_u32(&bar_q_empty), 1);      // every QK^T product of an item has completed: Q may be overwritten
+        tc::mbar_init(tc::smem_u32(&bar_q_empty), kOwn ? 2 : 1);      // every QK^T product of an item has completed: Q may be overwritten
         for (int s = 0; s < kStages; ++s) {
             tc::mbar_init(tc::smem_u32(&bar_k_full[s]), 1);
-            tc::mbar_init(tc::smem_u32(&bar_k_empty[s]), 1);
+            tc::mbar_init(tc::smem_u32(&bar_k_empty[s]), kOwn ? 2 : 1);
             tc::mbar_init(tc::smem_u32(&bar_v_full[s]), 1);
-            tc::mbar_init(tc::smem_u32(&bar_v_empty[s]), 1);
+            tc::mbar_init(tc::smem_u32(&bar_v_empty[s]), kOwn ? 2 : 1);
         }
         for (int q = 0; q < 2; ++q) {
             tc::mbar_init(tc::smem_u32(&bar_s_full[q]), 1);     // scores of query tile q are in S
@@ -345,8 +365,8 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = tmem_base_s;
-    const uint32_t tm_s = tmem;
-    const uint32_t tm_p[2] = {tmem + 128, tmem + 192};
+    const uint32_t tm_s[2] = {tmem, kOwn ? tmem + 128 : tmem};
+    const uint32_t tm_p[2] = {kOwn ? tmem : tmem + 128, kOwn ? tmem + 128 : tmem + 192};
     const uint32_t tm_o[2] = {tmem + 256, tmem + 256 + D};
 
     // Each role runs its own copy of the item loop.  Nothing brings all of them together between two
@@ -356,7 +376,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
     // first P of the next item (written after its epilogue) is what lets the PV issuer overwrite O.
     struct ItemView {
         Item it;
-        int f, rp, h, nt, rows_here, NQ;
+        int f, rp, h, nt, NQ;
     };
     auto view_item = [&](long long pos) {
         ItemView v;
@@ -369,8 +389,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
         v.rp = idx % p.row_pairs; idx /= p.row_pairs;
         v.h = idx;
         v.nt = v.it.t1 - v.it.t0;
-        v.rows_here = min(256, p.R - v.rp * 256);
-        v.NQ = v.rows_here > 128 ? 2 : 1;
+        v.NQ = min(2, p.q_tiles - v.rp * 2);
         return v;
     };
 
@@ -397,11 +416,11 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                     }
                     if (ok && tc::elect_one()) {
                         tc::prefetch_tmap(&maps.q);
-                        tc::mbar_arrive_expect_tx(bq, v.NQ * Shape::kTileBytes);
+                        tc::mbar_arrive_expect_tx(bq, v.NQ * Shape::kChunks * p.tile_rows * 128);
                         for (int q = 0; q < v.NQ; ++q)
                             for (int ch = 0; ch < Shape::kChunks; ++ch)
                                 tc::tma_load_4d(q_s + q * Shape::kTileBytes + ch * Shape::kChunkBytes, &maps.q, bq, ch * 64,
-                                                v.h * p.G, (v.rp * 2 + q) * (128 / p.G), v.f);
+                                                v.h * p.G, (v.rp * 2 + q) * p.tile_pos, v.f);
                     }
                     __syncwarp();
                     for (int jl = 0; jl < v.nt && ok; ++jl) {
@@ -488,8 +507,8 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
 #pragma unroll
                         for (int k = 0; k < D / 16; ++k) {
                             const uint32_t off = ((k >> 2) * Shape::kChunkBytes + (k & 3) * 32) >> 4;
-                            if (k == 0) tc::mma_ss_first(tm_s, dq + off, dk + off, kIdescQK);
-                            else tc::mma_ss_acc(tm_s, dq + off, dk + off, kIdescQK);
+                            if (k == 0) tc::mma_ss_first(tm_s[q], dq + off, dk + off, kIdescQK);
+                            else tc::mma_ss_acc(tm_s[q], dq + off, dk + off, kIdescQK);
                         }
                     };
                     // O[q] (+)= P[q] . V
@@ -500,6 +519,12 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
 #pragma unroll
                         for (int j = 1; j < kKeysPerTile / 16; ++j)
                             tc::mma_ts_acc(tm_o[q], tm_p[q] + j * 8, dv + static_cast<uint32_t>((j * 2048) >> 4), kIdescPV);
+                        if (kOwn) {
+                            // the low halves of the probabilities
+#pragma unroll
+                            for (int j = 0; j < kKeysPerTile / 16; ++j)
+                                tc::mma_ts_acc(tm_o[q], tm_p[q] + 64 + j * 8, dv + static_cast<uint32_t>((j * 2048) >> 4), kIdescPV);
+                        }
                     };
                     auto stage_of = [&](int jl) { return static_cast<int>((kv_cnt + jl) % kStages); };
                     auto phase_of = [&](int jl) { return ((kv_cnt + jl) / kStages) & 1u; };
@@ -550,7 +575,50 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                         s_has_prev = true;
                         return true;
                     };
-                    if (qk_role) {
+                    if (kOwn) {
+                        // one chain per query tile and warp: scores, (soft-max), output, the next tile's scores
+                        const int q = warp - 9;
+                        const bool mine = q < NQ;
+                        ok = __shfl_sync(0xFFFFFFFFu, wait(&bar_q_full, item_cnt) ? 1 : 0, 0) != 0;
+                        for (int jl = 0; jl < nt && ok; ++jl) {
+                            const int s = stage_of(jl);
+                            bool good = wait(&bar_k_full[s], phase_of(jl));
+                            // P[q] of the tile before lies in the same columns: its product has to be complete
+                            if (mine && sp_cnt[0] + jl > 0) good = good && wait(&bar_o_done[q], sp_cnt[0] + jl - 1);
+                            ok = __shfl_sync(0xFFFFFFFFu, good ? 1 : 0, 0) != 0;
+                            if (!ok) break;
+                            tc::fence_after_sync();
+                            if (tc::elect_one()) {
+                                if (mine) {
+                                    issue_qk(q, s);
+                                    tc::mma_commit(tc::smem_u32(&bar_s_full[q]));
+                                    tc::mma_commit(tc::smem_u32(&bar_k_empty[s]));
+                                    if (jl == nt - 1) tc::mma_commit(tc::smem_u32(&bar_q_empty));
+                                } else {
+                                    // no such query tile in this item: hand the stages on
+                                    tc::mbar_arrive(tc::smem_u32(&bar_k_empty[s]));
+                                    if (jl == nt - 1) tc::mbar_arrive(tc::smem_u32(&bar_q_empty));
+                                }
+                            }
+                            __syncwarp();
+                            good = wait(&bar_v_full[s], phase_of(jl));
+                            if (mine) good = good && wait(&bar_p_full[q], sp_cnt[0] + jl);
+                            ok = __shfl_sync(0xFFFFFFFFu, good ? 1 : 0, 0) != 0;
+                            if (!ok) break;
+                            tc::fence_after_sync();
+                            if (tc::elect_one()) {
+                                if (mine) {
+                                    issue_pv(q, s, jl > 0);
+                                    tc::mma_commit(tc::smem_u32(&bar_o_done[q]));
+                                    tc::mma_commit(tc::smem_u32(&bar_v_empty[s]));
+                                    if (jl == nt - 1) tc::mma_commit(tc::smem_u32(&bar_o_final[q]));
+                                } else {
+                                    tc::mbar_arrive(tc::smem_u32(&bar_v_empty[s]));
+                                }
+                            }
+                            __syncwarp();
+                        }
+                    } else if (qk_role) {
                         // scores: QK(0,0) | QK(1,j) QK(0,j+1) | ...   (S is one buffer: each product waits
                         // until the group that owned the previous scores has copied them out)
                         ok = __shfl_sync(0xFFFFFFFFu, wait(&bar_q_full, item_cnt) ? 1 : 0, 0) != 0;
@@ -574,7 +642,11 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                 }
                 __syncwarp();
                 kv_cnt += nt;
-                for (int q = 0; q < NQ; ++q) sp_cnt[q] += nt;
+                if (kOwn) {
+                    if (warp - 9 < NQ) sp_cnt[0] += nt;          // (this warp's query tile)
+                } else {
+                    for (int q = 0; q < NQ; ++q) sp_cnt[q] += nt;
+                }
                 ++item_cnt;
                 pos += nt;
             }
@@ -597,10 +669,11 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
             const SetParams& p = a.sets[it.s];
             const int f = v.f, rp = v.rp, h = v.h, nt = v.nt;
             const bool active = q < v.NQ;
-            const int r = rp * 256 + q * 128 + row_local;       // row inside the unit
-            const bool row_ok = r < p.R;
-            const int qi = row_ok ? r / p.G : 0;
-            const int qg = row_ok ? r - qi * p.G : 0;
+            const int pos_in_tile = row_local / p.G;
+            int qi = (rp * 2 + q) * p.tile_pos + pos_in_tile;   // block position of this row
+            const bool row_ok = row_local < p.tile_rows && qi < p.d;
+            if (!row_ok) qi = 0;
+            const int qg = row_ok ? row_local - pos_in_tile * p.G : 0;
             float m_used = -CUDART_INF_F, l = 0.0f;
             bool ok = *abort_flag == 0;
             if (active && ok) {
@@ -616,10 +689,12 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                     tc::fence_after_sync();
                     uint32_t sr[128];
 #pragma unroll
-                    for (int cc = 0; cc < 4; ++cc) tc::tmem_ld32(tm_s + lane_base + cc * 32, sr + cc * 32);
+                    for (int cc = 0; cc < 4; ++cc) tc::tmem_ld32(tm_s[q] + lane_base + cc * 32, sr + cc * 32);
                     tc::wait_ld();
-                    tc::fence_before_sync();
-                    tc::mbar_arrive(bf);                                // S may be overwritten now
+                    if (!kOwn) {
+                        tc::fence_before_sync();
+                        tc::mbar_arrive(bf);                            // S may be overwritten now
+                    }
                     int limit = t.nvalid;                               // keys [0, limit) are visible
                     if (p.causal && t.segment == 2) limit = min(limit, qi - t.index * kKeysPerTile + 1);
                     if (limit < kKeysPerTile) {
@@ -645,17 +720,20 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                     if (!(m_tile > -CUDART_INF_F)) m_tile = m_used > -CUDART_INF_F ? m_used : 0.0f;
                     // The previous PV of this query tile must be complete before P is overwritten and
                     // before O is rescaled (it is one phase behind at most).  Usually only the first
-                    // matters, so the wait sits after the exponentials.
-                    bool pv_done = jl == 0;
+                    // matters, so the wait sits after the exponentials.  (With a score buffer per query tile these
+                    // scores were only computed once that product was complete.)
+                    bool pv_done = kOwn || jl == 0;
                     if (jl == 0) {
                         m_used = m_tile;
                     } else {
                         const bool need = m_tile > m_used + 8.0f;
                         if (__any_sync(0xFFFFFFFFu, need)) {
-                            ok = tc::mbar_wait(bo, (sp0 + jl - 1) & 1, abort_flag, kWaitLimit);
-                            if (!ok) break;
-                            pv_done = true;
-                            tc::fence_after_sync();
+                            if (!kOwn) {
+                                ok = tc::mbar_wait(bo, (sp0 + jl - 1) & 1, abort_flag, kWaitLimit);
+                                if (!ok) break;
+                                pv_done = true;
+                                tc::fence_after_sync();
+                            }
                             const float alpha = need ? exp2f(m_used - m_tile) : 1.0f;
 #pragma unroll
                             for (int cc = 0; cc < D / 32; ++cc) {
@@ -674,7 +752,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                     // P = 2^(S * c - m): the first 128 - EMU scores through ex2.approx, the rest
                     // through the polynomial; row sums in four packed accumulators.
                     uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
-                    uint32_t packed[64];
+                    uint32_t packed[64], packed_lo[kOwn ? 32 : 1];
                     const uint64_t nm2 = tc::pack2(-m_used, -m_used);
 #pragma unroll
                     for (int i = 0; i < (128 - EMU) / 2; ++i) {
@@ -685,6 +763,16 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                         acc[i & 3] = tc::add2(acc[i & 3], tc::pack2(e0, e1));
                         const __nv_bfloat162 pk = __floats2bfloat162_rn(e0, e1);
                         packed[i] = *reinterpret_cast<const uint32_t*>(&pk);
+                        if (kOwn) {
+                            // what the rounding to bf16 left over (exact in fp32), again as bf16: 16 bits in all
+                            const float r0 = e0 - __uint_as_float(packed[i] << 16), r1 = e1 - __uint_as_float(packed[i] & 0xFFFF0000u);
+                            const __nv_bfloat162 pl = __floats2bfloat162_rn(r0, r1);
+                            packed_lo[i % 32] = *reinterpret_cast<const uint32_t*>(&pl);
+                            if (i % 32 == 31) {
+                                tc::tmem_st32(tm_p[q] + lane_base + i - 31, packed + i - 31);
+                                tc::tmem_st32(tm_p[q] + 64 + lane_base + i - 31, packed_lo);
+                            }
+                        }
                     }
                     if (EMU > 0) {
                         // y = (S * c - m + 112) / 128 clamped to [0, 1]; 2^(128 y - 112) = 2^n * 2^f with
@@ -727,8 +815,10 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                         if (!ok) break;
                         tc::fence_after_sync();
                     }
-                    tc::tmem_st32(tm_p[q] + lane_base, packed);
-                    tc::tmem_st32(tm_p[q] + lane_base + 32, packed + 32);
+                    if (!kOwn) {
+                        tc::tmem_st32(tm_p[q] + lane_base, packed);
+                        tc::tmem_st32(tm_p[q] + lane_base + 32, packed + 32);
+                    }
                     tc::wait_st();
                     tc::fence_before_sync();
                     tc::mbar_arrive(bp);
@@ -943,7 +1033,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                 const int n_pieces = dfr.n_pieces;
                 const int* slots = slot2_s[e];
                 // this CTA's share of the rows; a row is split between `col_groups` threads
-                const int rows_here = min(256, p.R - dfr.rp * 256);
+                const int rows_here = min(2 * p.tile_rows, p.d * p.G - dfr.rp * 2 * p.tile_rows);
                 const int mine = static_cast<int>(blockIdx.x) - dfr.c_first;
                 const int row_lo = rows_here * mine / n_pieces, row_hi = rows_here * (mine + 1) / n_pieces;
                 const int share = row_hi - row_lo;                    // <= 86 (three pieces or more)
@@ -952,9 +1042,10 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                 const int ct = (D / 4) / col_groups;                  // float4 columns per thread
                 const int row_in_share = lt / col_groups, cg = lt - row_in_share * col_groups;
                 if (share > 0 && row_in_share < share) {
-                    const int rowu = row_lo + row_in_share;
-                    const int r = dfr.rp * 256 + rowu;
-                    const int qi2 = r / p.G, qg2 = r - qi2 * p.G;
+                    const int rc = row_lo + row_in_share;             // row of the unit without the gap behind a tile's last row
+                    const int rowu = rc < p.tile_rows ? rc : rc - p.tile_rows + 128;
+                    const int pos2 = rc / p.G;
+                    const int qi2 = dfr.rp * 2 * p.tile_pos + pos2, qg2 = rc - pos2 * p.G;
                     __nv_bfloat16* op = p.out + ((static_cast<size_t>(dfr.f) * p.d + qi2) * p.n_q_heads + dfr.h * p.G + qg2) * D;
                     const int col0 = cg * ct;
                     switch (ct) {
@@ -991,7 +1082,7 @@ bool make_call_maps(const AttnProblem& a, int D, TcSetMaps* m) {
     {
         uint64_t dims[4] = {(uint64_t)D, (uint64_t)a.n_q_heads, (uint64_t)a.d, (uint64_t)a.n_forks};
         uint64_t str[3] = {D * eb, a.n_q_heads * D * eb, (uint64_t)a.d * a.n_q_heads * D * eb};
-        uint32_t box[4] = {64, (uint32_t)G, (uint32_t)(128 / G), 1};
+        uint32_t box[4] = {64, (uint32_t)G, (uint32_t)(128 / G), 1};   // one query tile: every head of the group at 128 / G positions
         if (!tmap::encode_bf16(&m->q, a.q, 4, dims, str, box)) return false;
     }
     {
@@ -1075,7 +1166,7 @@ int emulated_exponentials() {
     return value;
 }
 
-template <int D, int MAXSETS, int EMU>
+template <int D, int MAXSETS, int EMU, int MODE>
 cudaError_t launch_one(const TcArgs<MAXSETS>& args, unsigned ctas, int device, cudaStream_t st) {
     const int smem = TcShape<D>::kSmemBytes;
     // the kernel's shared-memory size is a per-device attribute: set on the first launch on each device
@@ -1083,7 +1174,7 @@ cudaError_t launch_one(const TcArgs<MAXSETS>& args, unsigned ctas, int device, c
     static std::atomic<bool> configured[kMaxDevices];
     if (device < 0 || device >= kMaxDevices) return cudaErrorInvalidDevice;
     if (!configured[device].load(std::memory_order_acquire)) {
-        cudaError_t e = cudaFuncSetAttribute(attn_ptc_kernel<D, MAXSETS, EMU>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t e = cudaFuncSetAttribute(attn_ptc_kernel<D, MAXSETS, EMU, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         configured[device].store(true, std::memory_order_release);
     }
@@ -1106,7 +1197,7 @@ cudaError_t launch_one(const TcArgs<MAXSETS>& args, unsigned ctas, int device, c
     cfg.attrs = attr;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const bool capturing = cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
-    const void* fn = reinterpret_cast<const void*>(&attn_ptc_kernel<D, MAXSETS, EMU>);
+    const void* fn = reinterpret_cast<const void*>(&attn_ptc_kernel<D, MAXSETS, EMU, MODE>);
     if (!capturing && !early_start_refused[device].load(std::memory_order_relaxed)) {
         cfg.numAttrs = 2;
         const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, params);
@@ -1120,11 +1211,17 @@ cudaError_t launch_one(const TcArgs<MAXSETS>& args, unsigned ctas, int device, c
 
 template <int MAXSETS>
 cudaError_t launch_emu(const TcArgs<MAXSETS>& args, int head_dim, unsigned ctas, int device, cudaStream_t st) {
-    if (head_dim == 64) return launch_one<64, MAXSETS, 0>(args, ctas, device, st);
+    const int G = args.sets[0].G;                          // (the same for every scene of a context)
+    if ((G & (G - 1)) != 0) {
+        // Groups that are not a power of two keep 16 bits of every probability (see the top of the file).
+        if (head_dim == 64) return launch_one<64, MAXSETS, 0, kOwnScoresSplit>(args, ctas, device, st);
+        return launch_one<128, MAXSETS, 0, kOwnScoresSplit>(args, ctas, device, st);
+    }
+    if (head_dim == 64) return launch_one<64, MAXSETS, 0, kSharedScores>(args, ctas, device, st);
     switch (emulated_exponentials()) {
-        case 16: return launch_one<128, MAXSETS, 16>(args, ctas, device, st);
-        case 32: return launch_one<128, MAXSETS, 32>(args, ctas, device, st);
-        default: return launch_one<128, MAXSETS, 0>(args, ctas, device, st);
+        case 16: return launch_one<128, MAXSETS, 16, kSharedScores>(args, ctas, device, st);
+        case 32: return launch_one<128, MAXSETS, 32, kSharedScores>(args, ctas, device, st);
+        default: return launch_one<128, MAXSETS, 0, kSharedScores>(args, ctas, device, st);
     }
 }
 
@@ -1147,13 +1244,15 @@ cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* con
         p.page_table = a.page_table;
         p.n_forks = a.n_forks; p.d = a.d; p.n_q_heads = a.n_q_heads;
         p.G = a.n_q_heads / a.n_kv_heads;
-        p.R = a.d * p.G;
+        p.tile_pos = 128 / p.G;
+        p.tile_rows = p.tile_pos * p.G;
+        p.q_tiles = (a.d + p.tile_pos - 1) / p.tile_pos;
         p.prefix_len = a.prefix_len; p.page_tokens = a.page_tokens; p.n_phys_pages = a.prefix_capacity;
         p.suffix_len = a.suffix_len;
         p.tiles_prefix = (a.prefix_len + kKeysPerTile - 1) / kKeysPerTile;
         p.tiles_suffix = (a.suffix_len + kKeysPerTile - 1) / kKeysPerTile;
         p.tiles_total = p.tiles_prefix + p.tiles_suffix + (a.d + kKeysPerTile - 1) / kKeysPerTile;
-        p.row_pairs = (p.R + 255) / 256;
+        p.row_pairs = (p.q_tiles + 1) / 2;
         p.units_per_fork = a.n_kv_heads * p.row_pairs;
         p.causal = a.causal_in_block;
         p.gate = a.gate;
@@ -1186,15 +1285,6 @@ cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* con
 }
 
 }  // namespace
-
-// Whether the tensor-core kernel covers this problem.
-bool attention_tc_supported(const AttnProblem& a, int head_dim) {
-    const int G = a.n_q_heads / a.n_kv_heads;
-    if (head_dim != 64 && head_dim != 128) return false;
-    if (G < 1 || G > 16 || (G & (G - 1)) != 0) return false;
-    if (a.page_tokens != 0 && a.page_tokens != 64) return false;
-    return tmap::encode_fn() != nullptr;
-}
 
 // Scratch of the split-unit merge: two partial slots per CTA, each D / 4 float4 columns of 256 rows
 // plus the rows' log-sum-exps.

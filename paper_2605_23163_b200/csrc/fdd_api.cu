@@ -138,9 +138,10 @@ fdd_status fdd_create(const fdd_config* cfg, fdd_ctx** out) {
         e = cudaMalloc(&ctx->ws_attn, ctx->ws_attn_bytes);
     }
     if (e == cudaSuccess) {
-        // one counter per attention unit: (KV head, pair of 128-row tiles, rollout)
+        // one counter per attention unit: (KV head, pair of query tiles of 128 / G positions, rollout)
         const int G = cfg->n_q_heads / cfg->n_kv_heads;
-        const int row_pairs = (cfg->max_block * G + 255) / 256;
+        const int tile_pos = 128 / G;
+        const int row_pairs = ((cfg->max_block + tile_pos - 1) / tile_pos + 1) / 2;
         ctx->attn_max_units = cfg->n_kv_heads * row_pairs * cfg->max_forks;
         // two counters per unit: pieces written, CTAs done with their share of the merge
         e = cudaMalloc(&ctx->attn_unit_count, sizeof(int) * 2 * ctx->attn_max_units);
@@ -308,8 +309,8 @@ fdd_status fdd_block_attn_gated(fdd_ctx* ctx, fdd_forkset* const* sets, int n_se
     cudaStream_t st_ = static_cast<cudaStream_t>(stream);
     size_t q_off = 0, kv_off = 0;
     int fork_off = 0;
-    std::vector<AttnProblem> tc_probs;
-    std::vector<TcMapCache*> tc_caches;
+    std::vector<AttnProblem> probs;
+    std::vector<TcMapCache*> caches;
     for (int s = 0; s < n_sets; ++s) {
         fdd_forkset* fs = sets[s];
         AttnProblem p;
@@ -335,23 +336,15 @@ fdd_status fdd_block_attn_gated(fdd_ctx* ctx, fdd_forkset* const* sets, int n_se
         p.scale = scale;
         p.gate = gate ? gate + fork_off : nullptr;
         fork_off += fs->n_forks;
-        if (attention_tc_supported(p, c.head_dim)) {
-            // the tensor-core kernel takes many scenes per launch
-            tc_probs.push_back(p);
-            tc_caches.push_back(&fs->map_cache[layer]);
-        } else {
-            // the CUDA-core kernel covers the remaining shapes (GQA groups that are not a power of two)
-            cudaError_t e = launch_attention_simple(p, c.head_dim, st_);
-            ctx->launches += 1;
-            if (e != cudaSuccess) return cuda_fail(ctx, e, "fdd_block_attn launch");
-        }
+        probs.push_back(p);
+        caches.push_back(&fs->map_cache[layer]);
         q_off += static_cast<size_t>(fs->n_forks) * p.d * c.n_q_heads * c.head_dim;
         kv_off += static_cast<size_t>(fs->n_forks) * p.d * c.n_kv_heads * c.head_dim;
     }
-    for (size_t first = 0; first < tc_probs.size(); first += kTcMaxSets) {
-        const int n = static_cast<int>(std::min<size_t>(kTcMaxSets, tc_probs.size() - first));
+    for (size_t first = 0; first < probs.size(); first += kTcMaxSets) {   // many scenes per launch
+        const int n = static_cast<int>(std::min<size_t>(kTcMaxSets, probs.size() - first));
         int n_launches = 0;
-        cudaError_t e = launch_attention_ptc(ctx, tc_probs.data() + first, tc_caches.data() + first, n, c.head_dim, st_,
+        cudaError_t e = launch_attention_ptc(ctx, probs.data() + first, caches.data() + first, n, c.head_dim, st_,
                                              &n_launches);
         ctx->launches += n_launches;
         if (e != cudaSuccess) return cuda_fail(ctx, e, "fdd_block_attn launch");

@@ -169,8 +169,6 @@ static inline int unmask_items_per_row(int vocab, int tiles_per_item) {
 }
 size_t unmask_workspace_bytes(int vocab, int max_rows);
 
-cudaError_t launch_attention_simple(const AttnProblem& p, int head_dim, cudaStream_t st);
-bool attention_tc_supported(const AttnProblem& a, int head_dim);
 size_t attention_ptc_workspace_bytes(int head_dim, int max_ctas);
 cudaError_t launch_attention_ptc(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* const* caches, int n,
                                  int head_dim, cudaStream_t st, int* n_launches);

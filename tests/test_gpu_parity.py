@@ -411,6 +411,26 @@ def test_attention_group_of_three_uses_the_cuda_core_kernel():
     _attention_case(w)
 
 
+@pytest.mark.parametrize("group,dim,forks,block,prefix,page,blocks_before", [
+    (3, 128, 2, 43, 150, 0, 0),       # 42 positions a tile: the second tile holds one position
+    (5, 64, 1, 128, 2100, 0, 1),      # the longest block: six tiles, units cut into many pieces
+    (6, 128, 3, 21, 700, 64, 1),      # exactly one tile
+    (7, 128, 6, 27, 3001, 0, 0),      # units in two pieces and in more
+    (7, 128, 2, 19, 1, 0, 1),         # one key of prefix, the second tile holds one position
+    (15, 64, 2, 9, 333, 64, 0),       # 8 positions a tile, 120 rows
+    (12, 128, 1, 1, 0, 0, 0),         # a single key
+])
+@pytest.mark.parametrize("causal", [False, True])
+def test_attention_groups_that_are_not_a_power_of_two_keep_full_precision(group, dim, forks, block, prefix, page, blocks_before,
+                                                                           causal):
+    # both halves of every probability enter the product, so the rounding of the output to bf16 is all
+    # that is left: at most half an ulp, 2^-9 of each value (one bf16 half alone gives 2.3e-3)
+    sc = synth.Scene(prefix, forks, block, 0, blocks_before + 1)
+    w = synth.Workload(f"g{group}", 2 * group, 2, dim, 512, "bf16", "peaked", 0.9, 1.0, (sc,), page_tokens=page, seed=60 + group)
+    _, rel_l2 = _attention_case(w, n_blocks_before=blocks_before, causal=causal)
+    assert rel_l2 <= 2.0 ** -9 + 1e-5
+
+
 def test_more_scenes_and_rows_than_one_launch_takes():
     # 18 scenes (more than the 16 of one attention / unmask launch) and, separately, three sets of
     # 4096 rows each (more than the 8192 rows of one unmask launch): the calls split the work
