@@ -697,6 +697,29 @@ def test_unmask_noise_decides_on_flat_and_equal_rows(recipe, dtype, vocab, tempe
             assert len(set(got["tokens"][masked].tolist())) >= 8        # the winners are spread over the vocabulary
 
 
+@pytest.mark.parametrize("dtype,vocab,offset", [
+    ("bf16", 50257, 0), ("bf16", 4096, 3), ("bf16", 2047, 7), ("bf16", 2049, 1), ("bf16", 63, 5), ("bf16", 3, 1),
+    ("f32", 4099, 0), ("f32", 8192, 1), ("f32", 2050, 3), ("f32", 65, 2), ("f32", 2, 1)])
+@pytest.mark.parametrize("temperature", [0.0, 0.8])
+def test_unmask_rows_that_start_anywhere(dtype, vocab, offset, temperature, monkeypatch):
+    # a row pitch or a base that is not a multiple of 16 bytes: what lies around the logits must not
+    # enter (it would win every arg-max), nor a row's neighbours
+    sc = synth.Scene(prefix_len=16, n_forks=3, block_len=9, n_scaffold=0, n_blocks=1)
+    w = synth.Workload("ragged", 4, 1, 64, vocab, dtype, "normal_sigma2" if dtype == "f32" else "peaked", 0.4, temperature, (sc,),
+                       seed=70 + vocab)
+
+    def placed(w, arr, device="cuda", plain=harness.logits_tensor):
+        t = plain(w, arr, device)
+        buf = torch.full((t.numel() + 32,), 1e30, dtype=t.dtype, device=device)
+        buf[offset:offset + t.numel()] = t.reshape(-1)
+        return buf[offset:offset + t.numel()]
+
+    monkeypatch.setattr(harness, "logits_tensor", placed)
+    for step in (0, 2):
+        info, got, ref = _unmask_step_case(w, step=step)
+        assert info["rows"] == 3 * 9
+
+
 def test_unmask_threshold_extremes():
     w = synth.small_variant(synth.workload("tts"), prefix_len=64, vocab=4096, n_forks=2, n_blocks=1)
     info, got, ref = _unmask_step_case(w, threshold=1.5)          # nothing passes: one commit each
