@@ -15,6 +15,21 @@
 // written (the launch is cooperative, so the CTAs it waits for are running; the wait is bounded)
 // and merges an equal share of the unit's rows into the bf16 output.
 //
+// Fewer units than CTAs (BYUNIT).  Equal ranges then give most CTAs the end of one unit and the start of the
+// next: two pieces to write and two merges to wait for, which take longer than the two or three tile steps
+// between them.  Instead every unit is cut into equal pieces of its own, one per CTA, with the fewest
+// steps per piece that fit on the SMs; where even single query tiles leave SMs idle, a unit is one
+// query tile and a piece one step.  Equal ranges remain where the pieces would be over kUnitSlack steps
+// longer than an equal share.  Units of at most kWholeTiles steps are not cut at all: publishing a piece
+// and merging takes 8 us, as long as they do (stamps at 16 / 2 heads, prefix 4096, one rollout: 1.0 us to the
+// layout, 3.4 to the first scores, 1.6 for the one tile step, 1.5 to write the piece, 0.5 for the fence,
+// 1.5 until the last piece is seen, 4 for the merge).  Measured, launches one behind the other (equal ranges ->
+// pieces by unit): one rollout, prefix 4096: 24.6 -> 18.5-20 us; eight rollouts: 33-36 -> 27-29 us; 28 / 4
+// heads, six rollouts, prefix 3001: 41 -> 35 us; a block of 36 layers with eight rollouts: 6.3 -> 5.3 ms.
+// These launches also set themselves up ahead of the wait for the kernel before them and keep the scenes'
+// sizes in shared memory; a launch with more units than CTAs lost 2-3 % by the same (a block at 32 rollouts,
+// prefix 16384: 1815-1850 us against 1770-1790), so it does neither.
+//
 // Warp roles (384 threads): warps 0-3 and 4-7 are the two soft-max groups (thread = one query
 // row = one TMEM lane), warp 8 lane 0 drives TMA, warps 9 and 10 issue the tcgen05.mma (one lane each:
 // warp 9 the score products, warp 10 the output products), warp
@@ -64,7 +79,10 @@ constexpr int kTcThreads = 384;
 constexpr int kKeysPerTile = 128;
 constexpr long long kWaitLimit = 4000000000LL;   // about two seconds of SM clocks
 constexpr int kMaxGatedForks = kAttnMaxGatedForks;   // rollouts of one launch when any scene has a gate
-constexpr int kMinTilesPerCta = 3;               // do not cut the work finer than this (every cut costs a piece to write and merge)
+constexpr int kMinTilesPerCta = 3;               // do not cut equal ranges finer than this (every cut costs a piece to write and merge)
+constexpr int kUnitSlack = 4;                    // tile steps by which the longest piece of a unit may exceed an equal share
+constexpr int kWholeTiles = 6;                   // units up to this long are not cut
+constexpr int kSingleSteps = 1;                  // units of one query tile while no CTA gets more than this many steps of them
 // Registers per thread after the hand-over.  The CTA starts with 384 x 168; 8 soft-max warps x
 // kRegsSoftmax + 4 other warps x kRegsOther must not exceed that (2 * 208 + 88 = 3 * 168).
 constexpr int kRegsSoftmax = 208;
@@ -76,13 +94,12 @@ struct SetParams {
     const int32_t* page_table;
     const int32_t* gate;       // per rollout, 0 = skip it; nullptr = every rollout takes part
     int fork_base;             // rollouts of the scenes before this one (index into the kernel's list)
-    int units_per_fork;        // Hkv * row_pairs
+    int n_kv_heads;
     int n_forks, d, n_q_heads, G;
     int tile_pos, tile_rows;   // block positions of one query tile (128 / G) and the rows they make (tile_pos * G)
     int q_tiles;               // query tiles of a (rollout, KV head)
     int prefix_len, page_tokens, n_phys_pages, suffix_len;
     int tiles_prefix, tiles_suffix, tiles_total;
-    int row_pairs;
     int causal;
 };
 
@@ -96,6 +113,7 @@ struct TcArgs {
     int max_units;
     int* status;
     int min_tiles;             // do not cut the work into ranges shorter than this
+    int min_piece;             // nor a unit into pieces shorter than this
     int n_sets;
     float scale_log2;
     long long merge_wait_limit; // SM clocks a CTA waits for the other pieces of a cut unit before it gives up
@@ -176,14 +194,15 @@ struct Item {
 
 // step_base[s]: first global tile step of scene s (scenes laid end to end, skipped rollouts left out)
 template <int MAXSETS>
-__device__ __forceinline__ Item locate(const TcArgs<MAXSETS>& a, const long long* step_base, long long pos, long long end) {
+__device__ __forceinline__ Item locate(const TcArgs<MAXSETS>& a, const SetParams* sets, const long long* step_base, long long pos, long long end) {
     Item it;
     int s = 0;
     while (s + 1 < a.n_sets && pos >= step_base[s + 1]) ++s;
-    const SetParams& p = a.sets[s];
+    const SetParams& p = sets[s];
     const long long rel = pos - step_base[s];
     it.s = s;
-    it.unit = static_cast<int>(rel / p.tiles_total);
+    it.unit = rel <= 0xFFFFFFFFLL ? static_cast<int>(static_cast<uint32_t>(rel) / static_cast<uint32_t>(p.tiles_total))
+                                  : static_cast<int>(rel / p.tiles_total);
     it.t0 = static_cast<int>(rel - static_cast<long long>(it.unit) * p.tiles_total);
     it.unit_begin = pos - it.t0;
     const long long left = end - pos;
@@ -203,7 +222,7 @@ constexpr float kRoundMagic = 12582912.0f;                    // 1.5 * 2^23: add
 
 // Merge of a unit cut between CTAs:  out = sum_k w_k O_k / sum_k w_k,  w_k = 2^(lse_k - M), M = max_k lse_k.
 // Every CTA that holds a piece merges an equal share of the unit's rows.  A thread takes CT float4
-// columns of one row: 32 / CT pieces are read per round trip, 32 independent 16-byte reads (and the
+// columns of one row: 40 / CT pieces are read per round trip, 40 independent 16-byte reads (and the
 // pieces' log-sum-exps) in flight.  M is not known in advance: the sums are kept relative to the
 // largest log-sum-exp seen so far and rescaled when a chunk raises it, so the pieces are read once.
 // Partials lie column-major in their slots ([D / 4][256 rows] float4).
@@ -211,7 +230,7 @@ template <int D, int CT>
 __device__ __forceinline__ void merge_columns(const float* part_o, const float* part_lse, const int* slot_s, int n_pieces,
                                               int row, int col0, __nv_bfloat16* op) {
     constexpr int NC4 = D / 4;
-    constexpr int PC = 32 / CT;                     // pieces per chunk
+    constexpr int PC = CT == 1 ? 36 : 40 / CT;      // pieces per chunk (as many as the registers hold)
     const float4* po4 = reinterpret_cast<const float4*>(part_o);
     float4 acc[CT];
 #pragma unroll
@@ -261,11 +280,82 @@ __device__ __forceinline__ void merge_columns(const float* part_o, const float* 
 
 // A unit whose merge this CTA takes part in once its range is done.
 struct Deferred {
-    int s, unit, f, rp, h, c_first, n_pieces, gu;
+    int s, unit, f, tile0, h, c_first, n_pieces, gu;   // tile0: the unit's first query tile
     long long unit_begin;
 };
 
-template <int D, int MAXSETS, int EMU, int MODE>
+// How the tile steps of a launch are handed out (see the top of the file); every CTA derives the same.
+struct Layout {
+    long long T;               // tile steps
+    int ctas;                  // CTAs that take part
+    int per_unit;              // query tiles of a unit: 2, or 1 where that gives every tile step a CTA of its own
+    int by_unit;               // > 0: every unit is cut into equal pieces of at most this many steps; 0: equal ranges
+};
+
+// The layout of a launch: one warp, lane s looks after scene s (n_sets <= 16).
+template <int MAXSETS, bool BYUNIT>
+__device__ __forceinline__ void plan(const TcArgs<MAXSETS>& a, const SetParams* sets, const int* n_act, long long* step_base,
+                                     int* unit_base, int* cta_base, int* pieces, Layout* out, int lane) {
+    const unsigned full = 0xFFFFFFFFu;
+    const bool mine = lane < a.n_sets;
+    const int tiles = mine ? sets[lane].tiles_total : 1;
+    const int q_tiles = mine ? sets[lane].q_tiles : 0;
+    const int heads_forks = mine ? sets[lane].n_kv_heads * n_act[lane] : 0;
+    auto sum = [&](long long v) {
+        if (MAXSETS == 1) return __shfl_sync(full, v, 0);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(full, v, off);
+        return v;
+    };
+    auto before = [&](long long v) {                    // sum over the lanes below this one
+        long long incl = v;
+#pragma unroll
+        for (int off = 1; off < MAXSETS; off <<= 1) {
+            const long long up = __shfl_up_sync(full, incl, off);
+            if (lane >= off) incl += up;
+        }
+        return incl - v;
+    };
+    const int grid = static_cast<int>(gridDim.x);
+    Layout l;
+    l.per_unit = 1;
+    long long units = static_cast<long long>(heads_forks) * q_tiles;
+    l.T = sum(units * tiles);
+    if (!BYUNIT || l.T > grid * kSingleSteps) {
+        l.per_unit = 2;
+        units = static_cast<long long>(heads_forks) * ((q_tiles + 1) / 2);
+        l.T = sum(units * tiles);
+    }
+    const long long U = sum(units);
+    int n = 1;                                          // pieces of a unit of this lane's scene
+    l.by_unit = 0;
+    l.ctas = static_cast<int>(max(1LL, min(static_cast<long long>(grid), l.T / a.min_tiles)));
+    if (BYUNIT && l.T > 0 && U <= grid) {
+        const int even = max(a.min_piece, static_cast<int>((l.T + grid - 1) / grid));
+        for (int c = even; c <= even + kUnitSlack; ++c) {
+            n = tiles <= kWholeTiles ? 1 : (tiles + c - 1) / c;
+            const long long need = sum(units * n);
+            if (need <= grid) {
+                l.by_unit = c;
+                l.ctas = static_cast<int>(need);
+                break;
+            }
+        }
+    }
+    const long long steps_before = before(units * tiles), units_before = before(units), ctas_before = before(units * n);
+    if (mine) {
+        step_base[lane] = steps_before;
+        unit_base[lane] = static_cast<int>(units_before);
+        cta_base[lane] = static_cast<int>(ctas_before);  // (only used by unit, where it is below the grid's size)
+        pieces[lane] = n;
+    }
+    if (lane == 0) {
+        step_base[a.n_sets] = l.T;
+        *out = l;
+    }
+}
+
+template <int D, int MAXSETS, int EMU, int MODE, bool BYUNIT>
 __global__ void __launch_bounds__(kTcThreads, 1)
 attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
     using Shape = TcShape<D>;
@@ -291,19 +381,61 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
     // The rollouts that take part (gate != 0), scene after scene, and the layout of the work that
     // follows from them.  Every CTA derives the same lists from the same gate values.
     __shared__ unsigned short fork_s[kMaxGatedForks];
-    __shared__ int n_act_s[MAXSETS], unit_base_s[MAXSETS];
+    __shared__ int n_act_s[MAXSETS], unit_base_s[MAXSETS], cta_base_s[MAXSETS], pieces_s[MAXSETS];
     __shared__ long long step_base_s[MAXSETS + 1];
+    __shared__ Layout layout_s;
+    __shared__ SetParams sets_s[BYUNIT ? MAXSETS : 1];
+    const SetParams* const sets = BYUNIT ? sets_s : a.sets;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // A kernel launched behind this one for an early start (the unmasking step's streaming kernel)
     // may be made resident on SMs as their CTA of this launch exits; it waits for the whole of this
     // launch before it reads anything.
     tc::grid_launch_dependents();
-    // (and this launch may itself have started early: the gate below is written by the kernel ahead of it)
+    // This launch may itself have started early: what does not depend on the kernel ahead of it (barriers,
+    // TMEM, the tensor maps, the scenes' sizes) is set up while that one drains; the gate below is written
+    // by it.
+    auto set_up = [&]() {
+        if (tid == 0) {
+            abort_s = 0;
+            n_deferred_s = 0;
+            tc::mbar_init(tc::smem_u32(&bar_q_full), 1);
+            tc::mbar_init(tc::smem_u32(&bar_q_empty), kOwn ? 2 : 1);      // every QK^T product of an item has completed: Q may be overwritten
+            for (int s = 0; s < kStages; ++s) {
+                tc::mbar_init(tc::smem_u32(&bar_k_full[s]), 1);
+                tc::mbar_init(tc::smem_u32(&bar_k_empty[s]), kOwn ? 2 : 1);
+                tc::mbar_init(tc::smem_u32(&bar_v_full[s]), 1);
+                tc::mbar_init(tc::smem_u32(&bar_v_empty[s]), kOwn ? 2 : 1);
+            }
+            for (int q = 0; q < 2; ++q) {
+                tc::mbar_init(tc::smem_u32(&bar_s_full[q]), 1);     // scores of query tile q are in S
+                tc::mbar_init(tc::smem_u32(&bar_s_free[q]), 128);   // group q has copied them out of S
+                tc::mbar_init(tc::smem_u32(&bar_p_full[q]), 128);   // group q has written P[q]
+                tc::mbar_init(tc::smem_u32(&bar_o_done[q]), 1);     // a PV product of query tile q has completed
+                tc::mbar_init(tc::smem_u32(&bar_o_final[q]), 1);    // the last PV product of query tile q in an item has completed
+            }
+            tc::fence_barrier_init();
+        }
+        if (warp == 9) {
+            tc::tmem_alloc(tc::smem_u32(&tmem_base_s), 512);
+            tc::tmem_relinquish();
+        }
+    };
+    if (BYUNIT) {
+        for (int i = tid; i < a.n_sets * static_cast<int>(sizeof(SetParams) / 4); i += kTcThreads)
+            reinterpret_cast<uint32_t*>(sets_s)[i] = reinterpret_cast<const uint32_t*>(a.sets)[i];
+        set_up();
+        if (warp == 8 && lane < a.n_sets) {
+            tc::prefetch_tmap(&a.maps[lane].q);
+            tc::prefetch_tmap(&a.maps[lane].pk);
+            tc::prefetch_tmap(&a.maps[lane].pv);
+        }
+        __syncthreads();
+    }
     tc::grid_dependency_wait();
 
     for (int s = warp; s < a.n_sets; s += kTcThreads / 32) {
-        const SetParams& p = a.sets[s];
+        const SetParams& p = sets[s];
         int cnt = p.n_forks;
         if (p.gate != nullptr) {
             cnt = 0;
@@ -318,54 +450,41 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
         if (lane == 0) n_act_s[s] = cnt;
     }
     __syncthreads();
-    if (tid == 0) {
-        long long steps = 0;
-        int units = 0;
-        for (int s = 0; s < a.n_sets; ++s) {
-            step_base_s[s] = steps;
-            unit_base_s[s] = units;
-            const int u = a.sets[s].units_per_fork * n_act_s[s];
-            steps += static_cast<long long>(u) * a.sets[s].tiles_total;
-            units += u;
-        }
-        step_base_s[a.n_sets] = steps;
-    }
+    if (warp == 0) plan<MAXSETS, BYUNIT>(a, sets, n_act_s, step_base_s, unit_base_s, cta_base_s, pieces_s, &layout_s, lane);
+    if (BYUNIT) tc::fence_before_sync();
     __syncthreads();
-    const long long T = step_base_s[a.n_sets];
-    const long long C = max(1LL, min(static_cast<long long>(gridDim.x), T / a.min_tiles));
-    if (T == 0 || blockIdx.x >= C) return;          // nothing (left) to do: before any barrier or TMEM exists
-    const long long range_begin = T * blockIdx.x / C;
-    const long long range_end = T * (blockIdx.x + 1) / C;
+    if (BYUNIT) tc::fence_after_sync();
+    const Layout lay = layout_s;
+    const int per_unit = BYUNIT ? lay.per_unit : 2;
+    const bool by_unit = BYUNIT && lay.by_unit > 0;
+    const long long T = lay.T;
+    const long long C = lay.ctas;
+    if (T == 0 || blockIdx.x >= C) {                // nothing (left) to do
+        if (BYUNIT && warp == 9) tc::tmem_dealloc(tmem_base_s, 512);
+        return;
+    }
+    if (!BYUNIT) {
+        set_up();
+        tc::fence_before_sync();
+        __syncthreads();
+        tc::fence_after_sync();
+    }
+    long long range_begin, range_end;
+    if (by_unit) {
+        int s = 0;
+        while (s + 1 < a.n_sets && static_cast<int>(blockIdx.x) >= cta_base_s[s + 1]) ++s;
+        const int rel = static_cast<int>(blockIdx.x) - cta_base_s[s], unit = rel / pieces_s[s], piece = rel - unit * pieces_s[s];
+        const int tiles = sets[s].tiles_total;
+        const long long unit_begin = step_base_s[s] + static_cast<long long>(unit) * tiles;
+        range_begin = unit_begin + tiles * piece / pieces_s[s];
+        range_end = unit_begin + tiles * (piece + 1) / pieces_s[s];
+    } else {
+        range_begin = T * blockIdx.x / C;
+        range_end = T * (blockIdx.x + 1) / C;
+    }
 
-    if (tid == 0) {
-        abort_s = 0;
-        n_deferred_s = 0;
-        tc::mbar_init(tc::smem_u32(&bar_q_full), 1);
-        tc::mbar_init(tc::smem_u32(&bar_q_empty), kOwn ? 2 : 1);      // every QK^T product of an item has completed: Q may be overwritten
-        for (int s = 0; s < kStages; ++s) {
-            tc::mbar_init(tc::smem_u32(&bar_k_full[s]), 1);
-            tc::mbar_init(tc::smem_u32(&bar_k_empty[s]), kOwn ? 2 : 1);
-            tc::mbar_init(tc::smem_u32(&bar_v_full[s]), 1);
-            tc::mbar_init(tc::smem_u32(&bar_v_empty[s]), kOwn ? 2 : 1);
-        }
-        for (int q = 0; q < 2; ++q) {
-            tc::mbar_init(tc::smem_u32(&bar_s_full[q]), 1);     // scores of query tile q are in S
-            tc::mbar_init(tc::smem_u32(&bar_s_free[q]), 128);   // group q has copied them out of S
-            tc::mbar_init(tc::smem_u32(&bar_p_full[q]), 128);   // group q has written P[q]
-            tc::mbar_init(tc::smem_u32(&bar_o_done[q]), 1);     // a PV product of query tile q has completed
-            tc::mbar_init(tc::smem_u32(&bar_o_final[q]), 1);    // the last PV product of query tile q in an item has completed
-        }
-        tc::fence_barrier_init();
-    }
-    if (warp == 9) {
-        tc::tmem_alloc(tc::smem_u32(&tmem_base_s), 512);
-        tc::tmem_relinquish();
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
     const uint32_t tmem = tmem_base_s;
-    const uint32_t tm_s[2] = {tmem, kOwn ? tmem + 128 : tmem};
+    const uint32_t tm_s = tmem;                         // (+ 128 q where every query tile has its own scores)
     const uint32_t tm_p[2] = {kOwn ? tmem : tmem + 128, kOwn ? tmem + 128 : tmem + 192};
     const uint32_t tm_o[2] = {tmem + 256, tmem + 256 + D};
 
@@ -376,20 +495,21 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
     // first P of the next item (written after its epilogue) is what lets the PV issuer overwrite O.
     struct ItemView {
         Item it;
-        int f, rp, h, nt, NQ;
+        int f, tile0, h, nt, NQ;
     };
     auto view_item = [&](long long pos) {
         ItemView v;
-        v.it = locate(a, step_base_s, pos, range_end);
-        const SetParams& p = a.sets[v.it.s];
+        v.it = locate(a, sets, step_base_s, pos, range_end);
+        const SetParams& p = sets[v.it.s];
         int idx = v.it.unit;
         const int n_act = n_act_s[v.it.s];
         v.f = idx % n_act; idx /= n_act;
         if (p.gate != nullptr) v.f = fork_s[p.fork_base + v.f];
-        v.rp = idx % p.row_pairs; idx /= p.row_pairs;
-        v.h = idx;
+        const int per_head = per_unit == 2 ? (p.q_tiles + 1) / 2 : p.q_tiles;
+        v.h = idx / per_head;
+        v.tile0 = (idx - v.h * per_head) * per_unit;
         v.nt = v.it.t1 - v.it.t0;
-        v.NQ = min(2, p.q_tiles - v.rp * 2);
+        v.NQ = min(per_unit, p.q_tiles - v.tile0);
         return v;
     };
 
@@ -406,7 +526,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                 const ItemView v = view_item(pos);
                 {
                     // warp-uniform loop, one elected lane issues the copies
-                    const SetParams& p = a.sets[v.it.s];
+                    const SetParams& p = sets[v.it.s];
                     const TcSetMaps& maps = a.maps[v.it.s];
                     const uint32_t bq = tc::smem_u32(&bar_q_full);
                     if (item_cnt > 0) {
@@ -415,12 +535,11 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                         ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
                     }
                     if (ok && tc::elect_one()) {
-                        tc::prefetch_tmap(&maps.q);
                         tc::mbar_arrive_expect_tx(bq, v.NQ * Shape::kChunks * p.tile_rows * 128);
                         for (int q = 0; q < v.NQ; ++q)
                             for (int ch = 0; ch < Shape::kChunks; ++ch)
                                 tc::tma_load_4d(q_s + q * Shape::kTileBytes + ch * Shape::kChunkBytes, &maps.q, bq, ch * 64,
-                                                v.h * p.G, (v.rp * 2 + q) * p.tile_pos, v.f);
+                                                v.h * p.G, (v.tile0 + q) * p.tile_pos, v.f);
                     }
                     __syncwarp();
                     for (int jl = 0; jl < v.nt && ok; ++jl) {
@@ -507,8 +626,8 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
 #pragma unroll
                         for (int k = 0; k < D / 16; ++k) {
                             const uint32_t off = ((k >> 2) * Shape::kChunkBytes + (k & 3) * 32) >> 4;
-                            if (k == 0) tc::mma_ss_first(tm_s[q], dq + off, dk + off, kIdescQK);
-                            else tc::mma_ss_acc(tm_s[q], dq + off, dk + off, kIdescQK);
+                            if (k == 0) tc::mma_ss_first(tm_s + (kOwn ? q * 128 : 0), dq + off, dk + off, kIdescQK);
+                            else tc::mma_ss_acc(tm_s + (kOwn ? q * 128 : 0), dq + off, dk + off, kIdescQK);
                         }
                     };
                     // O[q] (+)= P[q] . V
@@ -667,10 +786,10 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
             const ItemView v = view_item(pos);
             const Item& it = v.it;
             const SetParams& p = a.sets[it.s];
-            const int f = v.f, rp = v.rp, h = v.h, nt = v.nt;
+            const int f = v.f, h = v.h, nt = v.nt;
             const bool active = q < v.NQ;
             const int pos_in_tile = row_local / p.G;
-            int qi = (rp * 2 + q) * p.tile_pos + pos_in_tile;   // block position of this row
+            int qi = (v.tile0 + q) * p.tile_pos + pos_in_tile;   // block position of this row
             const bool row_ok = row_local < p.tile_rows && qi < p.d;
             if (!row_ok) qi = 0;
             const int qg = row_ok ? row_local - pos_in_tile * p.G : 0;
@@ -689,7 +808,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                     tc::fence_after_sync();
                     uint32_t sr[128];
 #pragma unroll
-                    for (int cc = 0; cc < 4; ++cc) tc::tmem_ld32(tm_s[q] + lane_base + cc * 32, sr + cc * 32);
+                    for (int cc = 0; cc < 4; ++cc) tc::tmem_ld32(tm_s + (kOwn ? q * 128 : 0) + lane_base + cc * 32, sr + cc * 32);
                     tc::wait_ld();
                     if (!kOwn) {
                         tc::fence_before_sync();
@@ -829,10 +948,19 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
             }
 
             // ---------------------------------------------------------------- epilogue
-            const long long unit_end = it.unit_begin + p.tiles_total;
-            const int c_first = static_cast<int>(((it.unit_begin + 1) * C + T - 1) / T) - 1;   // CTA of the unit's first step
-            const int c_last = static_cast<int>((unit_end * C + T - 1) / T) - 1;                // CTA of its last step
-            const int n_pieces = c_last - c_first + 1;
+            int c_first, n_pieces;                              // CTA of the unit's first step, CTAs that hold a piece of it
+            if (by_unit) {
+                n_pieces = pieces_s[it.s];
+                c_first = cta_base_s[it.s] + it.unit * n_pieces;
+            } else {
+                const long long unit_end = it.unit_begin + p.tiles_total;
+                c_first = static_cast<int>(((it.unit_begin + 1) * C + T - 1) / T) - 1;
+                n_pieces = static_cast<int>((unit_end * C + T - 1) / T) - c_first;
+            }
+            // the scratch slot of the unit's piece in CTA c: 0 if the CTA's range starts inside the unit
+            auto slot_of = [&](int c, long long unit_begin) {
+                return c * 2 + (by_unit || unit_begin <= T * c / C ? 0 : 1);
+            };
             const float inv = l > 0.0f ? 1.0f / l : 0.0f;
             if (n_pieces == 1) {
                 if (active && ok) {
@@ -875,7 +1003,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                         // count, ahead of the barrier behind which the others read the piece
                         if (there) __threadfence();
                         last_s = there;
-                        slot_s[0] = c_first * 2 + (it.unit_begin <= T * c_first / C ? 0 : 1);
+                        slot_s[0] = slot_of(c_first, it.unit_begin);
                         slot_s[1] = (c_first + 1) * 2;           // the second piece starts its CTA's range
                     }
                     tc::named_barrier(1, 256);
@@ -959,7 +1087,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                             __threadfence();
                         }
                         last_s = last;
-                        slot_s[0] = c_first * 2 + (it.unit_begin <= T * c_first / C ? 0 : 1);
+                        slot_s[0] = slot_of(c_first, it.unit_begin);
                         slot_s[1] = (c_first + 1) * 2;           // the second piece starts its CTA's range
                     }
                     tc::named_barrier(1, 256);
@@ -980,7 +1108,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                     __threadfence();
                     atomicAdd(a.unit_count + gu, 1);
                     Deferred& dfr = deferred_s[n_deferred_s++];
-                    dfr.s = it.s; dfr.unit = it.unit; dfr.f = f; dfr.rp = rp; dfr.h = h;
+                    dfr.s = it.s; dfr.unit = it.unit; dfr.f = f; dfr.tile0 = v.tile0; dfr.h = h;
                     dfr.c_first = c_first; dfr.n_pieces = n_pieces; dfr.gu = gu;
                     dfr.unit_begin = it.unit_begin;
                 }
@@ -1005,6 +1133,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
         tc::named_barrier(1, 256);
         const int n_deferred = *abort_flag ? 0 : n_deferred_s;
         if (n_deferred > 0) {
+            int seen[2] = {0, 0};                                     // (thread 0) CTAs that saw the unit complete before this one
             if (tid == 0) {
                 const long long t0 = clock64();
                 for (int e = 0; e < n_deferred; ++e) {
@@ -1016,36 +1145,39 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                             break;
                         }
                     }
+                    // nobody looks at the unit's count any more once every holder of a piece has seen it complete
+                    seen[e] = atomicAdd(a.unit_count + a.max_units + deferred_s[e].gu, 1);
                 }
                 __threadfence();                                      // the pieces were published before their counts
             }
             for (int e = 0; e < n_deferred; ++e)
                 if (tid < deferred_s[e].n_pieces && tid < kMaxPieces) {
                     const int pc = deferred_s[e].c_first + tid;
-                    slot2_s[e][tid] = pc * 2 + (deferred_s[e].unit_begin <= T * pc / C ? 0 : 1);
+                    slot2_s[e][tid] = pc * 2 + (by_unit || deferred_s[e].unit_begin <= T * pc / C ? 0 : 1);
                 }
             tc::named_barrier(1, 256);
             if (*abort_flag == 0) {
                 const int threads_e = 256 / n_deferred;               // threads per unit
                 const int e = tid / threads_e, lt = tid - e * threads_e;
                 const Deferred dfr = deferred_s[e];
-                const SetParams& p = a.sets[dfr.s];
+                const SetParams& p = sets[dfr.s];
                 const int n_pieces = dfr.n_pieces;
                 const int* slots = slot2_s[e];
                 // this CTA's share of the rows; a row is split between `col_groups` threads
-                const int rows_here = min(2 * p.tile_rows, p.d * p.G - dfr.rp * 2 * p.tile_rows);
+                const int rows_here = min(per_unit * p.tile_rows, p.d * p.G - dfr.tile0 * p.tile_rows);
                 const int mine = static_cast<int>(blockIdx.x) - dfr.c_first;
                 const int row_lo = rows_here * mine / n_pieces, row_hi = rows_here * (mine + 1) / n_pieces;
                 const int share = row_hi - row_lo;                    // <= 86 (three pieces or more)
                 int col_groups = 1;                                   // a power of two, share * col_groups <= threads_e
                 while (col_groups < D / 4 && share * col_groups * 2 <= threads_e) col_groups *= 2;
                 const int ct = (D / 4) / col_groups;                  // float4 columns per thread
-                const int row_in_share = lt / col_groups, cg = lt - row_in_share * col_groups;
-                if (share > 0 && row_in_share < share) {
+                // (neighbouring lanes take neighbouring rows, whose partials lie side by side)
+                const int cg = share > 0 ? lt / share : col_groups, row_in_share = lt - cg * share;
+                if (cg < col_groups) {
                     const int rc = row_lo + row_in_share;             // row of the unit without the gap behind a tile's last row
                     const int rowu = rc < p.tile_rows ? rc : rc - p.tile_rows + 128;
                     const int pos2 = rc / p.G;
-                    const int qi2 = dfr.rp * 2 * p.tile_pos + pos2, qg2 = rc - pos2 * p.G;
+                    const int qi2 = dfr.tile0 * p.tile_pos + pos2, qg2 = rc - pos2 * p.G;
                     __nv_bfloat16* op = p.out + ((static_cast<size_t>(dfr.f) * p.d + qi2) * p.n_q_heads + dfr.h * p.G + qg2) * D;
                     const int col0 = cg * ct;
                     switch (ct) {
@@ -1057,16 +1189,13 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                         default: merge_columns<D, 32>(a.part_o, a.part_lse, slots, n_pieces, rowu, col0, op); break;
                     }
                 }
-                tc::named_barrier(1, 256);
-                if (tid < n_deferred) {
-                    // the last CTA to finish its share leaves both counters at zero for the next launch
-                    const Deferred& d2 = deferred_s[tid];
-                    int* done = a.unit_count + a.max_units + d2.gu;
-                    if (atomicAdd(done, 1) == d2.n_pieces - 1) {
-                        *done = 0;
-                        a.unit_count[d2.gu] = 0;
-                    }
-                }
+                if (tid == 0)
+                    // the last of them leaves both counters at zero for the next launch
+                    for (int e = 0; e < n_deferred; ++e)
+                        if (seen[e] == deferred_s[e].n_pieces - 1) {
+                            a.unit_count[deferred_s[e].gu] = 0;
+                            a.unit_count[a.max_units + deferred_s[e].gu] = 0;
+                        }
             }
         }
     }
@@ -1166,20 +1295,21 @@ int emulated_exponentials() {
     return value;
 }
 
-template <int D, int MAXSETS, int EMU, int MODE>
-cudaError_t launch_one(const TcArgs<MAXSETS>& args, unsigned ctas, int device, cudaStream_t st) {
+template <int D, int MAXSETS, int EMU, int MODE, bool BYUNIT>
+cudaError_t launch_one(const TcArgs<MAXSETS>& args, unsigned ctas, bool waits, int device, cudaStream_t st) {
     const int smem = TcShape<D>::kSmemBytes;
     // the kernel's shared-memory size is a per-device attribute: set on the first launch on each device
     constexpr int kMaxDevices = 64;
     static std::atomic<bool> configured[kMaxDevices];
     if (device < 0 || device >= kMaxDevices) return cudaErrorInvalidDevice;
     if (!configured[device].load(std::memory_order_acquire)) {
-        cudaError_t e = cudaFuncSetAttribute(attn_ptc_kernel<D, MAXSETS, EMU, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t e = cudaFuncSetAttribute(attn_ptc_kernel<D, MAXSETS, EMU, MODE, BYUNIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         configured[device].store(true, std::memory_order_release);
     }
-    // The CTAs wait for one another's pieces at the end: a cooperative launch makes the runtime
-    // guarantee that all of them are resident at once (or fail the launch).  The launch also asks for
+    // Where CTAs may wait for one another's pieces at the end (`waits`), a cooperative launch makes the runtime
+    // guarantee that all of them are resident at once (or fail the launch).  (It costs about a microsecond:
+    // a launch that cuts no unit goes without.)  The launch also asks for
     // an early start behind the kernel ahead of it on the stream (the kernel waits before it reads
     // anything); a runtime that does not take the two attributes together gets the first one alone.
     void* params[] = {const_cast<TcArgs<MAXSETS>*>(&args)};
@@ -1189,16 +1319,16 @@ cudaError_t launch_one(const TcArgs<MAXSETS>& args, unsigned ctas, int device, c
     cfg.blockDim = dim3(kTcThreads);
     cfg.dynamicSmemBytes = static_cast<size_t>(smem);
     cfg.stream = st;
+    const void* fn = reinterpret_cast<const void*>(&attn_ptc_kernel<D, MAXSETS, EMU, MODE, BYUNIT>);
     cudaLaunchAttribute attr[2];
+    cfg.attrs = attr;
+    if (!waits) {
+        cfg.numAttrs = overlap_launch_attribute(st, attr);
+        return cudaLaunchKernelExC(&cfg, fn, params);
+    }
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    const bool capturing = cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
-    const void* fn = reinterpret_cast<const void*>(&attn_ptc_kernel<D, MAXSETS, EMU, MODE>);
-    if (!capturing && !early_start_refused[device].load(std::memory_order_relaxed)) {
+    if (!early_start_refused[device].load(std::memory_order_relaxed) && overlap_launch_attribute(st, attr + 1) == 1) {
         cfg.numAttrs = 2;
         const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, params);
         if (e == cudaSuccess) return e;
@@ -1209,20 +1339,23 @@ cudaError_t launch_one(const TcArgs<MAXSETS>& args, unsigned ctas, int device, c
     return cudaLaunchKernelExC(&cfg, fn, params);
 }
 
-template <int MAXSETS>
-cudaError_t launch_emu(const TcArgs<MAXSETS>& args, int head_dim, unsigned ctas, int device, cudaStream_t st) {
+template <int MAXSETS, bool BYUNIT>
+cudaError_t launch_shape(const TcArgs<MAXSETS>& args, int head_dim, unsigned ctas, bool waits, int device, cudaStream_t st) {
     const int G = args.sets[0].G;                          // (the same for every scene of a context)
     if ((G & (G - 1)) != 0) {
         // Groups that are not a power of two keep 16 bits of every probability (see the top of the file).
-        if (head_dim == 64) return launch_one<64, MAXSETS, 0, kOwnScoresSplit>(args, ctas, device, st);
-        return launch_one<128, MAXSETS, 0, kOwnScoresSplit>(args, ctas, device, st);
+        if (head_dim == 64) return launch_one<64, MAXSETS, 0, kOwnScoresSplit, BYUNIT>(args, ctas, waits, device, st);
+        return launch_one<128, MAXSETS, 0, kOwnScoresSplit, BYUNIT>(args, ctas, waits, device, st);
     }
-    if (head_dim == 64) return launch_one<64, MAXSETS, 0, kSharedScores>(args, ctas, device, st);
-    switch (emulated_exponentials()) {
-        case 16: return launch_one<128, MAXSETS, 16, kSharedScores>(args, ctas, device, st);
-        case 32: return launch_one<128, MAXSETS, 32, kSharedScores>(args, ctas, device, st);
-        default: return launch_one<128, MAXSETS, 0, kSharedScores>(args, ctas, device, st);
+    if (head_dim == 64) return launch_one<64, MAXSETS, 0, kSharedScores, BYUNIT>(args, ctas, waits, device, st);
+    if (!BYUNIT) {
+        switch (emulated_exponentials()) {
+            case 16: return launch_one<128, MAXSETS, 16, kSharedScores, false>(args, ctas, waits, device, st);
+            case 32: return launch_one<128, MAXSETS, 32, kSharedScores, false>(args, ctas, waits, device, st);
+            default: break;
+        }
     }
+    return launch_one<128, MAXSETS, 0, kSharedScores, BYUNIT>(args, ctas, waits, device, st);
 }
 
 template <int MAXSETS>
@@ -1231,9 +1364,9 @@ cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* con
     // 1-20 KB, kept off the stack in the context's own buffer (a context is used by one host thread at a time)
     if (ctx->attn_args.size() * sizeof(uint64_t) < sizeof(TcArgs<MAXSETS>)) ctx->attn_args.resize((sizeof(TcArgs<MAXSETS>) + 7) / 8);
     TcArgs<MAXSETS>& args = *reinterpret_cast<TcArgs<MAXSETS>*>(ctx->attn_args.data());
-    long long steps = 0;
-    int units = 0, forks = 0;
-    bool gated = false;
+    long long pieces = 0;                                  // CTAs that the finest cut could occupy
+    int units = 0, pairs = 0, forks = 0;
+    bool gated = false, cut = false;
     for (int s = 0; s < n; ++s) {
         const AttnProblem& a = probs[s];
         const TcSetMaps* m = maps_for(a, head_dim, caches[s]);
@@ -1252,24 +1385,30 @@ cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* con
         p.tiles_prefix = (a.prefix_len + kKeysPerTile - 1) / kKeysPerTile;
         p.tiles_suffix = (a.suffix_len + kKeysPerTile - 1) / kKeysPerTile;
         p.tiles_total = p.tiles_prefix + p.tiles_suffix + (a.d + kKeysPerTile - 1) / kKeysPerTile;
-        p.row_pairs = (p.q_tiles + 1) / 2;
-        p.units_per_fork = a.n_kv_heads * p.row_pairs;
+        p.n_kv_heads = a.n_kv_heads;
         p.causal = a.causal_in_block;
         p.gate = a.gate;
         p.fork_base = forks;
         gated = gated || a.gate != nullptr;
         forks += a.n_forks;
-        steps += static_cast<long long>(p.units_per_fork) * a.n_forks * p.tiles_total;
-        units += p.units_per_fork * a.n_forks;
+        const int units_here = a.n_kv_heads * p.q_tiles * a.n_forks;
+        pieces += static_cast<long long>(units_here) * (p.tiles_total <= kWholeTiles ? 1 : p.tiles_total);
+        cut = cut || p.tiles_total > kWholeTiles;
+        units += units_here;
+        pairs += a.n_kv_heads * ((p.q_tiles + 1) / 2) * a.n_forks;
     }
     if (units > ctx->attn_max_units) return cudaErrorInvalidValue;
     if (gated && forks > kMaxGatedForks) return cudaErrorInvalidValue;
-    static int min_tiles = 0;
-    if (min_tiles == 0) {
-        min_tiles = kMinTilesPerCta;
-        if (const char* e = std::getenv("FDD_ATTN_MIN_TILES")) { const int v = std::atoi(e); if (v >= 1 && v <= 64) min_tiles = v; }
-    }
-    long long ctas = steps / min_tiles;
+    // FDD_ATTN_MIN_TILES overrides how finely the work is cut
+    static const int min_tiles = [] {
+        const char* e = std::getenv("FDD_ATTN_MIN_TILES");
+        const int v = e ? std::atoi(e) : 0;
+        return v >= 1 && v <= 64 ? v : 0;
+    }();
+    // one CTA per SM, fewer when there is not a piece for each
+    long long ctas = pieces;
+    // short units, each with a CTA of its own: none is cut, no CTA waits for another
+    const bool waits = cut || ctas > ctx->attn_max_ctas;
     if (ctas > ctx->attn_max_ctas) ctas = ctx->attn_max_ctas;
     if (ctas < 1) ctas = 1;
     args.part_o = static_cast<float*>(ctx->ws_attn);
@@ -1277,11 +1416,13 @@ cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* con
     args.unit_count = ctx->attn_unit_count;
     args.max_units = ctx->attn_max_units;
     args.status = ctx->d_status;
-    args.min_tiles = min_tiles;
+    args.min_tiles = min_tiles ? min_tiles : kMinTilesPerCta;
+    args.min_piece = min_tiles ? min_tiles : 1;
     args.n_sets = n;
     args.scale_log2 = probs[0].scale * 1.4426950408889634f;
     args.merge_wait_limit = ctx->attn_merge_wait_limit;
-    return launch_emu<MAXSETS>(args, head_dim, static_cast<unsigned>(ctas), ctx->device, st);
+    if (pairs <= ctx->attn_max_ctas) return launch_shape<MAXSETS, true>(args, head_dim, static_cast<unsigned>(ctas), waits, ctx->device, st);
+    return launch_shape<MAXSETS, false>(args, head_dim, static_cast<unsigned>(ctas), waits, ctx->device, st);
 }
 
 }  // namespace

@@ -138,11 +138,11 @@ fdd_status fdd_create(const fdd_config* cfg, fdd_ctx** out) {
         e = cudaMalloc(&ctx->ws_attn, ctx->ws_attn_bytes);
     }
     if (e == cudaSuccess) {
-        // one counter per attention unit: (KV head, pair of query tiles of 128 / G positions, rollout)
+        // one counter per attention unit: (KV head, query tile of 128 / G positions, rollout): a unit has one or two query tiles
         const int G = cfg->n_q_heads / cfg->n_kv_heads;
         const int tile_pos = 128 / G;
-        const int row_pairs = ((cfg->max_block + tile_pos - 1) / tile_pos + 1) / 2;
-        ctx->attn_max_units = cfg->n_kv_heads * row_pairs * cfg->max_forks;
+        const int q_tiles = (cfg->max_block + tile_pos - 1) / tile_pos;
+        ctx->attn_max_units = cfg->n_kv_heads * q_tiles * cfg->max_forks;
         // two counters per unit: pieces written, CTAs done with their share of the merge
         e = cudaMalloc(&ctx->attn_unit_count, sizeof(int) * 2 * ctx->attn_max_units);
         if (e == cudaSuccess) e = cudaMemset(ctx->attn_unit_count, 0, sizeof(int) * 2 * ctx->attn_max_units);

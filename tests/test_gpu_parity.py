@@ -431,6 +431,43 @@ def test_attention_groups_that_are_not_a_power_of_two_keep_full_precision(group,
     assert rel_l2 <= 2.0 ** -9 + 1e-5
 
 
+@pytest.mark.parametrize("hq,hkv,dim,prefix,forks,block,live", [
+    (8, 2, 128, 700, 3, 32, None),       # seven tiles: the shortest units that are cut, one query tile each
+    (8, 2, 128, 639, 3, 32, None),       # six tiles: the longest that are not
+    (8, 1, 128, 1500, 1, 3, None),       # more pieces than rows to share out
+    (32, 8, 128, 900, 8, 64, None),      # 64 units of a pair of query tiles, in two pieces each
+    (32, 8, 64, 1300, 18, 17, None),     # 144 units: one CTA each, four left over
+    (32, 8, 64, 1300, 12, 64, (0, 7)),   # few live rollouts of many
+    (16, 2, 128, 4096, 4, 36, (2,)),     # odd number of query tiles per rollout (3), units of one
+    (16, 2, 128, 2000, 8, 36, None),     # the same, units of two and one
+])
+def test_attention_units_cut_into_pieces_of_their_own(hq, hkv, dim, prefix, forks, block, live):
+    sc = synth.Scene(prefix, forks, block, 0, 1)
+    w = synth.Workload("units", hq, hkv, dim, 512, "bf16", "peaked", 0.9, 1.0, (sc,), seed=80 + prefix)
+    ctx = harness.create_context(w)
+    try:
+        scene = harness.GpuScene(ctx, w, 0)
+        pk, pv = synth.make_prefix(w, 0)
+        empty = ([np.zeros((0, hkv, dim), dtype=np.uint16)] * forks,) * 2
+        q, k, v = synth.make_qkv(w, 0, 0, 0, 0)
+        qd, kd, vd = harness.bf16_tensor(q), harness.bf16_tensor(k), harness.bf16_tensor(v)
+        on = list(range(forks)) if live is None else list(live)
+        gate = None
+        if live is not None:
+            gate = torch.zeros(forks, dtype=torch.int32, device="cuda")
+            gate[on] = 1
+        for _ in range(2):                   # (the second call finds the counters of the first)
+            out = torch.full_like(qd, float("nan"))
+            fdd.fdd_block_attn_gated(ctx, [scene.forkset], 0, qd, kd, vd, out, [block], 1.0 / np.sqrt(dim), 0, gate)
+            fdd.fdd_poll_status(ctx)
+            got = out.float().cpu().numpy().astype(np.float64).reshape(q.shape)
+            ref = pu.attention_oracle(w, (pk, pv), empty, q, k, v, forks=on)
+            pu.assert_attention_close(got[on], ref)
+            assert np.all(np.isnan(got[np.setdiff1d(np.arange(forks), on)]))
+    finally:
+        fdd.fdd_destroy(ctx)
+
+
 def test_more_scenes_and_rows_than_one_launch_takes():
     # 18 scenes (more than the 16 of one attention / unmask launch) and, separately, three sets of
     # 4096 rows each (more than the 8192 rows of one unmask launch): the calls split the work
