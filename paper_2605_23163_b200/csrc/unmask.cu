@@ -899,34 +899,58 @@ unmask_finalize_kernel(const UnmaskPartial* __restrict__ partial, int32_t* __res
 // every DRAFT row, the verifier's token (arg-max of its perturbed logits).  Going left to right, a
 // draft is accepted while it equals the verifier's token; at the first mismatch the verifier's token
 // replaces it and every later draft goes back to MASKED.
-__global__ void __launch_bounds__(128)
+// Bound by latencies: the records of the DRAFT rows (a dozen per row when few rollouts decode) are fetched by
+// groups of lanes in one round trip, as in unmask_finalize_kernel, and the kernel starts early behind
+// the streaming kernel.
+__global__ void __launch_bounds__(kFinalizeThreads)
 ss_accept_kernel(const UnmaskPartial* __restrict__ partial, int32_t* __restrict__ tokens,
                  uint8_t* __restrict__ state, int32_t* __restrict__ n_accepted, int32_t* __restrict__ n_left,
                  const __grid_constant__ UnmaskSets sets, int items_per_row) {
+    tc::grid_launch_dependents();
+    tc::grid_dependency_wait();                         // the streaming kernel's records are complete and visible
     const int fork = blockIdx.x;
-    const int i = threadIdx.x;
+    const int i = threadIdx.x, warp = i >> 5, lane = i & 31;
     int set = 0;
     while (set + 1 < sets.n_sets && fork >= sets.fork_off[set + 1]) ++set;
     const int d = sets.d[set];
-    const int row = sets.row_off[set] + (fork - sets.fork_off[set]) * d + i;
-    __shared__ int s_first_mismatch, s_accepted, s_masked;
-    if (i == 0) { s_first_mismatch = 0x7FFFFFFF; s_accepted = 0; s_masked = 0; }
+    const int row0 = sets.row_off[set] + (fork - sets.fork_off[set]) * d, row = row0 + i;
+    __shared__ int s_first_mismatch, s_accepted, s_masked, s_drafts, s_max_rec;
+    __shared__ int s_tok[128], s_nrec[128], s_rows[128];
+    if (i == 0) { s_first_mismatch = 0x7FFFFFFF; s_accepted = 0; s_masked = 0; s_drafts = 0; s_max_rec = 1; }
     __syncthreads();
-    int st = FDD_SCAFFOLD, tok = 0;
-    bool draft = false, mismatch = false;
-    if (i < d) {
-        st = state[row];
-        draft = st == FDD_DRAFT;
-        if (draft) {
-            const UnmaskPartial* p = partial + static_cast<size_t>(row) * items_per_row;
-            const int n_rec = p[0].pad[0];
-            Best B{-CUDART_INF_F, -CUDART_INF_F, 0x7FFFFFFF};
-            for (int c = 0; c < n_rec; ++c) B = better(B, Best{p[c].best_score, p[c].best_logit, p[c].best_index});
-            tok = B.index;
-            mismatch = tok != tokens[row];
-            if (mismatch) atomicMin(&s_first_mismatch, i);
-        }
+    const int st = i < d ? state[row] : FDD_SCAFFOLD;
+    const bool draft = st == FDD_DRAFT;
+    if (draft) {
+        const int n_rec = max(1, min(items_per_row, partial[static_cast<size_t>(row) * items_per_row].pad[0]));
+        s_nrec[i] = n_rec;
+        s_rows[atomicAdd(&s_drafts, 1)] = i;
+        atomicMax(&s_max_rec, n_rec);
     }
+    __syncthreads();
+    const int n_drafts = s_drafts;
+    int w = 1;
+    while (w < s_max_rec && w < 32) w <<= 1;
+    const int per = 32 / w, sub = lane / w, sl = lane - sub * w;
+    for (int base = warp * per; base < n_drafts; base += (kFinalizeThreads / 32) * per) {   // (warp-uniform bounds)
+        const int k = base + sub;
+        const bool valid = k < n_drafts;
+        const int j = valid ? s_rows[k] : 0;
+        const int nr = valid ? s_nrec[j] : 0;
+        const UnmaskPartial* p = partial + static_cast<size_t>(row0 + j) * items_per_row;
+        Best B{-CUDART_INF_F, -CUDART_INF_F, 0x7FFFFFFF};
+        for (int c = sl; c < nr; c += w) B = better(B, Best{p[c].best_score, p[c].best_logit, p[c].best_index});
+        for (int off = w >> 1; off > 0; off >>= 1) {
+            Best o;
+            o.score = __shfl_xor_sync(0xFFFFFFFFu, B.score, off);
+            o.logit = __shfl_xor_sync(0xFFFFFFFFu, B.logit, off);
+            o.index = __shfl_xor_sync(0xFFFFFFFFu, B.index, off);
+            B = better(B, o);
+        }
+        if (valid && sl == 0) s_tok[j] = B.index;
+    }
+    __syncthreads();
+    const int tok = draft ? s_tok[i] : 0;
+    if (draft && tok != tokens[row]) atomicMin(&s_first_mismatch, i);
     __syncthreads();
     const int stop = s_first_mismatch;                  // position of the replacement token, if any
     if (draft) {
@@ -1046,17 +1070,17 @@ cudaError_t launch_unmask_kernels(const UnmaskProblem& p, UnmaskPartial* partial
     launches[which](p, partial, tiles_per_item, select_state, status, sm_count * per_sm[which], st);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (mode == 2)
-        ss_accept_kernel<<<forks, 128, 0, st>>>(partial, p.tokens, p.state, p.n_committed, p.n_left, p.sets, items_per_row);
-    else
-    {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(forks);
-        cfg.blockDim = dim3(kFinalizeThreads);
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        cfg.numAttrs = overlap_launch_attribute(st, attr);
-        cfg.attrs = attr;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(forks);
+    cfg.blockDim = dim3(kFinalizeThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    cfg.numAttrs = overlap_launch_attribute(st, attr);
+    cfg.attrs = attr;
+    if (mode == 2) {
+        cudaLaunchKernelEx(&cfg, ss_accept_kernel, static_cast<const UnmaskPartial*>(partial), p.tokens, p.state, p.n_committed,
+                           p.n_left, p.sets, items_per_row);
+    } else {
         cudaLaunchKernelEx(&cfg, unmask_finalize_kernel, static_cast<const UnmaskPartial*>(partial), p.tokens, p.state,
                            p.n_committed, p.n_left, p.conf, p.sets, items_per_row, p.threshold,
                            mode == 1 ? static_cast<int>(FDD_DRAFT) : static_cast<int>(FDD_COMMITTED),

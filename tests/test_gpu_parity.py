@@ -872,6 +872,38 @@ def test_ss_draft_and_accept_cycles_match_oracle(temperature):
         fdd.fdd_destroy(ctx)
 
 
+@pytest.mark.parametrize("forks,block,vocab,right", [
+    (1, 5, 151936, 3),       # a record per tile: 75 of them for every row
+    (1, 5, 151936, 5),       # every draft right
+    (3, 128, 2048, 100),     # the longest block, one record per row
+    (2, 1, 5000, 0),         # a single draft, wrong
+])
+def test_ss_accept_merges_any_number_of_records(forks, block, vocab, right):
+    from oracle.ss import DRAFT, ss_accept
+    sc = synth.Scene(16, forks, block, 0, 1)
+    w = synth.Workload("accept", 4, 1, 64, vocab, "bf16", "peaked", 0.9, 0.0, (sc,), seed=90 + block)
+    ctx = harness.create_context(w)
+    try:
+        scene = harness.GpuScene(ctx, w, 0)
+        g = np.random.default_rng(vocab + right)
+        tokens = g.integers(0, vocab, (forks, block)).astype(np.int32)
+        state = np.full((forks, block), DRAFT, dtype=np.uint8)
+        ar = (g.standard_normal((forks, block, vocab)) * 0.5).astype(np.float32)
+        for f in range(forks):
+            for i in range(block):
+                ar[f, i, tokens[f, i] if i < right else (tokens[f, i] + 1) % vocab] = 12.0
+        bits = synth.f32_to_bf16_bits(ar)
+        tok_d, st_d = torch.from_numpy(tokens).cuda(), torch.from_numpy(state).cuda()
+        n_a, n_l = (torch.full((forks,), -7, dtype=torch.int32, device="cuda") for _ in range(2))
+        fdd.fdd_ss_accept(ctx, [scene.forkset], harness.bf16_tensor(bits), tok_d, st_d, [block], 0.0, 0, 0, n_a, n_l)
+        fdd.fdd_poll_status(ctx)
+        ref = ss_accept(pu.widen_logits(w, bits), tokens, state, scene.seeds, 0.0, 0, 0)
+        assert np.array_equal(tok_d.cpu().numpy(), ref["tokens"]) and np.array_equal(st_d.cpu().numpy(), ref["state"])
+        assert np.array_equal(n_a.cpu().numpy(), ref["n_accepted"]) and np.array_equal(n_l.cpu().numpy(), ref["n_left"])
+    finally:
+        fdd.fdd_destroy(ctx)
+
+
 # ---------------------------------------------------------------------------------------------
 # whole block loop, averaging
 # ---------------------------------------------------------------------------------------------
