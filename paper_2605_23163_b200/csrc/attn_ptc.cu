@@ -1092,7 +1092,9 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                     }
                     tc::named_barrier(1, 256);
                     if (last_s) {
-                        if (row_ok) {                            // thread = row
+                        // thread = row; the second group of an item with one query tile has none (its positions
+                        // would be those of another unit)
+                        if (active && row_ok) {
                             __nv_bfloat16* op = p.out + ((static_cast<size_t>(f) * p.d + qi) * p.n_q_heads + h * p.G + qg) * D;
 #pragma unroll
                             for (int col0 = 0; col0 < D / 4; col0 += 16)

@@ -1,4 +1,8 @@
 """GPU parity: every C-ABI call against the CPU fp64 oracle on the same seeded inputs."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -466,6 +470,24 @@ def test_attention_units_cut_into_pieces_of_their_own(hq, hkv, dim, prefix, fork
             assert np.all(np.isnan(got[np.setdiff1d(np.arange(forks), on)]))
     finally:
         fdd.fdd_destroy(ctx)
+
+
+def _in_child(code, **env):
+    # settings that the library reads once per process
+    here = os.path.dirname(os.path.abspath(__file__))
+    head = f"import sys; sys.path[:0] = [{os.path.dirname(here)!r}, {here!r}]; import test_gpu_parity as t\n"
+    res = subprocess.run([sys.executable, "-c", head + code], env={**os.environ, **env}, capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0, res.stdout + res.stderr
+
+
+def test_attention_units_of_one_query_tile_in_two_pieces():
+    # FDD_ATTN_MIN_TILES = 4 cuts units of one query tile (seven or eight key tiles) into two pieces: the piece that
+    # comes second merges its own rows only (even and odd numbers of query tiles, both layouts of TMEM)
+    _in_child("""
+for hq, hkv, dim, prefix, forks, block in [(8, 2, 128, 768, 1, 48), (8, 2, 64, 896, 1, 80), (4, 1, 128, 768, 3, 64),
+                                           (14, 2, 128, 768, 1, 27), (12, 2, 64, 896, 2, 50)]:
+    t.test_attention_units_cut_into_pieces_of_their_own(hq, hkv, dim, prefix, forks, block, None)
+""", FDD_ATTN_MIN_TILES="4")
 
 
 def test_more_scenes_and_rows_than_one_launch_takes():
