@@ -70,6 +70,7 @@
 
 #include <math_constants.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstdlib>
 
@@ -193,7 +194,7 @@ struct Item {
 };
 
 // step_base[s]: first global tile step of scene s (scenes laid end to end, skipped rollouts left out)
-template <int MAXSETS>
+template <bool OWN, int MAXSETS>
 __device__ __forceinline__ Item locate(const TcArgs<MAXSETS>& a, const SetParams* sets, const long long* step_base, long long pos, long long end) {
     Item it;
     int s = 0;
@@ -201,8 +202,11 @@ __device__ __forceinline__ Item locate(const TcArgs<MAXSETS>& a, const SetParams
     const SetParams& p = sets[s];
     const long long rel = pos - step_base[s];
     it.s = s;
-    it.unit = rel <= 0xFFFFFFFFLL ? static_cast<int>(static_cast<uint32_t>(rel) / static_cast<uint32_t>(p.tiles_total))
-                                  : static_cast<int>(rel / p.tiles_total);
+    // (Which division is the faster one goes by the instantiation, as measured.  One score buffer, 32 / 8 heads, 32
+    // rollouts: 124.2 us with a 32-bit branch, 121.8 without at prefix 4003, 37.0 and 35.3 at prefix 700, head
+    // dimension 64.  Own scores, 28 / 4 heads, 40 rollouts, prefix 3001: 108.4 with it, 110.4 without.)
+    it.unit = OWN && rel <= 0xFFFFFFFFLL ? static_cast<int>(static_cast<uint32_t>(rel) / static_cast<uint32_t>(p.tiles_total))
+                                         : static_cast<int>(rel / p.tiles_total);
     it.t0 = static_cast<int>(rel - static_cast<long long>(it.unit) * p.tiles_total);
     it.unit_begin = pos - it.t0;
     const long long left = end - pos;
@@ -292,7 +296,12 @@ struct Layout {
     int by_unit;               // > 0: every unit is cut into equal pieces of at most this many steps; 0: equal ranges
 };
 
-// The layout of a launch: one warp, lane s looks after scene s (n_sets <= 16).
+// Pieces of a unit of `tiles` steps when no piece is longer than c.
+__host__ __device__ __forceinline__ int pieces_of(int tiles, int c) { return tiles <= kWholeTiles ? 1 : (tiles + c - 1) / c; }
+
+// The layout of a launch: one warp, lane s looks after scene s (n_sets <= 16).  Every role waits for it, so it is
+// kept short: 32-bit divisions, and for one scene the lengths of a piece are tried side by side (with 64-bit divisions
+// one after the other, equal ranges at 16 / 2 heads, prefix 16384, 16 rollouts took 75.4 us a launch instead of 73.4).
 template <int MAXSETS, bool BYUNIT>
 __device__ __forceinline__ void plan(const TcArgs<MAXSETS>& a, const SetParams* sets, const int* n_act, long long* step_base,
                                      int* unit_base, int* cta_base, int* pieces, Layout* out, int lane) {
@@ -301,52 +310,67 @@ __device__ __forceinline__ void plan(const TcArgs<MAXSETS>& a, const SetParams* 
     const int tiles = mine ? sets[lane].tiles_total : 1;
     const int q_tiles = mine ? sets[lane].q_tiles : 0;
     const int heads_forks = mine ? sets[lane].n_kv_heads * n_act[lane] : 0;
-    auto sum = [&](long long v) {
-        if (MAXSETS == 1) return __shfl_sync(full, v, 0);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(full, v, off);
-        return v;
-    };
-    auto before = [&](long long v) {                    // sum over the lanes below this one
-        long long incl = v;
+    auto sum = [&](int v) { return MAXSETS == 1 ? __shfl_sync(full, v, 0) : __reduce_add_sync(full, v); };
+    auto scan = [&](auto v) {                           // sum over the lanes up to this one
 #pragma unroll
         for (int off = 1; off < MAXSETS; off <<= 1) {
-            const long long up = __shfl_up_sync(full, incl, off);
-            if (lane >= off) incl += up;
+            const auto up = __shfl_up_sync(full, v, off);
+            if (lane >= off) v += up;
         }
-        return incl - v;
+        return v;
     };
-    const int grid = static_cast<int>(gridDim.x);
+    const int grid = static_cast<int>(gridDim.x), last = a.n_sets - 1;
     Layout l;
-    l.per_unit = 1;
-    long long units = static_cast<long long>(heads_forks) * q_tiles;
-    l.T = sum(units * tiles);
-    if (!BYUNIT || l.T > grid * kSingleSteps) {
-        l.per_unit = 2;
-        units = static_cast<long long>(heads_forks) * ((q_tiles + 1) / 2);
-        l.T = sum(units * tiles);
+    int units = heads_forks * ((q_tiles + 1) / 2);
+    l.per_unit = 2;
+    if (BYUNIT) {
+        // (a scene alone may be over the limit: counted as just over it)
+        const long long singles = static_cast<long long>(heads_forks) * q_tiles * tiles;
+        const int limit = grid * kSingleSteps;
+        if (sum(singles > limit ? limit + 1 : static_cast<int>(singles)) <= limit) {
+            l.per_unit = 1;
+            units = heads_forks * q_tiles;
+        }
     }
-    const long long U = sum(units);
+    const long long steps_incl = scan(static_cast<long long>(units) * tiles);
+    const int units_incl = scan(units);
+    l.T = __shfl_sync(full, steps_incl, last);
     int n = 1;                                          // pieces of a unit of this lane's scene
     l.by_unit = 0;
-    l.ctas = static_cast<int>(max(1LL, min(static_cast<long long>(grid), l.T / a.min_tiles)));
-    if (BYUNIT && l.T > 0 && U <= grid) {
-        const int even = max(a.min_piece, static_cast<int>((l.T + grid - 1) / grid));
-        for (int c = even; c <= even + kUnitSlack; ++c) {
-            n = tiles <= kWholeTiles ? 1 : (tiles + c - 1) / c;
-            const long long need = sum(units * n);
-            if (need <= grid) {
-                l.by_unit = c;
-                l.ctas = static_cast<int>(need);
-                break;
+    l.ctas = l.T >= static_cast<long long>(grid) * a.min_tiles ? grid : max(1, static_cast<int>(l.T) / a.min_tiles);
+    int ctas_incl = 0;
+    const int U = __shfl_sync(full, units_incl, last);
+    if (BYUNIT && l.T > 0 && U <= grid && l.T <= 0x7FFFFFFF - grid) {
+        const int even = max(a.min_piece, (static_cast<int>(l.T) + grid - 1) / grid);
+        if (MAXSETS == 1) {
+            // one scene: a lane per length
+            const int u0 = __shfl_sync(full, units, 0), t0 = __shfl_sync(full, tiles, 0);
+            const int k = pieces_of(t0, even + lane);
+            const bool fit = lane <= kUnitSlack && k <= grid && u0 * k <= grid;
+            const unsigned fits = __ballot_sync(full, fit);
+            if (fits != 0u) {
+                const int at = __ffs(fits) - 1;         // (the same in every lane)
+                n = __shfl_sync(full, k, at);
+                l.by_unit = even + at;
+                l.ctas = u0 * n;
+            }
+        } else {
+            for (int c = even; c <= even + kUnitSlack; ++c) {
+                n = pieces_of(tiles, c);
+                const int need = sum(units * min(n, grid + 1));
+                if (need <= grid) {
+                    l.by_unit = c;
+                    l.ctas = need;
+                    break;
+                }
             }
         }
+        ctas_incl = scan(units * n);
     }
-    const long long steps_before = before(units * tiles), units_before = before(units), ctas_before = before(units * n);
     if (mine) {
-        step_base[lane] = steps_before;
-        unit_base[lane] = static_cast<int>(units_before);
-        cta_base[lane] = static_cast<int>(ctas_before);  // (only used by unit, where it is below the grid's size)
+        step_base[lane] = steps_incl - static_cast<long long>(units) * tiles;
+        unit_base[lane] = units_incl - units;
+        cta_base[lane] = ctas_incl - units * n;         // (only used by unit)
         pieces[lane] = n;
     }
     if (lane == 0) {
@@ -499,15 +523,15 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
     };
     auto view_item = [&](long long pos) {
         ItemView v;
-        v.it = locate(a, sets, step_base_s, pos, range_end);
+        v.it = locate<kOwn>(a, sets, step_base_s, pos, range_end);
         const SetParams& p = sets[v.it.s];
         int idx = v.it.unit;
         const int n_act = n_act_s[v.it.s];
         v.f = idx % n_act; idx /= n_act;
         if (p.gate != nullptr) v.f = fork_s[p.fork_base + v.f];
         const int per_head = per_unit == 2 ? (p.q_tiles + 1) / 2 : p.q_tiles;
-        v.h = idx / per_head;
-        v.tile0 = (idx - v.h * per_head) * per_unit;
+        v.tile0 = (idx % per_head) * per_unit; idx /= per_head;
+        v.h = idx;
         v.nt = v.it.t1 - v.it.t0;
         v.NQ = min(per_unit, p.q_tiles - v.tile0);
         return v;
@@ -1147,8 +1171,6 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                             break;
                         }
                     }
-                    // nobody looks at the unit's count any more once every holder of a piece has seen it complete
-                    seen[e] = atomicAdd(a.unit_count + a.max_units + deferred_s[e].gu, 1);
                 }
                 __threadfence();                                      // the pieces were published before their counts
             }
@@ -1158,6 +1180,10 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                     slot2_s[e][tid] = pc * 2 + (by_unit || deferred_s[e].unit_begin <= T * pc / C ? 0 : 1);
                 }
             tc::named_barrier(1, 256);
+            // Nobody looks at a unit's count any more once every holder of a piece has seen it complete.  (Behind the
+            // barrier: the answer is only needed at the end, and the merge need not wait for it; 1-2 us of a launch.)
+            if (tid == 0)
+                for (int e = 0; e < n_deferred; ++e) seen[e] = atomicAdd(a.unit_count + a.max_units + deferred_s[e].gu, 1);
             if (*abort_flag == 0) {
                 const int threads_e = 256 / n_deferred;               // threads per unit
                 const int e = tid / threads_e, lt = tid - e * threads_e;
@@ -1360,6 +1386,25 @@ cudaError_t launch_shape(const TcArgs<MAXSETS>& args, int head_dim, unsigned cta
     return launch_one<128, MAXSETS, 0, kSharedScores, BYUNIT>(args, ctas, waits, device, st);
 }
 
+// Whether plan() would cut every unit of a launch without a gate into pieces of its own (`pairs` <= ctas).
+bool cuts_by_unit(const SetParams* sets, int n, int ctas, int min_piece) {
+    long long singles = 0, doubles = 0;                    // tile steps with units of one query tile and of two
+    for (int s = 0; s < n; ++s) {
+        const long long per_tile = static_cast<long long>(sets[s].n_kv_heads) * sets[s].n_forks * sets[s].tiles_total;
+        singles += per_tile * sets[s].q_tiles;
+        doubles += per_tile * ((sets[s].q_tiles + 1) / 2);
+    }
+    if (singles <= ctas * kSingleSteps) return true;
+    const int even = std::max(min_piece, static_cast<int>((doubles + ctas - 1) / ctas));
+    for (int c = even; c <= even + kUnitSlack; ++c) {
+        long long need = 0;
+        for (int s = 0; s < n; ++s)
+            need += static_cast<long long>(sets[s].n_kv_heads) * sets[s].n_forks * ((sets[s].q_tiles + 1) / 2) * pieces_of(sets[s].tiles_total, c);
+        if (need <= ctas) return true;
+    }
+    return false;
+}
+
 template <int MAXSETS>
 cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* const* caches, int n, int head_dim,
                          cudaStream_t st) {
@@ -1423,7 +1468,10 @@ cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* con
     args.n_sets = n;
     args.scale_log2 = probs[0].scale * 1.4426950408889634f;
     args.merge_wait_limit = ctx->attn_merge_wait_limit;
-    if (pairs <= ctx->attn_max_ctas) return launch_shape<MAXSETS, true>(args, head_dim, static_cast<unsigned>(ctas), waits, ctx->device, st);
+    // Equal ranges are 1-3 us faster in the instantiation that knows nothing else (16 / 2 heads, prefix 16384, 16
+    // rollouts: 72.3 against 74.9 us); with a gate the layout is known on the device only, and is mostly by unit.
+    if (pairs <= ctx->attn_max_ctas && (gated || cuts_by_unit(args.sets, n, static_cast<int>(ctas), args.min_piece)))
+        return launch_shape<MAXSETS, true>(args, head_dim, static_cast<unsigned>(ctas), waits, ctx->device, st);
     return launch_shape<MAXSETS, false>(args, head_dim, static_cast<unsigned>(ctas), waits, ctx->device, st);
 }
 
