@@ -416,9 +416,8 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
     // may be made resident on SMs as their CTA of this launch exits; it waits for the whole of this
     // launch before it reads anything.
     tc::grid_launch_dependents();
-    // This launch may itself have started early: what does not depend on the kernel ahead of it (barriers,
-    // TMEM, the tensor maps, the scenes' sizes) is set up while that one drains; the gate below is written
-    // by it.
+    // This launch may itself have started early: what does not depend on the kernel ahead of it (barriers, the
+    // tensor maps, the scenes' sizes) is set up while that one drains; the gate below is written by it.
     auto set_up = [&]() {
         if (tid == 0) {
             abort_s = 0;
@@ -440,10 +439,6 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
             }
             tc::fence_barrier_init();
         }
-        if (warp == 9) {
-            tc::tmem_alloc(tc::smem_u32(&tmem_base_s), 512);
-            tc::tmem_relinquish();
-        }
     };
     if (BYUNIT) {
         for (int i = tid; i < a.n_sets * static_cast<int>(sizeof(SetParams) / 4); i += kTcThreads)
@@ -457,6 +452,16 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
         __syncthreads();
     }
     tc::grid_dependency_wait();
+    // TMEM only now: the kernel ahead may be a caller's, whose CTAs allow this launch to start before they have
+    // allocated theirs.  Holding all columns while waiting for it would leave the two waiting for each other.
+    // (While the other warps read the gate: no launch got slower by it.)
+    auto take_tmem = [&]() {
+        if (warp == 9) {
+            tc::tmem_alloc(tc::smem_u32(&tmem_base_s), 512);
+            tc::tmem_relinquish();
+        }
+    };
+    if (BYUNIT) take_tmem();
 
     for (int s = warp; s < a.n_sets; s += kTcThreads / 32) {
         const SetParams& p = sets[s];
@@ -489,6 +494,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
     }
     if (!BYUNIT) {
         set_up();
+        take_tmem();
         tc::fence_before_sync();
         __syncthreads();
         tc::fence_after_sync();

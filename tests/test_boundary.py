@@ -34,3 +34,15 @@ def test_status_codes_match_header():
     text = open(os.path.join(ROOT, "include", "fdd.h")).read()
     for name, val in re.findall(r"#define\s+(FDD_[A-Z_0-9]+)\s+\(?(-?\d+)\)?", text):
         assert getattr(fdd, name) == int(val), name
+
+
+def test_tensor_memory_is_taken_behind_the_wait_for_the_kernel_ahead():
+    # A kernel that starts early and holds tensor memory while it waits can be waited for by the kernel it waits for
+    # (a caller's, which has not allocated its own yet).  That cannot be tried out on a GPU, so the order is read here.
+    seen = 0
+    for path in build.sources():
+        code = re.sub(r"//[^\n]*", "", open(path).read())
+        if "tc::tmem_alloc(" in code:
+            seen += 1
+            assert "grid_dependency_wait()" in code[:code.index("tc::tmem_alloc(")], path
+    assert seen == 1
