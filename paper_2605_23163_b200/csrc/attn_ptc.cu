@@ -1316,8 +1316,8 @@ const TcSetMaps* maps_for(const AttnProblem& a, int D, TcMapCache* cache) {
 }
 
 int emulated_exponentials() {
-    // How many of the 128 exponentials of a key tile go through the polynomial.  FDD_ATTN_EMU
-    // (0, 16 or 32) overrides the default; every choice computes the same thing.
+    // How many of the 128 exponentials of a key tile go through the polynomial (head dimension 128, groups that are a
+    // power of two).  FDD_ATTN_EMU (0, 16 or 32) overrides the default; every choice computes the same thing.
     static int value = -1;
     if (value < 0) {
         value = 0;
@@ -1382,14 +1382,11 @@ cudaError_t launch_shape(const TcArgs<MAXSETS>& args, int head_dim, unsigned cta
         return launch_one<128, MAXSETS, 0, kOwnScoresSplit, BYUNIT>(args, ctas, waits, device, st);
     }
     if (head_dim == 64) return launch_one<64, MAXSETS, 0, kSharedScores, BYUNIT>(args, ctas, waits, device, st);
-    if (!BYUNIT) {
-        switch (emulated_exponentials()) {
-            case 16: return launch_one<128, MAXSETS, 16, kSharedScores, false>(args, ctas, waits, device, st);
-            case 32: return launch_one<128, MAXSETS, 32, kSharedScores, false>(args, ctas, waits, device, st);
-            default: break;
-        }
+    switch (emulated_exponentials()) {
+        case 16: return launch_one<128, MAXSETS, 16, kSharedScores, BYUNIT>(args, ctas, waits, device, st);
+        case 32: return launch_one<128, MAXSETS, 32, kSharedScores, BYUNIT>(args, ctas, waits, device, st);
+        default: return launch_one<128, MAXSETS, 0, kSharedScores, BYUNIT>(args, ctas, waits, device, st);
     }
-    return launch_one<128, MAXSETS, 0, kSharedScores, BYUNIT>(args, ctas, waits, device, st);
 }
 
 // Whether plan() would cut every unit of a launch without a gate into pieces of its own (`pairs` <= ctas).

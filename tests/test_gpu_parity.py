@@ -1,4 +1,5 @@
 """GPU parity: every C-ABI call against the CPU fp64 oracle on the same seeded inputs."""
+import hashlib
 import os
 import subprocess
 import sys
@@ -478,6 +479,29 @@ def _in_child(code, **env):
     head = f"import sys; sys.path[:0] = [{os.path.dirname(here)!r}, {here!r}]; import test_gpu_parity as t\n"
     res = subprocess.run([sys.executable, "-c", head + code], env={**os.environ, **env}, capture_output=True, text=True, timeout=300)
     assert res.returncode == 0, res.stdout + res.stderr
+    return res.stdout
+
+
+def _small_launch_digest():
+    w = synth.small_variant(synth.workload("tts"), prefix_len=900, vocab=512, n_forks=2, n_blocks=1)
+    ctx = harness.create_context(w)
+    try:
+        scene = harness.GpuScene(ctx, w, 0)
+        pk, pv = synth.make_prefix(w, 0)
+        q, k, v = synth.make_qkv(w, 0, 0, 0, 0)
+        got = pu.attention_gpu(ctx, scene, q, k, v)
+        empty = ([np.zeros((0, w.n_kv_heads, w.head_dim), dtype=np.uint16)] * 2,) * 2
+        pu.assert_attention_close(got, pu.attention_oracle(w, (pk, pv), empty, q, k, v))
+        return hashlib.sha256(got.tobytes()).hexdigest()
+    finally:
+        fdd.fdd_destroy(ctx)
+
+
+def test_attention_small_launches_honour_the_share_of_emulated_exponentials():
+    # the polynomial rounds differently, so the setting shows in the bits (and in nothing else)
+    run = "print('digest', t._small_launch_digest())"
+    digests = [_in_child(run, FDD_ATTN_EMU=str(n)).split("digest ")[1].split()[0] for n in (0, 16, 32)]
+    assert len(set(digests)) == 3
 
 
 def test_attention_units_of_one_query_tile_in_two_pieces():
