@@ -104,10 +104,17 @@ struct SetParams {
     int causal;
 };
 
+// Plain addresses of a scene's operands (redo_columns).
+struct RawSet {
+    const __nv_bfloat16 *q, *k_blk, *v_blk, *prefix_k, *prefix_v, *suffix_k, *suffix_v;
+    int prefix_capacity, suffix_capacity;
+};
+
 template <int MAXSETS>
 struct TcArgs {
     TcSetMaps maps[MAXSETS];
     SetParams sets[MAXSETS];
+    RawSet raw[MAXSETS];
     float* part_o;             // [2 * ctas][D / 4][256] float4: normalised partial outputs, column-major per slot
     float* part_lse;           // [2 * ctas][256] log2-domain log-sum-exp of the partial
     int* unit_count;           // [2][max_units]: pieces written per unit, CTAs done with the unit's merge (self-resetting)
@@ -280,6 +287,65 @@ __device__ __forceinline__ void merge_columns(const float* part_o, const float* 
         *reinterpret_cast<uint2*>(op + (col0 + c) * 4) =
             make_uint2(*reinterpret_cast<const uint32_t*>(&b0), *reinterpret_cast<const uint32_t*>(&b1));
     }
+}
+
+// One row's output over the key tiles [t0, t1) once more, in fp32 on the CUDA cores: 32 columns from col0, not yet
+// divided by the row sum.  For rows whose product on the tensor cores came out as an infinity or NaN although their
+// row sum is finite.  With an infinity in V the two halves of a probability make NaN of it (the low half can be zero or
+// negative), and V near the end of the range overflows under probabilities of up to 2^8.  Neither happens here: every
+// weight is one fp32 number and at most 1.  Rare, so one thread takes one row, and nothing is kept between columns.
+template <int D>
+__device__ __noinline__ void redo_columns(const SetParams& p, const RawSet& r, int h, int f, int qi, int qg, int t0, int t1,
+                                          float scale_log2, int col0, uint32_t* out, float* m_out, float* l_out) {
+    const __nv_bfloat16* qp = r.q + ((static_cast<size_t>(f) * p.d + qi) * p.n_q_heads + h * p.G + qg) * D;
+    float acc[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) acc[i] = 0.0f;
+    float m = -CUDART_INF_F, l = 0.0f;
+    for (int g = t0; g < t1; ++g) {
+        const TileInfo t = tile_info(p, g);
+        int limit = t.nvalid;
+        if (p.causal && t.segment == 2) limit = min(limit, qi - t.index * kKeysPerTile + 1);
+        for (int j = 0; j < limit; ++j) {
+            const int key = t.index * kKeysPerTile + j;            // inside its segment
+            const __nv_bfloat16 *kp, *vp;
+            size_t at;
+            if (t.segment == 0) {
+                if (p.page_tokens == 0) at = static_cast<size_t>(h) * r.prefix_capacity + key;
+                else at = (static_cast<size_t>(p.page_table[key / p.page_tokens]) * p.n_kv_heads + h) * p.page_tokens + key % p.page_tokens;
+                kp = r.prefix_k; vp = r.prefix_v;
+            } else if (t.segment == 1) {
+                at = (static_cast<size_t>(f) * p.n_kv_heads + h) * r.suffix_capacity + key;
+                kp = r.suffix_k; vp = r.suffix_v;
+            } else {
+                at = (static_cast<size_t>(f) * p.d + key) * p.n_kv_heads + h;
+                kp = r.k_blk; vp = r.v_blk;
+            }
+            kp += at * D;
+            vp += at * D + col0;
+            float dot = 0.0f;
+            for (int c = 0; c < D; c += 2) {
+                const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(qp + c));
+                const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(kp + c));
+                dot = fmaf(a.y, b.y, fmaf(a.x, b.x, dot));
+            }
+            const float s = dot * scale_log2, mn = fmaxf(m, s);
+            if (!(mn > -CUDART_INF_F)) continue;
+            const float back = exp2f(m - mn), w = exp2f(s - mn);
+            m = mn;
+            l = fmaf(l, back, w);
+#pragma unroll
+            for (int i = 0; i < 32; i += 2) {
+                const float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(vp + i));
+                acc[i] = fmaf(w, v.x, acc[i] * back);
+                acc[i + 1] = fmaf(w, v.y, acc[i + 1] * back);
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 32; ++i) out[i] = __float_as_uint(acc[i]);
+    *m_out = m;
+    *l_out = l;
 }
 
 // A unit whose merge this CTA takes part in once its range is done.
@@ -975,6 +1041,37 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                 // the item's last PV product of this query tile (and with it every product before it)
                 if (ok) ok = tc::mbar_wait(tc::smem_u32(&bar_o_final[q]), items_mine & 1, abort_flag, kWaitLimit);
                 if (ok) tc::fence_after_sync();
+                if (kOwn && ok) {
+                    // rows with an infinity or NaN in them are computed again (see redo_columns); a row sum that is not
+                    // finite comes from the scores, and nothing is to be mended then
+                    uint64_t zeros[2] = {0ull, 0ull};               // sums of 0 * value: NaN once a value is not finite
+#pragma unroll
+                    for (int cc = 0; cc < D / 32; ++cc) {
+                        uint32_t o[32];
+                        tc::tmem_ld32(tm_o[q] + lane_base + cc * 32, o);
+                        tc::wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 32; i += 2)
+                            zeros[(i >> 1) & 1] = tc::fma2(tc::pack2(__uint_as_float(o[i]), __uint_as_float(o[i + 1])), 0ull, zeros[(i >> 1) & 1]);
+                    }
+                    float z0, z1;
+                    tc::unpack2(tc::add2(zeros[0], zeros[1]), z0, z1);
+                    const bool redo = row_ok && !(z0 + z1 == 0.0f) && l < CUDART_INF_F;
+                    if (__any_sync(0xFFFFFFFFu, redo)) {
+                        float m_new = m_used, l_new = l;
+                        for (int cc = 0; cc < D / 32; ++cc) {
+                            uint32_t o[32];
+                            tc::tmem_ld32(tm_o[q] + lane_base + cc * 32, o);
+                            tc::wait_ld();
+                            if (redo) redo_columns<D>(p, a.raw[it.s], h, f, qi, qg, it.t0, it.t1, a.scale_log2, cc * 32, o, &m_new, &l_new);
+                            __syncwarp();
+                            tc::tmem_st32(tm_o[q] + lane_base + cc * 32, o);
+                        }
+                        tc::wait_st();
+                        m_used = m_new;
+                        l = l_new;
+                    }
+                }
             }
 
             // ---------------------------------------------------------------- epilogue
@@ -1435,6 +1532,7 @@ cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* con
         p.tiles_prefix = (a.prefix_len + kKeysPerTile - 1) / kKeysPerTile;
         p.tiles_suffix = (a.suffix_len + kKeysPerTile - 1) / kKeysPerTile;
         p.tiles_total = p.tiles_prefix + p.tiles_suffix + (a.d + kKeysPerTile - 1) / kKeysPerTile;
+        args.raw[s] = {a.q, a.k_blk, a.v_blk, a.prefix_k, a.prefix_v, a.suffix_k, a.suffix_v, a.prefix_capacity, a.suffix_capacity};
         p.n_kv_heads = a.n_kv_heads;
         p.causal = a.causal_in_block;
         p.gate = a.gate;

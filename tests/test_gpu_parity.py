@@ -436,6 +436,60 @@ def test_attention_groups_that_are_not_a_power_of_two_keep_full_precision(group,
     assert rel_l2 <= 2.0 ** -9 + 1e-5
 
 
+def _write_prefix(scene, cache, bits):
+    if scene.w.page_tokens:
+        x = harness.pack_prefix_paged(bits, scene.w.page_tokens, scene.page_table.cpu().numpy(), scene.pool_pages, "cuda")
+    else:
+        x = harness.pack_prefix_contiguous(bits, scene.prefix_capacity, "cuda")
+    cache.copy_(x)
+
+
+@pytest.mark.parametrize("hq,hkv,dim,prefix,page,forks", [
+    (14, 2, 128, 1500, 0, 12),        # pieces of two and three key tiles
+    (6, 2, 64, 700, 64, 3),           # paged, pieces of one
+    (28, 4, 128, 300, 0, 40),         # more units than CTAs
+])
+@pytest.mark.parametrize("causal", [False, True])
+def test_attention_groups_that_are_not_a_power_of_two_with_values_out_of_range(hq, hkv, dim, prefix, page, forks, causal):
+    block = 20
+    sc = synth.Scene(prefix, forks, block, 0, 1)
+    w = synth.Workload("range", hq, hkv, dim, 512, "bf16", "peaked", 0.9, 1.0, (sc,), page_tokens=page, seed=91)
+    ctx = harness.create_context(w)
+    try:
+        scene = harness.GpuScene(ctx, w, 0)
+        pk, pv = synth.make_prefix(w, 0)
+        q, k, v = synth.make_qkv(w, 0, 0, 0, 0)
+        empty = ([np.zeros((0, hkv, dim), dtype=np.uint16)] * forks,) * 2
+        want = pu.attention_oracle(w, (pk, pv), empty, q, k, v, causal=causal, forks=[0, 1]).reshape(2, block, hkv, hq // hkv, dim).copy()
+        # A visible infinity in V makes its column infinite, two of opposite signs or a NaN make it NaN; the other columns
+        # stay as they were, and keys hidden by the causal mask do not count.
+        inf, minus_inf, nan = 0x7F80, 0xFF80, 0x7FC0
+        bad_v, bad_pv = v.copy(), pv.copy()
+        bad_v[1, block - 1, 0, 7] = inf
+        bad_pv[5, 1, 3] = inf
+        bad_pv[prefix - 1, 1, 4] = minus_inf
+        bad_pv[3, 1, 5], bad_pv[prefix // 2, 1, 5] = inf, minus_inf
+        bad_pv[1, 1, 6] = nan
+        want[:, :, 1, :, 3], want[:, :, 1, :, 4], want[:, :, 1, :, 5:7] = np.inf, -np.inf, np.nan
+        want[1, block - 1 if causal else 0:, 0, :, 7] = np.inf
+        _write_prefix(scene, scene.prefix_v[0], bad_pv)
+        got = pu.attention_gpu(ctx, scene, q, k, bad_v, causal=causal)[[0, 1]].reshape(want.shape)
+        for special in (np.isnan, np.isposinf, np.isneginf):
+            assert np.array_equal(special(got), special(want))
+        pu.assert_attention_close(got[np.isfinite(want)], want[np.isfinite(want)])
+        # Large values: every key tile's scores lie 7 (in powers of two) above the tile before, so weights taken under the
+        # reference of the tile before are 2^7, and 128 of them times 2^116 are beyond fp32; the average is 2^116.
+        step = 7.0 / (np.sqrt(dim) * np.log2(np.e))
+        ramp = synth.f32_to_bf16_bits((step * (np.arange(prefix + block) // 128)).astype(np.float32))
+        _write_prefix(scene, scene.prefix_k[0], np.broadcast_to(ramp[:prefix, None, None], pk.shape).copy())
+        _write_prefix(scene, scene.prefix_v[0], np.full_like(pv, 0x7980))
+        got = pu.attention_gpu(ctx, scene, np.full_like(q, 0x3F80), np.broadcast_to(ramp[None, prefix:, None, None], k.shape).copy(),
+                               np.full_like(v, 0x7980), causal=causal)
+        assert np.all(np.abs(got / 2.0 ** 116 - 1.0) <= 2.0 ** -8)
+    finally:
+        fdd.fdd_destroy(ctx)
+
+
 @pytest.mark.parametrize("hq,hkv,dim,prefix,forks,block,live", [
     (8, 2, 128, 700, 3, 32, None),       # seven tiles: the shortest units that are cut, one query tile each
     (8, 2, 128, 639, 3, 32, None),       # six tiles: the longest that are not
