@@ -127,6 +127,9 @@ def compare_unmask(got, ref, tokens_in, state_in, threshold):
             assert got["n_committed"][f] == int((got["state"][f, masked] != MASKED).sum())
             assert got["n_left"][f] == int((got["state"][f, masked] == MASKED).sum())
             continue
+        assert np.array_equal(got["state"][f], ref["state"][f]), f"rollout {f}: commit set differs"
+        assert np.array_equal(got["tokens"][f], ref["tokens"][f]), f"rollout {f}: token ids differ"
+        assert got["n_committed"][f] == ref["n_committed"][f] and got["n_left"][f] == ref["n_left"][f]
     return dict(ambiguous_forks=ambiguous, low_margin_rows=low_margin, rows=rows)
 
 
