@@ -265,7 +265,7 @@ def test_attention_gated_rollouts_are_skipped_and_the_rest_is_unchanged():
                 off += ref.size; fork += sc.n_forks
     finally:
         fdd.fdd_destroy(ctx)
-    # the CUDA-core kernel (GQA group of three) honours the gate as well
+    # the layout of groups that are not a power of two (three here) honours the gate as well
     w = synth.Workload("g3_gated", 6, 2, 64, 256, "f32", "peaked", 0.9, 0.0,
                        (synth.Scene(prefix_len=100, n_forks=3, block_len=16, n_scaffold=5, n_blocks=1),), seed=13)
     ctx = harness.create_context(w)
@@ -409,8 +409,8 @@ def test_attention_largest_block_and_group():
         fdd.fdd_destroy(ctx)
 
 
-def test_attention_group_of_three_uses_the_cuda_core_kernel():
-    # a GQA group that is not a power of two is outside the tensor-core kernel's row stacking
+def test_attention_group_of_three():
+    # 126 of a query tile's 128 rows are in use
     sc = synth.Scene(prefix_len=150, n_forks=2, block_len=20, n_scaffold=5, n_blocks=1)
     w = synth.Workload("g3", 6, 2, 64, 512, "bf16", "peaked", 0.9, 1.0, (sc,), qkv_sigma=0.5, seed=32)
     _attention_case(w)
@@ -420,14 +420,14 @@ def test_attention_group_of_three_uses_the_cuda_core_kernel():
     (3, 128, 2, 43, 150, 0, 0),       # 42 positions a tile: the second tile holds one position
     (5, 64, 1, 128, 2100, 0, 1),      # the longest block: six tiles, units cut into many pieces
     (6, 128, 3, 21, 700, 64, 1),      # exactly one tile
-    (7, 128, 6, 27, 3001, 0, 0),      # units in two pieces and in more
+    (7, 128, 6, 27, 3001, 0, 0),      # units in nine pieces
     (7, 128, 2, 19, 1, 0, 1),         # one key of prefix, the second tile holds one position
     (15, 64, 2, 9, 333, 64, 0),       # 8 positions a tile, 120 rows
     (12, 128, 1, 1, 0, 0, 0),         # a single key
 ])
 @pytest.mark.parametrize("causal", [False, True])
-def test_attention_groups_that_are_not_a_power_of_two_keep_full_precision(group, dim, forks, block, prefix, page, blocks_before,
-                                                                           causal):
+def test_attention_groups_that_are_not_a_power_of_two_keep_sixteen_bits_of_the_weights(group, dim, forks, block, prefix, page,
+                                                                                      blocks_before, causal):
     # both halves of every probability enter the product, so the rounding of the output to bf16 is all
     # that is left: at most half an ulp, 2^-9 of each value (one bf16 half alone gives 2.3e-3)
     sc = synth.Scene(prefix, forks, block, 0, blocks_before + 1)
@@ -490,6 +490,51 @@ def test_attention_groups_that_are_not_a_power_of_two_with_values_out_of_range(h
         fdd.fdd_destroy(ctx)
 
 
+@pytest.mark.parametrize("hq,hkv,dim,page,scenes", [
+    (28, 4, 128, 0, [(200, 48, 27)]),                                  # more units than CTAs, two or three items per CTA
+    (28, 4, 128, 0, [(300, 30, 43)]),                                  # the same, items with one query tile between items with two
+    (12, 2, 64, 64, [(700, 40, 50)]),                                  # the same, paged, head dimension 64
+    (28, 4, 128, 0, [(1500, 18, 27)]),                                 # units in two pieces
+    (28, 4, 128, 64, [(300, 3, 27), (329, 2, 9), (1, 1, 40), (900, 4, 18)]),     # several scenes, pieces by unit
+    (28, 4, 64, 0, [(130, 20, 43), (70, 16, 9), (300, 12, 20)]),       # several scenes, more units than CTAs
+    (20, 4, 128, 0, [(8000, 10, 64), (130, 2, 5)]),                    # equal ranges over fewer units than CTAs
+])
+@pytest.mark.parametrize("gated", [False, True])
+def test_attention_groups_that_are_not_a_power_of_two_over_several_items_and_scenes(hq, hkv, dim, page, scenes, gated):
+    scenes = tuple(synth.Scene(p, n, d, 0, 1) for p, n, d in scenes)
+    w = synth.Workload("items", hq, hkv, dim, 512, "bf16", "peaked", 0.9, 1.0, scenes, page_tokens=page, seed=70 + len(scenes))
+    ctx = harness.create_context(w)
+    try:
+        gs = [harness.GpuScene(ctx, w, i) for i in range(len(scenes))]
+        qs, ks, vs = zip(*[synth.make_qkv(w, i, 0, 0, 0) for i in range(len(scenes))])
+        pack = lambda xs: harness.bf16_tensor(np.concatenate([x.reshape(-1) for x in xs]))
+        qd, kd, vd = pack(qs), pack(ks), pack(vs)
+        on = np.ones(sum(sc.n_forks for sc in scenes), np.int32)
+        if gated:
+            on[1::3] = 0
+        for _ in range(2):                   # (the second call finds the counters of the first)
+            out = torch.full_like(qd, float("nan"))
+            fdd.fdd_block_attn_gated(ctx, [g.forkset for g in gs], 0, qd, kd, vd, out, [sc.block_len for sc in scenes],
+                                     1.0 / np.sqrt(dim), 0, torch.from_numpy(on).cuda() if gated else None)
+            fdd.fdd_poll_status(ctx)
+            got = out.float().cpu().numpy().astype(np.float64)
+            off = fork = 0
+            for i, sc in enumerate(scenes):
+                rows = got[off:off + qs[i].size].reshape(qs[i].shape)
+                live = np.flatnonzero(on[fork:fork + sc.n_forks])
+                empty = ([np.zeros((0, hkv, dim), dtype=np.uint16)] * sc.n_forks,) * 2
+                if len(live):
+                    some = live if sc.prefix_len < 4000 else live[[0, -1]]
+                    ref = pu.attention_oracle(w, synth.make_prefix(w, i), empty, qs[i], ks[i], vs[i], forks=list(some))
+                    _, rel_l2 = pu.assert_attention_close(rows[some], ref)
+                    assert rel_l2 <= 2.0 ** -9 + 1e-5        # (the rounding of the output, as above)
+                    assert np.all(np.isfinite(rows[live]))
+                assert np.all(np.isnan(rows[np.setdiff1d(np.arange(sc.n_forks), live)]))
+                off += qs[i].size; fork += sc.n_forks
+    finally:
+        fdd.fdd_destroy(ctx)
+
+
 @pytest.mark.parametrize("hq,hkv,dim,prefix,forks,block,live", [
     (8, 2, 128, 700, 3, 32, None),       # seven tiles: the shortest units that are cut, one query tile each
     (8, 2, 128, 639, 3, 32, None),       # six tiles: the longest that are not
@@ -497,7 +542,8 @@ def test_attention_groups_that_are_not_a_power_of_two_with_values_out_of_range(h
     (32, 8, 128, 900, 8, 64, None),      # 64 units of a pair of query tiles, in two pieces each
     (32, 8, 64, 1300, 18, 17, None),     # 144 units: one CTA each, four left over
     (32, 8, 64, 1300, 12, 64, (0, 7)),   # few live rollouts of many
-    (16, 2, 128, 4096, 4, 36, (2,)),     # odd number of query tiles per rollout (3), units of one
+    (16, 2, 128, 4096, 4, 36, (2,)),     # odd number of query tiles per rollout (3), units of two and one
+    (16, 2, 128, 2000, 4, 36, (2,)),     # the same, units of one
     (16, 2, 128, 2000, 8, 36, None),     # the same, units of two and one
 ])
 def test_attention_units_cut_into_pieces_of_their_own(hq, hkv, dim, prefix, forks, block, live):
