@@ -132,7 +132,8 @@ fdd_status fdd_forkset_reset(fdd_ctx* ctx, fdd_forkset* set);
  * each other and causally to everything before the block.  For rollout f of a set the keys
  * are the shared prefix, f's private suffix and all block_len keys of f's block:
  *   out[f,i,h,:] = sum_j softmax_j(scale * q[f,i,h,:] . k_j[h/G,:]) v_j[h/G,:]
- * computed with bf16 operands, fp32 accumulation, bf16 output.
+ * computed with bf16 operands, fp32 accumulation, bf16 output; the probabilities enter the product
+ * with 8 bits, or with 16 where Hq / Hkv is not a power of two.
  *
  *   sets, n_sets   host array of fork sets handled in this call (independent scenes).
  *   layer          which per-layer cache to read, 0 <= layer < L.
@@ -197,10 +198,11 @@ fdd_status fdd_block_attn_gated(fdd_ctx* ctx, fdd_forkset* const* sets, int n_se
  * is committed.  Nothing else is written; rollouts without MASKED positions are no-ops.
  *
  *   logits        device, packed like q: [N_s][d_s][V], fp32 or bf16 per cfg.logits_dtype.
- *                 Only rows of MASKED positions are read.  N_s * d_s <= 8192 per set
- *                 (FDD_ERR_CAPACITY otherwise); the bulk copies need 16-byte aligned rows
- *                 (V % 8 == 0 for bf16, V % 4 == 0 for fp32, 16-byte aligned base), else a
- *                 slower path runs.
+ *                 Only rows of MASKED positions are used.  Where rows do not all start on a
+ *                 16-byte boundary (V % 8 != 0 for bf16, V % 4 != 0 for fp32, or such a base) up
+ *                 to 15 bytes on either side of such a row are fetched with it, never beyond the
+ *                 call's logits, and not looked at; otherwise nothing else is read.
+ *                 N_s * d_s <= 8192 per set (FDD_ERR_CAPACITY otherwise).
  *   tokens        device int32 [N_s][d_s], in/out.     state: device uint8, in/out.
  *   n_committed   device int32 [sum N_s]: commits of this step per rollout (written).
  *   n_left        device int32 [sum N_s]: MASKED positions remaining per rollout (written).
@@ -246,7 +248,7 @@ fdd_status fdd_unmask_counted(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets
  * verifier of Sec. 3.4); at the first mismatch the verifier's token replaces the draft and is
  * accepted, and every later FDD_DRAFT position goes back to MASKED for the next draft / verify
  * cycle.  n_accepted: positions that became COMMITTED in this call; n_left: MASKED afterwards.
- * Only rows in state FDD_DRAFT are read.  Limits as for fdd_unmask.
+ * Only rows in state FDD_DRAFT are used (as for fdd_unmask).  Limits as for fdd_unmask.
  */
 fdd_status fdd_ss_draft(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, const void* logits,
                         int32_t* tokens, uint8_t* state, const int32_t* block_len,

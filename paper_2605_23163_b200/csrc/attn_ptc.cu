@@ -26,9 +26,9 @@
 // 1.5 until the last piece is seen, 4 for the merge).  Measured, launches one behind the other (equal ranges ->
 // pieces by unit): one rollout, prefix 4096: 24.6 -> 18.5-20 us; eight rollouts: 33-36 -> 27-29 us; 28 / 4
 // heads, six rollouts, prefix 3001: 41 -> 35 us; a block of 36 layers with eight rollouts: 6.3 -> 5.3 ms.
-// These launches also set themselves up ahead of the wait for the kernel before them and keep the scenes'
+// These launches also initialise their barriers ahead of the wait for the kernel before them and keep the scenes'
 // sizes in shared memory; a launch with more units than CTAs lost 2-3 % by the same (a block at 32 rollouts,
-// prefix 16384: 1815-1850 us against 1770-1790), so it does neither.
+// prefix 16384: 1815-1850 us against 1770-1790), so it does neither.  TMEM is taken behind the wait everywhere.
 //
 // Warp roles (384 threads): warps 0-3 and 4-7 are the two soft-max groups (thread = one query
 // row = one TMEM lane), warp 8 lane 0 drives TMA, warps 9 and 10 issue the tcgen05.mma (one lane each:
@@ -47,7 +47,10 @@
 // probability, P = P_hi + P_lo with both halves bf16 (P_lo the rounding error of P_hi), as two products into
 // the same O: these shapes were computed in fp32 on the CUDA cores before, and with one bf16 P they would
 // lose precision (error against 64 bits: 1.66e-3 with both halves as before, the rounding of the output;
-// 2.3e-3 with P_hi alone).  TMEM is S0 | S1 | O0 | O1 for them: each query tile has scores of its own, and
+// 2.3e-3 with P_hi alone).  16 bits are fewer than the 24 of the fp32 weights: at most 2^-17 of each weight, which
+// the rounding of the output hides; over 24 shapes (groups of 3 to 15, prefix 100 to 16384) the error against 64 bits is
+// the fp32 kernel's to 4e-6 of itself.  What two halves cannot do, infinities in V and weights above 1 on very
+// large V, is done again in fp32 (redo_columns).  TMEM is S0 | S1 | O0 | O1 for them: each query tile has scores of its own, and
 // the two halves of P overwrite them.  The chain of a query tile (scores, soft-max, output, the next scores)
 // is then a serial one, one issuing warp each; the other tile's chain fills the gaps.  Three products of a
 // tile step instead of two are 3072 clocks of the tensor pipe, what a step of the other layout takes with
@@ -233,8 +236,8 @@ constexpr float kRoundMagic = 12582912.0f;                    // 1.5 * 2^23: add
 
 // Merge of a unit cut between CTAs:  out = sum_k w_k O_k / sum_k w_k,  w_k = 2^(lse_k - M), M = max_k lse_k.
 // Every CTA that holds a piece merges an equal share of the unit's rows.  A thread takes CT float4
-// columns of one row: 40 / CT pieces are read per round trip, 40 independent 16-byte reads (and the
-// pieces' log-sum-exps) in flight.  M is not known in advance: the sums are kept relative to the
+// columns of one row: 40 / CT pieces are read per round trip (36 for CT = 1), up to 40 independent 16-byte
+// reads (and the pieces' log-sum-exps) in flight.  M is not known in advance: the sums are kept relative to the
 // largest log-sum-exp seen so far and rescaled when a chunk raises it, so the pieces are read once.
 // Partials lie column-major in their slots ([D / 4][256 rows] float4).
 template <int D, int CT>

@@ -9,7 +9,8 @@
 // memory, three tiles deep; a lane takes 64 consecutive ids of a tile (16-byte reads, chunk order
 // rotated by the lane so that the banks do not collide) and keeps running soft-max statistics.
 // There is no CTA-wide barrier after the set-up, and nothing but the few logits that can win the
-// arg-max is looked at twice.  Rows that are not MASKED are never read.
+// arg-max is looked at twice.  Rows that are not MASKED are not read (ragged rows: but for the bytes that share a
+// 16-byte granule with a row that is).
 //
 // Noise (temperature > 0).  The Gumbel draws are g = -ln(E) with E an exponential race over groups
 // of 16 consecutive ids: group j has the 32-bit word R = word j % 4 of Philox block j / 4 (so the 64
@@ -113,7 +114,6 @@ template <typename T> struct Logit;
 template <> struct Logit<__nv_bfloat16> {
     static constexpr int kPerChunk = 8;                  // logits per 16-byte chunk
     __device__ static float load1(const __nv_bfloat16* p) { return __bfloat162float(*p); }
-    __device__ static __nv_bfloat16 minus_inf() { return __ushort_as_bfloat16(0xFF80u); }
     __device__ static void widen(const uint4& w, float* out) {
         const uint32_t x[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
@@ -137,7 +137,6 @@ template <> struct Logit<__nv_bfloat16> {
 template <> struct Logit<float> {
     static constexpr int kPerChunk = 4;
     __device__ static float load1(const float* p) { return *p; }
-    __device__ static float minus_inf() { return -CUDART_INF_F; }
     __device__ static void widen(const uint4& w, float* out) {
         out[0] = __uint_as_float(w.x); out[1] = __uint_as_float(w.y);
         out[2] = __uint_as_float(w.z); out[3] = __uint_as_float(w.w);
