@@ -331,6 +331,8 @@ fdd_status fdd_average_rollouts_jmt(fdd_ctx* ctx, const float* traj, int n, int 
  * library issues step t + 1 before it reads the counts of step t, so the GPU never waits for the
  * host; if step t completed the block, the kernels of step t + 1 find every rollout gated off and
  * no MASKED row and return at once (n_committed and n_left then hold that step's zeros).
+ * The layers of a step, whose inputs are all in place before it, share launches where no layer's output
+ * overlaps what another layer reads or writes (else they are issued one behind the other, as above).
  *   q, k_blk, v_blk, out   host arrays [n_inputs][n_layers] of device pointers, each laid out as for
  *                          fdd_block_attn; step t uses row t mod n_inputs (a caller whose model
  *                          writes every step into the same buffers passes n_inputs = 1)

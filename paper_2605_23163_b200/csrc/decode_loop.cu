@@ -102,12 +102,10 @@ fdd_status fdd_decode_block(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, 
     auto enqueue = [&](int t) -> fdd_status {
         if (before_step) before_step(user, t, stream);
         const int in = t % n_inputs;
-        for (int layer = 0; layer < n_layers; ++layer) {
-            const int i = in * n_layers + layer;
-            const fdd_status rc = fdd_block_attn_gated(ctx, sets, n_sets, layer, q[i], k_blk[i], v_blk[i], out[i], block_len,
-                                                       scale, causal_in_block, t == 0 ? nullptr : n_left, stream);
-            if (rc != FDD_OK) return rc;
-        }
+        const size_t at = static_cast<size_t>(in) * n_layers;
+        fdd_status rc = block_attn_layers(ctx, sets, n_sets, 0, n_layers, q + at, k_blk + at, v_blk + at, out + at, block_len,
+                                          scale, causal_in_block, t == 0 ? nullptr : n_left, stream);
+        if (rc != FDD_OK) return rc;
         // the unmasking step also writes (n_left, stamp) of every rollout into host memory that the
         // device can address: the host sees the counts the moment they land, without a copy and
         // without an event on the stream (which would sit between this step and the next one's early start)
@@ -115,11 +113,10 @@ fdd_status fdd_decode_block(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, 
         stamp_of[t & 1] = ctx->count_stamp;
         ctx->unmask_left_mirror = ctx->d_counts[t & 1];
         ctx->unmask_mirror_stamp = ctx->count_stamp;
-        const fdd_status rc = fdd_unmask(ctx, sets, n_sets, logits[in], tokens, state, block_len, threshold, temperature,
-                                         block_idx, static_cast<uint32_t>(t), n_committed, n_left, nullptr, stream);
+        rc = fdd_unmask(ctx, sets, n_sets, logits[in], tokens, state, block_len, threshold, temperature,
+                        block_idx, static_cast<uint32_t>(t), n_committed, n_left, nullptr, stream);
         ctx->unmask_left_mirror = nullptr;
-        if (rc != FDD_OK) return rc;
-        return FDD_OK;
+        return rc;
     };
 
     fdd_status rc = enqueue(0);
@@ -140,12 +137,10 @@ fdd_status fdd_decode_block(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, 
     if (commit_kv && left == 0) {
         // the block is complete: its keys and values, as the last step projected them, join every
         // rollout's private cache
-        const int in = (t - 1) % n_inputs;
-        for (int layer = 0; layer < n_layers; ++layer) {
-            rc = fdd_kv_commit(ctx, sets, n_sets, layer, k_blk[in * n_layers + layer], v_blk[in * n_layers + layer], block_len,
-                               layer == n_layers - 1 ? 1 : 0, stream);
-            if (rc != FDD_OK) return rc;
-        }
+        const size_t at = static_cast<size_t>((t - 1) % n_inputs) * n_layers;
+        CallRange commit_range("fdd_kv_commit");
+        rc = commit_layers(ctx, sets, n_sets, 0, n_layers, k_blk + at, v_blk + at, block_len, 1, stream, false);
+        if (rc != FDD_OK) return rc;
     }
     return FDD_OK;
 }

@@ -75,6 +75,38 @@ bool set_alive(const fdd_ctx* ctx, const fdd_forkset* s) {
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// Bytes [lo, hi) of device memory that a call reads or writes.
+struct Range {
+    uintptr_t lo, hi;
+};
+Range range_of(const void* p, size_t bytes) {
+    const uintptr_t at = reinterpret_cast<uintptr_t>(p);
+    return {at, at + bytes};
+}
+
+// Whether calls issued together do what they do one behind the other: nothing that one of them writes is
+// written or read by another (or by itself).
+bool independent(std::vector<Range>& writes, const std::vector<Range>& reads) {
+    const auto before = [](const Range& a, const Range& b) { return a.lo < b.lo; };
+    if (!std::is_sorted(writes.begin(), writes.end(), before)) std::sort(writes.begin(), writes.end(), before);
+    for (size_t i = 1; i < writes.size(); ++i)
+        if (writes[i].lo < writes[i - 1].hi) return false;
+    for (const Range& r : reads) {
+        // the first written range that ends behind the start of this one
+        const auto w = std::upper_bound(writes.begin(), writes.end(), r.lo, [](uintptr_t lo, const Range& x) { return lo < x.hi; });
+        if (w != writes.end() && w->lo < r.hi) return false;
+    }
+    return true;
+}
+
+// Bytes of one layer's prefix and suffix cache of a fork set.
+size_t prefix_cache_bytes(const fdd_config& c, const fdd_forkset* fs) {
+    return sizeof(__nv_bfloat16) * static_cast<size_t>(fs->prefix_capacity) * (c.page_tokens > 0 ? c.page_tokens : 1) * c.n_kv_heads * c.head_dim;
+}
+size_t suffix_cache_bytes(const fdd_config& c, const fdd_forkset* fs) {
+    return sizeof(__nv_bfloat16) * static_cast<size_t>(fs->n_forks) * fs->suffix_capacity * c.n_kv_heads * c.head_dim;
+}
+
 // Common checks of a batched call; fills total rollouts and per-set row offsets.
 fdd_status check_sets(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, const int32_t* block_len,
                       int* total_forks) {
@@ -93,6 +125,224 @@ fdd_status check_sets(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, const 
 }
 
 }  // namespace
+
+// Layers of a step are calls of their own to the caller, but their inputs are all in place before the first of them
+// (fdd_decode_block), so they go to the kernel like the scenes of one call: equal ranges over the tile steps of up to
+// kTcMaxSets (scene, layer) pairs fill the chip, where a layer of a few rollouts alone is cut into many pieces that have
+// to be merged.  Where a layer's output overlaps another one's output or inputs they go one behind the other.
+fdd_status block_attn_layers(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, int first_layer, int n_layers,
+                             const void* const* q, const void* const* k_blk, const void* const* v_blk, void* const* out,
+                             const int32_t* block_len, float scale, int causal_in_block, const int32_t* gate, void* stream) {
+    CallRange range("fdd_block_attn");
+    if (!ctx) return FDD_ERR_INVALID_ARG;
+    int total = 0;
+    fdd_status st = check_sets(ctx, sets, n_sets, block_len, &total);
+    if (st != FDD_OK) return st;
+    for (int l = 0; l < n_layers; ++l) {
+        if (!q[l] || !k_blk[l] || !v_blk[l] || !out[l]) return fail(ctx, FDD_ERR_INVALID_ARG, "q/k_blk/v_blk/out is NULL");
+        if (!aligned16(q[l]) || !aligned16(k_blk[l]) || !aligned16(v_blk[l]) || (reinterpret_cast<uintptr_t>(out[l]) & 31u) != 0)
+            return fail(ctx, FDD_ERR_INVALID_ARG, "q/k_blk/v_blk must be 16-byte aligned, out 32-byte aligned");
+    }
+    if (first_layer < 0 || first_layer >= ctx->cfg.n_layers || n_layers > ctx->cfg.n_layers - first_layer)
+        return fail(ctx, FDD_ERR_SHAPE, "layer %d outside [0, %d)", first_layer, ctx->cfg.n_layers);
+    if (!(scale > 0.0f)) return fail(ctx, FDD_ERR_INVALID_ARG, "scale must be positive");
+    if (gate && total > kAttnMaxGatedForks)
+        return fail(ctx, FDD_ERR_CAPACITY, "%d rollouts in one gated call exceed %d", total, kAttnMaxGatedForks);
+    const fdd_config& c = ctx->cfg;
+    cudaStream_t st_ = static_cast<cudaStream_t>(stream);
+    size_t rows = 0;
+    for (int s = 0; s < n_sets; ++s) rows += static_cast<size_t>(sets[s]->n_forks) * block_len[s];
+    bool together = n_layers > 1;
+    if (together) {
+        const size_t q_bytes = rows * c.n_q_heads * c.head_dim * sizeof(__nv_bfloat16), kv_bytes = rows * c.n_kv_heads * c.head_dim * sizeof(__nv_bfloat16);
+        std::vector<Range> writes, reads;
+        writes.reserve(n_layers);
+        reads.reserve(static_cast<size_t>(n_layers) * (3 + 4 * n_sets) + n_sets + 1);
+        for (int l = 0; l < n_layers; ++l) {
+            writes.push_back(range_of(out[l], q_bytes));
+            reads.push_back(range_of(q[l], q_bytes));
+            reads.push_back(range_of(k_blk[l], kv_bytes));
+            reads.push_back(range_of(v_blk[l], kv_bytes));
+            for (int s = 0; s < n_sets; ++s) {
+                const fdd_forkset* fs = sets[s];
+                const size_t pb = prefix_cache_bytes(c, fs), sb = suffix_cache_bytes(c, fs);
+                reads.push_back(range_of(fs->prefix_k[first_layer + l], pb));
+                reads.push_back(range_of(fs->prefix_v[first_layer + l], pb));
+                reads.push_back(range_of(fs->suffix_k[first_layer + l], sb));
+                reads.push_back(range_of(fs->suffix_v[first_layer + l], sb));
+            }
+        }
+        for (int s = 0; s < n_sets; ++s)
+            if (c.page_tokens > 0)
+                reads.push_back(range_of(sets[s]->page_table, sizeof(int32_t) * ((static_cast<size_t>(sets[s]->prefix_len) + c.page_tokens - 1) / c.page_tokens)));
+        if (gate) reads.push_back(range_of(gate, sizeof(int32_t) * total));
+        together = independent(writes, reads);
+    }
+    std::vector<AttnProblem> probs;
+    std::vector<TcMapCache*> caches;
+    probs.reserve(static_cast<size_t>(n_sets) * (together ? n_layers : 1));
+    caches.reserve(probs.capacity());
+    for (int l = 0; l < n_layers; ++l) {
+        const int layer = first_layer + l;
+        size_t q_off = 0, kv_off = 0;
+        int fork_off = 0;
+        for (int s = 0; s < n_sets; ++s) {
+            fdd_forkset* fs = sets[s];
+            AttnProblem p;
+            p.q = static_cast<const __nv_bfloat16*>(q[l]) + q_off;
+            p.k_blk = static_cast<const __nv_bfloat16*>(k_blk[l]) + kv_off;
+            p.v_blk = static_cast<const __nv_bfloat16*>(v_blk[l]) + kv_off;
+            p.out = static_cast<__nv_bfloat16*>(out[l]) + q_off;
+            p.prefix_k = static_cast<const __nv_bfloat16*>(fs->prefix_k[layer]);
+            p.prefix_v = static_cast<const __nv_bfloat16*>(fs->prefix_v[layer]);
+            p.page_table = fs->page_table;
+            p.suffix_k = static_cast<const __nv_bfloat16*>(fs->suffix_k[layer]);
+            p.suffix_v = static_cast<const __nv_bfloat16*>(fs->suffix_v[layer]);
+            p.n_forks = fs->n_forks;
+            p.d = block_len[s];
+            p.n_q_heads = c.n_q_heads;
+            p.n_kv_heads = c.n_kv_heads;
+            p.prefix_len = fs->prefix_len;
+            p.prefix_capacity = fs->prefix_capacity;
+            p.page_tokens = c.page_tokens;
+            p.suffix_len = fs->suffix_len;
+            p.suffix_capacity = fs->suffix_capacity;
+            p.causal_in_block = causal_in_block ? 1 : 0;
+            p.scale = scale;
+            p.gate = gate ? gate + fork_off : nullptr;
+            fork_off += fs->n_forks;
+            probs.push_back(p);
+            caches.push_back(&fs->map_cache[layer]);
+            q_off += static_cast<size_t>(fs->n_forks) * p.d * c.n_q_heads * c.head_dim;
+            kv_off += static_cast<size_t>(fs->n_forks) * p.d * c.n_kv_heads * c.head_dim;
+        }
+        if (together && l + 1 < n_layers) continue;
+        // as few launches as take all problems, of about the same size
+        const int count = static_cast<int>(probs.size());
+        const int launches = (count + kTcMaxSets - 1) / kTcMaxSets, most = (count + launches - 1) / launches;
+        for (int first = 0; first < count;) {
+            int n = 0, forks = 0;
+            while (n < most && first + n < count && (n == 0 || !gate || forks + probs[first + n].n_forks <= kAttnMaxGatedForks))
+                forks += probs[first + n++].n_forks;
+            int n_launches = 0;
+            cudaError_t e = launch_attention_ptc(ctx, probs.data() + first, caches.data() + first, n, c.head_dim, st_, &n_launches);
+            ctx->launches += n_launches;
+            if (e != cudaSuccess) return cuda_fail(ctx, e, "fdd_block_attn launch");
+            first += n;
+        }
+        probs.clear();
+        caches.clear();
+    }
+    return FDD_OK;
+}
+
+// Common body of fdd_kv_commit (to_prefix = false) and fdd_prefix_extend (to_prefix = true), for consecutive layers.
+fdd_status commit_layers(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, int first_layer, int n_layers,
+                         const void* const* k_blk, const void* const* v_blk, const int32_t* block_len,
+                         int advance, void* stream, bool to_prefix) {
+    if (!ctx) return FDD_ERR_INVALID_ARG;
+    int total = 0;
+    fdd_status st = check_sets(ctx, sets, n_sets, block_len, &total);
+    if (st != FDD_OK) return st;
+    for (int l = 0; l < n_layers; ++l) {
+        if (!k_blk[l] || !v_blk[l]) return fail(ctx, FDD_ERR_INVALID_ARG, "k_blk/v_blk is NULL");
+        if (!aligned16(k_blk[l]) || !aligned16(v_blk[l])) return fail(ctx, FDD_ERR_INVALID_ARG, "k_blk/v_blk must be 16-byte aligned");
+    }
+    if (first_layer < 0 || first_layer >= ctx->cfg.n_layers || n_layers > ctx->cfg.n_layers - first_layer)
+        return fail(ctx, FDD_ERR_SHAPE, "layer %d outside [0, %d)", first_layer, ctx->cfg.n_layers);
+    const fdd_config& c = ctx->cfg;
+    for (int s = 0; s < n_sets; ++s) {
+        const fdd_forkset* fs = sets[s];
+        if (!to_prefix) {
+            if (fs->suffix_len + block_len[s] > fs->suffix_capacity)
+                return fail(ctx, FDD_ERR_CAPACITY, "set %d: suffix %d + block %d exceeds capacity %d", s,
+                            fs->suffix_len, block_len[s], fs->suffix_capacity);
+            continue;
+        }
+        if (fs->n_forks != 1)
+            return fail(ctx, FDD_ERR_STATE, "set %d has %d rollouts: only a set of one rollout extends its prefix", s, fs->n_forks);
+        if (fs->suffix_len != 0)
+            return fail(ctx, FDD_ERR_STATE, "set %d has a private suffix of %d tokens: the prefix must stay in front of it", s, fs->suffix_len);
+        const int need = fs->prefix_len + block_len[s];
+        const bool fits = c.page_tokens == 0 ? need <= fs->prefix_capacity
+                                             : (need + c.page_tokens - 1) / c.page_tokens <= fs->prefix_capacity;
+        if (!fits)
+            return fail(ctx, FDD_ERR_CAPACITY, "set %d: prefix %d + block %d exceeds the cache (%d %s)", s, fs->prefix_len,
+                        block_len[s], fs->prefix_capacity, c.page_tokens ? "pages" : "tokens");
+        if (c.page_tokens != 0 && !fs->page_table)
+            return fail(ctx, FDD_ERR_INVALID_ARG, "set %d: a paged prefix needs its page table", s);
+    }
+    bool together = n_layers > 1;
+    if (together) {
+        // layers of one launch are copied in any order
+        size_t rows = 0;
+        for (int s = 0; s < n_sets; ++s) rows += static_cast<size_t>(sets[s]->n_forks) * block_len[s];
+        const size_t kv_bytes = rows * c.n_kv_heads * c.head_dim * sizeof(__nv_bfloat16);
+        std::vector<Range> writes, reads;
+        for (int l = 0; l < n_layers; ++l) {
+            reads.push_back(range_of(k_blk[l], kv_bytes));
+            reads.push_back(range_of(v_blk[l], kv_bytes));
+            for (int s = 0; s < n_sets; ++s) {
+                const fdd_forkset* fs = sets[s];
+                const size_t bytes = to_prefix ? prefix_cache_bytes(c, fs) : suffix_cache_bytes(c, fs);
+                writes.push_back(range_of(to_prefix ? fs->prefix_k[first_layer + l] : fs->suffix_k[first_layer + l], bytes));
+                writes.push_back(range_of(to_prefix ? fs->prefix_v[first_layer + l] : fs->suffix_v[first_layer + l], bytes));
+            }
+        }
+        together = independent(writes, reads);
+    }
+    CommitArgs a;
+    a.n = 0;
+    a.n_kv_heads = c.n_kv_heads;
+    a.vec_per_row = c.head_dim / 8;
+    a.status = ctx->d_status;
+    a.total = 0;
+    for (int l = 0; l < n_layers; ++l) {
+        const int layer = first_layer + l;
+        size_t kv_off = 0;
+        for (int s = 0; s < n_sets; ++s) {
+            const fdd_forkset* fs = sets[s];
+            CommitSet& cs = a.set[a.n++];
+            cs.k_src = static_cast<const __nv_bfloat16*>(k_blk[l]) + kv_off;
+            cs.v_src = static_cast<const __nv_bfloat16*>(v_blk[l]) + kv_off;
+            cs.n_forks = fs->n_forks;
+            cs.d = block_len[s];
+            cs.page_table = fs->page_table;
+            cs.page_tokens = c.page_tokens > 0 ? c.page_tokens : 1;
+            if (to_prefix) {
+                // the prefix caches are the caller's and read-only for every other call
+                cs.k_dst = const_cast<void*>(fs->prefix_k[layer]);
+                cs.v_dst = const_cast<void*>(fs->prefix_v[layer]);
+                cs.len = fs->prefix_len;
+                cs.cap = fs->prefix_capacity;
+                cs.mode = c.page_tokens == 0 ? kCommitPrefix : kCommitPagedPrefix;
+            } else {
+                cs.k_dst = fs->suffix_k[layer];
+                cs.v_dst = fs->suffix_v[layer];
+                cs.len = fs->suffix_len;
+                cs.cap = fs->suffix_capacity;
+                cs.mode = kCommitSuffix;
+            }
+            cs.vec_begin = a.total;
+            const size_t elems = static_cast<size_t>(fs->n_forks) * cs.d * c.n_kv_heads * c.head_dim;
+            a.total += static_cast<long long>(elems / 8);
+            kv_off += elems;
+            const bool layer_done = s + 1 == n_sets;
+            if (a.n < kCommitMaxSets && !(layer_done && (!together || l + 1 == n_layers))) continue;
+            cudaError_t e = launch_kv_commit(a, ctx->sm_count, static_cast<cudaStream_t>(stream));
+            ctx->launches += 1;
+            if (e != cudaSuccess) return cuda_fail(ctx, e, to_prefix ? "fdd_prefix_extend launch" : "fdd_kv_commit launch");
+            a.n = 0;
+            a.total = 0;
+        }
+    }
+    if (advance)
+        for (int s = 0; s < n_sets; ++s) {
+            if (to_prefix) sets[s]->prefix_len += block_len[s];
+            else sets[s]->suffix_len += block_len[s];
+        }
+    return FDD_OK;
+}
 
 extern "C" {
 
@@ -142,7 +392,8 @@ fdd_status fdd_create(const fdd_config* cfg, fdd_ctx** out) {
         const int G = cfg->n_q_heads / cfg->n_kv_heads;
         const int tile_pos = 128 / G;
         const int q_tiles = (cfg->max_block + tile_pos - 1) / tile_pos;
-        ctx->attn_max_units = cfg->n_kv_heads * q_tiles * cfg->max_forks;
+        // (a launch takes up to kTcMaxSets layers of a call)
+        ctx->attn_max_units = cfg->n_kv_heads * q_tiles * cfg->max_forks * std::min(cfg->n_layers, kTcMaxSets);
         // two counters per unit: pieces written, CTAs done with their share of the merge
         e = cudaMalloc(&ctx->attn_unit_count, sizeof(int) * 2 * ctx->attn_max_units);
         if (e == cudaSuccess) e = cudaMemset(ctx->attn_unit_count, 0, sizeof(int) * 2 * ctx->attn_max_units);
@@ -293,63 +544,7 @@ fdd_status fdd_block_attn_gated(fdd_ctx* ctx, fdd_forkset* const* sets, int n_se
                                 const void* q, const void* k_blk, const void* v_blk, void* out,
                                 const int32_t* block_len, float scale, int causal_in_block,
                                 const int32_t* gate, void* stream) {
-    CallRange range("fdd_block_attn");
-    if (!ctx) return FDD_ERR_INVALID_ARG;
-    int total = 0;
-    fdd_status st = check_sets(ctx, sets, n_sets, block_len, &total);
-    if (st != FDD_OK) return st;
-    if (!q || !k_blk || !v_blk || !out) return fail(ctx, FDD_ERR_INVALID_ARG, "q/k_blk/v_blk/out is NULL");
-    if (!aligned16(q) || !aligned16(k_blk) || !aligned16(v_blk) || (reinterpret_cast<uintptr_t>(out) & 31u) != 0)
-        return fail(ctx, FDD_ERR_INVALID_ARG, "q/k_blk/v_blk must be 16-byte aligned, out 32-byte aligned");
-    if (layer < 0 || layer >= ctx->cfg.n_layers) return fail(ctx, FDD_ERR_SHAPE, "layer %d outside [0, %d)", layer, ctx->cfg.n_layers);
-    if (!(scale > 0.0f)) return fail(ctx, FDD_ERR_INVALID_ARG, "scale must be positive");
-    if (gate && total > kAttnMaxGatedForks)
-        return fail(ctx, FDD_ERR_CAPACITY, "%d rollouts in one gated call exceed %d", total, kAttnMaxGatedForks);
-    const fdd_config& c = ctx->cfg;
-    cudaStream_t st_ = static_cast<cudaStream_t>(stream);
-    size_t q_off = 0, kv_off = 0;
-    int fork_off = 0;
-    std::vector<AttnProblem> probs;
-    std::vector<TcMapCache*> caches;
-    for (int s = 0; s < n_sets; ++s) {
-        fdd_forkset* fs = sets[s];
-        AttnProblem p;
-        p.q = static_cast<const __nv_bfloat16*>(q) + q_off;
-        p.k_blk = static_cast<const __nv_bfloat16*>(k_blk) + kv_off;
-        p.v_blk = static_cast<const __nv_bfloat16*>(v_blk) + kv_off;
-        p.out = static_cast<__nv_bfloat16*>(out) + q_off;
-        p.prefix_k = static_cast<const __nv_bfloat16*>(fs->prefix_k[layer]);
-        p.prefix_v = static_cast<const __nv_bfloat16*>(fs->prefix_v[layer]);
-        p.page_table = fs->page_table;
-        p.suffix_k = static_cast<const __nv_bfloat16*>(fs->suffix_k[layer]);
-        p.suffix_v = static_cast<const __nv_bfloat16*>(fs->suffix_v[layer]);
-        p.n_forks = fs->n_forks;
-        p.d = block_len[s];
-        p.n_q_heads = c.n_q_heads;
-        p.n_kv_heads = c.n_kv_heads;
-        p.prefix_len = fs->prefix_len;
-        p.prefix_capacity = fs->prefix_capacity;
-        p.page_tokens = c.page_tokens;
-        p.suffix_len = fs->suffix_len;
-        p.suffix_capacity = fs->suffix_capacity;
-        p.causal_in_block = causal_in_block ? 1 : 0;
-        p.scale = scale;
-        p.gate = gate ? gate + fork_off : nullptr;
-        fork_off += fs->n_forks;
-        probs.push_back(p);
-        caches.push_back(&fs->map_cache[layer]);
-        q_off += static_cast<size_t>(fs->n_forks) * p.d * c.n_q_heads * c.head_dim;
-        kv_off += static_cast<size_t>(fs->n_forks) * p.d * c.n_kv_heads * c.head_dim;
-    }
-    for (size_t first = 0; first < probs.size(); first += kTcMaxSets) {   // many scenes per launch
-        const int n = static_cast<int>(std::min<size_t>(kTcMaxSets, probs.size() - first));
-        int n_launches = 0;
-        cudaError_t e = launch_attention_ptc(ctx, probs.data() + first, caches.data() + first, n, c.head_dim, st_,
-                                             &n_launches);
-        ctx->launches += n_launches;
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "fdd_block_attn launch");
-    }
-    return FDD_OK;
+    return block_attn_layers(ctx, sets, n_sets, layer, 1, &q, &k_blk, &v_blk, &out, block_len, scale, causal_in_block, gate, stream);
 }
 
 static fdd_status unmask_like(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, const void* logits,
@@ -459,99 +654,18 @@ fdd_status fdd_ss_accept(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, con
                        n_accepted, n_left, nullptr, stream, 2);
 }
 
-// Common body of fdd_kv_commit (to_prefix = false) and fdd_prefix_extend (to_prefix = true).
-static fdd_status commit_like(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, int layer,
-                              const void* k_blk, const void* v_blk, const int32_t* block_len,
-                              int advance, void* stream, bool to_prefix) {
-    if (!ctx) return FDD_ERR_INVALID_ARG;
-    int total = 0;
-    fdd_status st = check_sets(ctx, sets, n_sets, block_len, &total);
-    if (st != FDD_OK) return st;
-    if (!k_blk || !v_blk) return fail(ctx, FDD_ERR_INVALID_ARG, "k_blk/v_blk is NULL");
-    if (!aligned16(k_blk) || !aligned16(v_blk)) return fail(ctx, FDD_ERR_INVALID_ARG, "k_blk/v_blk must be 16-byte aligned");
-    if (layer < 0 || layer >= ctx->cfg.n_layers) return fail(ctx, FDD_ERR_SHAPE, "layer %d outside [0, %d)", layer, ctx->cfg.n_layers);
-    const fdd_config& c = ctx->cfg;
-    for (int s = 0; s < n_sets; ++s) {
-        const fdd_forkset* fs = sets[s];
-        if (!to_prefix) {
-            if (fs->suffix_len + block_len[s] > fs->suffix_capacity)
-                return fail(ctx, FDD_ERR_CAPACITY, "set %d: suffix %d + block %d exceeds capacity %d", s,
-                            fs->suffix_len, block_len[s], fs->suffix_capacity);
-            continue;
-        }
-        if (fs->n_forks != 1)
-            return fail(ctx, FDD_ERR_STATE, "set %d has %d rollouts: only a set of one rollout extends its prefix", s, fs->n_forks);
-        if (fs->suffix_len != 0)
-            return fail(ctx, FDD_ERR_STATE, "set %d has a private suffix of %d tokens: the prefix must stay in front of it", s, fs->suffix_len);
-        const int need = fs->prefix_len + block_len[s];
-        const bool fits = c.page_tokens == 0 ? need <= fs->prefix_capacity
-                                             : (need + c.page_tokens - 1) / c.page_tokens <= fs->prefix_capacity;
-        if (!fits)
-            return fail(ctx, FDD_ERR_CAPACITY, "set %d: prefix %d + block %d exceeds the cache (%d %s)", s, fs->prefix_len,
-                        block_len[s], fs->prefix_capacity, c.page_tokens ? "pages" : "tokens");
-        if (c.page_tokens != 0 && !fs->page_table)
-            return fail(ctx, FDD_ERR_INVALID_ARG, "set %d: a paged prefix needs its page table", s);
-    }
-    size_t kv_off = 0;
-    for (int first = 0; first < n_sets; first += kCommitMaxSets) {
-        CommitArgs a;
-        a.n = std::min(kCommitMaxSets, n_sets - first);
-        a.n_kv_heads = c.n_kv_heads;
-        a.vec_per_row = c.head_dim / 8;
-        a.status = ctx->d_status;
-        a.total = 0;
-        for (int k = 0; k < a.n; ++k) {
-            fdd_forkset* fs = sets[first + k];
-            CommitSet& cs = a.set[k];
-            cs.k_src = static_cast<const __nv_bfloat16*>(k_blk) + kv_off;
-            cs.v_src = static_cast<const __nv_bfloat16*>(v_blk) + kv_off;
-            cs.n_forks = fs->n_forks;
-            cs.d = block_len[first + k];
-            cs.page_table = fs->page_table;
-            cs.page_tokens = c.page_tokens > 0 ? c.page_tokens : 1;
-            if (to_prefix) {
-                // the prefix caches are the caller's and read-only for every other call
-                cs.k_dst = const_cast<void*>(fs->prefix_k[layer]);
-                cs.v_dst = const_cast<void*>(fs->prefix_v[layer]);
-                cs.len = fs->prefix_len;
-                cs.cap = fs->prefix_capacity;
-                cs.mode = c.page_tokens == 0 ? kCommitPrefix : kCommitPagedPrefix;
-            } else {
-                cs.k_dst = fs->suffix_k[layer];
-                cs.v_dst = fs->suffix_v[layer];
-                cs.len = fs->suffix_len;
-                cs.cap = fs->suffix_capacity;
-                cs.mode = kCommitSuffix;
-            }
-            cs.vec_begin = a.total;
-            const size_t elems = static_cast<size_t>(fs->n_forks) * cs.d * c.n_kv_heads * c.head_dim;
-            a.total += static_cast<long long>(elems / 8);
-            kv_off += elems;
-        }
-        cudaError_t e = launch_kv_commit(a, ctx->sm_count, static_cast<cudaStream_t>(stream));
-        ctx->launches += 1;
-        if (e != cudaSuccess) return cuda_fail(ctx, e, to_prefix ? "fdd_prefix_extend launch" : "fdd_kv_commit launch");
-    }
-    if (advance)
-        for (int s = 0; s < n_sets; ++s) {
-            if (to_prefix) sets[s]->prefix_len += block_len[s];
-            else sets[s]->suffix_len += block_len[s];
-        }
-    return FDD_OK;
-}
-
 fdd_status fdd_kv_commit(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, int layer,
                          const void* k_blk, const void* v_blk, const int32_t* block_len,
                          int advance, void* stream) {
     CallRange range("fdd_kv_commit");
-    return commit_like(ctx, sets, n_sets, layer, k_blk, v_blk, block_len, advance, stream, false);
+    return commit_layers(ctx, sets, n_sets, layer, 1, &k_blk, &v_blk, block_len, advance, stream, false);
 }
 
 fdd_status fdd_prefix_extend(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, int layer,
                              const void* k_blk, const void* v_blk, const int32_t* block_len,
                              int advance, void* stream) {
     CallRange range("fdd_prefix_extend");
-    return commit_like(ctx, sets, n_sets, layer, k_blk, v_blk, block_len, advance, stream, true);
+    return commit_layers(ctx, sets, n_sets, layer, 1, &k_blk, &v_blk, block_len, advance, stream, true);
 }
 
 int fdd_forkset_prefix_len(const fdd_forkset* set) { return set ? set->prefix_len : FDD_ERR_INVALID_ARG; }

@@ -28,7 +28,7 @@ struct TcSetMaps {
     CUtensorMap pk, pv;             // contiguous: (D, P, Hkv); paged: (D, 64, Hkv, pages)
     CUtensorMap pk_tail, pv_tail;   // paged only: token dimension cut to the last page's fill
 };
-constexpr int kTcMaxSets = 16;      // scenes per attention launch
+constexpr int kTcMaxSets = 16;      // (scene, layer) pairs per attention launch
 
 // The maps last built for one (fork set, layer) and what they were built from.
 struct TcMapCache {
@@ -175,7 +175,7 @@ cudaError_t launch_attention_ptc(fdd_ctx* ctx, const AttnProblem* probs, TcMapCa
 cudaError_t launch_unmask(fdd_ctx* ctx, const UnmaskProblem& p, cudaStream_t st, int* n_launches, int mode = 0);
 // One scene's part of a cache append.
 constexpr int kCommitSuffix = 0, kCommitPrefix = 1, kCommitPagedPrefix = 2;
-constexpr int kCommitMaxSets = 16;          // scenes per append launch
+constexpr int kCommitMaxSets = 48;          // (scene, layer) pairs per append launch (4 KB of arguments)
 struct CommitSet {
     const void* k_src;       // this scene's rows of k_blk / v_blk
     const void* v_src;
@@ -203,7 +203,16 @@ inline int overlap_launch_attribute(cudaStream_t st, cudaLaunchAttribute* attr) 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     return 1;
 }
+static_assert(sizeof(CommitArgs) <= 4096, "the arguments of an append launch");
 cudaError_t launch_kv_commit(const CommitArgs& a, int sm_count, cudaStream_t st);
+// fdd_block_attn_gated and fdd_kv_commit (to_prefix: fdd_prefix_extend) of layers [first_layer, first_layer + n_layers);
+// the pointer arrays have one entry per layer.
+fdd_status block_attn_layers(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, int first_layer, int n_layers,
+                             const void* const* q, const void* const* k_blk, const void* const* v_blk, void* const* out,
+                             const int32_t* block_len, float scale, int causal_in_block, const int32_t* gate, void* stream);
+fdd_status commit_layers(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, int first_layer, int n_layers,
+                         const void* const* k_blk, const void* const* v_blk, const int32_t* block_len,
+                         int advance, void* stream, bool to_prefix);
 cudaError_t launch_average(const float* traj, int n, int w, float* out, cudaStream_t st);
 bool jmt_weights(int w, int w_out, std::vector<double>* weights);
 cudaError_t launch_average_jmt(const float* traj, int n, int w, int w_out, const double* d_weights, float* out,

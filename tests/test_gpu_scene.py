@@ -365,3 +365,59 @@ def test_library_block_loop_with_more_scenes_than_one_unmask_launch_takes():
             off += n
     finally:
         fdd.fdd_destroy(ctx)
+
+
+@pytest.mark.parametrize("layers,shared", [(2, ""), (18, ""), (50, ""), (3, "one output"), (3, "output feeds the next layer"),
+                                           (3, "one suffix cache")])
+def test_library_block_loop_does_what_calls_layer_by_layer_do(layers, shared):
+    # The layers of a step go to the GPU together where none touches what another writes, one behind the other
+    # elsewhere; either way the result is that of the calls made one by one.  50 layers take four attention launches
+    # and two appends.
+    hq, hkv, dim, vocab, n, d, prefix = 8, 2, 64, 512, 3, 16, 300
+    scale = 1.0 / np.sqrt(dim)
+
+    def decode(by_library):
+        gen = torch.Generator(device="cuda")
+        gen.manual_seed(5)
+        normal = lambda *shape: torch.randn(shape, generator=gen, device="cuda").to(torch.bfloat16)
+        ctx = fdd.fdd_create(hq, hkv, dim, vocab, layers, 0, d, n, fdd.FDD_LOGITS_BF16)
+        try:
+            pk, pv = normal(layers, hkv, prefix, dim), normal(layers, hkv, prefix, dim)
+            sk, sv = (torch.zeros((layers, n, hkv, 2 * d, dim), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+            q, out = [normal(n * d * hq * dim) for _ in range(layers)], [torch.full((n * d * hq * dim,), float("nan"), dtype=torch.bfloat16, device="cuda")
+                                                                         for _ in range(layers)]
+            k, v = [normal(n * d * hkv * dim) for _ in range(layers)], [normal(n * d * hkv * dim) for _ in range(layers)]
+            logits = 2.0 * torch.randn((n * d, vocab), generator=gen, device="cuda").to(torch.bfloat16)
+            suffix_k = [sk[0]] * layers if shared == "one suffix cache" else list(sk)
+            if shared == "one output":
+                out = [out[0]] * layers
+            elif shared == "output feeds the next layer":
+                out = q[1:] + out[-1:]
+            forkset = fdd.fdd_fork(ctx, list(pk), list(pv), None, prefix, prefix, n, [11, 12, 13], suffix_k, list(sv), 2 * d)
+            for block in range(2):
+                tokens = torch.full((n * d,), vocab - 1, dtype=torch.int32, device="cuda")
+                state = torch.full((n * d,), MASKED, dtype=torch.uint8, device="cuda")
+                state.view(n, d)[1, 4:] = fdd.FDD_COMMITTED          # this rollout is through long before the others
+                n_c, n_l = (torch.zeros(n, dtype=torch.int32, device="cuda") for _ in range(2))
+                if by_library:
+                    fdd.fdd_decode_block(ctx, [forkset], layers, d, [q], [k], [v], [out], [logits], tokens, state, [d], scale, 0, 0.9, 0.0,
+                                         block, 1, n_c, n_l)
+                    continue
+                for t in range(d):
+                    for layer in range(layers):
+                        fdd.fdd_block_attn_gated(ctx, [forkset], layer, q[layer], k[layer], v[layer], out[layer], [d], scale, 0,
+                                                 n_l if t else None)
+                    fdd.fdd_unmask(ctx, [forkset], logits, tokens, state, [d], 0.9, 0.0, block, t, n_c, n_l, None)
+                    if int(n_l.sum()) == 0:
+                        break
+                for layer in range(layers):
+                    fdd.fdd_kv_commit(ctx, [forkset], layer, k[layer], v[layer], [d], 1 if layer == layers - 1 else 0)
+            fdd.fdd_poll_status(ctx)
+            return torch.stack(out).float().cpu().numpy().astype(np.float64), tokens.cpu(), state.cpu(), sk.cpu(), sv.cpu()
+        finally:
+            fdd.fdd_destroy(ctx)
+
+    got, ref = decode(True), decode(False)
+    pu.assert_attention_close(got[0], ref[0])
+    for a, b in zip(got[1:], ref[1:]):
+        assert torch.equal(a, b)
