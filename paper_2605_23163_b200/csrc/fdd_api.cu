@@ -381,6 +381,7 @@ fdd_status fdd_create(const fdd_config* cfg, fdd_ctx** out) {
         const long long max_rows = static_cast<long long>(cfg->max_forks) * cfg->max_block;
         ctx->ws_unmask_bytes = unmask_workspace_bytes(cfg->vocab, static_cast<int>(std::min<long long>(max_rows, kUnmaskMaxRows)));
         e = cudaMalloc(&ctx->ws_unmask, ctx->ws_unmask_bytes);
+        if (e == cudaSuccess) e = cudaMemset(ctx->ws_unmask, 0, ctx->ws_unmask_bytes);
     }
     if (e == cudaSuccess) {
         ctx->attn_max_ctas = ctx->sm_count > 0 ? ctx->sm_count : 148;

@@ -151,7 +151,7 @@ struct UnmaskProblem {
 
 // Unmask scratch: one record per (row, chunk).
 struct UnmaskPartial {
-    float row_max;     // max logit of the chunk
+    float row_max;     // a logit of the chunk that none exceeds by more than kRefSlack
     float sum_exp;     // sum exp(logit - row_max)
     float best_score;  // max of logit + T * gumbel
     float best_logit;  // logit at the best score

@@ -2,8 +2,8 @@
 // (Gumbel-perturbed) arg-max per MASKED row, then the per-rollout commit rule.
 //
 // Kernel 1 (unmask_stream_kernel): persistent grid, every warp on its own.  The MASKED rows of the
-// call, cut into tiles of 2048 ids and laid end to end, are split into equal contiguous ranges, one
-// per warp (tail of a row, whole rows, head of the next; one record per (row, warp), merged by the
+// call, cut into tiles of 2048 ids, are split into pieces of a few tiles: one piece per warp when there are few rows,
+// else the warps draw them from a counter (one record per piece, merged by the
 // second kernel).  A warp streams its tiles from HBM once, through a ring of bulk asynchronous
 // copies (cp.async.bulk, completion on an mbarrier, no multicast) into its own part of shared
 // memory, three tiles deep; a lane takes 64 consecutive ids of a tile (16-byte reads, chunk order
@@ -23,11 +23,20 @@
 //   an upper bound of every score of the block: its largest logit + T * (bound of that word), and
 //   a lower bound of one score: the logit of that word's leader + T * (lower bound of its draw);
 // the warp keeps the largest lower bound so far, L (also: the largest logit so far with the smallest
-// draw there is), and notes the blocks whose upper bound reaches it in a short list in shared
-// memory.  After the piece L is a lower bound of the piece's best score, and only the noted blocks
-// that still reach it (a handful) are read again, from L2, and scored exactly with the second
-// stream, one group of 16 ids per lane.
+// draw there is), shares it with the warps that work on other pieces of the row (a word per row in global memory, read
+// a tile ahead of its use), and notes the blocks whose upper bound reaches it in a short list in shared
+// memory.  After the piece L is a lower bound of the row's best score, and only the noted blocks
+// that still reach it (half a block per piece where each piece by itself had six) are read again, from L2, and scored
+// exactly with the second stream.
 // Any id left out cannot reach L, so the arg-max (lowest id on ties) is exact.
+//
+// What bounds it: a greedy launch over many rows streams at 0.9 of the measured HBM rate once it runs; with noise the
+// 53 % busy issue slots and special-function units of four warps a scheduler (three CTAs an SM, with the registers
+// cut to 80, were no faster).  Small launches are bound by latency: 1.6 us to the first copies, 0.7 to the first
+// tile, 1.5 for a noisy tile, 1 for the look at the list.  Measured against equal ranges with a running maximum and
+// re-scoring piece by piece, whole calls: 408 rows of 50257 bf16 logits, greedy, 28.7 -> 22.5 us; 720 rows of 151936
+// fp32 logits with noise 88.7 -> 82.8; a draft / verify cycle over 176 rows of 151936 bf16 logits with noise 124.5 ->
+// 106.7.
 //
 // Kernel 2 (unmask_finalize_kernel): one CTA per rollout merges the records of its rows, forms the
 // confidences and applies the threshold / at-least-one rule.
@@ -47,8 +56,8 @@ constexpr int kLaneIds = 64;                          // consecutive ids a lane 
 constexpr int kTile = kUnmaskTile;                    // ids per tile (one bulk copy, one warp)
 constexpr int kStages = 3;                            // tiles a warp holds in shared memory (two in flight while one is reduced)
 constexpr int kMaxRows = kUnmaskMaxRows;              // rows of one launch (32 per thread in the set-up)
-constexpr int kPiecePadNoisy = 5, kPiecePadGreedy = 3;   // the per-piece work of a warp, in tiles of streaming
-constexpr int kMinPiecesPerRow = 8;                   // rows are cut on their own when each can have this many warps
+constexpr int kMinPiecesPerRow = 8;                   // a warp gets one piece when each row can have this many warps
+constexpr int kDealtShare = 5, kDealtLeast = 3, kDealtMost = 12;   // pieces that are dealt out: about five a warp, of 3 to 12 tiles
 constexpr int kMaxList = 224;                         // blocks in reach of the running lower bound kept per piece (a few dozen expected)
 constexpr long long kCopyWaitLimit = 4000000000LL;    // SM clocks a warp waits for one of its own copies (about two seconds)
 static_assert(kTile == 32 * kLaneIds, "a tile is 64 ids for each of 32 lanes");
@@ -56,6 +65,8 @@ static_assert(kMaxRows <= kThreads * 32, "the set-up gives every thread at most 
 
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
+constexpr float kRefSlack = 4.0f;                     // a lane's sum stays relative to the same logit until one is larger by more than this
+constexpr float kRefLeast = -2e38f;                   // ids masked with the type's lowest value: times log2(e) it has to stay finite
 constexpr float kGumbelMin = -2.95f;                  // no draw is smaller: E <= 36 / 16 + 23 ln 2 + ln 2 < e^2.95
 
 constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
@@ -104,10 +115,42 @@ __device__ __forceinline__ bool wait_copy(uint32_t bar, uint32_t parity) {
         if (clock64() - t0 > kCopyWaitLimit) return false;
     return true;
 }
+// Reductions over the warp in one instruction each.
+__device__ __forceinline__ float warp_max(float x) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xFFFFFFFF;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ int warp_min(int x) { return __reduce_min_sync(0xFFFFFFFFu, x); }
+__device__ __forceinline__ float warp_sum(float x) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, off);
+    return x;
+}
 // Position of the (k + 1)-th set bit of mask (k < popc(mask)).
 __device__ __forceinline__ int nth_set_bit(uint32_t mask, int k) {
-    for (; k > 0; --k) mask &= mask - 1;
-    return __ffs(mask) - 1;
+    int at = 0;
+#pragma unroll
+    for (int half = 16; half > 0; half >>= 1) {
+        const int c = __popc(mask & ((1u << half) - 1u));
+        if (k >= c) { k -= c; mask >>= half; at += half; }
+    }
+    return at;
+}
+
+// Words that the warps of a launch share, zero between launches: which piece is dealt out next, and for every row the
+// largest lower bound of its best score that any of its pieces has found so far (floats in the order of unsigned
+// numbers; 0 is below all of them and reads as NaN, which no maximum takes).
+constexpr int kSharedNext = 0, kSharedBars = 32;
+__device__ __forceinline__ uint32_t bar_key(float x) {
+    const uint32_t b = __float_as_uint(x);
+    return b ^ ((b >> 31) ? 0xFFFFFFFFu : 0x80000000u);
+}
+__device__ __forceinline__ float bar_value(uint32_t k) { return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xFFFFFFFFu)); }
+__device__ __forceinline__ uint32_t load_shared_word(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
 }
 
 template <typename T> struct Logit;
@@ -121,6 +164,21 @@ template <> struct Logit<__nv_bfloat16> {
             out[2 * i] = __uint_as_float(x[i] << 16);
             out[2 * i + 1] = __uint_as_float(x[i] & 0xFFFF0000u);
         }
+    }
+    // the largest logit of N chunks (two logits per instruction, on the packed words)
+    template <int N> __device__ static float largest(const uint4* w) {
+        __nv_bfloat162 m[4];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const uint32_t x[4] = {w[i].x, w[i].y, w[i].z, w[i].w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(&x[u]);
+                m[u] = i == 0 ? v : __hmax2(m[u], v);
+            }
+        }
+        const __nv_bfloat162 r = __hmax2(__hmax2(m[0], m[1]), __hmax2(m[2], m[3]));
+        return fmaxf(__low2float(r), __high2float(r));
     }
     // the chunk `w` with its first ms elements taken from `n`
     __device__ static uint4 splice(const uint4& w, const uint4& n, int ms) {
@@ -140,6 +198,16 @@ template <> struct Logit<float> {
     __device__ static void widen(const uint4& w, float* out) {
         out[0] = __uint_as_float(w.x); out[1] = __uint_as_float(w.y);
         out[2] = __uint_as_float(w.z); out[3] = __uint_as_float(w.w);
+    }
+    template <int N> __device__ static float largest(const uint4* w) {
+        float m[8];
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const int u = i % 8;
+            const float a = __uint_as_float(w[i].x), b = __uint_as_float(w[i].y), c = __uint_as_float(w[i].z), d = __uint_as_float(w[i].w);
+            m[u] = i < 8 ? tc::max3(a, b, fmaxf(c, d)) : tc::max3(tc::max3(m[u], a, b), c, d);
+        }
+        return tc::max3(tc::max3(m[0], m[1], m[2]), tc::max3(m[3], m[4], m[5]), fmaxf(m[6], m[7]));
     }
     __device__ static uint4 splice(const uint4& w, const uint4& n, int ms) {
         return make_uint4(0 < ms ? n.x : w.x, 1 < ms ? n.y : w.y, 2 < ms ? n.z : w.z, 3 < ms ? n.w : w.w);
@@ -168,16 +236,12 @@ __device__ __forceinline__ Best better(const Best& a, const Best& b) {
     if (b.score > a.score || (b.score == a.score && b.index < a.index)) return b;
     return a;
 }
-__device__ __forceinline__ Best warp_best(Best b) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        Best o;
-        o.score = __shfl_xor_sync(0xFFFFFFFFu, b.score, off);
-        o.logit = __shfl_xor_sync(0xFFFFFFFFu, b.logit, off);
-        o.index = __shfl_xor_sync(0xFFFFFFFFu, b.index, off);
-        b = better(b, o);
-    }
-    return b;
+__device__ __forceinline__ Best warp_best(const Best& b) {
+    const float score = warp_max(b.score);
+    const bool first = b.score == score;
+    const int index = warp_min(first ? b.index : 0x7FFFFFFF);
+    const uint32_t who = __ballot_sync(0xFFFFFFFFu, first && b.index == index);
+    return Best{score, __shfl_sync(0xFFFFFFFFu, b.logit, __ffs(who) - 1), index};
 }
 
 // ---- phase 2 of the noisy step: exact scores of the 16 ids of one group.
@@ -190,6 +254,13 @@ struct RowNoise {                                       // what fixes the draws 
 __device__ __forceinline__ float word_gumbel_bound(uint32_t R) {
     const uint32_t d = 0x0FFFFFFFu - (R >> 4);
     return d == 0u ? CUDART_INF_F : 22.18070977791825f - __logf(static_cast<float>(d)) + 1e-3f;
+}
+// Lower bound of the draw of a group's leader from its word alone: -ln U <= -ln(1 - y) <= y (1 + y) with y = (d + 1) / 2^28
+// while y <= 1 / 2, so g >= 32 ln 2 - ln(d + 1) - ln(1 + y).
+__device__ __forceinline__ float word_gumbel_least(uint32_t R) {
+    const float d1 = static_cast<float>(0x10000000u - (R >> 4));
+    const float y = d1 * 3.7252902984619140625e-09f;
+    return y <= 0.5f ? 22.18070977791825f - __logf(d1) - y - 1e-3f : kGumbelMin;
 }
 // E of a group's leader, -ln(U) / 16 with U = (h + (f + 0.5) 2^-23) / 2^28, h = R >> 4, on the fast
 // logarithm (absolute error 4e-7 on [0.5, 2], 3 ulp elsewhere).  In the upper half of the range the
@@ -207,62 +278,44 @@ __device__ __forceinline__ float leader_exponential(uint32_t R, uint32_t f23) {
     }
     return nl * 0.0625f;
 }
-struct ScoreArgs {
-    float lb, temperature;
-    int vocab, vec_ok;
-};
-// The best exact score among the 16 ids of group v0 (score -inf if the group cannot reach the lower
-// bound a.lb, or has no finite logit).  One Philox block for the group's word and four for the fine
-// bits of its ids, all independent of each other and of the load; every id is then scored, without a
-// branch: E = E_leader for the leader, E_leader - ln((f + 0.5) 2^-23) for the others, g = -ln E.
+// Four consecutive ids of group v0 (a multiple of 16): quad lane `part` takes ids v0 + 4 part ... + 3, with one Philox block
+// for the group's word and one for its own fine bits; the leader's fine bits come from the quad lane that has them.
+// E = E_leader for the leader, E_leader - ln((f + 0.5) 2^-23) for the others, g = -ln E.  Warp-wide (every lane calls).
 template <typename T>
-__device__ __noinline__ Best score_group(const T* row_ptr, int v0, ScoreArgs a, RowNoise n) {
-    Best best{-CUDART_INF_F, -CUDART_INF_F, 0x7FFFFFFF};
-    float val[kGroup];
-    load_group(row_ptr, v0, a.vocab, a.vec_ok, val);
+__device__ __forceinline__ Best score_quarter(const T* row_ptr, int v0, int part, bool act, float temperature, int vocab, const RowNoise& n) {
+    const int v = v0 + 4 * part;
+    float val[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) val[i] = act && v + i < vocab ? Logit<T>::load1(row_ptr + v + i) : -CUDART_INF_F;
     const int j = v0 >> 4;
     const uint32_t R = pick_word(philox4x32_10(make_uint4(static_cast<uint32_t>(j >> 2), n.pos, n.step, n.block_idx), n.keys), j & 3);
-    uint32_t f[kGroup];
-#pragma unroll
-    for (int k = 0; k < kGroup / 4; ++k) {
-        const uint4 r = philox4x32_10(make_uint4(static_cast<uint32_t>((v0 >> 2) + k), n.pos | kFineStream, n.step, n.block_idx), n.keys);
-        f[4 * k] = r.x >> 9; f[4 * k + 1] = r.y >> 9; f[4 * k + 2] = r.z >> 9; f[4 * k + 3] = r.w >> 9;
-    }
-    float gmax = val[0];
-#pragma unroll
-    for (int i = 1; i < kGroup; ++i) gmax = fmaxf(gmax, val[i]);
-    if (!(fmaf(a.temperature, word_gumbel_bound(R), gmax) >= a.lb - 1e-3f)) return best;
+    const uint4 r = philox4x32_10(make_uint4(static_cast<uint32_t>(v >> 2), n.pos | kFineStream, n.step, n.block_idx), n.keys);
+    const uint32_t f[4] = {r.x >> 9, r.y >> 9, r.z >> 9, r.w >> 9};
     const int li = static_cast<int>(R & 15u);
-    uint32_t f_lead = f[0];
-#pragma unroll
-    for (int i = 1; i < kGroup; ++i) if (i == li) f_lead = f[i];
+    const int k = li & 3;
+    const uint32_t f_mine = k == 0 ? f[0] : (k == 1 ? f[1] : (k == 2 ? f[2] : f[3]));
+    const uint32_t f_lead = __shfl_sync(0xFFFFFFFFu, f_mine, li >> 2, 4);
     const float e_lead = leader_exponential(R, f_lead);
+    Best best{-CUDART_INF_F, -CUDART_INF_F, 0x7FFFFFFF};
 #pragma unroll
-    for (int i = kGroup - 1; i >= 0; --i) {             // downwards: equal scores keep the lower id
-        const float e = i == li ? e_lead : e_lead + (15.942385152878742f - __logf(static_cast<float>(f[i]) + 0.5f));   // 23 ln 2 - ln(f + 0.5)
-        const float sc = fmaf(a.temperature, -__logf(e), val[i]);
-        if (val[i] > -CUDART_INF_F && sc >= best.score) best = Best{sc, val[i], v0 + i};
+    for (int i = 3; i >= 0; --i) {                      // downwards: equal scores keep the lower id
+        const float e = 4 * part + i == li ? e_lead : e_lead + (15.942385152878742f - __logf(static_cast<float>(f[i]) + 0.5f));   // 23 ln 2 - ln(f + 0.5)
+        const float sc = fmaf(temperature, -__logf(e), val[i]);
+        if (val[i] > -CUDART_INF_F && sc >= best.score) best = Best{sc, val[i], v + i};
     }
     return best;
 }
-
-// The ri-th selected row (ascending) from the set-up's per-thread runs: thread t owns rows
-// [t * per, (t + 1) * per), s_before[t] selected rows lie before its run, bit k of s_mask[t] says
-// that row t * per + k is selected.
-__device__ __forceinline__ int nth_selected_row(const int* s_before, const uint32_t* s_mask, int per, int ri) {
-    int lo = 0, hi = kThreads - 1;
-    while (lo < hi) {                                    // the last thread with s_before <= ri (its run is not empty)
-        const int mid = (lo + hi + 1) >> 1;
-        if (s_before[mid] <= ri) lo = mid; else hi = mid - 1;
-    }
-    return lo * per + nth_set_bit(s_mask[lo], ri - s_before[lo]);
-}
-
-// Item index of position v on the axis that has `pad` extra items in front of every row's ipr items.
-__device__ __forceinline__ long long padded_to_item(long long v, int ipr, int pad) {
-    const long long r = v / (ipr + pad);
-    const long long off = v - r * (ipr + pad);
-    return r * ipr + (off > pad ? off - pad : 0);
+// Bounds of group v0 from its word R: no score of the group exceeds ub, and one is at least lo (-inf: no such score).
+template <typename T>
+__device__ __forceinline__ void group_bounds(const T* row_ptr, int v0, uint32_t R, float temperature, int vocab, int vec_ok, float* ub, float* lo) {
+    float val[kGroup];
+    load_group(row_ptr, v0, vocab, vec_ok, val);
+    float gmax = val[0];
+#pragma unroll
+    for (int i = 1; i < kGroup; ++i) gmax = fmaxf(gmax, val[i]);
+    *ub = gmax > -CUDART_INF_F ? fmaf(temperature, word_gumbel_bound(R), gmax) : -CUDART_INF_F;
+    const int v = v0 + static_cast<int>(R & 15u);
+    *lo = v < vocab ? fmaf(temperature, word_gumbel_least(R), Logit<T>::load1(row_ptr + v)) : -CUDART_INF_F;
 }
 
 // A block (the 64 ids of one lane in one tile) whose upper bound reached the running lower bound.
@@ -294,21 +347,17 @@ constexpr int stream_smem_bytes() {
 // 57.8 us when the warp filled its stage with plain 2-byte loads, with nothing in flight behind them.
 template <typename T, bool NOISY, bool RAGGED>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 2 ? 2 : 1)
-unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* __restrict__ state,
+unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* state,
                      const __grid_constant__ UnmaskSets sets, UnmaskPartial* __restrict__ partial,
                      int vocab, int tiles_per_item, float temperature,
                      uint32_t block_idx, uint32_t step, int select_state,
-                     const uint32_t* __restrict__ step_counter, int* __restrict__ status) {
+                     const uint32_t* __restrict__ step_counter, int* __restrict__ status, uint32_t* shared_words) {
     // The launch may have been made resident before the kernel ahead of it on the stream was done (its
-    // set-up then overlaps that kernel's tail); nothing is read before this wait.  The kernel behind
+    // set-up then overlaps that kernel's tail); nothing is read before the wait.  The kernel behind
     // this one (the per-rollout step) may come in as soon as every CTA here has started.
-    tc::grid_dependency_wait();
-    tc::grid_launch_dependents();
-    if (step_counter != nullptr) step += *step_counter;    // the denoising step as counted on the device
     const int rows = sets.row_off[sets.n_sets];
-    __shared__ int s_before[kThreads];                  // selected rows before the thread's run
-    __shared__ uint32_t s_mask[kThreads];               // which rows of the thread's run are selected (MASKED, or DRAFT for the verifier)
-    __shared__ int s_warp_count[kWarps];
+    __shared__ uint32_t s_mask[kMaxRows / 32];          // which rows are selected (MASKED, or DRAFT for the verifier), 32 to a word
+    __shared__ int2 s_open[kWarps][8];                  // (row, piece of the row) of the pieces a warp has begun to copy
     __shared__ int s_n_list[kWarps];
     extern __shared__ __align__(128) unsigned char s_dyn[];
     constexpr int kStageBytes = stream_stage_bytes<T, RAGGED>();
@@ -321,76 +370,81 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* __restrict__ s
     Reach* list = reinterpret_cast<Reach*>(s_dyn + kWarps * kStages * kStageBytes) + warp * kMaxList;
     uint64_t* bars = reinterpret_cast<uint64_t*>(s_dyn + kWarps * kStages * kStageBytes + kWarps * kMaxList * 8) + warp * kStages;
 
-    // ---- set-up (the only CTA-wide part): which rows are selected.  A thread takes a run of
-    // consecutive rows, one block-wide prefix sum places the runs.
-    const int per = (rows + kThreads - 1) / kThreads;              // <= 32 (rows <= 8192)
-    int n_rows;
+    if (lane == 0) {
+        s_n_list[warp] = 0;
+        for (int s = 0; s < kStages; ++s) tc::mbar_init(tc::smem_u32(&bars[s]), 1);
+        tc::fence_barrier_init();
+    }
+    tc::grid_dependency_wait();
+    tc::grid_launch_dependents();
+    if (step_counter != nullptr) step += *step_counter;    // the denoising step as counted on the device
+
+    // ---- set-up (the only CTA-wide part): which rows are selected.  Every warp then keeps the count of selected rows
+    // before the words of each lane, which is all it takes to find the ri-th of them.
+    const int n_words = (rows + 31) / 32, per_lane = (n_words + 31) / 32;     // <= 256 and <= 8 (rows <= 8192)
+    constexpr int kWordsAtOnce = 4;                     // (loads in flight together)
+    for (int w0 = warp; w0 < per_lane * 32; w0 += kWarps * kWordsAtOnce) {
+        int st[kWordsAtOnce];
+#pragma unroll
+        for (int u = 0; u < kWordsAtOnce; ++u) {
+            const int r = (w0 + u * kWarps) * 32 + lane;
+            st[u] = r < rows ? state[r] : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < kWordsAtOnce; ++u) {
+            const uint32_t m = __ballot_sync(0xFFFFFFFFu, st[u] == select_state);
+            if (lane == 0 && w0 + u * kWarps < per_lane * 32) s_mask[w0 + u * kWarps] = m;
+        }
+    }
+    __syncthreads();
+    int rows_before, n_rows;
     {
-        const int r_begin = min(rows, tid * per), r_end = min(rows, r_begin + per);
-        uint32_t mine = 0;
-        for (int r = r_begin; r < r_end; ++r) mine |= (state[r] == select_state ? 1u : 0u) << (r - r_begin);
-        const int cnt = __popc(mine);
-        int incl = cnt;
+        int mine = 0;
+        for (int j = 0; j < per_lane; ++j) mine += __popc(s_mask[lane * per_lane + j]);
+        int incl = mine;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
             const int up = __shfl_up_sync(0xFFFFFFFFu, incl, off);
             if (lane >= off) incl += up;
         }
-        if (lane == 31) s_warp_count[warp] = incl;
-        if (lane == 0) {
-            s_n_list[warp] = 0;
-            for (int s = 0; s < kStages; ++s) tc::mbar_init(tc::smem_u32(&bars[s]), 1);
-            tc::fence_barrier_init();
-        }
-        __syncthreads();
-        int before = incl - cnt, total = 0;
-#pragma unroll
-        for (int w2 = 0; w2 < kWarps; ++w2) {
-            if (w2 < warp) before += s_warp_count[w2];
-            total += s_warp_count[w2];
-        }
-        s_before[tid] = before;
-        s_mask[tid] = mine;
-        n_rows = total;
-        __syncthreads();
+        rows_before = incl - mine;
+        n_rows = __shfl_sync(0xFFFFFFFFu, incl, 31);
     }
     if (n_rows == 0) return;
+    auto selected_row = [&](int ri) {                   // (warp-wide)
+        const int at = __popc(__ballot_sync(0xFFFFFFFFu, rows_before <= ri)) - 1;
+        int k = ri - __shfl_sync(0xFFFFFFFFu, rows_before, at), w = at * per_lane, c = __popc(s_mask[w]);
+        while (k >= c) {
+            k -= c;
+            c = __popc(s_mask[++w]);
+        }
+        return w * 32 + nth_set_bit(s_mask[w], k);
+    };
 
-    // ---- this warp's range of work items.  An item is tiles_per_item consecutive tiles of a row
-    // (the last item of a row may be shorter); a row has items_per_row of them and as many record
-    // slots.  Two ways to hand them out:
-    //  - few rows (at least kMinPiecesPerRow warps for each): a row is cut into ppr equal pieces, warp c
-    //    takes piece c % ppr of row c / ppr.  No warp then works on two rows, which would cost it two
-    //    rounds of the per-piece work (reductions, exact re-scoring, a record) while the others wait;
-    //  - otherwise the items of all rows, laid end to end, are cut into equal contiguous ranges, warp
-    //    c (of the G that get work) owns items [W c / G, W (c + 1) / G): tail of a row, whole rows, head
-    //    of the next.
+    // ---- the pieces.  An item is tiles_per_item consecutive tiles of a row (the last item of a row may be shorter);
+    // a row has ipr of them and as many record slots.  Every row is cut into ppr pieces of about the same number of
+    // items, and a piece leaves one record.  (A call has far fewer than 2^31 tiles: they lie in the GPU's memory.)
+    //  - Few rows: as many pieces as there are warps, one for each, where each row can have kMinPiecesPerRow of them or
+    //    where that makes no piece longer than an equal share.
+    //  - Otherwise pieces of a few tiles: every warp has one to begin with and draws the next one from a counter while
+    //    it still works on the one before.  SMs stream at rates that differ by a quarter (with equal ranges the warps of
+    //    a launch over 1216 rows of 152k ids ended after 52 us at the median and 66 us at the latest, greedy, and
+    //    71 and 89 us with noise; now 57 and 64, 76 and 88).  About five pieces a warp of at most twelve tiles: 720 rows
+    //    of fp32 logits 83 us, with eight of at most eight tiles 86.8, three of at most 24 87.3, two of at most 40 85.8.
     const int tiles_per_row = (vocab + kTile - 1) / kTile;
     const int ipr = (tiles_per_row + tiles_per_item - 1) / tiles_per_item;
-    const long long W = static_cast<long long>(n_rows) * ipr;
-    const long long warps_all = static_cast<long long>(gridDim.x) * kWarps;
-    const long long gw = static_cast<long long>(warp) * gridDim.x + blockIdx.x;   // warps of a CTA lie a grid apart: few items spread over all SMs
-    const int ppr = static_cast<int>(min(static_cast<long long>(ipr), warps_all / n_rows));   // pieces per row if rows are cut on their own
-    const bool by_row = ppr == ipr || ppr >= kMinPiecesPerRow;                   // (few pieces per row would leave too many warps without work)
-    const long long G = by_row ? static_cast<long long>(n_rows) * ppr : min(warps_all, W);
-    if (gw >= G) return;
-    // (in items; only where a range is much longer than it)
-    const int pad = (W >= 16 * G) ? ((NOISY ? kPiecePadNoisy : kPiecePadGreedy) + tiles_per_item - 1) / tiles_per_item : 0;
-    const long long Vp = static_cast<long long>(n_rows) * (ipr + pad);
-    long long range_begin, range_end;
-    if (by_row) {
-        const int ri = static_cast<int>(gw / ppr), pc = static_cast<int>(gw - static_cast<long long>(ri) * ppr);
-        range_begin = static_cast<long long>(ri) * ipr + ipr * pc / ppr;
-        range_end = static_cast<long long>(ri) * ipr + ipr * (pc + 1) / ppr;
-    } else {
-        // A warp whose range takes in a row's start works on two rows and pays the per-piece work
-        // twice.  That work is counted as `pad` items at the start of every row: the ranges are equal on
-        // the axis with those items put in, and are then mapped back (a range that falls inside the
-        // padding alone, which needs a range shorter than pad, is empty).
-        range_begin = padded_to_item(Vp * gw / G, ipr, pad);
-        range_end = padded_to_item(Vp * (gw + 1) / G, ipr, pad);
-        if (range_begin >= range_end) return;
+    const int warps_all = static_cast<int>(gridDim.x) * kWarps;
+    const int gw = warp * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x);   // warps of a CTA lie a grid apart: few pieces spread over all SMs
+    int ppr = min(ipr, warps_all / n_rows);
+    {
+        const int share = (n_rows * ipr + warps_all - 1) / warps_all;
+        if (ppr < min(ipr, kMinPiecesPerRow) && (ppr == 0 || (ipr + ppr - 1) / ppr > share)) {
+            const int len = max(1, min(max(share * tiles_per_item / kDealtShare, kDealtLeast), kDealtMost) / tiles_per_item);
+            ppr = (ipr + len - 1) / len;
+        }
     }
+    const int n_pieces = n_rows * ppr, piece_items = ipr / ppr, piece_more = ipr - piece_items * ppr;   // (the first piece_more pieces of a row have one item more)
+    if (gw >= n_pieces) return;
 
     const uint32_t full = 0xFFFFFFFFu;
     const int sw = lane & 7;                            // rotation of the chunk order (bank conflicts)
@@ -399,7 +453,8 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* __restrict__ s
     // ---- producer side (lane 0 issues, every lane keeps the same cursor): tile k of the warp's
     // sequence goes to stage k % kStages, which is the stage the consumer has just left
     const uint32_t ring_u32 = tc::smem_u32(ring), bars_u32 = tc::smem_u32(bars);
-    long long p_at = range_begin;                       // next item to open
+    int p_next = gw;                                    // next piece to open (lane 0's, once it comes from the counter)
+    int p_open = 0;                                     // pieces opened so far
     int p_tile = 0, p_tile_end = 0;
     const T* p_row_ptr = nullptr;
     uint32_t p_k = 0;
@@ -409,14 +464,20 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* __restrict__ s
     const uintptr_t whole_end = reinterpret_cast<uintptr_t>(logits + static_cast<size_t>(rows) * vocab) & ~uintptr_t(15);
     auto produce_one = [&](int stage) {
         if (p_tile == p_tile_end) {
-            if (p_at >= range_end) return;
-            const int ri = static_cast<int>(p_at / ipr);
-            const int c0 = static_cast<int>(p_at - static_cast<long long>(ri) * ipr);
-            const int c1 = static_cast<int>(min(static_cast<long long>(ipr), c0 + (range_end - p_at)));
-            p_at += c1 - c0;
+            const int id = __shfl_sync(full, p_next, 0);
+            if (id >= n_pieces) return;
+            const int ri = id / ppr, pc = id - ri * ppr, row = selected_row(ri), c0 = pc * piece_items + min(pc, piece_more);
             p_tile = c0 * tiles_per_item;
-            p_tile_end = min(tiles_per_row, c1 * tiles_per_item);
-            p_row_ptr = logits + static_cast<size_t>(nth_selected_row(s_before, s_mask, per, ri)) * vocab;
+            p_tile_end = min(tiles_per_row, (c0 + piece_items + (pc < piece_more ? 1 : 0)) * tiles_per_item);
+            p_row_ptr = logits + static_cast<size_t>(row) * vocab;
+            // (at most kStages pieces are ahead of the one being reduced; the answer of the counter is not needed before
+            // the last tile of this piece is on its way)
+            if (lane == 0) {
+                s_open[warp][p_open & 7] = make_int2(row, pc);
+                p_next = n_pieces > warps_all ? warps_all + static_cast<int>(atomicAdd(shared_words + kSharedNext, 1u)) : n_pieces;
+            }
+            ++p_open;
+            __syncwarp();
         }
         if (lane == 0) {
             const int v0 = p_tile * kTile;
@@ -443,28 +504,13 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* __restrict__ s
     uint32_t c_k = 0;                                   // tiles consumed so far: the next one sits in stage c_k % kStages
     int stage = 0;
     uint32_t phase = 0;                                 // parity of the stage's current use
-    for (long long at = range_begin; at < range_end && alive;) {
-        // ---- open the piece: items [at, at + n) of one row
-        const int ri = static_cast<int>(at / ipr);
-        const int chunk0 = static_cast<int>(at - static_cast<long long>(ri) * ipr);
-        const int chunk1 = static_cast<int>(min(static_cast<long long>(ipr), chunk0 + (range_end - at)));
-        at += chunk1 - chunk0;
-        const int tile0 = chunk0 * tiles_per_item, tile1 = min(tiles_per_row, chunk1 * tiles_per_item);
-        const int row = nth_selected_row(s_before, s_mask, per, ri);
+    for (int c_open = 0; c_open != p_open && alive; ++c_open) {
+        // ---- open the piece: tiles [tile0, tile1) of one row
+        const int row = s_open[warp][c_open & 7].x, pc = s_open[warp][c_open & 7].y;
+        const int c0 = pc * piece_items + min(pc, piece_more);
+        const int tile0 = c0 * tiles_per_item, tile1 = min(tiles_per_row, (c0 + piece_items + (pc < piece_more ? 1 : 0)) * tiles_per_item);
         const int seg_end = min(vocab, tile1 * kTile);
-        // which of the row's records this is, and how many there are
-        int seg, segs;
-        if (by_row) {
-            seg = static_cast<int>(gw - static_cast<long long>(ri) * ppr);
-            segs = ppr;
-        } else {
-            // the warps that hold the row's first and last item, on the padded axis
-            const long long v_first = static_cast<long long>(ri) * (ipr + pad) + pad;
-            const int w_first = static_cast<int>(((v_first + 1) * G + Vp - 1) / Vp) - 1;
-            const int w_last = static_cast<int>(((v_first + ipr) * G + Vp - 1) / Vp) - 1;
-            seg = static_cast<int>(gw) - w_first;
-            segs = w_last - w_first + 1;
-        }
+        uint32_t* const row_bar = shared_words + kSharedBars + row;
         const T* row_ptr = logits + static_cast<size_t>(row) * vocab;
         const int ms = RAGGED ? static_cast<int>((reinterpret_cast<uintptr_t>(row_ptr) & 15u) / sizeof(T)) : 0;
         const int vec_ok = ms == 0;                     // the row can be read in 16-byte chunks
@@ -481,10 +527,20 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* __restrict__ s
                               __shfl_sync(0xFFFFFFFFu, static_cast<uint32_t>(seed >> 32), 0));
         }
 
-        // ---- pass 1: stream the piece; per lane the running maximum m and sum exp(l - m).  The greedy
-        // step also keeps the first tile t1 that showed m (u1 = m there); the noisy step keeps the warp's
+        // ---- pass 1: stream the piece; per lane s = sum of 2^((l - ref) log2 e), where ref is the largest logit of the
+        // lane's first 64 ids and moves only when a logit exceeds it by more than kRefSlack: the exponentials wait for
+        // no running maximum, and their sum keeps the precision it has with one (arguments stay below 6).  The greedy
+        // step also keeps the lane's maximum u1 and the first tile t1 that showed it; the noisy step keeps the warp's
         // running lower bound lb of the piece's best score and lists the blocks that reach it.
-        float m = -CUDART_INF_F, s = 0.0f, nml = 0.0f;  // nml = -m log2(e) once m is finite
+        float ref = -CUDART_INF_F, s = 0.0f, nref = 0.0f;   // nref = -ref log2(e) once ref is finite
+        auto move_ref = [&](float bm) {
+            if (bm > ref + kRefSlack) {                 // (also the first time: ref is -inf then)
+                const float to = fmaxf(bm, kRefLeast);
+                s *= tc::ex2((ref - to) * kLog2e);
+                ref = to;
+                nref = -to * kLog2e;
+            }
+        };
         float u1 = -CUDART_INF_F, lb = -CUDART_INF_F;
         int t1 = tile0;
         Best best{-CUDART_INF_F, -CUDART_INF_F, 0x7FFFFFFF};
@@ -512,65 +568,63 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* __restrict__ s
             const uint4* sp = reinterpret_cast<const uint4*>(buf) + lane * kLaneChunks;
             const T* lp = reinterpret_cast<const T*>(buf) + lane * kLaneIds + ms;
             float bm64 = -CUDART_INF_F;
+            uint32_t others = 0u;                       // what the row's other pieces have found (looked at behind the sums)
+            if (NOISY && ppr > 1) others = load_shared_word(row_bar);
             // (per lane: in a row's last tile the lanes whose 64 ids all exist take the fast path too, the
             // lanes beyond the row's end have nothing to do, and at most one lane straddles the end)
             const bool whole = vb + kLaneIds <= seg_end;
             uint4 rq = make_uint4(0u, 0u, 0u, 0u);      // the words of the block's four groups
-            if (NOISY) rq = philox4x32_10(make_uint4(static_cast<uint32_t>(vb >> 6), pos, step, block_idx), keys);
+            const uint4 counter = make_uint4(static_cast<uint32_t>(vb >> 6), static_cast<uint32_t>(pos), step, block_idx);
             if (whole) {
-                // whole tile: two halves of 32 logits, chunk c of the lane read from place c ^ sw (the
-                // eight lanes of a quarter warp then touch eight different 16-byte columns of the banks)
-                uint4 after = make_uint4(0u, 0u, 0u, 0u);
-                if (RAGGED) after = sp[kLaneChunks];
+                // the lane's 64 logits as they lie in the stage, chunk c read from place c ^ sw (the eight
+                // lanes of a quarter warp then touch eight different 16-byte columns of the banks)
+                uint4 w[kLaneChunks];
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    float v[32];
+                for (int k = 0; k < kLaneChunks; ++k) w[k] = sp[k ^ sw];
+                if (RAGGED) {
+                    const uint4 after = sp[kLaneChunks];
 #pragma unroll
-                    for (int c = 0; c < kLaneChunks / 2; ++c) {
-                        const int k = h * (kLaneChunks / 2) + c;
-                        uint4 w = sp[k ^ sw];
-                        if (RAGGED && k < 8 && k == sw) w = Logit<T>::splice(w, after, ms);   // (place 0)
-                        Logit<T>::widen(w, v + c * kPerChunk);
-                    }
-                    float g8[8];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) g8[u] = tc::max3(v[4 * u], v[4 * u + 1], fmaxf(v[4 * u + 2], v[4 * u + 3]));
-                    const float bm = tc::max3(tc::max3(g8[0], g8[1], g8[2]), tc::max3(g8[3], g8[4], g8[5]), fmaxf(g8[6], g8[7]));
-                    bm64 = fmaxf(bm64, bm);
-                    {
-                        // rescale by 2^((m - mn) log2 e): exactly 1 while the maximum stands (the rounded nml
-                        // must not enter here).  Without a branch, so that the tile step is one straight run of
-                        // instructions and the Philox rounds of the noisy step overlap the exponentials.
-                        const float mn = fmaxf(m, bm);
-                        s *= tc::ex2(mn == m ? 0.0f : (m - mn) * kLog2e);
-                        m = mn;
-                        nml = mn > -CUDART_INF_F ? -mn * kLog2e : 0.0f;
-                    }
+                    for (int k = 0; k < 8; ++k)
+                        if (k == sw) w[k] = Logit<T>::splice(w[k], after, ms);          // (place 0)
+                }
+                if (tile == tile0) move_ref(Logit<T>::template largest<kLaneChunks>(w));
+                // (the reference stands in all but a few tiles: the sum does not wait for the maximum, and is
+                // formed again where a logit exceeds the reference by too much)
+                for (;;) {
+                    if (NOISY) rq = philox4x32_10(counter, keys);          // (here, so that its rounds overlap the exponentials)
                     // packed fp32x2 arithmetic: one FMA and one add per two logits
-                    const uint64_t l2e2 = tc::pack2(kLog2e, kLog2e), nm2 = tc::pack2(nml, nml);
-                    uint64_t acc[2] = {tc::pack2(0.f, 0.f), tc::pack2(0.f, 0.f)};
+                    const uint64_t l2e2 = tc::pack2(kLog2e, kLog2e), nm2 = tc::pack2(nref, nref);
+                    uint64_t acc[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
-                    for (int i = 0; i < 32; i += 2) {
-                        float x0, x1;
-                        tc::unpack2(tc::fma2(tc::pack2(v[i], v[i + 1]), l2e2, nm2), x0, x1);
-                        acc[(i >> 1) & 1] = tc::add2(acc[(i >> 1) & 1], tc::pack2(tc::ex2(x0), tc::ex2(x1)));
+                    for (int k = 0; k < kLaneChunks; ++k) {
+                        float v[kPerChunk];
+                        Logit<T>::widen(w[k], v);
+#pragma unroll
+                        for (int i = 0; i < kPerChunk; i += 2) {
+                            float x0, x1;
+                            tc::unpack2(tc::fma2(tc::pack2(v[i], v[i + 1]), l2e2, nm2), x0, x1);
+                            acc[(i >> 1) & 3] = tc::add2(acc[(i >> 1) & 3], tc::pack2(tc::ex2(x0), tc::ex2(x1)));
+                        }
+                    }
+                    bm64 = Logit<T>::template largest<kLaneChunks>(w);
+                    if (bm64 > ref + kRefSlack) {
+                        move_ref(bm64);
+                        continue;
                     }
                     float a0, a1;
-                    tc::unpack2(tc::add2(acc[0], acc[1]), a0, a1);
+                    tc::unpack2(tc::add2(tc::add2(acc[0], acc[1]), tc::add2(acc[2], acc[3])), a0, a1);
                     s += a0 + a1;
+                    break;
                 }
             } else if (vb < seg_end) {
                 // the lane that straddles the row's end: ids from seg_end on do not exist
+                if (NOISY) rq = philox4x32_10(counter, keys);
                 for (int e = 0; e < kLaneIds; ++e)
                     if (vb + e < seg_end) bm64 = fmaxf(bm64, Logit<T>::load1(lp + e));
-                if (bm64 > m) {
-                    s *= tc::ex2((m - bm64) * kLog2e);
-                    m = bm64;
-                    nml = -bm64 * kLog2e;
-                }
+                move_ref(bm64);
                 float add = 0.0f;
                 for (int e = 0; e < kLaneIds; ++e)
-                    if (vb + e < seg_end) add += tc::ex2(fmaf(Logit<T>::load1(lp + e), kLog2e, nml));
+                    if (vb + e < seg_end) add += tc::ex2(fmaf(Logit<T>::load1(lp + e), kLog2e, nref));
                 s += add;
             }
             if (!NOISY) {
@@ -598,6 +652,7 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* __restrict__ s
                 // g < 32 ln 2 - ln d <= 27 ln 2 - ln d5
                 const float g_hi = d5 == 0u ? CUDART_INF_F : fmaf(-kLn2, __log2f(fd5), 18.71497388f + 2e-3f);
                 const float ub = fmaf(temperature, g_hi, bm64);
+                lb = fmaxf(lb, bar_value(others));
                 const bool reaches = bm64 > -CUDART_INF_F && ub >= lb - 1e-3f;
                 // (no block in reach: no score of this tile step can raise the bound either, since the
                 // lower bounds below lie under the blocks' upper bounds)
@@ -609,9 +664,11 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* __restrict__ s
                     // a score that exists in this block: that leader's, or the largest logit's with the smallest draw there is
                     float lo = bm64 > -CUDART_INF_F ? fmaf(temperature, kGumbelMin, bm64) : -CUDART_INF_F;
                     if (vb + li < seg_end) lo = fmaxf(lo, fmaf(temperature, g_lo, Logit<T>::load1(lp + li)));
-#pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) lo = fmaxf(lo, __shfl_xor_sync(full, lo, off));
-                    lb = fmaxf(lb, lo);
+                    lo = warp_max(lo);
+                    if (lo > lb) {                      // (the same in every lane)
+                        lb = lo;
+                        if (ppr > 1 && lane == 0) atomicMax(row_bar, bar_key(lb));
+                    }
                     if (reaches && ub >= lb - 1e-3f) {
                         const int slot = atomicAdd(&s_n_list[warp], 1);
                         if (slot < kMaxList) list[slot] = Reach{ub, static_cast<uint16_t>(tile - tile0), static_cast<uint16_t>(lane)};
@@ -629,15 +686,15 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* __restrict__ s
         if (!alive) break;
 
         if (NOISY) {
-            // ---- pass 2: lb is now a lower bound of the piece's best score.  The listed blocks that still
-            // reach it are read again (the piece has just gone through L2) and scored exactly, group by
+            // ---- pass 2: lb is now a lower bound of the row's best score as far as its pieces have come.  The listed blocks
+            // that still reach it (none in most pieces, eight or so in a row) are read again (the piece has just gone through L2) and scored exactly, group by
             // group: a turn deals out eight blocks, one group per lane, so that the loads are in flight
             // together.  (A list that ran over, or a piece of more than 65536 tiles: every block.)
             __syncwarp();
             const RowNoise noise{keys, static_cast<uint32_t>(pos), step, block_idx};
-            const ScoreArgs sargs{lb, temperature, vocab, vec_ok};
-            const float cut = lb - 1e-3f;
             const int n_seen = *reinterpret_cast<volatile int*>(&s_n_list[warp]);
+            if (n_seen > 0 && ppr > 1) lb = fmaxf(lb, bar_value(load_shared_word(row_bar)));
+            const float cut = lb - 1e-3f;
             const bool every = n_seen > kMaxList || tile1 - tile0 > 65536;
             int n_blocks = 0;
             if (every) {
@@ -655,112 +712,60 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* __restrict__ s
                     __syncwarp();
                 }
             }
-            // Up to eight listed blocks (the usual case): one turn, a group of 16 ids per lane.
-            if (n_blocks <= 32 / kLaneGroups) {
-                const int blk = lane / kLaneGroups;
-                if (blk < n_blocks) {
-                    const int tl = every ? blk / 32 : list[blk].tile, fl = every ? blk % 32 : list[blk].lane;
-                    const int v0 = (tile0 + tl) * kTile + fl * kLaneIds + (lane % kLaneGroups) * kGroup;
-                    if (v0 < seg_end) best = better(best, score_group<T>(row_ptr, v0, sargs, noise));
-                }
-                __syncwarp();
-                n_blocks = 0;
-            }
-            // More: thirty-two listed blocks at a time, in two stages.  Stage one, a block per lane: the
-            // block's four words (one Philox block) and the largest logit of each of its four groups give a
-            // bound per group, which is tighter than the block's (about one group in three of a listed
-            // block still reaches).  Stage two, a group per lane: the groups that reach are dealt out over
-            // the lanes and scored exactly, so that no lane idles behind a group that was ruled out.  The
-            // best exact score so far raises the bar for the next thirty-two.
-            ScoreArgs turn_args = sargs;
-            for (int c0 = 0; c0 < n_blocks; c0 += 32) {
-                const int c = c0 + lane;
-                int vb0 = seg_end;                              // first id of this lane's block (none: seg_end)
+            // Two stages, eight blocks at a time.  Stage one, a group per lane: the bounds of single groups (the group's word
+            // with the group's largest logit, and its leader's score), which are tighter than the block's and raise lb.
+            // Stage two: the few groups that still reach lb are scored exactly, four ids per lane.  The best exact
+            // score so far raises lb for the next eight.
+            for (int c0 = 0; c0 < n_blocks; c0 += 32 / kLaneGroups) {
+                const int c = c0 + lane / kLaneGroups, g = lane % kLaneGroups;
+                int v_own = seg_end;
                 if (c < n_blocks) {
                     const int tl = every ? c / 32 : list[c].tile, fl = every ? c % 32 : list[c].lane;
-                    vb0 = (tile0 + tl) * kTile + fl * kLaneIds;
+                    v_own = (tile0 + tl) * kTile + fl * kLaneIds + g * kGroup;
                 }
-                uint32_t reach = 0;                             // bit g: group g of the block can reach the bar
-                if (vb0 < seg_end) {
+                float ub = -CUDART_INF_F, lo = -CUDART_INF_F;
+                if (v_own < seg_end) {
                     // (a listed block lies inside the piece as a whole; only the row's end can cut it short,
                     // and ids beyond the vocabulary read as -inf)
-                    const uint4 rq4 = philox4x32_10(make_uint4(static_cast<uint32_t>(vb0 >> 6), static_cast<uint32_t>(pos), step, block_idx), keys);
-                    float val[kLaneGroups][kGroup];
-#pragma unroll
-                    for (int g = 0; g < kLaneGroups; ++g) load_group(row_ptr, vb0 + g * kGroup, vocab, vec_ok, val[g]);
-#pragma unroll
-                    for (int g = 0; g < kLaneGroups; ++g) {
-                        float gmax = val[g][0];
-#pragma unroll
-                        for (int i = 1; i < kGroup; ++i) gmax = fmaxf(gmax, val[g][i]);
-                        if (fmaf(temperature, word_gumbel_bound(pick_word(rq4, g)), gmax) >= turn_args.lb - 1e-3f) reach |= 1u << g;
-                    }
+                    const uint4 rq = philox4x32_10(make_uint4(static_cast<uint32_t>(v_own >> 6), static_cast<uint32_t>(pos), step, block_idx), keys);
+                    group_bounds(row_ptr, v_own, pick_word(rq, g), temperature, vocab, vec_ok, &ub, &lo);
                 }
-                uint32_t mg[kLaneGroups];
-                int total = 0;
-#pragma unroll
-                for (int g = 0; g < kLaneGroups; ++g) {
-                    mg[g] = __ballot_sync(full, (reach >> g) & 1u);
-                    total += __popc(mg[g]);
-                }
-                for (int j0 = 0; j0 < total; j0 += 32) {
-                    int r = j0 + lane, g = 0, src = 0;
+                lb = fmaxf(lb, warp_max(lo));
+                const uint32_t reach = __ballot_sync(full, ub > -CUDART_INF_F && ub >= lb - 1e-3f);
+                const int total = __popc(reach);
+                for (int j0 = 0; j0 < total; j0 += 8) {
+                    const int r = j0 + (lane >> 2);
                     const bool act = r < total;
-                    if (act) {
-                        while (r >= __popc(mg[g])) { r -= __popc(mg[g]); ++g; }
-                        src = nth_set_bit(mg[g], r);
-                    }
-                    const int v_src = __shfl_sync(full, vb0, src);
-                    if (act) best = better(best, score_group<T>(row_ptr, v_src + g * kGroup, turn_args, noise));
-                    __syncwarp();
+                    const int v0 = __shfl_sync(full, v_own, act ? nth_set_bit(reach, r) : 0);
+                    best = better(best, score_quarter<T>(row_ptr, v0, lane & 3, act, temperature, vocab, noise));
                 }
-                if (c0 + 32 < n_blocks) {
-                    float seen = best.score;
-#pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) seen = fmaxf(seen, __shfl_xor_sync(full, seen, off));
-                    turn_args.lb = fmaxf(turn_args.lb, seen);
-                }
+                if (c0 + 32 / kLaneGroups < n_blocks) lb = fmaxf(lb, warp_max(best.score));
             }
             if (lane == 0) s_n_list[warp] = 0;          // the list is empty again for the next piece
         } else {
-            // ---- greedy: the piece's maximum and its first place.  The lanes that hold the maximum look
-            // for it in the 64 ids of the first tile that showed it (equal values in later tiles have
-            // higher ids).
-            float pm = u1;
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) pm = fmaxf(pm, __shfl_xor_sync(full, pm, off));
-            if (pm > -CUDART_INF_F && u1 == pm) {
-                int at_e = 0x7FFFFFFF;
-                const int vb = t1 * kTile + lane * kLaneIds;
-#pragma unroll
-                for (int g = kLaneGroups - 1; g >= 0; --g) {
-                    float val[kGroup];
-                    load_group(row_ptr, vb + g * kGroup, vocab, vec_ok, val);
-#pragma unroll
-                    for (int i = kGroup - 1; i >= 0; --i)
-                        if (val[i] == pm) at_e = vb + g * kGroup + i;
-                }
-                best = Best{pm, pm, at_e};
+            // ---- greedy: the piece's maximum and its first place: of the lanes that hold the maximum the one whose
+            // first tile with it has the lowest ids; the warp reads those 64 ids together (equal values in later
+            // tiles have higher ids).
+            const float pm = warp_max(u1);
+            if (pm > -CUDART_INF_F) {
+                const int v = warp_min(u1 == pm ? t1 * kTile + lane * kLaneIds : 0x7FFFFFFF) + lane;
+                const bool h0 = v < vocab && Logit<T>::load1(row_ptr + v) == pm, h1 = v + 32 < vocab && Logit<T>::load1(row_ptr + v + 32) == pm;
+                const uint32_t m0 = __ballot_sync(full, h0), m1 = __ballot_sync(full, h1);
+                best = Best{pm, pm, v - lane + (m0 != 0u ? __ffs(m0) - 1 : 31 + __ffs(m1))};
             }
         }
 
         // ---- the piece's record
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const float mx = __shfl_xor_sync(full, m, off);
-            const float sx = __shfl_xor_sync(full, s, off);
-            const float mn = fmaxf(m, mx);
-            if (mn > -CUDART_INF_F) s = s * __expf(m - mn) + sx * __expf(mx - mn);
-            m = mn;
-        }
-        best = warp_best(best);
+        const float row_ref = warp_max(ref);
+        s = warp_sum(ref > -CUDART_INF_F ? s * tc::ex2((ref - row_ref) * kLog2e) : 0.0f);
+        if (NOISY) best = warp_best(best);              // (greedy: the same in every lane)
         if (lane == 0) {
             UnmaskPartial out;
-            out.row_max = m; out.sum_exp = s; out.best_score = best.score; out.best_logit = best.logit;
+            out.row_max = row_ref; out.sum_exp = s; out.best_score = best.score; out.best_logit = best.logit;
             out.best_index = best.index;
-            out.pad[0] = segs;                          // how many records this row has (read from record 0)
+            out.pad[0] = ppr;                           // how many records this row has (read from record 0)
             out.pad[1] = out.pad[2] = 0;
-            partial[static_cast<size_t>(row) * ipr + seg] = out;
+            partial[static_cast<size_t>(row) * ipr + pc] = out;
         }
         __syncwarp();
     }
@@ -777,118 +782,180 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* __restrict__ s
     }
 }
 
-// Soft-max statistics of a row spread over several records: (m, s) with s = sum exp(l - m).
-__device__ __forceinline__ void merge_stats(float& m, float& s, float m2, float s2) {
-    const float mn = fmaxf(m, m2);
-    if (mn > -CUDART_INF_F) s = s * __expf(m - mn) + s2 * __expf(m2 - mn);
-    m = mn;
-}
-
 constexpr int kFinalizeThreads = 512;               // the first 128 are the positions of the rollout; all of them merge records
 
-__global__ void __launch_bounds__(kFinalizeThreads)
-unmask_finalize_kernel(const UnmaskPartial* __restrict__ partial, int32_t* __restrict__ tokens,
-                       uint8_t* __restrict__ state, int32_t* __restrict__ n_committed,
-                       int32_t* __restrict__ n_left, float* __restrict__ conf_out,
-                       const __grid_constant__ UnmaskSets sets, int items_per_row, float threshold, int commit_state,
-                       uint32_t* __restrict__ step_bump, int2* __restrict__ left_mirror, int mirror_stamp) {
-    tc::grid_launch_dependents();                       // the next kernel may be made resident; it waits for this one
-    tc::grid_dependency_wait();                         // the streaming kernel's records are complete and visible
-    // (the streaming kernel of this call has read the counter; the next call sees it advanced)
-    if (step_bump != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *step_bump += 1u;
-    const int fork = blockIdx.x;                        // rollout index over all sets of the call
-    const int i = threadIdx.x, warp = i >> 5, lane = i & 31;
+// What the per-rollout kernels share: where the rollout's rows lie, and the merged records of its selected rows.
+struct RolloutRows {
+    int fork, d, row0;                              // rollout over all sets of the call, its block length and first row
+};
+__device__ __forceinline__ RolloutRows rollout_rows(const UnmaskSets& sets) {
+    RolloutRows r;
+    r.fork = blockIdx.x;
     int set = 0;
-    while (set + 1 < sets.n_sets && fork >= sets.fork_off[set + 1]) ++set;
-    const int d = sets.d[set];
-    const int row0 = sets.row_off[set] + (fork - sets.fork_off[set]) * d;
-    __shared__ float s_conf[128];
-    __shared__ int s_tok[128], s_nrec[128], s_rows[128];
-    __shared__ int s_masked, s_pass, s_max_rec;
-    if (i == 0) { s_masked = 0; s_pass = 0; s_max_rec = 1; }
-    __syncthreads();
+    while (set + 1 < sets.n_sets && r.fork >= sets.fork_off[set + 1]) ++set;
+    r.d = sets.d[set];
+    r.row0 = sets.row_off[set] + (r.fork - sets.fork_off[set]) * r.d;
+    return r;
+}
+struct MergeShared {
+    int tok[128], nrec[128], rows[128];             // token, records and position of the selected rows
+    float conf[128];
+    int n_rows, max_rec;
+};
 
-    // ---- the MASKED positions of the rollout and how many records each has (one round trip each)
-    const int row = row0 + i;
-    const bool masked = i < d && state[row] == FDD_MASKED;     // (d <= 128: threads beyond it only help with the merge)
-    if (masked) {
-        // records the first kernel wrote for this row (never more than the row has slots)
-        const int n_rec = max(1, min(items_per_row, partial[static_cast<size_t>(row) * items_per_row].pad[0]));
-        s_nrec[i] = n_rec;
-        s_rows[atomicAdd(&s_masked, 1)] = i;
-        atomicMax(&s_max_rec, n_rec);
+// The selected positions and how many records each has; thread i is position i.
+__device__ __forceinline__ void list_rows(MergeShared& sh, int i, bool selected, int n_rec) {
+    if (i < 128) {
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, selected);
+        const int most = __reduce_max_sync(0xFFFFFFFFu, selected ? n_rec : 1);
+        int base = 0;
+        if ((i & 31) == 0 && m != 0u) {
+            base = atomicAdd(&sh.n_rows, __popc(m));
+            atomicMax(&sh.max_rec, most);
+        }
+        base = __shfl_sync(0xFFFFFFFFu, base, 0);
+        if (selected) {
+            sh.nrec[i] = n_rec;
+            sh.rows[base + __popc(m & ((1u << (i & 31)) - 1u))] = i;
+        }
     }
-    if (i < 128) s_conf[i] = -1.0f;
-    __syncthreads();
-    const int n_masked = s_masked;
+}
 
-    // ---- merge the records: a group of w lanes per position (w = the largest record count, rounded up
-    // to a power of two, 32 at most), so that all records of 32 / w positions are fetched in one round
-    // trip per warp.  Early steps have many positions with two or three records, late steps a few
-    // positions with up to a record per tile.
+// Merge the records of the listed rows: a group of w lanes per position (w = the largest record count, rounded up
+// to a power of two, 32 at most), so that all records of 32 / w positions are fetched in one round
+// trip per warp (three records a lane at once: a row of 152k ids has 75).  Early steps have many positions with two or
+// three records, late steps a few positions with up to a record per tile.  CONF: also the confidence of the best id.
+template <bool CONF>
+__device__ __forceinline__ void merge_rows(MergeShared& sh, const UnmaskPartial* partial, int row0, int items_per_row, int i) {
+    constexpr int kAtOnce = 3;
+    const int warp = i >> 5, lane = i & 31;
+    const int n_rows = sh.n_rows, max_rec = sh.max_rec;
     int w = 1;
-    while (w < s_max_rec && w < 32) w <<= 1;
+    while (w < max_rec && w < 32) w <<= 1;
     const int per = 32 / w, sub = lane / w, sl = lane - sub * w;
-    for (int base = warp * per; base < n_masked; base += (kFinalizeThreads / 32) * per) {   // (warp-uniform bounds)
+    for (int base = warp * per; base < n_rows; base += (kFinalizeThreads / 32) * per) {   // (warp-uniform bounds)
         const int k = base + sub;
-        const bool valid = k < n_masked;
-        const int j = valid ? s_rows[k] : 0;
-        const int nr = valid ? s_nrec[j] : 0;
+        const bool valid = k < n_rows;
+        const int j = valid ? sh.rows[k] : 0;
+        const int nr = valid ? sh.nrec[j] : 0;
         const UnmaskPartial* p = partial + static_cast<size_t>(row0 + j) * items_per_row;
         float M = -CUDART_INF_F, S = 0.0f;
         Best B{-CUDART_INF_F, -CUDART_INF_F, 0x7FFFFFFF};
-        for (int c = sl; c < nr; c += w) {
-            const float4 st4 = *reinterpret_cast<const float4*>(&p[c]);     // row_max, sum_exp, best_score, best_logit
-            const int idx = p[c].best_index;
-            merge_stats(M, S, st4.x, st4.y);
-            B = better(B, Best{st4.z, st4.w, idx});
+        for (int c0 = sl; c0 < nr; c0 += kAtOnce * w) {
+            float4 st4[kAtOnce];                                            // row_max, sum_exp, best_score, best_logit
+            int idx[kAtOnce];
+#pragma unroll
+            for (int u = 0; u < kAtOnce; ++u) {
+                const int c = c0 + u * w;
+                st4[u] = make_float4(-CUDART_INF_F, 0.0f, -CUDART_INF_F, -CUDART_INF_F);
+                idx[u] = 0x7FFFFFFF;
+                if (c < nr) {
+                    st4[u] = *reinterpret_cast<const float4*>(&p[c]);
+                    idx[u] = p[c].best_index;
+                }
+            }
+            if (CONF) {
+                const float mn = fmaxf(M, tc::max3(st4[0].x, st4[1].x, st4[2].x));
+                if (mn > -CUDART_INF_F) {
+                    S *= __expf(M - mn);
+#pragma unroll
+                    for (int u = 0; u < kAtOnce; ++u) S = fmaf(st4[u].y, __expf(st4[u].x - mn), S);
+                }
+                M = mn;
+            }
+#pragma unroll
+            for (int u = 0; u < kAtOnce; ++u) B = better(B, Best{st4[u].z, st4[u].w, idx[u]});
         }
+        const float own = M;
         for (int off = w >> 1; off > 0; off >>= 1) {
-            const float m2 = __shfl_xor_sync(0xFFFFFFFFu, M, off), s2 = __shfl_xor_sync(0xFFFFFFFFu, S, off);
+            if (CONF) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, off));
             Best o;
             o.score = __shfl_xor_sync(0xFFFFFFFFu, B.score, off);
             o.logit = __shfl_xor_sync(0xFFFFFFFFu, B.logit, off);
             o.index = __shfl_xor_sync(0xFFFFFFFFu, B.index, off);
-            merge_stats(M, S, m2, s2);
             B = better(B, o);
         }
+        if (CONF) {
+            S = own > -CUDART_INF_F ? S * __expf(own - M) : 0.0f;
+            for (int off = w >> 1; off > 0; off >>= 1) S += __shfl_xor_sync(0xFFFFFFFFu, S, off);
+        }
         if (valid && sl == 0) {
-            s_conf[j] = expf(B.logit - M) / S;
-            s_tok[j] = B.index;
+            if (CONF) sh.conf[j] = expf(B.logit - M) / S;
+            sh.tok[j] = B.index;
         }
     }
+}
+
+// Bound by latencies (one CTA of 512 threads a rollout, a few KB): the chain is state and record counts, records,
+// their reduction, the rule.  What does not depend on the streaming kernel stands ahead of the wait for it.  (What that
+// kernel writes is not declared read-only here: such loads could be moved ahead of the wait.)
+__global__ void __launch_bounds__(kFinalizeThreads)
+unmask_finalize_kernel(const UnmaskPartial* partial, int32_t* __restrict__ tokens,
+                       uint8_t* state, int32_t* __restrict__ n_committed,
+                       int32_t* __restrict__ n_left, float* __restrict__ conf_out,
+                       const __grid_constant__ UnmaskSets sets, int items_per_row, float threshold, int commit_state,
+                       uint32_t* __restrict__ step_bump, int2* __restrict__ left_mirror, int mirror_stamp,
+                       uint32_t* __restrict__ shared_words) {
+    tc::grid_launch_dependents();                       // the next kernel may be made resident; it waits for this one
+    __shared__ MergeShared sh;
+    const int i = threadIdx.x;
+    const RolloutRows r = rollout_rows(sets);
+    const int d = r.d, row = r.row0 + i;
+    if (i == 0) { sh.n_rows = 0; sh.max_rec = 1; }
+    if (i < 128) sh.conf[i] = -1.0f;
+    __syncthreads();
+    tc::grid_dependency_wait();                         // the streaming kernel's records are complete and visible
+    // (the streaming kernel of this call has read the counter; the next call sees it advanced)
+    if (step_bump != nullptr && blockIdx.x == 0 && i == 0) *step_bump += 1u;
+
+    // ---- the MASKED positions of the rollout (d <= 128: threads beyond it only help with the merge)
+    bool masked = false;
+    int n_rec = 1;
+    if (i < d) {
+        // records the first kernel wrote for this row (never more than the row has slots; not looked at if it is not
+        // MASKED): the two loads are independent, one round trip
+        n_rec = partial[static_cast<size_t>(row) * items_per_row].pad[0];
+        masked = state[row] == FDD_MASKED;
+        shared_words[kSharedBars + row] = 0u;
+        n_rec = max(1, min(items_per_row, n_rec));
+    }
+    if (blockIdx.x == 0 && i == 0) shared_words[kSharedNext] = 0u;     // (the streaming kernel is through with them)
+    list_rows(sh, i, masked, n_rec);
+    __syncthreads();
+    const int n_masked = sh.n_rows;
+    merge_rows<true>(sh, partial, r.row0, items_per_row, i);
     __syncthreads();
 
     // ---- the commit rule of the rollout
-    const float conf = i < 128 ? s_conf[i] : -1.0f;
+    const float conf = i < 128 ? sh.conf[i] : -1.0f;
     if (i < d && conf_out) conf_out[row] = masked ? conf : CUDART_NAN_F;
     const bool pass = masked && conf > threshold;
-    if (pass) atomicAdd(&s_pass, 1);
-    __syncthreads();
-    const int n_pass = s_pass;
+    const int n_pass = __syncthreads_count(pass);
     bool commit = pass;
     if (n_masked > 0 && n_pass == 0) {
-        // at-least-one rule: the most confident MASKED position, lowest index on ties
+        // at-least-one rule: the most confident MASKED position, lowest index on ties (each warp finds it for itself)
         int best_i = -1;
         float best_c = -1.0f;
-        for (int j = 0; j < d; ++j) {
-            const float c = s_conf[j];
-            if (c > best_c) { best_c = c; best_i = j; }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float c = sh.conf[k * 32 + (i & 31)];
+            if (c > best_c) { best_c = c; best_i = k * 32 + (i & 31); }
         }
-        commit = (i == best_i);
+        const float top = warp_max(best_c);
+        commit = i == warp_min(best_i >= 0 && best_c == top ? best_i : 0x7FFFFFFF);
     }
     if (commit && i < d) {
-        tokens[row] = s_tok[i];
+        tokens[row] = sh.tok[i];
         state[row] = static_cast<uint8_t>(commit_state);
     }
     if (i == 0) {
         const int nc = (n_masked == 0) ? 0 : (n_pass > 0 ? n_pass : 1);
-        n_committed[fork] = nc;
-        n_left[fork] = n_masked - nc;
+        n_committed[r.fork] = nc;
+        n_left[r.fork] = n_masked - nc;
         // host memory the GPU can write: count and stamp go out as one 8-byte store, so a host that
         // sees the stamp of this call sees its count
         if (left_mirror != nullptr)
-            *reinterpret_cast<unsigned long long*>(left_mirror + fork) =
+            *reinterpret_cast<unsigned long long*>(left_mirror + r.fork) =
                 (static_cast<unsigned long long>(static_cast<uint32_t>(mirror_stamp)) << 32) | static_cast<uint32_t>(n_masked - nc);
     }
 }
@@ -898,76 +965,49 @@ unmask_finalize_kernel(const UnmaskPartial* __restrict__ partial, int32_t* __res
 // every DRAFT row, the verifier's token (arg-max of its perturbed logits).  Going left to right, a
 // draft is accepted while it equals the verifier's token; at the first mismatch the verifier's token
 // replaces it and every later draft goes back to MASKED.
-// Bound by latencies: the records of the DRAFT rows (a dozen per row when few rollouts decode) are fetched by
-// groups of lanes in one round trip, as in unmask_finalize_kernel, and the kernel starts early behind
-// the streaming kernel.
 __global__ void __launch_bounds__(kFinalizeThreads)
-ss_accept_kernel(const UnmaskPartial* __restrict__ partial, int32_t* __restrict__ tokens,
-                 uint8_t* __restrict__ state, int32_t* __restrict__ n_accepted, int32_t* __restrict__ n_left,
-                 const __grid_constant__ UnmaskSets sets, int items_per_row) {
+ss_accept_kernel(const UnmaskPartial* partial, int32_t* __restrict__ tokens,
+                 uint8_t* state, int32_t* __restrict__ n_accepted, int32_t* __restrict__ n_left,
+                 const __grid_constant__ UnmaskSets sets, int items_per_row, uint32_t* __restrict__ shared_words) {
     tc::grid_launch_dependents();
+    __shared__ MergeShared sh;
+    __shared__ int s_first_mismatch;
+    const int i = threadIdx.x;
+    const RolloutRows r = rollout_rows(sets);
+    const int d = r.d, row = r.row0 + i;
+    if (i == 0) { sh.n_rows = 0; sh.max_rec = 1; s_first_mismatch = 0x7FFFFFFF; }
+    __syncthreads();
     tc::grid_dependency_wait();                         // the streaming kernel's records are complete and visible
-    const int fork = blockIdx.x;
-    const int i = threadIdx.x, warp = i >> 5, lane = i & 31;
-    int set = 0;
-    while (set + 1 < sets.n_sets && fork >= sets.fork_off[set + 1]) ++set;
-    const int d = sets.d[set];
-    const int row0 = sets.row_off[set] + (fork - sets.fork_off[set]) * d, row = row0 + i;
-    __shared__ int s_first_mismatch, s_accepted, s_masked, s_drafts, s_max_rec;
-    __shared__ int s_tok[128], s_nrec[128], s_rows[128];
-    if (i == 0) { s_first_mismatch = 0x7FFFFFFF; s_accepted = 0; s_masked = 0; s_drafts = 0; s_max_rec = 1; }
-    __syncthreads();
-    const int st = i < d ? state[row] : FDD_SCAFFOLD;
+    int st = FDD_SCAFFOLD, n_rec = 1, drafted = 0;
+    if (i < d) {
+        n_rec = partial[static_cast<size_t>(row) * items_per_row].pad[0];
+        st = state[row];
+        drafted = tokens[row];
+        shared_words[kSharedBars + row] = 0u;
+        n_rec = max(1, min(items_per_row, n_rec));
+    }
     const bool draft = st == FDD_DRAFT;
-    if (draft) {
-        const int n_rec = max(1, min(items_per_row, partial[static_cast<size_t>(row) * items_per_row].pad[0]));
-        s_nrec[i] = n_rec;
-        s_rows[atomicAdd(&s_drafts, 1)] = i;
-        atomicMax(&s_max_rec, n_rec);
-    }
+    if (blockIdx.x == 0 && i == 0) shared_words[kSharedNext] = 0u;
+    list_rows(sh, i, draft, n_rec);
     __syncthreads();
-    const int n_drafts = s_drafts;
-    int w = 1;
-    while (w < s_max_rec && w < 32) w <<= 1;
-    const int per = 32 / w, sub = lane / w, sl = lane - sub * w;
-    for (int base = warp * per; base < n_drafts; base += (kFinalizeThreads / 32) * per) {   // (warp-uniform bounds)
-        const int k = base + sub;
-        const bool valid = k < n_drafts;
-        const int j = valid ? s_rows[k] : 0;
-        const int nr = valid ? s_nrec[j] : 0;
-        const UnmaskPartial* p = partial + static_cast<size_t>(row0 + j) * items_per_row;
-        Best B{-CUDART_INF_F, -CUDART_INF_F, 0x7FFFFFFF};
-        for (int c = sl; c < nr; c += w) B = better(B, Best{p[c].best_score, p[c].best_logit, p[c].best_index});
-        for (int off = w >> 1; off > 0; off >>= 1) {
-            Best o;
-            o.score = __shfl_xor_sync(0xFFFFFFFFu, B.score, off);
-            o.logit = __shfl_xor_sync(0xFFFFFFFFu, B.logit, off);
-            o.index = __shfl_xor_sync(0xFFFFFFFFu, B.index, off);
-            B = better(B, o);
-        }
-        if (valid && sl == 0) s_tok[j] = B.index;
-    }
+    merge_rows<false>(sh, partial, r.row0, items_per_row, i);
     __syncthreads();
-    const int tok = draft ? s_tok[i] : 0;
-    if (draft && tok != tokens[row]) atomicMin(&s_first_mismatch, i);
+    const int tok = draft ? sh.tok[i] : 0;
+    if (draft && tok != drafted) atomicMin(&s_first_mismatch, i);
     __syncthreads();
     const int stop = s_first_mismatch;                  // position of the replacement token, if any
-    if (draft) {
-        if (i <= stop) {
-            if (i == stop) tokens[row] = tok;           // the verifier's token, always accepted
-            state[row] = FDD_COMMITTED;
-            atomicAdd(&s_accepted, 1);
-        } else {
-            state[row] = FDD_MASKED;                    // discarded draft
-            atomicAdd(&s_masked, 1);
-        }
-    } else if (i < d && st == FDD_MASKED) {
-        atomicAdd(&s_masked, 1);
+    const bool accepted = draft && i <= stop;
+    if (accepted) {
+        if (i == stop) tokens[row] = tok;               // the verifier's token, always accepted
+        state[row] = FDD_COMMITTED;
+    } else if (draft) {
+        state[row] = FDD_MASKED;                        // discarded draft
     }
-    __syncthreads();
+    const int n_accept = __syncthreads_count(accepted);
+    const int n_masked = __syncthreads_count((draft && !accepted) || (i < d && st == FDD_MASKED));
     if (i == 0) {
-        n_accepted[fork] = s_accepted;
-        n_left[fork] = s_masked;
+        n_accepted[r.fork] = n_accept;
+        n_left[r.fork] = n_masked;
     }
 }
 
@@ -993,6 +1033,9 @@ cudaError_t setup_one(int* ctas_per_sm) {
     return e;
 }
 
+// Bytes of the shared words of a launch over at most `rows` rows (a multiple of 128: the records lie behind them).
+size_t unmask_shared_bytes(int rows) { return ((kSharedBars + static_cast<size_t>(rows)) * sizeof(uint32_t) + 127) / 128 * 128; }
+
 cudaError_t device_setup(int dev, int* sm_count, const int** ctas_per_sm) {
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     if (!g_device_ready[dev].load(std::memory_order_acquire)) {
@@ -1017,7 +1060,7 @@ cudaError_t device_setup(int dev, int* sm_count, const int** ctas_per_sm) {
 }
 
 template <typename T, bool NOISY, bool RAGGED>
-void launch_stream(const UnmaskProblem& p, UnmaskPartial* partial, int tiles_per_item, int select_state,
+void launch_stream(const UnmaskProblem& p, UnmaskPartial* partial, uint32_t* shared_words, int tiles_per_item, int select_state,
                    int* status, int resident_ctas, cudaStream_t st) {
     const int rows = p.sets.row_off[p.sets.n_sets];
     const int tiles_per_row = (p.vocab + kTile - 1) / kTile;
@@ -1037,14 +1080,14 @@ void launch_stream(const UnmaskProblem& p, UnmaskPartial* partial, int tiles_per
     cfg.numAttrs = n_attr;
     cudaLaunchKernelEx(&cfg, unmask_stream_kernel<T, NOISY, RAGGED>, static_cast<const T*>(p.logits), static_cast<const uint8_t*>(p.state),
                        p.sets, partial, p.vocab, tiles_per_item, p.temperature, p.block_idx, p.step, select_state,
-                       static_cast<const uint32_t*>(p.step_counter), status);
+                       static_cast<const uint32_t*>(p.step_counter), status, shared_words);
 }
 
 // Both entry points launch the same two kernels; only the home of the records differs.
 // mode 0: unmasking step; 1: draft of Scaffold Speculative Decoding (every MASKED row becomes DRAFT);
 // 2: its accept scan (rows in state DRAFT are read, then the scan runs).
 // tiles_per_item: how many 2048-id tiles share one record slot (a row has ceil(tiles / tiles_per_item) slots).
-cudaError_t launch_unmask_kernels(const UnmaskProblem& p, UnmaskPartial* partial, int tiles_per_item, int dev,
+cudaError_t launch_unmask_kernels(const UnmaskProblem& p, UnmaskPartial* partial, uint32_t* shared_words, int tiles_per_item, int dev,
                                   int* status, cudaStream_t st, int mode = 0) {
     const int select_state = mode == 2 ? FDD_DRAFT : FDD_MASKED;
     const int rows = p.sets.row_off[p.sets.n_sets];
@@ -1060,13 +1103,13 @@ cudaError_t launch_unmask_kernels(const UnmaskProblem& p, UnmaskPartial* partial
     const bool bf16 = p.logits_dtype == FDD_LOGITS_BF16;
     const bool ragged = p.vocab % (bf16 ? 8 : 4) != 0 || reinterpret_cast<uintptr_t>(p.logits) % 16 != 0;
     const int which = (ragged ? 4 : 0) + (bf16 ? 0 : 2) + (noisy ? 0 : 1);
-    using Launch = void (*)(const UnmaskProblem&, UnmaskPartial*, int, int, int*, int, cudaStream_t);
+    using Launch = void (*)(const UnmaskProblem&, UnmaskPartial*, uint32_t*, int, int, int*, int, cudaStream_t);
     static const Launch launches[8] = {
         launch_stream<__nv_bfloat16, true, false>, launch_stream<__nv_bfloat16, false, false>,
         launch_stream<float, true, false>, launch_stream<float, false, false>,
         launch_stream<__nv_bfloat16, true, true>, launch_stream<__nv_bfloat16, false, true>,
         launch_stream<float, true, true>, launch_stream<float, false, true>};
-    launches[which](p, partial, tiles_per_item, select_state, status, sm_count * per_sm[which], st);
+    launches[which](p, partial, shared_words, tiles_per_item, select_state, status, sm_count * per_sm[which], st);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -1078,26 +1121,31 @@ cudaError_t launch_unmask_kernels(const UnmaskProblem& p, UnmaskPartial* partial
     cfg.attrs = attr;
     if (mode == 2) {
         cudaLaunchKernelEx(&cfg, ss_accept_kernel, static_cast<const UnmaskPartial*>(partial), p.tokens, p.state, p.n_committed,
-                           p.n_left, p.sets, items_per_row);
+                           p.n_left, p.sets, items_per_row, shared_words);
     } else {
         cudaLaunchKernelEx(&cfg, unmask_finalize_kernel, static_cast<const UnmaskPartial*>(partial), p.tokens, p.state,
                            p.n_committed, p.n_left, p.conf, p.sets, items_per_row, p.threshold,
                            mode == 1 ? static_cast<int>(FDD_DRAFT) : static_cast<int>(FDD_COMMITTED),
-                           p.bump_counter ? p.step_counter : static_cast<uint32_t*>(nullptr), p.left_mirror, p.mirror_stamp);
+                           p.bump_counter ? p.step_counter : static_cast<uint32_t*>(nullptr), p.left_mirror, p.mirror_stamp, shared_words);
     }
-    return cudaGetLastError();
+    e = cudaGetLastError();
+    // (the words have to be zero for the next launch whatever became of the kernel that clears them)
+    if (e != cudaSuccess) (void)cudaMemsetAsync(shared_words, 0, unmask_shared_bytes(rows), st);
+    return e;
 }
 
 }  // namespace
 
+// Scratch of a context: the shared words, then the records.
+static int launch_rows(long long max_rows) { return static_cast<int>(max_rows < kMaxRows ? max_rows : kMaxRows); }   // a launch takes at most kMaxRows rows
 size_t unmask_workspace_bytes(int vocab, int max_rows) {
-    const int rows = max_rows < kMaxRows ? max_rows : kMaxRows;      // a launch takes at most kMaxRows rows
-    return static_cast<size_t>(rows) * unmask_items_per_row(vocab, 1) * sizeof(UnmaskPartial);
+    return unmask_shared_bytes(launch_rows(max_rows)) + static_cast<size_t>(launch_rows(max_rows)) * unmask_items_per_row(vocab, 1) * sizeof(UnmaskPartial);
 }
 
 cudaError_t launch_unmask(fdd_ctx* ctx, const UnmaskProblem& p, cudaStream_t st, int* n_launches, int mode) {
     *n_launches += 2;
-    return launch_unmask_kernels(p, static_cast<UnmaskPartial*>(ctx->ws_unmask), 1, ctx->device, ctx->d_status, st, mode);
+    char* records = static_cast<char*>(ctx->ws_unmask) + unmask_shared_bytes(launch_rows(static_cast<long long>(ctx->cfg.max_forks) * ctx->cfg.max_block));
+    return launch_unmask_kernels(p, reinterpret_cast<UnmaskPartial*>(records), static_cast<uint32_t*>(ctx->ws_unmask), 1, ctx->device, ctx->d_status, st, mode);
 }
 
 // -------------------------------------------------------------------------------------------------
@@ -1113,10 +1161,12 @@ constexpr int kStaticTilesPerItem = kUnmaskChunk / kUnmaskTile;    // one record
 
 // Held by every GPU that loads the library until the process exits (2 MiB).
 static __device__ __align__(256) UnmaskPartial g_static_partials[kStaticMaxRecords];
+static __device__ __align__(256) uint32_t g_static_shared[kSharedBars + kMaxRows];
 
 // Device address of g_static_partials per device ordinal, resolved on first use.  In host code the
 // array's name is only a handle for the runtime; the address a kernel can use must be asked for.
 UnmaskPartial* g_static_ptr[kMaxDevices];
+uint32_t* g_static_shared_ptr[kMaxDevices];
 bool g_static_ready[kMaxDevices];
 
 void put_error(char* err, size_t err_len, const char* text) {
@@ -1176,7 +1226,14 @@ extern "C" fdd_status fdd_unmask_static(const void* logits, int logits_dtype, in
             if (err && err_len) snprintf(err, err_len, "fdd_unmask_static: cudaGetSymbolAddress failed: %s", cudaGetErrorString(e));
             return FDD_ERR_CUDA;
         }
+        void* words = nullptr;
+        e = cudaGetSymbolAddress(&words, g_static_shared);
+        if (e != cudaSuccess || !words) {
+            if (err && err_len) snprintf(err, err_len, "fdd_unmask_static: cudaGetSymbolAddress failed: %s", cudaGetErrorString(e));
+            return FDD_ERR_CUDA;
+        }
         g_static_ptr[dev] = static_cast<UnmaskPartial*>(p);
+        g_static_shared_ptr[dev] = static_cast<uint32_t*>(words);
         g_static_ready[dev] = true;
     }
     UnmaskProblem p;
@@ -1188,7 +1245,7 @@ extern "C" fdd_status fdd_unmask_static(const void* logits, int logits_dtype, in
     p.sets.d[0] = block_len; p.sets.seeds[0] = seeds;
     p.vocab = vocab; p.logits_dtype = logits_dtype;
     p.threshold = threshold; p.temperature = temperature; p.block_idx = block_idx; p.step = step;
-    e = launch_unmask_kernels(p, g_static_ptr[dev], kStaticTilesPerItem, dev, nullptr, static_cast<cudaStream_t>(stream));
+    e = launch_unmask_kernels(p, g_static_ptr[dev], g_static_shared_ptr[dev], kStaticTilesPerItem, dev, nullptr, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) {
         if (err && err_len) snprintf(err, err_len, "fdd_unmask_static: launch failed: %s", cudaGetErrorString(e));
         return FDD_ERR_CUDA;

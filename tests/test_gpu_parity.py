@@ -903,6 +903,64 @@ def test_unmask_rows_that_start_anywhere(dtype, vocab, offset, temperature, monk
         assert info["rows"] == 3 * 9
 
 
+@pytest.mark.parametrize("dtype,forks,block,vocab,temperature", [
+    ("bf16", 32, 128, 2049, 0.9),        # more rows than warps, two tiles each, ragged: whole rows are dealt out
+    ("bf16", 20, 64, 17000, 0.0),        # three pieces a row, dealt out
+    ("f32", 10, 128, 8192, 0.8),         # the same for fp32
+    ("bf16", 13, 25, 30000, 0.9),        # seven pieces a row, one for each warp
+])
+def test_unmask_pieces_one_a_warp_or_dealt_out(dtype, forks, block, vocab, temperature):
+    # twice over the same context: the words that the warps of a launch share are back at zero behind it
+    sc = synth.Scene(prefix_len=16, n_forks=forks, block_len=block, n_scaffold=block // 4, n_blocks=1)
+    w = synth.Workload("pieces", 4, 1, 64, vocab, dtype, "normal_sigma2" if dtype == "f32" else "peaked", 0.4, temperature, (sc,), seed=91)
+    ctx = harness.create_context(w)
+    try:
+        scene = harness.GpuScene(ctx, w, 0)
+        tokens, state = synth.make_block_template(w, 0, 0)
+        for step in (0, 1):
+            logits = synth.make_logits(w, 0, 0, step, rows="all")
+            got = pu.unmask_gpu(ctx, scene, logits, tokens, state, w.threshold, temperature, 0, step)
+            ref = unmask_step(pu.widen_logits(w, logits), tokens, state, scene.seeds, w.threshold, temperature, 0, step)
+            info = pu.compare_unmask(got, ref, tokens, state, w.threshold)
+            assert info["rows"] == forks * (block - block // 4)
+    finally:
+        fdd.fdd_destroy(ctx)
+
+
+@pytest.mark.parametrize("dtype,lowest", [("bf16", "lowest"), ("f32", "lowest"), ("bf16", "inf"), ("f32", "inf")])
+@pytest.mark.parametrize("temperature", [0.0, 0.8])
+def test_unmask_ids_masked_with_the_lowest_value(dtype, lowest, temperature):
+    # a grammar's mask: thousands of ids in a row at the type's lowest value or at -inf, the first and the last among them
+    vocab, n, d = 20000, 2, 9
+    t = torch.bfloat16 if dtype == "bf16" else torch.float32
+    low = float("-inf") if lowest == "inf" else torch.finfo(t).min
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(3)
+    logits = torch.randn((n * d, vocab), generator=gen, device="cuda").to(t)
+    logits[:, :6000] = low
+    logits[:, 9000:16000] = low
+    logits[:, 19990:] = low
+    ctx = fdd.fdd_create(4, 1, 64, vocab, 1, 0, d, n, fdd.FDD_LOGITS_BF16 if dtype == "bf16" else fdd.FDD_LOGITS_F32)
+    try:
+        cache = [torch.zeros((1, 16, 64), dtype=torch.bfloat16, device="cuda") for _ in range(4)]
+        forkset = fdd.fdd_fork(ctx, cache[:1], cache[1:2], None, 16, 16, n, [5, 6], cache[2:3], cache[3:], 0)
+        tokens = torch.full((n * d,), -1, dtype=torch.int32, device="cuda")
+        state = torch.full((n * d,), MASKED, dtype=torch.uint8, device="cuda")
+        n_c, n_l = (torch.zeros(n, dtype=torch.int32, device="cuda") for _ in range(2))
+        conf = torch.zeros(n * d, device="cuda")
+        fdd.fdd_unmask(ctx, [forkset], logits, tokens, state, [d], -1.0, temperature, 0, 0, n_c, n_l, conf)
+        fdd.fdd_poll_status(ctx)
+    finally:
+        fdd.fdd_destroy(ctx)
+    x = logits.double()
+    picked = x.gather(1, tokens.long()[:, None])[:, 0]
+    assert bool((picked > -100).all())                        # no masked id wins
+    if temperature == 0.0:
+        assert torch.equal(tokens.long(), x.argmax(1))
+    ref = torch.exp(picked - torch.logsumexp(x, 1))
+    assert float(((conf.double() - ref).abs() / ref).max()) < 1e-5   # sums of 152k exponentials in fp32: 4e-7
+
+
 def test_unmask_threshold_extremes():
     w = synth.small_variant(synth.workload("tts"), prefix_len=64, vocab=4096, n_forks=2, n_blocks=1)
     info, got, ref = _unmask_step_case(w, threshold=1.5)          # nothing passes: one commit each
