@@ -343,11 +343,14 @@ fdd_status fdd_average_rollouts_jmt(fdd_ctx* ctx, const float* traj, int n, int 
  *   before_step            NULL, or a function the library calls as before_step(user, t, stream)
  *                          before it issues step t: the place where a caller enqueues, on `stream`,
  *                          the model work that produces step t's q / k / v / logits
+ * Without a callback the attention of the steps runs on a stream of the context's own, beside the unmasking (unless they
+ * share memory that one of them writes); `stream` waits for it before the commits, and so does whatever
+ * the caller enqueues on `stream` after the call.
  * The counts reach the host through pinned host memory that the unmasking step writes itself
  * (count and a per-step stamp in one 8-byte store), which the call polls: no copy and no event sits
  * between two steps on the stream.  The poll is bounded: it ends with FDD_ERR_CUDA if the stream
  * reports an error or runs empty without the counts, and with FDD_ERR_DEVICE_TIMEOUT after 30 s.
- * The call returns when the counts of the last step have reached the host; the commits it issued
+ * The call returns when the counts of the last step have reached the host; the attention and the commits it issued
  * may still be running.
  * Errors as for the calls it makes; nothing is issued after the first failure.
  */

@@ -86,6 +86,7 @@ constexpr int kMaxGatedForks = kAttnMaxGatedForks;   // rollouts of one launch w
 constexpr int kMinTilesPerCta = 3;               // do not cut equal ranges finer than this (every cut costs a piece to write and merge)
 constexpr int kUnitSlack = 4;                    // tile steps by which the longest piece of a unit may exceed an equal share
 constexpr int kWholeTiles = 6;                   // units up to this long are not cut
+constexpr int kBesideSteps = 7, kBesideStepsSplit = 5;   // least steps per CTA beside other kernels (Split: probabilities in two halves)
 constexpr int kSingleSteps = 1;                  // units of one query tile while no CTA gets more than this many steps of them
 // Registers per thread after the hand-over.  The CTA starts with 384 x 168; 8 soft-max warps x
 // kRegsSoftmax + 4 other warps x kRegsOther must not exceed that (2 * 208 + 88 = 3 * 168).
@@ -1510,12 +1511,13 @@ bool cuts_by_unit(const SetParams* sets, int n, int ctas, int min_piece) {
 
 template <int MAXSETS>
 cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* const* caches, int n, int head_dim,
-                         cudaStream_t st) {
+                         cudaStream_t st, bool beside) {
     // 1-20 KB, kept off the stack in the context's own buffer (a context is used by one host thread at a time)
     if (ctx->attn_args.size() * sizeof(uint64_t) < sizeof(TcArgs<MAXSETS>)) ctx->attn_args.resize((sizeof(TcArgs<MAXSETS>) + 7) / 8);
     TcArgs<MAXSETS>& args = *reinterpret_cast<TcArgs<MAXSETS>*>(ctx->attn_args.data());
     long long pieces = 0;                                  // CTAs that the finest cut could occupy
     int units = 0, pairs = 0, forks = 0;
+    long long beside_ctas = 0;                             // CTAs with at least kBesideSteps steps each
     bool gated = false, cut = false;
     for (int s = 0; s < n; ++s) {
         const AttnProblem& a = probs[s];
@@ -1546,7 +1548,9 @@ cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* con
         pieces += static_cast<long long>(units_here) * (p.tiles_total <= kWholeTiles ? 1 : p.tiles_total);
         cut = cut || p.tiles_total > kWholeTiles;
         units += units_here;
-        pairs += a.n_kv_heads * ((p.q_tiles + 1) / 2) * a.n_forks;
+        const int pairs_here = a.n_kv_heads * ((p.q_tiles + 1) / 2) * a.n_forks;
+        pairs += pairs_here;
+        beside_ctas += static_cast<long long>(pairs_here) * std::max(1, p.tiles_total / ((p.G & (p.G - 1)) != 0 ? kBesideStepsSplit : kBesideSteps));
     }
     if (units > ctx->attn_max_units) return cudaErrorInvalidValue;
     if (gated && forks > kMaxGatedForks) return cudaErrorInvalidValue;
@@ -1558,10 +1562,15 @@ cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* con
     }();
     // one CTA per SM, fewer when there is not a piece for each
     long long ctas = pieces;
-    // short units, each with a CTA of its own: none is cut, no CTA waits for another
-    const bool waits = cut || ctas > ctx->attn_max_ctas;
     if (ctas > ctx->attn_max_ctas) ctas = ctx->attn_max_ctas;
+    // Beside other kernels SMs are worth something: a CTA spends 13 us outside its tile steps, as much as seven of them
+    // take, so it gets at least that many; half the chip a launch may have in any case, for the rollouts that are left
+    // late in a block.  (16 / 2 heads, prefix 4096, three blocks side by side with their unmasking: eight rollouts 677 ->
+    // 600 us, one rollout 323 -> 281; the launch by itself takes longer, 35 against 26 us.)
+    if (beside) ctas = std::min(ctas, std::max<long long>(ctx->attn_max_ctas / 2, beside_ctas));
     if (ctas < 1) ctas = 1;
+    // short units, each with a CTA of its own: none is cut, no CTA waits for another
+    const bool waits = cut || pieces > ctas;
     args.part_o = static_cast<float*>(ctx->ws_attn);
     args.part_lse = args.part_o + static_cast<size_t>(2) * ctx->attn_max_ctas * 256 * head_dim;
     args.unit_count = ctx->attn_unit_count;
@@ -1589,9 +1598,9 @@ size_t attention_ptc_workspace_bytes(int head_dim, int max_ctas) {
 
 // One launch for up to kTcMaxSets scenes (all with the same soft-max scale).
 cudaError_t launch_attention_ptc(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* const* caches, int n,
-                                 int head_dim, cudaStream_t st, int* n_launches) {
+                                 int head_dim, cudaStream_t st, bool beside, int* n_launches) {
     if (n < 1 || n > kTcMaxSets) return cudaErrorInvalidValue;
     *n_launches += 1;
-    if (n == 1) return launch_group<1>(ctx, probs, caches, n, head_dim, st);
-    return launch_group<kTcMaxSets>(ctx, probs, caches, n, head_dim, st);
+    if (n == 1) return launch_group<1>(ctx, probs, caches, n, head_dim, st, beside);
+    return launch_group<kTcMaxSets>(ctx, probs, caches, n, head_dim, st, beside);
 }

@@ -132,7 +132,7 @@ fdd_status check_sets(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, const 
 // to be merged.  Where a layer's output overlaps another one's output or inputs they go one behind the other.
 fdd_status block_attn_layers(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, int first_layer, int n_layers,
                              const void* const* q, const void* const* k_blk, const void* const* v_blk, void* const* out,
-                             const int32_t* block_len, float scale, int causal_in_block, const int32_t* gate, void* stream) {
+                             const int32_t* block_len, float scale, int causal_in_block, const int32_t* gate, void* stream, bool beside) {
     CallRange range("fdd_block_attn");
     if (!ctx) return FDD_ERR_INVALID_ARG;
     int total = 0;
@@ -225,7 +225,7 @@ fdd_status block_attn_layers(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets,
             while (n < most && first + n < count && (n == 0 || !gate || forks + probs[first + n].n_forks <= kAttnMaxGatedForks))
                 forks += probs[first + n++].n_forks;
             int n_launches = 0;
-            cudaError_t e = launch_attention_ptc(ctx, probs.data() + first, caches.data() + first, n, c.head_dim, st_, &n_launches);
+            cudaError_t e = launch_attention_ptc(ctx, probs.data() + first, caches.data() + first, n, c.head_dim, st_, beside, &n_launches);
             ctx->launches += n_launches;
             if (e != cudaSuccess) return cuda_fail(ctx, e, "fdd_block_attn launch");
             first += n;
@@ -234,6 +234,54 @@ fdd_status block_attn_layers(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets,
         caches.clear();
     }
     return FDD_OK;
+}
+
+bool attention_beside_unmasking(const fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, int n_layers, int n_inputs,
+                                const void* const* q, const void* const* k_blk, const void* const* v_blk, void* const* out,
+                                const void* const* logits, const int32_t* tokens, const uint8_t* state, const int32_t* block_len,
+                                const int32_t* n_committed, const int32_t* n_left) {
+    if (!block_len) return false;
+    const fdd_config& c = ctx->cfg;
+    size_t rows = 0, forks = 0;
+    for (int s = 0; s < n_sets; ++s) {
+        if (!set_alive(ctx, sets[s])) return false;
+        rows += static_cast<size_t>(sets[s]->n_forks) * block_len[s];
+        forks += sets[s]->n_forks;
+    }
+    const size_t q_bytes = rows * c.n_q_heads * c.head_dim * sizeof(__nv_bfloat16), kv_bytes = rows * c.n_kv_heads * c.head_dim * sizeof(__nv_bfloat16);
+    // the unmasking's ranges are few: every range of the attention is held against them
+    const std::vector<Range> written = {range_of(tokens, rows * sizeof(int32_t)), range_of(state, rows),
+                                        range_of(n_committed, forks * sizeof(int32_t)), range_of(n_left, forks * sizeof(int32_t))};
+    std::vector<Range> touched = written;
+    for (int i = 0; i < n_inputs; ++i)
+        if (i == 0 || logits[i] != logits[i - 1]) touched.push_back(range_of(logits[i], rows * c.vocab * (c.logits_dtype == FDD_LOGITS_BF16 ? 2 : 4)));
+    const auto apart = [](const std::vector<Range>& set, const Range& r) {
+        for (const Range& x : set)
+            if (x.lo < r.hi && r.lo < x.hi) return false;
+        return true;
+    };
+    for (int i = 0; i < n_inputs * n_layers; ++i) {
+        // (what the attention refuses it has to refuse before anything of the step is issued)
+        if (!q[i] || !k_blk[i] || !v_blk[i] || !out[i] || !aligned16(q[i]) || !aligned16(k_blk[i]) || !aligned16(v_blk[i]) ||
+            (reinterpret_cast<uintptr_t>(out[i]) & 31u) != 0)
+            return false;
+        const int before = i - n_layers;               // (a caller that reuses its buffers passes the same row again)
+        if ((before < 0 || out[i] != out[before]) && !apart(touched, range_of(out[i], q_bytes))) return false;
+        if ((before < 0 || q[i] != q[before]) && !apart(written, range_of(q[i], q_bytes))) return false;
+        if ((before < 0 || k_blk[i] != k_blk[before]) && !apart(written, range_of(k_blk[i], kv_bytes))) return false;
+        if ((before < 0 || v_blk[i] != v_blk[before]) && !apart(written, range_of(v_blk[i], kv_bytes))) return false;
+    }
+    for (int s = 0; s < n_sets; ++s) {
+        const fdd_forkset* fs = sets[s];
+        const size_t pb = prefix_cache_bytes(c, fs), sb = suffix_cache_bytes(c, fs);
+        for (int l = 0; l < n_layers; ++l)
+            if (!apart(written, range_of(fs->prefix_k[l], pb)) || !apart(written, range_of(fs->prefix_v[l], pb)) ||
+                !apart(written, range_of(fs->suffix_k[l], sb)) || !apart(written, range_of(fs->suffix_v[l], sb)))
+                return false;
+        if (c.page_tokens > 0 && !apart(written, range_of(fs->page_table, sizeof(int32_t) * ((static_cast<size_t>(fs->prefix_len) + c.page_tokens - 1) / c.page_tokens))))
+            return false;
+    }
+    return true;
 }
 
 // Common body of fdd_kv_commit (to_prefix = false) and fdd_prefix_extend (to_prefix = true), for consecutive layers.
@@ -399,6 +447,10 @@ fdd_status fdd_create(const fdd_config* cfg, fdd_ctx** out) {
         e = cudaMalloc(&ctx->attn_unit_count, sizeof(int) * 2 * ctx->attn_max_units);
         if (e == cudaSuccess) e = cudaMemset(ctx->attn_unit_count, 0, sizeof(int) * 2 * ctx->attn_max_units);
     }
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->gate_slots, sizeof(int32_t) * kGateSlots * static_cast<size_t>(cfg->max_forks));
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking);
+    for (cudaEvent_t* ev : {&ctx->ev_gate[0], &ctx->ev_gate[1], &ctx->ev_end})
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     if (e != cudaSuccess) {
         fdd_destroy(ctx);
         return FDD_ERR_CUDA;
@@ -422,6 +474,10 @@ void fdd_destroy(fdd_ctx* ctx) {
     if (ctx->ws_unmask) cudaFree(ctx->ws_unmask);
     if (ctx->ws_attn) cudaFree(ctx->ws_attn);
     if (ctx->attn_unit_count) cudaFree(ctx->attn_unit_count);
+    if (ctx->gate_slots) cudaFree(ctx->gate_slots);
+    for (cudaEvent_t ev : {ctx->ev_gate[0], ctx->ev_gate[1], ctx->ev_end})
+        if (ev) cudaEventDestroy(ev);
+    if (ctx->side_stream) cudaStreamDestroy(ctx->side_stream);
     delete static_cast<SeedChunk*>(ctx->seed_chunk);
     delete ctx;
 }
@@ -607,6 +663,7 @@ static fdd_status unmask_like(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets
         p.bump_counter = (step_counter != nullptr && s == n_sets) ? 1 : 0;      // the last group of the call advances it
         p.left_mirror = (mode == 0 && ctx->unmask_left_mirror) ? ctx->unmask_left_mirror + fork_off : nullptr;
         p.mirror_stamp = ctx->unmask_mirror_stamp;
+        p.gate_out = (mode == 0 && ctx->unmask_gate_out) ? ctx->unmask_gate_out + fork_off : nullptr;
         int n_launches = 0;
         cudaError_t e = launch_unmask(ctx, p, static_cast<cudaStream_t>(stream), &n_launches, mode);
         ctx->launches += n_launches;

@@ -72,6 +72,11 @@ struct fdd_ctx {
     std::vector<uint64_t> attn_args;  // host buffer for the attention kernel's argument block (8-byte aligned)
     long long attn_merge_wait_limit = 4000000000LL;   // SM clocks (about two seconds): wait for the pieces of a cut unit
     void* seed_chunk = nullptr;       // host staging of seeds on their way to the device as kernel arguments
+    // fdd_decode_block runs the attention of its steps on a stream of its own, beside the unmasking (decode_loop.cu)
+    cudaStream_t side_stream = nullptr;
+    cudaEvent_t ev_gate[2] = {nullptr, nullptr}, ev_end = nullptr;
+    int32_t* gate_slots = nullptr;    // device [kGateSlots][max_forks]: what every step left, for the attention of the next one
+    int32_t* unmask_gate_out = nullptr;   // where fdd_unmask puts n_left a second time (nullptr: nowhere)
     uint64_t launches = 0;
     std::string last_error;
     std::vector<fdd_forkset*> live_sets;
@@ -118,6 +123,7 @@ struct AttnProblem {
     const int32_t* gate;           // device [N], 0 = leave the rollout out; nullptr = all take part
 };
 
+constexpr int kGateSlots = 130;             // steps whose counts fdd_decode_block keeps (a block has at most 128 positions)
 constexpr int kJmtMaxWaypoints = 32;        // decoded waypoints per rollout the interpolation takes
 constexpr int kJmtMaxOutputs = 256;         // interpolated waypoints
 constexpr int kAttnMaxGatedForks = 2048;    // rollouts of one fdd_block_attn_gated call
@@ -147,6 +153,7 @@ struct UnmaskProblem {
     int bump_counter = 0;               // increment it once this launch pair is done
     int2* left_mirror = nullptr;        // host memory mapped for the device, [forks], or nullptr: (n_left, mirror_stamp) is written there too
     int mirror_stamp = 0;
+    int32_t* gate_out = nullptr;        // device [forks] or nullptr: n_left goes there too
 };
 
 // Unmask scratch: one record per (row, chunk).
@@ -171,7 +178,7 @@ size_t unmask_workspace_bytes(int vocab, int max_rows);
 
 size_t attention_ptc_workspace_bytes(int head_dim, int max_ctas);
 cudaError_t launch_attention_ptc(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* const* caches, int n,
-                                 int head_dim, cudaStream_t st, int* n_launches);
+                                 int head_dim, cudaStream_t st, bool beside, int* n_launches);
 cudaError_t launch_unmask(fdd_ctx* ctx, const UnmaskProblem& p, cudaStream_t st, int* n_launches, int mode = 0);
 // One scene's part of a cache append.
 constexpr int kCommitSuffix = 0, kCommitPrefix = 1, kCommitPagedPrefix = 2;
@@ -206,13 +213,19 @@ inline int overlap_launch_attribute(cudaStream_t st, cudaLaunchAttribute* attr) 
 static_assert(sizeof(CommitArgs) <= 4096, "the arguments of an append launch");
 cudaError_t launch_kv_commit(const CommitArgs& a, int sm_count, cudaStream_t st);
 // fdd_block_attn_gated and fdd_kv_commit (to_prefix: fdd_prefix_extend) of layers [first_layer, first_layer + n_layers);
-// the pointer arrays have one entry per layer.
+// the pointer arrays have one entry per layer.  beside: other kernels run at the same time.
 fdd_status block_attn_layers(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, int first_layer, int n_layers,
                              const void* const* q, const void* const* k_blk, const void* const* v_blk, void* const* out,
-                             const int32_t* block_len, float scale, int causal_in_block, const int32_t* gate, void* stream);
+                             const int32_t* block_len, float scale, int causal_in_block, const int32_t* gate, void* stream, bool beside = false);
 fdd_status commit_layers(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, int first_layer, int n_layers,
                          const void* const* k_blk, const void* const* v_blk, const int32_t* block_len,
                          int advance, void* stream, bool to_prefix);
+// Whether the attention of a block loop's steps and its unmasking share no memory but what both only read, and the
+// attention's pointers are in order (rows of inputs as for fdd_decode_block).
+bool attention_beside_unmasking(const fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, int n_layers, int n_inputs,
+                                const void* const* q, const void* const* k_blk, const void* const* v_blk, void* const* out,
+                                const void* const* logits, const int32_t* tokens, const uint8_t* state, const int32_t* block_len,
+                                const int32_t* n_committed, const int32_t* n_left);
 cudaError_t launch_average(const float* traj, int n, int w, float* out, cudaStream_t st);
 bool jmt_weights(int w, int w_out, std::vector<double>* weights);
 cudaError_t launch_average_jmt(const float* traj, int n, int w, int w_out, const double* d_weights, float* out,

@@ -895,7 +895,7 @@ unmask_finalize_kernel(const UnmaskPartial* partial, int32_t* __restrict__ token
                        int32_t* __restrict__ n_left, float* __restrict__ conf_out,
                        const __grid_constant__ UnmaskSets sets, int items_per_row, float threshold, int commit_state,
                        uint32_t* __restrict__ step_bump, int2* __restrict__ left_mirror, int mirror_stamp,
-                       uint32_t* __restrict__ shared_words) {
+                       uint32_t* __restrict__ shared_words, int32_t* __restrict__ gate_out) {
     tc::grid_launch_dependents();                       // the next kernel may be made resident; it waits for this one
     __shared__ MergeShared sh;
     const int i = threadIdx.x;
@@ -952,6 +952,7 @@ unmask_finalize_kernel(const UnmaskPartial* partial, int32_t* __restrict__ token
         const int nc = (n_masked == 0) ? 0 : (n_pass > 0 ? n_pass : 1);
         n_committed[r.fork] = nc;
         n_left[r.fork] = n_masked - nc;
+        if (gate_out != nullptr) gate_out[r.fork] = n_masked - nc;
         // host memory the GPU can write: count and stamp go out as one 8-byte store, so a host that
         // sees the stamp of this call sees its count
         if (left_mirror != nullptr)
@@ -1126,7 +1127,7 @@ cudaError_t launch_unmask_kernels(const UnmaskProblem& p, UnmaskPartial* partial
         cudaLaunchKernelEx(&cfg, unmask_finalize_kernel, static_cast<const UnmaskPartial*>(partial), p.tokens, p.state,
                            p.n_committed, p.n_left, p.conf, p.sets, items_per_row, p.threshold,
                            mode == 1 ? static_cast<int>(FDD_DRAFT) : static_cast<int>(FDD_COMMITTED),
-                           p.bump_counter ? p.step_counter : static_cast<uint32_t*>(nullptr), p.left_mirror, p.mirror_stamp, shared_words);
+                           p.bump_counter ? p.step_counter : static_cast<uint32_t*>(nullptr), p.left_mirror, p.mirror_stamp, shared_words, p.gate_out);
     }
     e = cudaGetLastError();
     // (the words have to be zero for the next launch whatever became of the kernel that clears them)

@@ -421,3 +421,50 @@ def test_library_block_loop_does_what_calls_layer_by_layer_do(layers, shared):
     pu.assert_attention_close(got[0], ref[0])
     for a, b in zip(got[1:], ref[1:]):
         assert torch.equal(a, b)
+
+
+def test_library_block_loop_leaves_the_stream_behind_its_attention():
+    # The attention may run on a stream of its own: what the caller enqueues after the call still comes behind it, and
+    # what the call refuses it refuses before anything of the step has happened.
+    hq, hkv, dim, vocab, n, d, prefix = 16, 2, 128, 512, 4, 32, 4000
+    scale = 1.0 / np.sqrt(dim)
+    ctx = fdd.fdd_create(hq, hkv, dim, vocab, 1, 0, d, n, fdd.FDD_LOGITS_BF16)
+    try:
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            gen = torch.Generator(device="cuda")
+            gen.manual_seed(6)
+            normal = lambda *shape: torch.randn(shape, generator=gen, device="cuda").to(torch.bfloat16)
+            pk, pv = normal(hkv, prefix, dim), normal(hkv, prefix, dim)
+            sk, sv = (torch.zeros((n, hkv, d, dim), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+            forkset = fdd.fdd_fork(ctx, [pk], [pv], None, prefix, prefix, n, [1, 2, 3, 4], [sk], [sv], d)
+            q, k, v = normal(n * d * hq * dim), normal(n * d * hkv * dim), normal(n * d * hkv * dim)
+            logits = 2.0 * normal(n * d, vocab)
+            ref = torch.zeros_like(q)
+            fdd.fdd_block_attn(ctx, [forkset], 0, q, k, v, ref, [d], scale, 0)
+            tokens = torch.full((n * d,), -1, dtype=torch.int32, device="cuda")
+            state = torch.full((n * d,), MASKED, dtype=torch.uint8, device="cuda")
+            n_c, n_l = (torch.zeros(n, dtype=torch.int32, device="cuda") for _ in range(2))
+            odd = torch.zeros(q.numel() + 1, dtype=torch.bfloat16, device="cuda")[1:]
+            launches = fdd.fdd_launch_count(ctx)
+            for bad in (dict(q=odd), dict(out=odd), dict(scale=0.0)):
+                with pytest.raises(fdd.FddError) as ei:
+                    fdd.fdd_decode_block(ctx, [forkset], 1, d, [[bad.get("q", q)]], [[k]], [[v]], [[bad.get("out", ref)]], [logits], tokens,
+                                         state, [d], bad.get("scale", scale), 0, 0.9, 0.0, 0, 0, n_c, n_l)
+                assert ei.value.status == fdd.FDD_ERR_INVALID_ARG
+            assert fdd.fdd_launch_count(ctx) == launches and bool((state == MASKED).all())
+            for _ in range(10):
+                qq, out = q.clone(), torch.zeros_like(q)
+                state.fill_(MASKED)
+                fdd.fdd_decode_block(ctx, [forkset], 1, d, [[qq]], [[k]], [[v]], [[out]], [logits], tokens, state, [d], scale, 0, 0.9, 0.0,
+                                     0, 0, n_c, n_l)
+                got = out.clone()                          # behind the last step's attention
+                qq.zero_()                                 # and so is this
+                out.zero_()
+                stream.synchronize()
+                assert bool((got != 0).any(dim=0).any())
+                pu.assert_attention_close(got.float().cpu().numpy().astype(np.float64), ref.float().cpu().numpy().astype(np.float64))
+                assert not bool(out.any())
+        fdd.fdd_poll_status(ctx)
+    finally:
+        fdd.fdd_destroy(ctx)
