@@ -26,6 +26,12 @@
 // 1.5 until the last piece is seen, 4 for the merge).  Measured, launches one behind the other (equal ranges ->
 // pieces by unit): one rollout, prefix 4096: 24.6 -> 18.5-20 us; eight rollouts: 33-36 -> 27-29 us; 28 / 4
 // heads, six rollouts, prefix 3001: 41 -> 35 us; a block of 36 layers with eight rollouts: 6.3 -> 5.3 ms.
+// Few units: clusters.  The pieces of a unit are the CTAs of a cluster of 16 or 8; each leaves its output in its own
+// shared memory (over the operand tiles), and behind a barrier of the cluster every CTA merges its share of the rows out
+// of all of them: no scratch, no counters, no cooperative launch; writing a piece, publishing it, waiting and
+// merging take 3 us instead of 7.5.  Seven clusters of 16 or 15 of 8 fit on the chip (one CTA per SM), so this is for
+// up to 15 units.  Launches one behind the other, 16 / 2 heads, pieces by unit -> clusters: one rollout, prefix
+// 4096 18.5 -> 14.9 us, prefix 12000 24.6 -> 18.7; two rollouts 20.5 -> 16.2; four 22.4 -> 21.6.
 // These launches also initialise their barriers ahead of the wait for the kernel before them and keep the scenes'
 // sizes in shared memory; a launch with more units than CTAs lost 2-3 % by the same (a block at 32 rollouts,
 // prefix 16384: 1815-1850 us against 1770-1790), so it does neither.  TMEM is taken behind the wait everywhere.
@@ -85,6 +91,7 @@ constexpr long long kWaitLimit = 4000000000LL;   // about two seconds of SM cloc
 constexpr int kMaxGatedForks = kAttnMaxGatedForks;   // rollouts of one launch when any scene has a gate
 constexpr int kMinTilesPerCta = 3;               // do not cut equal ranges finer than this (every cut costs a piece to write and merge)
 constexpr int kUnitSlack = 4;                    // tile steps by which the longest piece of a unit may exceed an equal share
+constexpr int kClusterSizes[2] = {16, 8};        // CTAs of a cluster
 constexpr int kWholeTiles = 6;                   // units up to this long are not cut
 constexpr int kBesideSteps = 7, kBesideStepsSplit = 5;   // least steps per CTA beside other kernels (Split: probabilities in two halves)
 constexpr int kSingleSteps = 1;                  // units of one query tile while no CTA gets more than this many steps of them
@@ -126,6 +133,7 @@ struct TcArgs {
     int* status;
     int min_tiles;             // do not cut the work into ranges shorter than this
     int min_piece;             // nor a unit into pieces shorter than this
+    int cluster_size, cluster_unit;   // units in clusters: CTAs of a cluster (pieces of a unit), query tiles of a unit
     int n_sets;
     float scale_log2;
     long long merge_wait_limit; // SM clocks a CTA waits for the other pieces of a cut unit before it gives up
@@ -449,10 +457,67 @@ __device__ __forceinline__ void plan(const TcArgs<MAXSETS>& a, const SetParams* 
     }
 }
 
-template <int D, int MAXSETS, int EMU, int MODE, bool BYUNIT>
+// Merge of a unit whose pieces lie in the shared memory of the CTAs of a cluster (piece k in CTA k): CT float4 columns of
+// one row, out = sum_k 2^(m_k - M) O_k / sum_k 2^(m_k - M) l_k.  All reads of eight pieces are in flight together.
+template <int D, int CT>
+__device__ __forceinline__ void merge_cluster(uint32_t part, uint32_t ml, int n_pieces, int row, int col0, __nv_bfloat16* op) {
+    constexpr int kAtOnce = 8;
+    float4 acc[CT];
+#pragma unroll
+    for (int c = 0; c < CT; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+    float M = -CUDART_INF_F, wsum = 0.0f;
+    for (int k0 = 0; k0 < n_pieces; k0 += kAtOnce) {
+        float2 st[kAtOnce];
+        float4 ov[kAtOnce][CT];
+#pragma unroll
+        for (int k = 0; k < kAtOnce; ++k) {
+            const uint32_t rank = min(k0 + k, n_pieces - 1);
+            const uint32_t from = tc::cluster_addr(part, rank);
+            st[k] = tc::cluster_ld2(tc::cluster_addr(ml, rank) + row * 8);
+#pragma unroll
+            for (int c = 0; c < CT; ++c) ov[k][c] = tc::cluster_ld4(from + ((col0 + c) * 256 + row) * 16);
+        }
+        float mn = M;
+#pragma unroll
+        for (int k = 0; k < kAtOnce; ++k)
+            if (k0 + k < n_pieces) mn = fmaxf(mn, st[k].x);
+        if (!(mn > -CUDART_INF_F)) continue;                        // nothing but pieces without a visible key so far
+        const float back = exp2f(M - mn);
+        wsum *= back;
+#pragma unroll
+        for (int c = 0; c < CT; ++c) { acc[c].x *= back; acc[c].y *= back; acc[c].z *= back; acc[c].w *= back; }
+        M = mn;
+#pragma unroll
+        for (int k = 0; k < kAtOnce; ++k) {
+            if (k0 + k >= n_pieces || st[k].x == -CUDART_INF_F) continue;
+            const float w = exp2f(st[k].x - M);
+            wsum = fmaf(w, st[k].y, wsum);
+#pragma unroll
+            for (int c = 0; c < CT; ++c) {
+                acc[c].x = fmaf(w, ov[k][c].x, acc[c].x); acc[c].y = fmaf(w, ov[k][c].y, acc[c].y);
+                acc[c].z = fmaf(w, ov[k][c].z, acc[c].z); acc[c].w = fmaf(w, ov[k][c].w, acc[c].w);
+            }
+        }
+    }
+    const float iw = wsum > 0.0f ? 1.0f / wsum : 0.0f;
+#pragma unroll
+    for (int c = 0; c < CT; ++c) {
+        const __nv_bfloat162 b0 = __floats2bfloat162_rn(acc[c].x * iw, acc[c].y * iw), b1 = __floats2bfloat162_rn(acc[c].z * iw, acc[c].w * iw);
+        *reinterpret_cast<uint2*>(op + (col0 + c) * 4) =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&b0), *reinterpret_cast<const uint32_t*>(&b1));
+    }
+}
+
+// How a launch is cut (see the top of the file).
+constexpr int kEqualRanges = 0, kByUnit = 1, kByCluster = 2;
+
+template <int D, int MAXSETS, int EMU, int MODE, int CUT>
 __global__ void __launch_bounds__(kTcThreads, 1)
 attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
     using Shape = TcShape<D>;
+    constexpr bool BYUNIT = CUT != kEqualRanges;        // (or by equal ranges, if the gate leaves nothing better)
+    constexpr bool CLUSTERED = CUT == kByCluster;
+    static_assert(!CLUSTERED || MAXSETS == 1, "units in clusters: one scene");
     constexpr int kStages = Shape::kStages;
     constexpr bool kOwn = MODE == kOwnScoresSplit;      // every query tile has a score buffer of its own, probabilities in two halves
     static_assert(EMU % 8 == 0 && EMU >= 0 && EMU <= 128, "EMU: emulated exponentials per 128-key tile");
@@ -479,6 +544,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
     __shared__ long long step_base_s[MAXSETS + 1];
     __shared__ Layout layout_s;
     __shared__ SetParams sets_s[BYUNIT ? MAXSETS : 1];
+    __shared__ float2 row_ml_s[CLUSTERED ? 256 : 1];    // reference maximum and row sum of this CTA's piece
     const SetParams* const sets = BYUNIT ? sets_s : a.sets;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -549,11 +615,22 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
         if (lane == 0) n_act_s[s] = cnt;
     }
     __syncthreads();
-    if (warp == 0) plan<MAXSETS, BYUNIT>(a, sets, n_act_s, step_base_s, unit_base_s, cta_base_s, pieces_s, &layout_s, lane);
+    if (!CLUSTERED && warp == 0) plan<MAXSETS, BYUNIT>(a, sets, n_act_s, step_base_s, unit_base_s, cta_base_s, pieces_s, &layout_s, lane);
     if (BYUNIT) tc::fence_before_sync();
     __syncthreads();
     if (BYUNIT) tc::fence_after_sync();
-    const Layout lay = layout_s;
+    Layout lay;
+    if (CLUSTERED) {
+        // a cluster per unit, a piece per CTA (all CTAs of a cluster take the same way here)
+        const SetParams& p = sets[0];
+        lay.per_unit = a.cluster_unit;
+        const int per_head = lay.per_unit == 2 ? (p.q_tiles + 1) / 2 : p.q_tiles;
+        lay.ctas = p.n_kv_heads * n_act_s[0] * per_head * a.cluster_size;
+        lay.T = lay.ctas;
+        lay.by_unit = 1;
+    } else {
+        lay = layout_s;
+    }
     const int per_unit = BYUNIT ? lay.per_unit : 2;
     const bool by_unit = BYUNIT && lay.by_unit > 0;
     const long long T = lay.T;
@@ -570,14 +647,21 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
         tc::fence_after_sync();
     }
     long long range_begin, range_end;
+    Item own = {0, 0, 0, 0, 0};                         // by unit: the CTA's only item
     if (by_unit) {
         int s = 0;
-        while (s + 1 < a.n_sets && static_cast<int>(blockIdx.x) >= cta_base_s[s + 1]) ++s;
-        const int rel = static_cast<int>(blockIdx.x) - cta_base_s[s], unit = rel / pieces_s[s], piece = rel - unit * pieces_s[s];
+        if (!CLUSTERED)
+            while (s + 1 < a.n_sets && static_cast<int>(blockIdx.x) >= cta_base_s[s + 1]) ++s;
+        const int pieces = CLUSTERED ? a.cluster_size : pieces_s[s];
+        const int rel = static_cast<int>(blockIdx.x) - (CLUSTERED ? 0 : cta_base_s[s]), piece = rel % pieces;
         const int tiles = sets[s].tiles_total;
-        const long long unit_begin = step_base_s[s] + static_cast<long long>(unit) * tiles;
-        range_begin = unit_begin + tiles * piece / pieces_s[s];
-        range_end = unit_begin + tiles * (piece + 1) / pieces_s[s];
+        own.s = s;
+        own.unit = rel / pieces;
+        own.t0 = tiles * piece / pieces;
+        own.t1 = tiles * (piece + 1) / pieces;
+        own.unit_begin = (CLUSTERED ? 0 : step_base_s[s]) + static_cast<long long>(own.unit) * tiles;
+        range_begin = own.unit_begin + own.t0;
+        range_end = own.unit_begin + own.t1;
     } else {
         range_begin = T * blockIdx.x / C;
         range_end = T * (blockIdx.x + 1) / C;
@@ -599,7 +683,8 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
     };
     auto view_item = [&](long long pos) {
         ItemView v;
-        v.it = locate<kOwn>(a, sets, step_base_s, pos, range_end);
+        if (by_unit) v.it = own;
+        else v.it = locate<kOwn>(a, sets, step_base_s, pos, range_end);
         const SetParams& p = sets[v.it.s];
         int idx = v.it.unit;
         const int n_act = n_act_s[v.it.s];
@@ -871,6 +956,11 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
             }
         }
         // (warp 11 has nothing to do but to have given up its registers)
+        if (CLUSTERED) {
+            __syncwarp();
+            tc::cluster_sync();                          // every piece of the unit lies in its CTA's shared memory
+            tc::cluster_sync();                          // and has been read
+        }
     } else {
         tc::reg_alloc<kRegsSoftmax>();
         // ---------------------------------------------------------------------- soft-max groups
@@ -1079,6 +1169,31 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
             }
 
             // ---------------------------------------------------------------- epilogue
+            if (CLUSTERED) {
+                // the piece goes over the operand tiles, column-major ([D / 4 float4 columns][256 rows]), once the products of
+                // both query tiles have read them
+                tc::named_barrier(1, 256);
+                if (active && ok) {
+                    float4* po = reinterpret_cast<float4*>(smem) + q * 128 + row_local;
+#pragma unroll
+                    for (int cc = 0; cc < D / 32; ++cc) {
+                        uint32_t o[32];
+                        tc::tmem_ld32(tm_o[q] + lane_base + cc * 32, o);
+                        tc::wait_ld();
+#pragma unroll
+                        for (int v4 = 0; v4 < 8; ++v4)
+                            po[(cc * 8 + v4) * 256] = make_float4(__uint_as_float(o[v4 * 4]), __uint_as_float(o[v4 * 4 + 1]),
+                                                                  __uint_as_float(o[v4 * 4 + 2]), __uint_as_float(o[v4 * 4 + 3]));
+                    }
+                }
+                // (a row that saw no key in this piece has a sum of 0 and counts for nothing)
+                row_ml_s[q * 128 + row_local] = make_float2(l == 0.0f ? -CUDART_INF_F : m_used, l);
+                if (!ok) {
+                    if (*abort_flag == 0) atomicCAS(a.status, 0, FDD_ERR_DEVICE_TIMEOUT);
+                    *abort_flag = 1;
+                }
+                break;
+            }
             int c_first, n_pieces;                              // CTA of the unit's first step, CTAs that hold a piece of it
             if (by_unit) {
                 n_pieces = pieces_s[it.s];
@@ -1258,6 +1373,34 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
             pos += nt;
         }
 
+        if (CLUSTERED) {
+            // Every CTA of the cluster merges an equal share of the unit's rows out of all their shared memories.  (A CTA
+            // that gave up has set the status and takes part all the same: nobody waits for ever.)
+            __syncwarp();
+            tc::cluster_sync();
+            const SetParams& p = sets[0];
+            const ItemView v = view_item(range_begin);
+            const int n_pieces = a.cluster_size, rank = static_cast<int>(blockIdx.x) % n_pieces;
+            const int rows_here = min(per_unit * p.tile_rows, p.d * p.G - v.tile0 * p.tile_rows);
+            const int row_lo = rows_here * rank / n_pieces, share = rows_here * (rank + 1) / n_pieces - row_lo;   // <= 128
+            int col_groups = 1;                                        // a power of two, share * col_groups <= 256
+            while (col_groups < D / 4 && share * col_groups * 2 <= 256) col_groups *= 2;
+            const int cg = share > 0 ? tid / share : col_groups, rc = row_lo + tid - cg * share;
+            if (cg < col_groups) {
+                const int rowu = rc < p.tile_rows ? rc : rc - p.tile_rows + 128;     // (without the gap behind a tile's last row)
+                const int pos2 = rc / p.G, qi2 = v.tile0 * p.tile_pos + pos2, qg2 = rc - pos2 * p.G;
+                __nv_bfloat16* op = p.out + ((static_cast<size_t>(v.f) * p.d + qi2) * p.n_q_heads + v.h * p.G + qg2) * D;
+                const uint32_t ml = tc::smem_u32(row_ml_s);
+                const int ct = (D / 4) / col_groups;
+                if (ct == 1) {
+                    merge_cluster<D, 1>(q_s, ml, n_pieces, rowu, cg, op);
+                } else {
+                    for (int c = 0; c < ct; c += 2) merge_cluster<D, 2>(q_s, ml, n_pieces, rowu, cg * ct + c, op);
+                }
+            }
+            __syncwarp();
+            tc::cluster_sync();
+        } else {
         // ------------------------------------------------------------ merges of the cut units
         // Every CTA that holds a piece of a unit (in more than two pieces) merges an equal share of
         // the unit's rows, once all pieces are there.  (All CTAs of the launch are resident at once:
@@ -1333,6 +1476,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                         }
             }
         }
+        }   // not in clusters
     }
 
     tc::fence_before_sync();
@@ -1430,7 +1574,7 @@ int emulated_exponentials() {
     return value;
 }
 
-template <int D, int MAXSETS, int EMU, int MODE, bool BYUNIT>
+template <int D, int MAXSETS, int EMU, int MODE, int CUT>
 cudaError_t launch_one(const TcArgs<MAXSETS>& args, unsigned ctas, bool waits, int device, cudaStream_t st) {
     const int smem = TcShape<D>::kSmemBytes;
     // the kernel's shared-memory size is a per-device attribute: set on the first launch on each device
@@ -1438,7 +1582,8 @@ cudaError_t launch_one(const TcArgs<MAXSETS>& args, unsigned ctas, bool waits, i
     static std::atomic<bool> configured[kMaxDevices];
     if (device < 0 || device >= kMaxDevices) return cudaErrorInvalidDevice;
     if (!configured[device].load(std::memory_order_acquire)) {
-        cudaError_t e = cudaFuncSetAttribute(attn_ptc_kernel<D, MAXSETS, EMU, MODE, BYUNIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t e = cudaFuncSetAttribute(attn_ptc_kernel<D, MAXSETS, EMU, MODE, CUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess && CUT == kByCluster) e = cudaFuncSetAttribute(attn_ptc_kernel<D, MAXSETS, EMU, MODE, CUT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
         configured[device].store(true, std::memory_order_release);
     }
@@ -1454,9 +1599,16 @@ cudaError_t launch_one(const TcArgs<MAXSETS>& args, unsigned ctas, bool waits, i
     cfg.blockDim = dim3(kTcThreads);
     cfg.dynamicSmemBytes = static_cast<size_t>(smem);
     cfg.stream = st;
-    const void* fn = reinterpret_cast<const void*>(&attn_ptc_kernel<D, MAXSETS, EMU, MODE, BYUNIT>);
+    const void* fn = reinterpret_cast<const void*>(&attn_ptc_kernel<D, MAXSETS, EMU, MODE, CUT>);
     cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
+    if (CUT == kByCluster) {
+        // the CTAs of a cluster are resident together by construction, and no cluster waits for another
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim = {static_cast<unsigned>(args.cluster_size), 1, 1};
+        cfg.numAttrs = 1 + overlap_launch_attribute(st, attr + 1);
+        return cudaLaunchKernelExC(&cfg, fn, params);
+    }
     if (!waits) {
         cfg.numAttrs = overlap_launch_attribute(st, attr);
         return cudaLaunchKernelExC(&cfg, fn, params);
@@ -1474,19 +1626,19 @@ cudaError_t launch_one(const TcArgs<MAXSETS>& args, unsigned ctas, bool waits, i
     return cudaLaunchKernelExC(&cfg, fn, params);
 }
 
-template <int MAXSETS, bool BYUNIT>
+template <int MAXSETS, int CUT>
 cudaError_t launch_shape(const TcArgs<MAXSETS>& args, int head_dim, unsigned ctas, bool waits, int device, cudaStream_t st) {
     const int G = args.sets[0].G;                          // (the same for every scene of a context)
     if ((G & (G - 1)) != 0) {
         // Groups that are not a power of two keep 16 bits of every probability (see the top of the file).
-        if (head_dim == 64) return launch_one<64, MAXSETS, 0, kOwnScoresSplit, BYUNIT>(args, ctas, waits, device, st);
-        return launch_one<128, MAXSETS, 0, kOwnScoresSplit, BYUNIT>(args, ctas, waits, device, st);
+        if (head_dim == 64) return launch_one<64, MAXSETS, 0, kOwnScoresSplit, CUT>(args, ctas, waits, device, st);
+        return launch_one<128, MAXSETS, 0, kOwnScoresSplit, CUT>(args, ctas, waits, device, st);
     }
-    if (head_dim == 64) return launch_one<64, MAXSETS, 0, kSharedScores, BYUNIT>(args, ctas, waits, device, st);
+    if (head_dim == 64) return launch_one<64, MAXSETS, 0, kSharedScores, CUT>(args, ctas, waits, device, st);
     switch (emulated_exponentials()) {
-        case 16: return launch_one<128, MAXSETS, 16, kSharedScores, BYUNIT>(args, ctas, waits, device, st);
-        case 32: return launch_one<128, MAXSETS, 32, kSharedScores, BYUNIT>(args, ctas, waits, device, st);
-        default: return launch_one<128, MAXSETS, 0, kSharedScores, BYUNIT>(args, ctas, waits, device, st);
+        case 16: return launch_one<128, MAXSETS, 16, kSharedScores, CUT>(args, ctas, waits, device, st);
+        case 32: return launch_one<128, MAXSETS, 32, kSharedScores, CUT>(args, ctas, waits, device, st);
+        default: return launch_one<128, MAXSETS, 0, kSharedScores, CUT>(args, ctas, waits, device, st);
     }
 }
 
@@ -1507,6 +1659,68 @@ bool cuts_by_unit(const SetParams* sets, int n, int ctas, int min_piece) {
         if (need <= ctas) return true;
     }
     return false;
+}
+
+// Clusters of kClusterSizes CTAs (one per SM) that a device holds at a time; asked for once per device.
+const int* resident_clusters(int device) {
+    constexpr int kMaxDevices = 64;
+    static std::atomic<bool> known[kMaxDevices];
+    static int most[kMaxDevices][2];
+    static const int none[2] = {0, 0};
+    if (device < 0 || device >= kMaxDevices) return none;
+    if (!known[device].load(std::memory_order_acquire)) {
+        auto kernel = attn_ptc_kernel<128, 1, 0, kSharedScores, kByCluster>;
+        const int smem = TcShape<128>::kSmemBytes;
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        for (int i = 0; i < 2; ++i) {
+            int n = 0;
+            cudaLaunchAttribute attr;
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim = {static_cast<unsigned>(kClusterSizes[i]), 1, 1};
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(static_cast<unsigned>(kClusterSizes[i]));
+            cfg.blockDim = dim3(kTcThreads);
+            cfg.dynamicSmemBytes = static_cast<size_t>(smem);
+            cfg.attrs = &attr;
+            cfg.numAttrs = 1;
+            if (e != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+                (void)cudaGetLastError();
+                n = 0;
+            }
+            most[device][i] = n;
+        }
+        known[device].store(true, std::memory_order_release);
+    }
+    return most[device];
+}
+
+// Whether the units of a launch over one scene go to clusters, of how many CTAs, and whether a unit has one query tile or
+// two: what takes least time by a fit to measured launches (nanoseconds; launches one behind the other, 16 / 2 heads,
+// prefix 1000 to 12000, one to eight rollouts).  Clusters of other sizes took 4 to 10 us more than the fit, whatever the
+// number of steps, and are not used.
+bool unit_clusters(const SetParams& p, int ctas, const int* resident, int* size, int* unit) {
+    if (p.tiles_total <= kWholeTiles) return false;
+    const int heads_forks = p.n_kv_heads * p.n_forks, pair_units = heads_forks * ((p.q_tiles + 1) / 2);
+    const int single_step = 1250, pair_step = 1650, step = p.q_tiles == 1 ? single_step : pair_step;
+    long long best = 18700 + static_cast<long long>(step) * ((static_cast<long long>(pair_units) * p.tiles_total + ctas - 1) / ctas);
+    bool found = false;
+    for (int u = 1; u <= 2; ++u) {
+        if (u == 2 && p.q_tiles == 1) break;
+        const int units = u == 1 ? heads_forks * p.q_tiles : pair_units;
+        for (int i = 0; i < 2; ++i) {
+            const int s = kClusterSizes[i];
+            if (units > resident[i] || s > p.tiles_total) continue;
+            const int steps = (p.tiles_total + s - 1) / s;
+            const long long cost = u == 1 ? 10500 + static_cast<long long>(single_step) * steps : 13000 + static_cast<long long>(pair_step) * steps;
+            if (cost >= best) continue;
+            best = cost;
+            *size = s;
+            *unit = u;
+            found = true;
+        }
+    }
+    return found;
 }
 
 template <int MAXSETS>
@@ -1581,11 +1795,20 @@ cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* con
     args.n_sets = n;
     args.scale_log2 = probs[0].scale * 1.4426950408889634f;
     args.merge_wait_limit = ctx->attn_merge_wait_limit;
+    if constexpr (MAXSETS == 1) {
+        // (the barrier of a cluster knows no limit: a caller who sets one gets the merge that has it)
+        if (!min_tiles && ctx->attn_merge_wait_limit == kMergeWaitDefault &&
+            unit_clusters(args.sets[0], ctx->attn_max_ctas, resident_clusters(ctx->device), &args.cluster_size, &args.cluster_unit)) {
+            const SetParams& p = args.sets[0];
+            const int clusters = p.n_kv_heads * p.n_forks * (args.cluster_unit == 2 ? (p.q_tiles + 1) / 2 : p.q_tiles);
+            return launch_shape<1, kByCluster>(args, head_dim, static_cast<unsigned>(clusters * args.cluster_size), false, ctx->device, st);
+        }
+    }
     // Equal ranges are 1-3 us faster in the instantiation that knows nothing else (16 / 2 heads, prefix 16384, 16
     // rollouts: 72.3 against 74.9 us); with a gate the layout is known on the device only, and is mostly by unit.
     if (pairs <= ctx->attn_max_ctas && (gated || cuts_by_unit(args.sets, n, static_cast<int>(ctas), args.min_piece)))
-        return launch_shape<MAXSETS, true>(args, head_dim, static_cast<unsigned>(ctas), waits, ctx->device, st);
-    return launch_shape<MAXSETS, false>(args, head_dim, static_cast<unsigned>(ctas), waits, ctx->device, st);
+        return launch_shape<MAXSETS, kByUnit>(args, head_dim, static_cast<unsigned>(ctas), waits, ctx->device, st);
+    return launch_shape<MAXSETS, kEqualRanges>(args, head_dim, static_cast<unsigned>(ctas), waits, ctx->device, st);
 }
 
 }  // namespace

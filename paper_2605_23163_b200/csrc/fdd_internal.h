@@ -51,6 +51,8 @@ struct TcMapPoolEntry {
     std::vector<TcMapCache> maps;
 };
 
+constexpr long long kMergeWaitDefault = 4000000000LL;   // SM clocks (about two seconds)
+
 struct fdd_ctx {
     fdd_config cfg;
     int device = 0;
@@ -70,7 +72,7 @@ struct fdd_ctx {
     int attn_max_units = 0;
     int attn_max_ctas = 0;
     std::vector<uint64_t> attn_args;  // host buffer for the attention kernel's argument block (8-byte aligned)
-    long long attn_merge_wait_limit = 4000000000LL;   // SM clocks (about two seconds): wait for the pieces of a cut unit
+    long long attn_merge_wait_limit = kMergeWaitDefault;   // SM clocks: wait for the pieces of a cut unit
     void* seed_chunk = nullptr;       // host staging of seeds on their way to the device as kernel arguments
     // fdd_decode_block runs the attention of its steps on a stream of its own, beside the unmasking (decode_loop.cu)
     cudaStream_t side_stream = nullptr;

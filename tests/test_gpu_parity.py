@@ -573,6 +573,46 @@ def test_attention_units_cut_into_pieces_of_their_own(hq, hkv, dim, prefix, fork
         fdd.fdd_destroy(ctx)
 
 
+@pytest.mark.parametrize("hq,hkv,dim,prefix,page,forks,block,live", [
+    (16, 2, 128, 1920, 0, 1, 32, None),      # sixteen tiles, one for each CTA of a cluster of 16
+    (16, 2, 128, 2100, 64, 1, 32, None),     # one more, paged, ragged
+    (16, 2, 128, 896, 0, 2, 32, (1,)),       # eight tiles and units in clusters of eight, half of them gated off
+    (16, 2, 128, 3000, 0, 4, 32, None),      # units of two query tiles
+    (16, 2, 128, 1100, 0, 3, 36, (0, 2)),    # the last unit of a rollout has one query tile
+    (28, 4, 128, 1500, 0, 3, 27, None),      # groups of seven: a gap behind a tile's last row
+    (3, 1, 64, 2500, 64, 2, 3, None),        # fewer rows than CTAs in a cluster
+    (4, 1, 64, 5000, 0, 1, 16, None),
+])
+@pytest.mark.parametrize("causal", [False, True])
+def test_attention_units_in_clusters(hq, hkv, dim, prefix, page, forks, block, live, causal):
+    sc = synth.Scene(prefix, forks, block, 0, 2)
+    w = synth.Workload("clusters", hq, hkv, dim, 512, "bf16", "peaked", 0.9, 1.0, (sc,), page_tokens=page, seed=60 + prefix)
+    ctx = harness.create_context(w)
+    try:
+        scene = harness.GpuScene(ctx, w, 0)
+        pk, pv = synth.make_prefix(w, 0)
+        q, k, v = synth.make_qkv(w, 0, 0, 0, 0)
+        fdd.fdd_kv_commit(ctx, [scene.forkset], 0, harness.bf16_tensor(k), harness.bf16_tensor(v), [block], 1)
+        suffix = ([k[f] for f in range(forks)], [v[f] for f in range(forks)])
+        q, k, v = synth.make_qkv(w, 0, 0, 1, 0)
+        qd, kd, vd = harness.bf16_tensor(q), harness.bf16_tensor(k), harness.bf16_tensor(v)
+        on = list(range(forks)) if live is None else list(live)
+        gate = None
+        if live is not None:
+            gate = torch.zeros(forks, dtype=torch.int32, device="cuda")
+            gate[on] = 1
+        for _ in range(2):
+            out = torch.full_like(qd, float("nan"))
+            fdd.fdd_block_attn_gated(ctx, [scene.forkset], 0, qd, kd, vd, out, [block], 1.0 / np.sqrt(dim), int(causal), gate)
+            fdd.fdd_poll_status(ctx)
+            got = out.float().cpu().numpy().astype(np.float64).reshape(q.shape)
+            ref = pu.attention_oracle(w, (pk, pv), suffix, q, k, v, forks=on, causal=causal)
+            pu.assert_attention_close(got[on], ref)
+            assert np.all(np.isnan(got[np.setdiff1d(np.arange(forks), on)]))
+    finally:
+        fdd.fdd_destroy(ctx)
+
+
 def _in_child(code, **env):
     # settings that the library reads once per process
     here = os.path.dirname(os.path.abspath(__file__))
