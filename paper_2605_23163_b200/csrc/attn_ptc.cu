@@ -26,12 +26,13 @@
 // 1.5 until the last piece is seen, 4 for the merge).  Measured, launches one behind the other (equal ranges ->
 // pieces by unit): one rollout, prefix 4096: 24.6 -> 18.5-20 us; eight rollouts: 33-36 -> 27-29 us; 28 / 4
 // heads, six rollouts, prefix 3001: 41 -> 35 us; a block of 36 layers with eight rollouts: 6.3 -> 5.3 ms.
-// Few units: clusters.  The pieces of a unit are the CTAs of a cluster of 16 or 8; each leaves its output in its own
+// Few units: clusters.  The pieces of a unit are the CTAs of a cluster of 16, 8 or 4; each leaves its output in its own
 // shared memory (over the operand tiles), and behind a barrier of the cluster every CTA merges its share of the rows out
 // of all of them: no scratch, no counters, no cooperative launch; writing a piece, publishing it, waiting and
-// merging take 3 us instead of 7.5.  Seven clusters of 16 or 15 of 8 fit on the chip (one CTA per SM), so this is for
-// up to 15 units.  Launches one behind the other, 16 / 2 heads, pieces by unit -> clusters: one rollout, prefix
-// 4096 18.5 -> 14.9 us, prefix 12000 24.6 -> 18.7; two rollouts 20.5 -> 16.2; four 22.4 -> 21.6.
+// merging take 3 us instead of 7.5.  7 clusters of 16, 15 of 8 or 33 of 4 fit on the chip (one CTA per SM), so this is for
+// up to 33 units.  Launches one behind the other, 16 / 2 heads, pieces by unit -> clusters: one rollout, prefix
+// 4096 18.5 -> 14.9 us, prefix 12000 24.6 -> 18.7; two rollouts 20.5 -> 16.2; four 22.4 -> 20.6; eight 24.8 -> 21.6,
+// prefix 1000 20.5 -> 14.4.
 // These launches also initialise their barriers ahead of the wait for the kernel before them and keep the scenes'
 // sizes in shared memory; a launch with more units than CTAs lost 2-3 % by the same (a block at 32 rollouts,
 // prefix 16384: 1815-1850 us against 1770-1790), so it does neither.  TMEM is taken behind the wait everywhere.
@@ -91,7 +92,7 @@ constexpr long long kWaitLimit = 4000000000LL;   // about two seconds of SM cloc
 constexpr int kMaxGatedForks = kAttnMaxGatedForks;   // rollouts of one launch when any scene has a gate
 constexpr int kMinTilesPerCta = 3;               // do not cut equal ranges finer than this (every cut costs a piece to write and merge)
 constexpr int kUnitSlack = 4;                    // tile steps by which the longest piece of a unit may exceed an equal share
-constexpr int kClusterSizes[2] = {16, 8};        // CTAs of a cluster
+constexpr int kClusterSizes[3] = {16, 8, 4};     // CTAs of a cluster
 constexpr int kWholeTiles = 6;                   // units up to this long are not cut
 constexpr int kBesideSteps = 7, kBesideStepsSplit = 5;   // least steps per CTA beside other kernels (Split: probabilities in two halves)
 constexpr int kSingleSteps = 1;                  // units of one query tile while no CTA gets more than this many steps of them
@@ -377,7 +378,7 @@ struct Layout {
 // Pieces of a unit of `tiles` steps when no piece is longer than c.
 __host__ __device__ __forceinline__ int pieces_of(int tiles, int c) { return tiles <= kWholeTiles ? 1 : (tiles + c - 1) / c; }
 
-// The layout of a launch: one warp, lane s looks after scene s (n_sets <= 16).  Every role waits for it, so it is
+// The layout of a launch: one warp, lane s looks after scene s (n_sets <= 32).  Every role waits for it, so it is
 // kept short: 32-bit divisions, and for one scene the lengths of a piece are tried side by side (with 64-bit divisions
 // one after the other, equal ranges at 16 / 2 heads, prefix 16384, 16 rollouts took 75.4 us a launch instead of 73.4).
 template <int MAXSETS, bool BYUNIT>
@@ -458,10 +459,9 @@ __device__ __forceinline__ void plan(const TcArgs<MAXSETS>& a, const SetParams* 
 }
 
 // Merge of a unit whose pieces lie in the shared memory of the CTAs of a cluster (piece k in CTA k): CT float4 columns of
-// one row, out = sum_k 2^(m_k - M) O_k / sum_k 2^(m_k - M) l_k.  All reads of eight pieces are in flight together.
-template <int D, int CT>
+// one row, out = sum_k 2^(m_k - M) O_k / sum_k 2^(m_k - M) l_k.  All reads of kAtOnce pieces are in flight together.
+template <int D, int CT, int kAtOnce>
 __device__ __forceinline__ void merge_cluster(uint32_t part, uint32_t ml, int n_pieces, int row, int col0, __nv_bfloat16* op) {
-    constexpr int kAtOnce = 8;
     float4 acc[CT];
 #pragma unroll
     for (int c = 0; c < CT; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1392,10 +1392,14 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                 __nv_bfloat16* op = p.out + ((static_cast<size_t>(v.f) * p.d + qi2) * p.n_q_heads + v.h * p.G + qg2) * D;
                 const uint32_t ml = tc::smem_u32(row_ml_s);
                 const int ct = (D / 4) / col_groups;
-                if (ct == 1) {
-                    merge_cluster<D, 1>(q_s, ml, n_pieces, rowu, cg, op);
+                if (!kOwn && n_pieces == 4) {
+                    if (ct == 1) merge_cluster<D, 1, 4>(q_s, ml, 4, rowu, cg, op);
+                    else
+                        for (int c = 0; c < ct; c += 2) merge_cluster<D, 2, 4>(q_s, ml, 4, rowu, cg * ct + c, op);
                 } else {
-                    for (int c = 0; c < ct; c += 2) merge_cluster<D, 2>(q_s, ml, n_pieces, rowu, cg * ct + c, op);
+                    if (ct == 1) merge_cluster<D, 1, 8>(q_s, ml, n_pieces, rowu, cg, op);
+                    else
+                        for (int c = 0; c < ct; c += 2) merge_cluster<D, 2, 8>(q_s, ml, n_pieces, rowu, cg * ct + c, op);
                 }
             }
             __syncwarp();
@@ -1665,15 +1669,15 @@ bool cuts_by_unit(const SetParams* sets, int n, int ctas, int min_piece) {
 const int* resident_clusters(int device) {
     constexpr int kMaxDevices = 64;
     static std::atomic<bool> known[kMaxDevices];
-    static int most[kMaxDevices][2];
-    static const int none[2] = {0, 0};
+    static int most[kMaxDevices][3];
+    static const int none[3] = {0, 0, 0};
     if (device < 0 || device >= kMaxDevices) return none;
     if (!known[device].load(std::memory_order_acquire)) {
         auto kernel = attn_ptc_kernel<128, 1, 0, kSharedScores, kByCluster>;
         const int smem = TcShape<128>::kSmemBytes;
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < 3; ++i) {
             int n = 0;
             cudaLaunchAttribute attr;
             attr.id = cudaLaunchAttributeClusterDimension;
@@ -1696,23 +1700,29 @@ const int* resident_clusters(int device) {
 }
 
 // Whether the units of a launch over one scene go to clusters, of how many CTAs, and whether a unit has one query tile or
-// two: what takes least time by a fit to measured launches (nanoseconds; launches one behind the other, 16 / 2 heads,
-// prefix 1000 to 12000, one to eight rollouts).  Clusters of other sizes took 4 to 10 us more than the fit, whatever the
-// number of steps, and are not used.
+// two: what takes least time by a fit to measured launches (nanoseconds: 16 / 2, 32 / 8, 4 / 1, 28 / 4 and 12 / 2 heads, prefix
+// 1000 to 12000, one to eight rollouts, launches one behind the other, within 10 %; two microseconds more for launches
+// that are not in clusters, which start later behind another kernel).  Clusters of other sizes than powers of two take 4 to
+// 10 us more than the fit.  Of two halves of the probabilities the query tiles' chains are serial: longer steps, and
+// four CTAs are never enough.
 bool unit_clusters(const SetParams& p, int ctas, const int* resident, int* size, int* unit) {
     if (p.tiles_total <= kWholeTiles) return false;
-    const int heads_forks = p.n_kv_heads * p.n_forks, pair_units = heads_forks * ((p.q_tiles + 1) / 2);
-    const int single_step = 1250, pair_step = 1650, step = p.q_tiles == 1 ? single_step : pair_step;
-    long long best = 18700 + static_cast<long long>(step) * ((static_cast<long long>(pair_units) * p.tiles_total + ctas - 1) / ctas);
+    struct Cost { int base, step; };
+    const bool split = (p.G & (p.G - 1)) != 0;
+    const Cost single = split ? Cost{12400, 2000} : Cost{10500, 1250}, pair = split ? Cost{15000, 2750} : Cost{13500, 1650};
+    const Cost pieces = split ? Cost{21000, 2900} : Cost{20700, p.q_tiles == 1 ? 1250 : 1650};
+    const int heads_forks = p.n_kv_heads * p.n_forks, single_units = heads_forks * p.q_tiles, pair_units = heads_forks * ((p.q_tiles + 1) / 2);
+    long long best = static_cast<long long>(single_units) * p.tiles_total <= static_cast<long long>(ctas) * kSingleSteps
+        ? 19500 : pieces.base + pieces.step * ((static_cast<long long>(pair_units) * p.tiles_total + ctas - 1) / ctas);
     bool found = false;
     for (int u = 1; u <= 2; ++u) {
         if (u == 2 && p.q_tiles == 1) break;
-        const int units = u == 1 ? heads_forks * p.q_tiles : pair_units;
-        for (int i = 0; i < 2; ++i) {
+        const Cost& c = u == 1 ? single : pair;
+        for (int i = 0; i < 3; ++i) {
             const int s = kClusterSizes[i];
-            if (units > resident[i] || s > p.tiles_total) continue;
-            const int steps = (p.tiles_total + s - 1) / s;
-            const long long cost = u == 1 ? 10500 + static_cast<long long>(single_step) * steps : 13000 + static_cast<long long>(pair_step) * steps;
+            if ((u == 1 ? single_units : pair_units) > resident[i] || s > p.tiles_total || (split && s == 4)) continue;
+            const long long steps = (p.tiles_total + s - 1) / s;
+            const long long cost = c.base + c.step * steps + (split && s == 16 ? 600 : 0);
             if (cost >= best) continue;
             best = cost;
             *size = s;
@@ -1824,6 +1834,8 @@ cudaError_t launch_attention_ptc(fdd_ctx* ctx, const AttnProblem* probs, TcMapCa
                                  int head_dim, cudaStream_t st, bool beside, int* n_launches) {
     if (n < 1 || n > kTcMaxSets) return cudaErrorInvalidValue;
     *n_launches += 1;
+    // (32 KB of arguments cost a launch a microsecond or two: 28 / 4 heads, two layers 303 -> 298 us a block without them)
     if (n == 1) return launch_group<1>(ctx, probs, caches, n, head_dim, st, beside);
+    if (n <= kTcFewSets) return launch_group<kTcFewSets>(ctx, probs, caches, n, head_dim, st, beside);
     return launch_group<kTcMaxSets>(ctx, probs, caches, n, head_dim, st, beside);
 }

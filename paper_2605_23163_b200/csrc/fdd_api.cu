@@ -219,7 +219,8 @@ fdd_status block_attn_layers(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets,
         if (together && l + 1 < n_layers) continue;
         // as few launches as take all problems, of about the same size
         const int count = static_cast<int>(probs.size());
-        const int launches = (count + kTcMaxSets - 1) / kTcMaxSets, most = (count + launches - 1) / launches;
+        const int room = n_layers > 1 ? kTcMaxSets : kTcMaxScenes;
+        const int launches = (count + room - 1) / room, most = (count + launches - 1) / launches;
         for (int first = 0; first < count;) {
             int n = 0, forks = 0;
             while (n < most && first + n < count && (n == 0 || !gate || forks + probs[first + n].n_forks <= kAttnMaxGatedForks))

@@ -28,7 +28,9 @@ struct TcSetMaps {
     CUtensorMap pk, pv;             // contiguous: (D, P, Hkv); paged: (D, 64, Hkv, pages)
     CUtensorMap pk_tail, pv_tail;   // paged only: token dimension cut to the last page's fill
 };
-constexpr int kTcMaxSets = 16;      // (scene, layer) pairs per attention launch
+constexpr int kTcMaxSets = 24;      // (scene, layer) pairs per attention launch: what 32 KB of kernel arguments hold
+constexpr int kTcFewSets = 4;       // launches of so few take a kernel with room for no more
+constexpr int kTcMaxScenes = 16;    // scenes of one layer per launch
 
 // The maps last built for one (fork set, layer) and what they were built from.
 struct TcMapCache {
