@@ -34,8 +34,8 @@
 // 53 % busy issue slots and special-function units of four warps a scheduler (three CTAs an SM, with the registers
 // cut to 80, were no faster).  Small launches are bound by latency: 1.6 us to the first copies, 0.7 to the first
 // tile, 1.5 for a noisy tile, 1 for the look at the list.  Measured against equal ranges with a running maximum and
-// re-scoring piece by piece, whole calls: 408 rows of 50257 bf16 logits, greedy, 28.7 -> 22.5 us; 720 rows of 151936
-// fp32 logits with noise 88.7 -> 82.8; a draft / verify cycle over 176 rows of 151936 bf16 logits with noise 124.5 ->
+// re-scoring piece by piece, whole calls: 408 rows of 50257 bf16 logits, greedy, 28.8 -> 22.5-23.3 us; 720 rows of 151936
+// fp32 logits with noise 90 -> 82-85; a draft / verify cycle over 176 rows of 151936 bf16 logits with noise 124.5 ->
 // 106.7.
 //
 // Kernel 2 (unmask_finalize_kernel): one CTA per rollout merges the records of its rows, forms the
@@ -57,7 +57,7 @@ constexpr int kTile = kUnmaskTile;                    // ids per tile (one bulk 
 constexpr int kStages = 3;                            // tiles a warp holds in shared memory (two in flight while one is reduced)
 constexpr int kMaxRows = kUnmaskMaxRows;              // rows of one launch (32 per thread in the set-up)
 constexpr int kMinPiecesPerRow = 8;                   // a warp gets one piece when each row can have this many warps
-constexpr int kDealtShare = 5, kDealtLeast = 3, kDealtMost = 12;   // pieces that are dealt out: about five a warp, of 3 to 12 tiles
+constexpr int kDealtShare = 6, kDealtLeast = 3, kDealtMost = 12;   // short pieces that are dealt out: a sixth of a warp's share, of 3 to 12 tiles
 constexpr int kMaxList = 224;                         // blocks in reach of the running lower bound kept per piece (a few dozen expected)
 constexpr long long kCopyWaitLimit = 4000000000LL;    // SM clocks a warp waits for one of its own copies (about two seconds)
 static_assert(kTile == 32 * kLaneIds, "a tile is 64 ids for each of 32 lanes");
@@ -426,24 +426,37 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* state,
     // items, and a piece leaves one record.  (A call has far fewer than 2^31 tiles: they lie in the GPU's memory.)
     //  - Few rows: as many pieces as there are warps, one for each, where each row can have kMinPiecesPerRow of them or
     //    where that makes no piece longer than an equal share.
-    //  - Otherwise pieces of a few tiles: every warp has one to begin with and draws the next one from a counter while
-    //    it still works on the one before.  SMs stream at rates that differ by a quarter (with equal ranges the warps of
-    //    a launch over 1216 rows of 152k ids ended after 52 us at the median and 66 us at the latest, greedy, and
-    //    71 and 89 us with noise; now 57 and 64, 76 and 88).  About five pieces a warp of at most twelve tiles: 720 rows
-    //    of fp32 logits 83 us, with eight of at most eight tiles 86.8, three of at most 24 87.3, two of at most 40 85.8.
+    //  - Otherwise most of every row goes into long pieces, about one for each warp, and the rest into pieces of a few
+    //    tiles, which the warps draw from a counter while they still work on the piece before.  SMs stream at rates that
+    //    differ by a quarter (with equal ranges the warps of a launch over 1216 rows of 152k ids ended after 52 us at the
+    //    median and 66 us at the latest, greedy, and 71 and 89 us with noise), and every piece costs about a microsecond.
+    //    Whole calls, equal ranges -> long and short pieces, us: 1216 rows of 151936 bf16 logits 67.5 -> 68.3 greedy and
+    //    93.6 -> 92.7 with noise, 608 rows 41.5 -> 43.5 and 59.9 -> 53.8, 1216 rows of 50257 49.6 -> 45.5 and 72.5 -> 63.2,
+    //    2048 rows of 32000 with noise 57.2 -> 51.2, 720 rows of fp32 logits 74.7 -> 72.5 and 86.4 -> 79.5.  With 0.7 and
+    //    0.9 of a share in long pieces 608 rows with noise took 55.3 and 55.4; short pieces alone 60.6.
     const int tiles_per_row = (vocab + kTile - 1) / kTile;
     const int ipr = (tiles_per_row + tiles_per_item - 1) / tiles_per_item;
     const int warps_all = static_cast<int>(gridDim.x) * kWarps;
     const int gw = warp * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x);   // warps of a CTA lie a grid apart: few pieces spread over all SMs
-    int ppr = min(ipr, warps_all / n_rows);
+    constexpr int kLongShare = sizeof(T) == 2 ? 8 : 6;            // tenths of a warp's share that are its long piece
+    int ppr = min(ipr, warps_all / n_rows), n_long = 0, long_items = 0;
     {
         const int share = (n_rows * ipr + warps_all - 1) / warps_all;
         if (ppr < min(ipr, kMinPiecesPerRow) && (ppr == 0 || (ipr + ppr - 1) / ppr > share)) {
             const int len = max(1, min(max(share * tiles_per_item / kDealtShare, kDealtLeast), kDealtMost) / tiles_per_item);
-            ppr = (ipr + len - 1) / len;
+            const int at_most = max(1, warps_all / n_rows), rounds = (n_rows * at_most + warps_all - 1) / warps_all;
+            long_items = min(share * kLongShare / 10 / rounds, ipr * kLongShare / 10 / at_most);
+            if (long_items > 2 * len) n_long = at_most;
+            ppr = n_long + (ipr - n_long * long_items + len - 1) / len;
         }
     }
-    const int n_pieces = n_rows * ppr, piece_items = ipr / ppr, piece_more = ipr - piece_items * ppr;   // (the first piece_more pieces of a row have one item more)
+    const int n_short = ppr - n_long, n_pieces = n_rows * ppr;
+    const int short_items = (ipr - n_long * long_items) / n_short, short_more = ipr - n_long * long_items - short_items * n_short;
+    // first item of a piece (the first short_more short pieces of a row have one item more)
+    auto first_item = [&](int pc) {
+        if (pc <= n_long) return pc * long_items;
+        return n_long * long_items + (pc - n_long) * short_items + min(pc - n_long, short_more);
+    };
     if (gw >= n_pieces) return;
 
     const uint32_t full = 0xFFFFFFFFu;
@@ -466,9 +479,12 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* state,
         if (p_tile == p_tile_end) {
             const int id = __shfl_sync(full, p_next, 0);
             if (id >= n_pieces) return;
-            const int ri = id / ppr, pc = id - ri * ppr, row = selected_row(ri), c0 = pc * piece_items + min(pc, piece_more);
-            p_tile = c0 * tiles_per_item;
-            p_tile_end = min(tiles_per_row, (c0 + piece_items + (pc < piece_more ? 1 : 0)) * tiles_per_item);
+            // (the long pieces of all rows come first)
+            const bool is_long = id < n_rows * n_long;
+            const int among = is_long ? id : id - n_rows * n_long, per_row = is_long ? n_long : n_short, ri = among / per_row;
+            const int pc = among - ri * per_row + (is_long ? 0 : n_long), row = selected_row(ri);
+            p_tile = first_item(pc) * tiles_per_item;
+            p_tile_end = min(tiles_per_row, first_item(pc + 1) * tiles_per_item);
             p_row_ptr = logits + static_cast<size_t>(row) * vocab;
             // (at most kStages pieces are ahead of the one being reduced; the answer of the counter is not needed before
             // the last tile of this piece is on its way)
@@ -507,8 +523,7 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* state,
     for (int c_open = 0; c_open != p_open && alive; ++c_open) {
         // ---- open the piece: tiles [tile0, tile1) of one row
         const int row = s_open[warp][c_open & 7].x, pc = s_open[warp][c_open & 7].y;
-        const int c0 = pc * piece_items + min(pc, piece_more);
-        const int tile0 = c0 * tiles_per_item, tile1 = min(tiles_per_row, (c0 + piece_items + (pc < piece_more ? 1 : 0)) * tiles_per_item);
+        const int tile0 = first_item(pc) * tiles_per_item, tile1 = min(tiles_per_row, first_item(pc + 1) * tiles_per_item);
         const int seg_end = min(vocab, tile1 * kTile);
         uint32_t* const row_bar = shared_words + kSharedBars + row;
         const T* row_ptr = logits + static_cast<size_t>(row) * vocab;
