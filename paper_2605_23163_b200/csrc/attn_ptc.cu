@@ -135,6 +135,7 @@ struct TcArgs {
     int min_tiles;             // do not cut the work into ranges shorter than this
     int min_piece;             // nor a unit into pieces shorter than this
     int cluster_size, cluster_unit;   // units in clusters: CTAs of a cluster (pieces of a unit), query tiles of a unit
+    int ref_ctas;              // > 0: pieces longer than an equal share among so many CTAs take their reference maximum anew (Layout::ref)
     int n_sets;
     float scale_log2;
     long long merge_wait_limit; // SM clocks a CTA waits for the other pieces of a cut unit before it gives up
@@ -373,7 +374,18 @@ struct Layout {
     int ctas;                  // CTAs that take part
     int per_unit;              // query tiles of a unit: 2, or 1 where that gives every tile step a CTA of its own
     int by_unit;               // > 0: every unit is cut into equal pieces of at most this many steps; 0: equal ranges
+    int ref;                   // key tiles after which a piece takes its reference maximum anew
 };
+constexpr int kKeepRef = 0x7FFFFFFF;
+// A tile's largest probability is exact in bf16 where the row's reference is that tile's maximum, as it is in the first
+// tile of every piece, so the error against 64 bits goes with the length of the pieces.  A launch that cuts longer pieces
+// than one over a single layer on all CTAs would (units in clusters, layers together, beside other kernels) takes
+// the maximum of the tile at hand as the reference whenever a piece has gone that far.  Errors with the first tile's maximum -> with
+// this, as those launches had in the finer cut: one rollout in clusters of 16, prefix 4096, 2.25e-3 -> 2.15e-3; eight rollouts 2.33e-3 ->
+// 2.28e-3; 36 layers 2.33e-3 -> 2.24e-3.  A rescaling of O costs a tile step 0.2 us.
+__device__ __forceinline__ int ref_length(long long steps, int ctas) {
+    return steps >= kKeepRef - ctas ? kKeepRef : max(1, (static_cast<int>(steps) + ctas - 1) / ctas);
+}
 
 // Pieces of a unit of `tiles` steps when no piece is longer than c.
 __host__ __device__ __forceinline__ int pieces_of(int tiles, int c) { return tiles <= kWholeTiles ? 1 : (tiles + c - 1) / c; }
@@ -414,6 +426,7 @@ __device__ __forceinline__ void plan(const TcArgs<MAXSETS>& a, const SetParams* 
     const long long steps_incl = scan(static_cast<long long>(units) * tiles);
     const int units_incl = scan(units);
     l.T = __shfl_sync(full, steps_incl, last);
+    l.ref = a.ref_ctas > 0 ? ref_length(l.T, a.ref_ctas) : kKeepRef;
     int n = 1;                                          // pieces of a unit of this lane's scene
     l.by_unit = 0;
     l.ctas = l.T >= static_cast<long long>(grid) * a.min_tiles ? grid : max(1, static_cast<int>(l.T) / a.min_tiles);
@@ -509,17 +522,18 @@ __device__ __forceinline__ void merge_cluster(uint32_t part, uint32_t ml, int n_
 }
 
 // How a launch is cut (see the top of the file).
-constexpr int kEqualRanges = 0, kByUnit = 1, kByCluster = 2;
+constexpr int kEqualRanges = 0, kByUnit = 1, kByCluster = 2, kRangesRef = 3;   // kRangesRef: equal ranges with Layout::ref
 
 template <int D, int MAXSETS, int EMU, int MODE, int CUT>
 __global__ void __launch_bounds__(kTcThreads, 1)
 attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
     using Shape = TcShape<D>;
-    constexpr bool BYUNIT = CUT != kEqualRanges;        // (or by equal ranges, if the gate leaves nothing better)
+    constexpr bool BYUNIT = CUT == kByUnit || CUT == kByCluster;        // (or by equal ranges, if the gate leaves nothing better)
     constexpr bool CLUSTERED = CUT == kByCluster;
     static_assert(!CLUSTERED || MAXSETS == 1, "units in clusters: one scene");
     constexpr int kStages = Shape::kStages;
     constexpr bool kOwn = MODE == kOwnScoresSplit;      // every query tile has a score buffer of its own, probabilities in two halves
+    constexpr bool kRef = !kOwn && CUT != kEqualRanges; // (two halves of a probability lose next to nothing)
     static_assert(EMU % 8 == 0 && EMU >= 0 && EMU <= 128, "EMU: emulated exponentials per 128-key tile");
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -628,6 +642,8 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
         lay.ctas = p.n_kv_heads * n_act_s[0] * per_head * a.cluster_size;
         lay.T = lay.ctas;
         lay.by_unit = 1;
+        const long long head_steps = static_cast<long long>(p.n_kv_heads) * n_act_s[0] * p.tiles_total;
+        lay.ref = head_steps * p.q_tiles <= a.ref_ctas * kSingleSteps ? 1 : ref_length(head_steps * ((p.q_tiles + 1) / 2), a.ref_ctas);
     } else {
         lay = layout_s;
     }
@@ -991,6 +1007,8 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                 const float c_emu = c * (1.0f / 128.0f);
                 const uint32_t bs = tc::smem_u32(&bar_s_full[q]), bf = tc::smem_u32(&bar_s_free[q]);
                 const uint32_t bp = tc::smem_u32(&bar_p_full[q]);
+                const int ref_length = p.tiles_total > kWholeTiles ? lay.ref : kKeepRef;
+                int ref_left = ref_length;
                 for (int jl = 0; jl < nt; ++jl) {
                     const TileInfo t = tile_info(p, it.t0 + jl);
                     ok = tc::mbar_wait(bs, (sp0 + jl) & 1, abort_flag, kWaitLimit);
@@ -1029,31 +1047,41 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                     if (!(m_tile > -CUDART_INF_F)) m_tile = m_used > -CUDART_INF_F ? m_used : 0.0f;
                     // The previous PV of this query tile must be complete before P is overwritten and
                     // before O is rescaled (it is one phase behind at most).  Usually only the first
-                    // matters, so the wait sits after the exponentials.  (With a score buffer per query tile these
-                    // scores were only computed once that product was complete.)
-                    bool pv_done = kOwn || jl == 0;
+                    // matters, so the wait sits after the exponentials; where the reference is taken anew every few tiles O is
+                    // rescaled there as well (36 layers: 1339 us a block, 1395 with the wait ahead of the exponentials).
+                    // (With a score buffer per query tile these scores were only computed once that product was complete.)
+                    auto rescale_o = [&](float alpha) {
+#pragma unroll
+                        for (int cc = 0; cc < D / 32; ++cc) {
+                            uint32_t o[32];
+                            tc::tmem_ld32(tm_o[q] + lane_base + cc * 32, o);
+                            tc::wait_ld();
+#pragma unroll
+                            for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                            tc::tmem_st32(tm_o[q] + lane_base + cc * 32, o);
+                        }
+                        tc::wait_st();
+                    };
+                    bool pv_done = kOwn || jl == 0, rescale = false;
+                    float alpha = 1.0f;
                     if (jl == 0) {
                         m_used = m_tile;
                     } else {
-                        const bool need = m_tile > m_used + 8.0f;
+                        bool need = m_tile > m_used + 8.0f;
+                        if (kRef && --ref_left == 0) {
+                            ref_left = ref_length;
+                            need = m_tile > m_used - 8.0f && m_tile != m_used;
+                        }
                         if (__any_sync(0xFFFFFFFFu, need)) {
-                            if (!kOwn) {
+                            if (!kOwn && !kRef) {
                                 ok = tc::mbar_wait(bo, (sp0 + jl - 1) & 1, abort_flag, kWaitLimit);
                                 if (!ok) break;
                                 pv_done = true;
                                 tc::fence_after_sync();
                             }
-                            const float alpha = need ? exp2f(m_used - m_tile) : 1.0f;
-#pragma unroll
-                            for (int cc = 0; cc < D / 32; ++cc) {
-                                uint32_t o[32];
-                                tc::tmem_ld32(tm_o[q] + lane_base + cc * 32, o);
-                                tc::wait_ld();
-#pragma unroll
-                                for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-                                tc::tmem_st32(tm_o[q] + lane_base + cc * 32, o);
-                            }
-                            tc::wait_st();
+                            alpha = need ? exp2f(m_used - m_tile) : 1.0f;
+                            if (kRef) rescale = true;                   // (the same in every lane)
+                            else rescale_o(alpha);
                             l *= alpha;
                             if (need) m_used = m_tile;
                         }
@@ -1124,6 +1152,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                         if (!ok) break;
                         tc::fence_after_sync();
                     }
+                    if (kRef && rescale) rescale_o(alpha);
                     if (!kOwn) {
                         tc::tmem_st32(tm_p[q] + lane_base, packed);
                         tc::tmem_st32(tm_p[q] + lane_base + 32, packed + 32);
@@ -1633,15 +1662,17 @@ cudaError_t launch_one(const TcArgs<MAXSETS>& args, unsigned ctas, bool waits, i
 template <int MAXSETS, int CUT>
 cudaError_t launch_shape(const TcArgs<MAXSETS>& args, int head_dim, unsigned ctas, bool waits, int device, cudaStream_t st) {
     const int G = args.sets[0].G;                          // (the same for every scene of a context)
+    // (16 bits of a probability need no reference anew; the shares of emulated exponentials are for trying out)
+    constexpr int kPlainCut = CUT == kRangesRef ? kEqualRanges : CUT;
     if ((G & (G - 1)) != 0) {
         // Groups that are not a power of two keep 16 bits of every probability (see the top of the file).
-        if (head_dim == 64) return launch_one<64, MAXSETS, 0, kOwnScoresSplit, CUT>(args, ctas, waits, device, st);
-        return launch_one<128, MAXSETS, 0, kOwnScoresSplit, CUT>(args, ctas, waits, device, st);
+        if (head_dim == 64) return launch_one<64, MAXSETS, 0, kOwnScoresSplit, kPlainCut>(args, ctas, waits, device, st);
+        return launch_one<128, MAXSETS, 0, kOwnScoresSplit, kPlainCut>(args, ctas, waits, device, st);
     }
     if (head_dim == 64) return launch_one<64, MAXSETS, 0, kSharedScores, CUT>(args, ctas, waits, device, st);
     switch (emulated_exponentials()) {
-        case 16: return launch_one<128, MAXSETS, 16, kSharedScores, CUT>(args, ctas, waits, device, st);
-        case 32: return launch_one<128, MAXSETS, 32, kSharedScores, CUT>(args, ctas, waits, device, st);
+        case 16: return launch_one<128, MAXSETS, 16, kSharedScores, kPlainCut>(args, ctas, waits, device, st);
+        case 32: return launch_one<128, MAXSETS, 32, kSharedScores, kPlainCut>(args, ctas, waits, device, st);
         default: return launch_one<128, MAXSETS, 0, kSharedScores, CUT>(args, ctas, waits, device, st);
     }
 }
@@ -1735,8 +1766,8 @@ bool unit_clusters(const SetParams& p, int ctas, const int* resident, int* size,
 
 template <int MAXSETS>
 cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* const* caches, int n, int head_dim,
-                         cudaStream_t st, bool beside) {
-    // 1-20 KB, kept off the stack in the context's own buffer (a context is used by one host thread at a time)
+                         cudaStream_t st, bool beside, int alone) {
+    // 2-32 KB, kept off the stack in the context's own buffer (a context is used by one host thread at a time)
     if (ctx->attn_args.size() * sizeof(uint64_t) < sizeof(TcArgs<MAXSETS>)) ctx->attn_args.resize((sizeof(TcArgs<MAXSETS>) + 7) / 8);
     TcArgs<MAXSETS>& args = *reinterpret_cast<TcArgs<MAXSETS>*>(ctx->attn_args.data());
     long long pieces = 0;                                  // CTAs that the finest cut could occupy
@@ -1791,8 +1822,10 @@ cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* con
     // take, so it gets at least that many; half the chip a launch may have in any case, for the rollouts that are left
     // late in a block.  (16 / 2 heads, prefix 4096, three blocks side by side with their unmasking: eight rollouts 677 ->
     // 600 us, one rollout 323 -> 281; the launch by itself takes longer, 35 against 26 us.)
+    const long long most_ctas = ctas;
     if (beside) ctas = std::min(ctas, std::max<long long>(ctx->attn_max_ctas / 2, beside_ctas));
     if (ctas < 1) ctas = 1;
+    args.ref_ctas = n > alone || ctas < most_ctas ? static_cast<int>(static_cast<long long>(ctx->attn_max_ctas) * std::max(n, alone) / alone) : 0;
     // short units, each with a CTA of its own: none is cut, no CTA waits for another
     const bool waits = cut || pieces > ctas;
     args.part_o = static_cast<float*>(ctx->ws_attn);
@@ -1811,6 +1844,7 @@ cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* con
             unit_clusters(args.sets[0], ctx->attn_max_ctas, resident_clusters(ctx->device), &args.cluster_size, &args.cluster_unit)) {
             const SetParams& p = args.sets[0];
             const int clusters = p.n_kv_heads * p.n_forks * (args.cluster_unit == 2 ? (p.q_tiles + 1) / 2 : p.q_tiles);
+            args.ref_ctas = ctx->attn_max_ctas;
             return launch_shape<1, kByCluster>(args, head_dim, static_cast<unsigned>(clusters * args.cluster_size), false, ctx->device, st);
         }
     }
@@ -1818,6 +1852,7 @@ cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* con
     // rollouts: 72.3 against 74.9 us); with a gate the layout is known on the device only, and is mostly by unit.
     if (pairs <= ctx->attn_max_ctas && (gated || cuts_by_unit(args.sets, n, static_cast<int>(ctas), args.min_piece)))
         return launch_shape<MAXSETS, kByUnit>(args, head_dim, static_cast<unsigned>(ctas), waits, ctx->device, st);
+    if (args.ref_ctas > 0) return launch_shape<MAXSETS, kRangesRef>(args, head_dim, static_cast<unsigned>(ctas), waits, ctx->device, st);
     return launch_shape<MAXSETS, kEqualRanges>(args, head_dim, static_cast<unsigned>(ctas), waits, ctx->device, st);
 }
 
@@ -1829,13 +1864,14 @@ size_t attention_ptc_workspace_bytes(int head_dim, int max_ctas) {
     return static_cast<size_t>(2) * max_ctas * 256 * (head_dim + 1) * sizeof(float);
 }
 
-// One launch for up to kTcMaxSets scenes (all with the same soft-max scale).
+// One launch for up to kTcMaxSets scenes (all with the same soft-max scale).  alone: how many of them a launch over one layer
+// would have.
 cudaError_t launch_attention_ptc(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* const* caches, int n,
-                                 int head_dim, cudaStream_t st, bool beside, int* n_launches) {
+                                 int head_dim, cudaStream_t st, bool beside, int alone, int* n_launches) {
     if (n < 1 || n > kTcMaxSets) return cudaErrorInvalidValue;
     *n_launches += 1;
     // (32 KB of arguments cost a launch a microsecond or two: 28 / 4 heads, two layers 303 -> 298 us a block without them)
-    if (n == 1) return launch_group<1>(ctx, probs, caches, n, head_dim, st, beside);
-    if (n <= kTcFewSets) return launch_group<kTcFewSets>(ctx, probs, caches, n, head_dim, st, beside);
-    return launch_group<kTcMaxSets>(ctx, probs, caches, n, head_dim, st, beside);
+    if (n == 1) return launch_group<1>(ctx, probs, caches, n, head_dim, st, beside, alone);
+    if (n <= kTcFewSets) return launch_group<kTcFewSets>(ctx, probs, caches, n, head_dim, st, beside, alone);
+    return launch_group<kTcMaxSets>(ctx, probs, caches, n, head_dim, st, beside, alone);
 }

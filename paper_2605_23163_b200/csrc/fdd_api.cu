@@ -178,6 +178,7 @@ fdd_status block_attn_layers(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets,
         if (gate) reads.push_back(range_of(gate, sizeof(int32_t) * total));
         together = independent(writes, reads);
     }
+    const int alone_launches = (n_sets + kTcMaxScenes - 1) / kTcMaxScenes, alone = (n_sets + alone_launches - 1) / alone_launches;
     std::vector<AttnProblem> probs;
     std::vector<TcMapCache*> caches;
     probs.reserve(static_cast<size_t>(n_sets) * (together ? n_layers : 1));
@@ -226,7 +227,7 @@ fdd_status block_attn_layers(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets,
             while (n < most && first + n < count && (n == 0 || !gate || forks + probs[first + n].n_forks <= kAttnMaxGatedForks))
                 forks += probs[first + n++].n_forks;
             int n_launches = 0;
-            cudaError_t e = launch_attention_ptc(ctx, probs.data() + first, caches.data() + first, n, c.head_dim, st_, beside, &n_launches);
+            cudaError_t e = launch_attention_ptc(ctx, probs.data() + first, caches.data() + first, n, c.head_dim, st_, beside, alone, &n_launches);
             ctx->launches += n_launches;
             if (e != cudaSuccess) return cuda_fail(ctx, e, "fdd_block_attn launch");
             first += n;

@@ -182,7 +182,7 @@ size_t unmask_workspace_bytes(int vocab, int max_rows);
 
 size_t attention_ptc_workspace_bytes(int head_dim, int max_ctas);
 cudaError_t launch_attention_ptc(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* const* caches, int n,
-                                 int head_dim, cudaStream_t st, bool beside, int* n_launches);
+                                 int head_dim, cudaStream_t st, bool beside, int alone, int* n_launches);
 cudaError_t launch_unmask(fdd_ctx* ctx, const UnmaskProblem& p, cudaStream_t st, int* n_launches, int mode = 0);
 // One scene's part of a cache append.
 constexpr int kCommitSuffix = 0, kCommitPrefix = 1, kCommitPagedPrefix = 2;

@@ -468,3 +468,60 @@ def test_library_block_loop_leaves_the_stream_behind_its_attention():
         fdd.fdd_poll_status(ctx)
     finally:
         fdd.fdd_destroy(ctx)
+
+
+def _attention64(q, k, v, pk, pv, scale):
+    """Attention of one layer in 64 bits: q [n, d, hq, dim], k and v [n, d, hkv, dim], pk and pv [hkv, prefix, dim]."""
+    n, d, hq, dim = q.shape
+    hkv = k.shape[2]
+    res = []
+    for f in range(n):
+        keys, vals = (torch.cat([p.double(), x[f].double().transpose(0, 1)], 1) for p, x in ((pk, k), (pv, v)))
+        qh = q[f].double().view(d, hkv, hq // hkv, dim).permute(1, 2, 0, 3).reshape(hkv, -1, dim)
+        o = torch.softmax(qh @ keys.transpose(1, 2) * scale, -1) @ vals
+        res.append(o.view(hkv, hq // hkv, d, dim).permute(2, 0, 1, 3).reshape(d, hq, dim))
+    return torch.stack(res)
+
+
+@pytest.mark.parametrize("layers,forks,prefix", [
+    (1, 1, 4096),        # a piece per tile step -> clusters of sixteen
+    (1, 8, 4096),        # pieces of four tile steps -> clusters of four
+    (1, 20, 2500),       # pieces of six -> of eleven, beside the unmasking
+    (6, 8, 4003),        # pieces of four -> layers together, up to whole units
+    (6, 1, 1500),
+])
+def test_longer_pieces_are_as_precise_as_the_finer_cut(layers, forks, prefix):
+    # The error against 64 bits goes with how often a row's reference is the maximum of the tile at hand; launches that
+    # cut longer pieces than a layer by itself on all SMs take the reference anew.  The finer cut is what a call takes that has a wait
+    # limit of its own.  The two errors are of the same distribution then, over 65536 values or more a layer: 1 % is four
+    # times their scatter, and half of what is lost (2.7 to 4.5 %) if a piece keeps its first reference.
+    hq, hkv, dim, d, vocab = 16, 2, 128, 32, 512
+    scale = 1.0 / np.sqrt(dim)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(prefix + forks)
+    normal = lambda *shape: torch.randn(shape, generator=gen, device="cuda").to(torch.bfloat16)
+    pk, pv = normal(layers, hkv, prefix, dim), normal(layers, hkv, prefix, dim)
+    sk, sv = (torch.zeros((layers, forks, hkv, d, dim), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    q, k, v = normal(layers, forks, d, hq, dim), normal(layers, forks, d, hkv, dim), normal(layers, forks, d, hkv, dim)
+    exact = torch.stack([_attention64(q[l], k[l], v[l], pk[l], pv[l], scale) for l in range(layers)])
+    error = lambda out: float(torch.linalg.vector_norm(out.double() - exact) / torch.linalg.vector_norm(exact))
+    ctx = fdd.fdd_create(hq, hkv, dim, vocab, layers, 0, d, forks, fdd.FDD_LOGITS_BF16)
+    try:
+        forkset = fdd.fdd_fork(ctx, list(pk), list(pv), None, prefix, prefix, forks, list(range(forks)), list(sk), list(sv), d)
+        finer, called, looped = (torch.full_like(q, float("nan")) for _ in range(3))
+        fdd.fdd_set_merge_wait_limit(ctx, 3_999_999_999)
+        for l in range(layers):
+            fdd.fdd_block_attn(ctx, [forkset], l, q[l], k[l], v[l], finer[l], [d], scale, 0)
+        fdd.fdd_set_merge_wait_limit(ctx, 4_000_000_000)
+        for l in range(layers):
+            fdd.fdd_block_attn(ctx, [forkset], l, q[l], k[l], v[l], called[l], [d], scale, 0)
+        tokens = torch.zeros(forks * d, dtype=torch.int32, device="cuda")
+        state = torch.full((forks * d,), MASKED, dtype=torch.uint8, device="cuda")
+        n_c, n_l = (torch.zeros(forks, dtype=torch.int32, device="cuda") for _ in range(2))
+        fdd.fdd_decode_block(ctx, [forkset], layers, 1, [list(q)], [list(k)], [list(v)], [list(looped)], [normal(forks * d, vocab)], tokens,
+                             state, [d], scale, 0, 0.9, 0.0, 0, 0, n_c, n_l)
+        fdd.fdd_poll_status(ctx)
+        for out in (called, looped):
+            assert error(out) <= 1.01 * error(finer), (error(out), error(finer))
+    finally:
+        fdd.fdd_destroy(ctx)
