@@ -472,7 +472,10 @@ __device__ __forceinline__ void plan(const TcArgs<MAXSETS>& a, const SetParams* 
 }
 
 // Merge of a unit whose pieces lie in the shared memory of the CTAs of a cluster (piece k in CTA k): CT float4 columns of
-// one row, out = sum_k 2^(m_k - M) O_k / sum_k 2^(m_k - M) l_k.  All reads of kAtOnce pieces are in flight together.
+// one row, out = sum_k w_k O_k / sum_k w_k with w_k = 2^(m_k - M) l_k.  All reads of kAtOnce pieces are in flight together.
+// The pieces lie there divided by their row sums, and the weights carry 2^-32 (row sums stay below 2^32: probabilities of up to
+// 2^8, 2^24 keys), so that the sum is no larger than the largest value of V: what does not overflow inside a piece does not
+// overflow here.
 template <int D, int CT, int kAtOnce>
 __device__ __forceinline__ void merge_cluster(uint32_t part, uint32_t ml, int n_pieces, int row, int col0, __nv_bfloat16* op) {
     float4 acc[CT];
@@ -503,8 +506,8 @@ __device__ __forceinline__ void merge_cluster(uint32_t part, uint32_t ml, int n_
 #pragma unroll
         for (int k = 0; k < kAtOnce; ++k) {
             if (k0 + k >= n_pieces || st[k].x == -CUDART_INF_F) continue;
-            const float w = exp2f(st[k].x - M);
-            wsum = fmaf(w, st[k].y, wsum);
+            const float w = exp2f(st[k].x - M) * (st[k].y * 2.3283064365386963e-10f);
+            wsum += w;
 #pragma unroll
             for (int c = 0; c < CT; ++c) {
                 acc[c].x = fmaf(w, ov[k][c].x, acc[c].x); acc[c].y = fmaf(w, ov[k][c].y, acc[c].y);
@@ -1203,6 +1206,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                 // both query tiles have read them
                 tc::named_barrier(1, 256);
                 if (active && ok) {
+                    const float inv = l > 0.0f ? 1.0f / l : 0.0f;
                     float4* po = reinterpret_cast<float4*>(smem) + q * 128 + row_local;
 #pragma unroll
                     for (int cc = 0; cc < D / 32; ++cc) {
@@ -1211,8 +1215,8 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                         tc::wait_ld();
 #pragma unroll
                         for (int v4 = 0; v4 < 8; ++v4)
-                            po[(cc * 8 + v4) * 256] = make_float4(__uint_as_float(o[v4 * 4]), __uint_as_float(o[v4 * 4 + 1]),
-                                                                  __uint_as_float(o[v4 * 4 + 2]), __uint_as_float(o[v4 * 4 + 3]));
+                            po[(cc * 8 + v4) * 256] = make_float4(__uint_as_float(o[v4 * 4]) * inv, __uint_as_float(o[v4 * 4 + 1]) * inv,
+                                                                  __uint_as_float(o[v4 * 4 + 2]) * inv, __uint_as_float(o[v4 * 4 + 3]) * inv);
                     }
                 }
                 // (a row that saw no key in this piece has a sum of 0 and counts for nothing)

@@ -613,6 +613,29 @@ def test_attention_units_in_clusters(hq, hkv, dim, prefix, page, forks, block, l
         fdd.fdd_destroy(ctx)
 
 
+@pytest.mark.parametrize("hq,hkv,forks", [(16, 2, 1), (16, 2, 8), (28, 4, 1)])
+def test_attention_units_in_clusters_with_large_values_spread_over_the_pieces(hq, hkv, forks):
+    # Equal scores: every key has the weight 1, and a row's output is the mean of V.  Over the keys of a piece (at most 1152
+    # of them) values of 2^117 add up to less than 2^128, over all 4096 they do not.
+    dim, prefix, block = 128, 4064, 32
+    sc = synth.Scene(prefix, forks, block, 0, 1)
+    w = synth.Workload("range", hq, hkv, dim, 512, "bf16", "peaked", 0.9, 1.0, (sc,), seed=90)
+    ctx = harness.create_context(w)
+    try:
+        scene = harness.GpuScene(ctx, w, 0)
+        scene.prefix_v[0].fill_(2.0 ** 117)
+        _, k, _ = synth.make_qkv(w, 0, 0, 0, 0)
+        kd = harness.bf16_tensor(k)
+        qd = torch.zeros(forks * block * hq * dim, dtype=torch.bfloat16, device="cuda")
+        vd = torch.full_like(kd, 2.0 ** 117)
+        out = torch.full_like(qd, float("nan"))
+        fdd.fdd_block_attn(ctx, [scene.forkset], 0, qd, kd, vd, out, [block], 1.0 / np.sqrt(dim), 0)
+        fdd.fdd_poll_status(ctx)
+        assert bool((out.float() == 2.0 ** 117).all())
+    finally:
+        fdd.fdd_destroy(ctx)
+
+
 def _in_child(code, **env):
     # settings that the library reads once per process
     here = os.path.dirname(os.path.abspath(__file__))
