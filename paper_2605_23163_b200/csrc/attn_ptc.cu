@@ -475,13 +475,15 @@ __device__ __forceinline__ void plan(const TcArgs<MAXSETS>& a, const SetParams* 
 // one row, out = sum_k w_k O_k / sum_k w_k with w_k = 2^(m_k - M) l_k.  All reads of kAtOnce pieces are in flight together.
 // The pieces lie there divided by their row sums, and the weights carry 2^-32 (row sums stay below 2^32: probabilities of up to
 // 2^8, 2^24 keys), so that the sum is no larger than the largest value of V: what does not overflow inside a piece does not
-// overflow here.
+// overflow here.  A row with a piece of a CTA that gave up (its row sum says so) is not written.
+constexpr float kGaveUp = -1.0f;
 template <int D, int CT, int kAtOnce>
 __device__ __forceinline__ void merge_cluster(uint32_t part, uint32_t ml, int n_pieces, int row, int col0, __nv_bfloat16* op) {
     float4 acc[CT];
 #pragma unroll
     for (int c = 0; c < CT; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
     float M = -CUDART_INF_F, wsum = 0.0f;
+    bool whole = true;                                              // no piece comes from a CTA that gave up
     for (int k0 = 0; k0 < n_pieces; k0 += kAtOnce) {
         float2 st[kAtOnce];
         float4 ov[kAtOnce][CT];
@@ -496,7 +498,10 @@ __device__ __forceinline__ void merge_cluster(uint32_t part, uint32_t ml, int n_
         float mn = M;
 #pragma unroll
         for (int k = 0; k < kAtOnce; ++k)
-            if (k0 + k < n_pieces) mn = fmaxf(mn, st[k].x);
+            if (k0 + k < n_pieces) {
+                mn = fmaxf(mn, st[k].x);
+                whole = whole && st[k].y != kGaveUp;
+            }
         if (!(mn > -CUDART_INF_F)) continue;                        // nothing but pieces without a visible key so far
         const float back = exp2f(M - mn);
         wsum *= back;
@@ -515,6 +520,7 @@ __device__ __forceinline__ void merge_cluster(uint32_t part, uint32_t ml, int n_
             }
         }
     }
+    if (!whole) return;
     const float iw = wsum > 0.0f ? 1.0f / wsum : 0.0f;
 #pragma unroll
     for (int c = 0; c < CT; ++c) {
@@ -1220,7 +1226,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                     }
                 }
                 // (a row that saw no key in this piece has a sum of 0 and counts for nothing)
-                row_ml_s[q * 128 + row_local] = make_float2(l == 0.0f ? -CUDART_INF_F : m_used, l);
+                row_ml_s[q * 128 + row_local] = ok ? make_float2(l == 0.0f ? -CUDART_INF_F : m_used, l) : make_float2(-CUDART_INF_F, kGaveUp);
                 if (!ok) {
                     if (*abort_flag == 0) atomicCAS(a.status, 0, FDD_ERR_DEVICE_TIMEOUT);
                     *abort_flag = 1;
@@ -1408,7 +1414,7 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
 
         if (CLUSTERED) {
             // Every CTA of the cluster merges an equal share of the unit's rows out of all their shared memories.  (A CTA
-            // that gave up has set the status and takes part all the same: nobody waits for ever.)
+            // that gave up has set the status, marked its rows and takes part all the same: nobody waits for ever.)
             __syncwarp();
             tc::cluster_sync();
             const SetParams& p = sets[0];
