@@ -1066,10 +1066,15 @@ attn_ptc_kernel(const __grid_constant__ TcArgs<MAXSETS> a) {
                             tc::tmem_ld32(tm_o[q] + lane_base + cc * 32, o);
                             tc::wait_ld();
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                            for (int i = 0; i < 32; i += 2) {
+                                float o0, o1;
+                                tc::unpack2(tc::fma2(tc::pack2(__uint_as_float(o[i]), __uint_as_float(o[i + 1])), tc::pack2(alpha, alpha), 0ull), o0, o1);
+                                o[i] = __float_as_uint(o0);
+                                o[i + 1] = __float_as_uint(o1);
+                            }
                             tc::tmem_st32(tm_o[q] + lane_base + cc * 32, o);
                         }
-                        tc::wait_st();
+                        if (!kRef) tc::wait_st();                       // (or with P's)
                     };
                     bool pv_done = kOwn || jl == 0, rescale = false;
                     float alpha = 1.0f;
