@@ -3,7 +3,7 @@
 //
 // Kernel 1 (unmask_stream_kernel): persistent grid, every warp on its own.  The MASKED rows of the
 // call, cut into tiles of 2048 ids, are split into pieces of a few tiles: one piece per warp when there are few rows,
-// else the warps draw them from a counter (one record per piece, merged by the
+// else equal ranges or pieces that the warps draw from a counter (one record per piece, merged by the
 // second kernel).  A warp streams its tiles from HBM once, through a ring of bulk asynchronous
 // copies (cp.async.bulk, completion on an mbarrier, no multicast) into its own part of shared
 // memory, three tiles deep; a lane takes 64 consecutive ids of a tile (16-byte reads, chunk order
@@ -56,6 +56,7 @@ constexpr int kLaneIds = 64;                          // consecutive ids a lane 
 constexpr int kTile = kUnmaskTile;                    // ids per tile (one bulk copy, one warp)
 constexpr int kStages = 3;                            // tiles a warp holds in shared memory (two in flight while one is reduced)
 constexpr int kMaxRows = kUnmaskMaxRows;              // rows of one launch (32 per thread in the set-up)
+constexpr int kPiecePad = 1;                          // items that stand for what a piece costs beside its tiles
 constexpr int kMinPiecesPerRow = 8;                   // a warp gets one piece when each row can have this many warps
 constexpr int kDealtShare = 6, kDealtLeast = 3, kDealtMost = 12;   // short pieces that are dealt out: a sixth of a warp's share, of 3 to 12 tiles
 constexpr int kMaxList = 224;                         // blocks in reach of the running lower bound kept per piece (a few dozen expected)
@@ -326,6 +327,13 @@ struct Reach {
 };
 static_assert(sizeof(Reach) == 8, "eight bytes per kept block");
 
+// Equal ranges over the rows' items, laid end to end: a row is row_axis places long, its items behind `pad` empty ones.
+struct Ranges {
+    int row_axis, pad;
+    int ppr;                                            // > 0: no ranges, every row is cut into ppr pieces
+    int axis;                                           // all rows
+};
+
 // Shared memory of the streaming kernel beyond its static arrays: the rings, the lists of kept blocks, the barriers.
 // A ragged row's tile comes with the 16-byte granules it shares with its neighbours.
 template <typename T, bool RAGGED>
@@ -359,6 +367,9 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* state,
     __shared__ uint32_t s_mask[kMaxRows / 32];          // which rows are selected (MASKED, or DRAFT for the verifier), 32 to a word
     __shared__ int2 s_open[kWarps][8];                  // (row, piece of the row) of the pieces a warp has begun to copy
     __shared__ int s_n_list[kWarps];
+    constexpr bool kEqual = sizeof(T) == 2 && !NOISY && !RAGGED;                      // all pieces are equal ranges
+    __shared__ Ranges s_ranges[kEqual ? kWarps : 1];    // (a copy for every warp: the tile loop has no registers to spare)
+    __shared__ int4 s_cut[kEqual ? kWarps : 1][8];      // ... and for the pieces in s_open: first tile, tile behind the last, pieces of the row
     extern __shared__ __align__(128) unsigned char s_dyn[];
     constexpr int kStageBytes = stream_stage_bytes<T, RAGGED>();
     constexpr int kPerChunk = Logit<T>::kPerChunk;
@@ -426,21 +437,45 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* state,
     // items, and a piece leaves one record.  (A call has far fewer than 2^31 tiles: they lie in the GPU's memory.)
     //  - Few rows: as many pieces as there are warps, one for each, where each row can have kMinPiecesPerRow of them or
     //    where that makes no piece longer than an equal share.
-    //  - Otherwise most of every row goes into long pieces, about one for each warp, and the rest into pieces of a few
-    //    tiles, which the warps draw from a counter while they still work on the piece before.  SMs stream at rates that
-    //    differ by a quarter (with equal ranges the warps of a launch over 1216 rows of 152k ids ended after 52 us at the
-    //    median and 66 us at the latest, greedy, and 71 and 89 us with noise), and every piece costs about a microsecond.
-    //    Whole calls, equal ranges -> long and short pieces, us: 1216 rows of 151936 bf16 logits 67.5 -> 68.3 greedy and
-    //    93.6 -> 92.7 with noise, 608 rows 41.5 -> 43.5 and 59.9 -> 53.8, 1216 rows of 50257 49.6 -> 45.5 and 72.5 -> 63.2,
-    //    2048 rows of 32000 with noise 57.2 -> 51.2, 720 rows of fp32 logits 74.7 -> 72.5 and 86.4 -> 79.5.  With 0.7 and
-    //    0.9 of a share in long pieces 608 rows with noise took 55.3 and 55.4; short pieces alone 60.6.
+    //  - Otherwise, greedy over bf16 rows that start on 16 bytes (kEqual): the rows' items end to end in equal ranges, a warp
+    //    each.  Every piece costs about as much as a tile beside its own (opening, look-up, record), so kPiecePad items in
+    //    front of every row stand for that where ranges are long.  These launches are bound by instructions more than the
+    //    others, most of all at the lower clocks of a loaded GPU, and pieces dealt out as below cost them more than an even finish
+    //    gives.  Whole calls, dealt out -> equal ranges, us, clocks free and (after heavy products) lowered, 151936 ids: 1216 rows 71.0 -> 70.9
+    //    (97.6 -> 95.5), 608 rows 60.5 -> 55.4 (62.9 -> 57.6), 800 rows 56.6 -> 52.7 (74.6 -> 69.7), 1520 rows 86.2 -> 84.6 (117.7 ->
+    //    113.7); 1216 rows of 128256 63.5 -> 60.7 (87.3 -> 83.3).  Without the padding 1520 rows took 86.5 (116.7).
+    //  - Otherwise most of every row goes into long pieces, as many for each row as there are whole warps for it, and the rest
+    //    into pieces of a few tiles, which the warps draw from a counter while they still work on the piece before (warps without
+    //    a long piece from the start).  SMs stream at rates that differ by a quarter (with equal ranges the warps of a
+    //    launch over 1216 rows of 152k ids with noise ended after 71 us at the median and 89 us at the latest).
+    //    Whole calls, equal ranges -> long and short pieces, us: 1216 rows of 151936 bf16 logits with noise 95.2 -> 91.2, 608 rows
+    //    60.4 -> 53.6, 1064 rows 86.1 -> 76.0, 1216 rows of 50257 49.3 -> 45.2 greedy and 73.1 -> 62.7 with noise, 720 rows of fp32
+    //    logits 78.6 -> 74.4 and 83.1 -> 80.1.  A long piece for every warp, whole rows' long parts cut into equal ranges or some
+    //    rows with one long piece more than others, was faster at 1216 rows (89.5 and 90.8 us with noise) and slower at 1064 (82.1 and 82.7).
     const int tiles_per_row = (vocab + kTile - 1) / kTile;
     const int ipr = (tiles_per_row + tiles_per_item - 1) / tiles_per_item;
     const int warps_all = static_cast<int>(gridDim.x) * kWarps;
     const int gw = warp * static_cast<int>(gridDim.x) + static_cast<int>(blockIdx.x);   // warps of a CTA lie a grid apart: few pieces spread over all SMs
     constexpr int kLongShare = sizeof(T) == 2 ? 8 : 6;            // tenths of a warp's share that are its long piece
     int ppr = min(ipr, warps_all / n_rows), n_long = 0, long_items = 0;
-    {
+    int r_at = 0, r_end = 0;                            // (kEqual) the warp's range, on the axis of all rows' items end to end
+    Ranges& R = s_ranges[kEqual ? warp : 0];
+    if (kEqual) {
+        const int share = (n_rows * ipr + warps_all - 1) / warps_all;
+        const bool by_row = !(ppr < min(ipr, kMinPiecesPerRow) && (ppr == 0 || (ipr + ppr - 1) / ppr > share));
+        const int pad = !by_row && share >= 16 * kPiecePad ? kPiecePad : 0, row_axis = ipr + pad;
+        if (lane == 0) R = Ranges{row_axis, pad, by_row ? ppr : 0, n_rows * row_axis};
+        if (by_row) {
+            const int ri = gw / ppr, pc = gw - ri * ppr;
+            if (ri >= n_rows) return;
+            r_at = ri * ipr + static_cast<int>(static_cast<long long>(ipr) * pc / ppr);
+            r_end = ri * ipr + static_cast<int>(static_cast<long long>(ipr) * (pc + 1) / ppr);
+        } else {
+            r_at = static_cast<int>(static_cast<long long>(n_rows * row_axis) * gw / warps_all);
+            r_end = static_cast<int>(static_cast<long long>(n_rows * row_axis) * (gw + 1) / warps_all);
+        }
+        __syncwarp();
+    } else {
         const int share = (n_rows * ipr + warps_all - 1) / warps_all;
         if (ppr < min(ipr, kMinPiecesPerRow) && (ppr == 0 || (ipr + ppr - 1) / ppr > share)) {
             const int len = max(1, min(max(share * tiles_per_item / kDealtShare, kDealtLeast), kDealtMost) / tiles_per_item);
@@ -450,14 +485,14 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* state,
             ppr = n_long + (ipr - n_long * long_items + len - 1) / len;
         }
     }
-    const int n_short = ppr - n_long, n_pieces = n_rows * ppr;
+    const int n_short = max(1, ppr - n_long), n_pieces = n_rows * ppr;
     const int short_items = (ipr - n_long * long_items) / n_short, short_more = ipr - n_long * long_items - short_items * n_short;
     // first item of a piece (the first short_more short pieces of a row have one item more)
     auto first_item = [&](int pc) {
         if (pc <= n_long) return pc * long_items;
         return n_long * long_items + (pc - n_long) * short_items + min(pc - n_long, short_more);
     };
-    if (gw >= n_pieces) return;
+    if (!kEqual && gw >= n_pieces) return;
 
     const uint32_t full = 0xFFFFFFFFu;
     const int sw = lane & 7;                            // rotation of the chunk order (bank conflicts)
@@ -476,7 +511,30 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* state,
     const uintptr_t whole_begin = (reinterpret_cast<uintptr_t>(logits) + 15) & ~uintptr_t(15);
     const uintptr_t whole_end = reinterpret_cast<uintptr_t>(logits + static_cast<size_t>(rows) * vocab) & ~uintptr_t(15);
     auto produce_one = [&](int stage) {
-        if (p_tile == p_tile_end) {
+        if (kEqual) {
+            while (p_tile == p_tile_end) {
+                if (r_at >= r_end) return;
+                const int ri = r_at / R.row_axis, o = r_at - ri * R.row_axis, o_end = min(R.row_axis, o + r_end - r_at);
+                r_at += o_end - o;
+                p_tile = max(0, o - R.pad) * tiles_per_item;
+                p_tile_end = min(tiles_per_row, max(0, o_end - R.pad) * tiles_per_item);
+                if (p_tile == p_tile_end) continue;     // (padding alone)
+                const int row = selected_row(ri);
+                p_row_ptr = logits + static_cast<size_t>(row) * vocab;
+                int first = ri * R.ppr, of = R.ppr;     // the warp that holds the row's first item, and how many hold one
+                if (R.ppr == 0) {
+                    const long long at = static_cast<long long>(ri) * R.row_axis;
+                    first = static_cast<int>(((at + R.pad + 1) * warps_all - 1) / R.axis);
+                    of = static_cast<int>(((at + R.row_axis) * warps_all - 1) / R.axis) - first + 1;
+                }
+                if (lane == 0) {
+                    s_open[warp][p_open & 7] = make_int2(row, gw - first);
+                    s_cut[kEqual ? warp : 0][p_open & 7] = make_int4(p_tile, p_tile_end, of, 0);
+                }
+                ++p_open;
+                __syncwarp();
+            }
+        } else if (p_tile == p_tile_end) {
             const int id = __shfl_sync(full, p_next, 0);
             if (id >= n_pieces) return;
             // (the long pieces of all rows come first)
@@ -523,7 +581,17 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* state,
     for (int c_open = 0; c_open != p_open && alive; ++c_open) {
         // ---- open the piece: tiles [tile0, tile1) of one row
         const int row = s_open[warp][c_open & 7].x, pc = s_open[warp][c_open & 7].y;
-        const int tile0 = first_item(pc) * tiles_per_item, tile1 = min(tiles_per_row, first_item(pc + 1) * tiles_per_item);
+        int tile0, tile1, of;                           // its tiles, and how many pieces the row has
+        if (kEqual) {
+            const int4 cut = s_cut[kEqual ? warp : 0][c_open & 7];
+            tile0 = cut.x;
+            tile1 = cut.y;
+            of = cut.z;
+        } else {
+            tile0 = first_item(pc) * tiles_per_item;
+            tile1 = min(tiles_per_row, first_item(pc + 1) * tiles_per_item);
+            of = ppr;
+        }
         const int seg_end = min(vocab, tile1 * kTile);
         uint32_t* const row_bar = shared_words + kSharedBars + row;
         const T* row_ptr = logits + static_cast<size_t>(row) * vocab;
@@ -778,7 +846,7 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* state,
             UnmaskPartial out;
             out.row_max = row_ref; out.sum_exp = s; out.best_score = best.score; out.best_logit = best.logit;
             out.best_index = best.index;
-            out.pad[0] = ppr;                           // how many records this row has (read from record 0)
+            out.pad[0] = of;                            // how many records this row has (read from record 0)
             out.pad[1] = out.pad[2] = 0;
             partial[static_cast<size_t>(row) * ipr + pc] = out;
         }

@@ -968,7 +968,9 @@ def test_unmask_rows_that_start_anywhere(dtype, vocab, offset, temperature, monk
 
 @pytest.mark.parametrize("dtype,forks,block,vocab,temperature", [
     ("bf16", 32, 128, 2049, 0.9),        # more rows than warps, two tiles each, ragged: whole rows are dealt out
-    ("bf16", 20, 64, 17000, 0.0),        # three pieces a row, dealt out
+    ("bf16", 20, 64, 17000, 0.0),        # equal ranges of three and four tiles
+    ("bf16", 26, 50, 79000, 0.0),        # equal ranges of sixteen, the rows padded
+    ("bf16", 20, 64, 17000, 0.7),        # three pieces a row, dealt out
     ("f32", 10, 128, 8192, 0.8),         # the same for fp32
     ("bf16", 13, 25, 30000, 0.9),        # seven pieces a row, one for each warp
 ])
