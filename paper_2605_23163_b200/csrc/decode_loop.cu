@@ -7,6 +7,7 @@
 // native code and runs one step ahead of the counts it reads.
 #include "fdd_internal.h"
 
+#include <algorithm>
 #include <chrono>
 
 namespace {
@@ -115,7 +116,7 @@ fdd_status fdd_decode_block(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, 
     auto follow = [&](cudaStream_t to, cudaStream_t from, cudaEvent_t ev) {
         return cuda_ok(cudaEventRecord(ev, from)) && cuda_ok(cudaStreamWaitEvent(to, ev, 0));
     };
-    auto gate_slot = [&](int t) { return ctx->gate_slots + static_cast<size_t>(t % kGateSlots) * ctx->cfg.max_forks; };
+    auto gate_slot = [&](int t) { return ctx->gate_slots + static_cast<size_t>(t % kGateSlots) * std::min(ctx->cfg.max_forks, kAttnMaxGatedForks); };
 
     int stamp_of[2] = {0, 0};
     // From the second step on, attention skips the rollouts that the step before left without a MASKED position.

@@ -30,6 +30,7 @@ fdd_status cuda_fail(fdd_ctx* ctx, cudaError_t e, const char* what) {
 // Seeds travel to the device as kernel arguments: stream-ordered like everything else, no
 // staging buffer, no allocation, no synchronisation.
 constexpr size_t kMapPoolEntries = 64;
+constexpr long long kLayeredUnits = 1 << 20;    // units up to which a launch takes several layers (8 MB of counters)
 constexpr int kSeedsPerLaunch = 240;
 struct SeedChunk {
     uint64_t value[kSeedsPerLaunch];
@@ -224,8 +225,16 @@ fdd_status block_attn_layers(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets,
         const int launches = (count + room - 1) / room, most = (count + launches - 1) / launches;
         for (int first = 0; first < count;) {
             int n = 0, forks = 0;
-            while (n < most && first + n < count && (n == 0 || !gate || forks + probs[first + n].n_forks <= kAttnMaxGatedForks))
-                forks += probs[first + n++].n_forks;
+            long long units = 0;
+            while (n < most && first + n < count) {
+                const AttnProblem& p = probs[first + n];
+                const int tile_pos = 128 / (p.n_q_heads / p.n_kv_heads);
+                const long long more = static_cast<long long>(p.n_kv_heads) * ((p.d + tile_pos - 1) / tile_pos) * p.n_forks;
+                if (n > 0 && ((gate && forks + p.n_forks > kAttnMaxGatedForks) || units + more > ctx->attn_max_units)) break;
+                forks += p.n_forks;
+                units += more;
+                ++n;
+            }
             int n_launches = 0;
             cudaError_t e = launch_attention_ptc(ctx, probs.data() + first, caches.data() + first, n, c.head_dim, st_, beside, alone, &n_launches);
             ctx->launches += n_launches;
@@ -443,13 +452,14 @@ fdd_status fdd_create(const fdd_config* cfg, fdd_ctx** out) {
         const int G = cfg->n_q_heads / cfg->n_kv_heads;
         const int tile_pos = 128 / G;
         const int q_tiles = (cfg->max_block + tile_pos - 1) / tile_pos;
-        // (a launch takes up to kTcMaxSets layers of a call)
-        ctx->attn_max_units = cfg->n_kv_heads * q_tiles * cfg->max_forks * std::min(cfg->n_layers, kTcMaxSets);
+        // (a launch takes up to kTcMaxSets layers of a call, fewer where a layer alone has very many units)
+        const long long one_layer = static_cast<long long>(cfg->n_kv_heads) * q_tiles * cfg->max_forks;
+        ctx->attn_max_units = static_cast<int>(std::max(one_layer, std::min(one_layer * std::min(cfg->n_layers, kTcMaxSets), kLayeredUnits)));
         // two counters per unit: pieces written, CTAs done with their share of the merge
-        e = cudaMalloc(&ctx->attn_unit_count, sizeof(int) * 2 * ctx->attn_max_units);
-        if (e == cudaSuccess) e = cudaMemset(ctx->attn_unit_count, 0, sizeof(int) * 2 * ctx->attn_max_units);
+        e = cudaMalloc(&ctx->attn_unit_count, sizeof(int) * 2 * static_cast<size_t>(ctx->attn_max_units));
+        if (e == cudaSuccess) e = cudaMemset(ctx->attn_unit_count, 0, sizeof(int) * 2 * static_cast<size_t>(ctx->attn_max_units));
     }
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->gate_slots, sizeof(int32_t) * kGateSlots * static_cast<size_t>(cfg->max_forks));
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->gate_slots, sizeof(int32_t) * kGateSlots * static_cast<size_t>(std::min(cfg->max_forks, kAttnMaxGatedForks)));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking);
     for (cudaEvent_t* ev : {&ctx->ev_gate[0], &ctx->ev_gate[1], &ctx->ev_end})
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
@@ -816,7 +826,7 @@ fdd_status fdd_poll_status(fdd_ctx* ctx, void* stream) {
     const int code = *ctx->h_status;
     if (code != FDD_OK) {
         // a kernel that gave up may have left piece counters of the attention merge half counted
-        cudaMemsetAsync(ctx->attn_unit_count, 0, sizeof(int) * 2 * ctx->attn_max_units, st);
+        cudaMemsetAsync(ctx->attn_unit_count, 0, sizeof(int) * 2 * static_cast<size_t>(ctx->attn_max_units), st);
         cudaStreamSynchronize(st);
         return fail(ctx, code, "a kernel recorded device status %d", code);
     }

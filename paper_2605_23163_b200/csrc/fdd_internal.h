@@ -79,7 +79,7 @@ struct fdd_ctx {
     // fdd_decode_block runs the attention of its steps on a stream of its own, beside the unmasking (decode_loop.cu)
     cudaStream_t side_stream = nullptr;
     cudaEvent_t ev_gate[2] = {nullptr, nullptr}, ev_end = nullptr;
-    int32_t* gate_slots = nullptr;    // device [kGateSlots][max_forks]: what every step left, for the attention of the next one
+    int32_t* gate_slots = nullptr;    // device [kGateSlots][rollouts a gate takes]: what every step left, for the attention of the next one
     int32_t* unmask_gate_out = nullptr;   // where fdd_unmask puts n_left a second time (nullptr: nowhere)
     uint64_t launches = 0;
     std::string last_error;

@@ -525,3 +525,29 @@ def test_longer_pieces_are_as_precise_as_the_finer_cut(layers, forks, prefix):
             assert error(out) <= 1.01 * error(finer), (error(out), error(finer))
     finally:
         fdd.fdd_destroy(ctx)
+
+
+def test_context_for_many_rollouts_and_layers():
+    # 24 layers times 128 units of each of 700,000 rollouts are more than 2^31 counters: a context keeps no more than one
+    # layer takes, and launches hold as many layers as that leaves room for.
+    hq, hkv, dim, d, layers, n, prefix = 128, 8, 64, 128, 24, 1, 130
+    ctx = fdd.fdd_create(hq, hkv, dim, 512, layers, 0, d, 700_000, fdd.FDD_LOGITS_BF16)
+    try:
+        gen = torch.Generator(device="cuda")
+        gen.manual_seed(7)
+        normal = lambda *shape: torch.randn(shape, generator=gen, device="cuda").to(torch.bfloat16)
+        pk, pv = normal(layers, hkv, prefix, dim), normal(layers, hkv, prefix, dim)
+        sk, sv = (torch.zeros((layers, n, hkv, d, dim), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        q, k, v = normal(layers, n, d, hq, dim), normal(layers, n, d, hkv, dim), normal(layers, n, d, hkv, dim)
+        out = torch.full_like(q, float("nan"))
+        forkset = fdd.fdd_fork(ctx, list(pk), list(pv), None, prefix, prefix, n, [1], list(sk), list(sv), d)
+        tokens, state = torch.zeros(d, dtype=torch.int32, device="cuda"), torch.full((d,), MASKED, dtype=torch.uint8, device="cuda")
+        n_c, n_l = (torch.zeros(n, dtype=torch.int32, device="cuda") for _ in range(2))
+        fdd.fdd_decode_block(ctx, [forkset], layers, 2, [list(q)], [list(k)], [list(v)], [list(out)], [normal(d, 512)], tokens, state, [d],
+                             dim ** -0.5, 0, 0.9, 0.0, 0, 0, n_c, n_l)
+        fdd.fdd_poll_status(ctx)
+        for l in (0, layers - 1):
+            ref = _attention64(q[l], k[l], v[l], pk[l], pv[l], dim ** -0.5)
+            pu.assert_attention_close(out[l].float().cpu().numpy().astype(np.float64), ref.cpu().numpy())
+    finally:
+        fdd.fdd_destroy(ctx)
