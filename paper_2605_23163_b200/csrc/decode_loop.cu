@@ -58,6 +58,35 @@ fdd_status wait_for_counts(fdd_ctx* ctx, int buf, int stamp, int forks, cudaStre
     return FDD_OK;
 }
 
+// Whether `st` belongs to a green context (a share of the SMs that its work is confined to).
+bool in_green_context(cudaStream_t st) {
+    using GetGreenCtx = CUresult (*)(CUstream, CUgreenCtx*);
+    static const GetGreenCtx get = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        const bool ok = cudaGetDriverEntryPoint("cuStreamGetGreenCtx", &p, cudaEnableDefault, &found) == cudaSuccess && found == cudaDriverEntryPointSuccess;
+        return ok ? reinterpret_cast<GetGreenCtx>(p) : nullptr;
+    }();
+    CUgreenCtx green = nullptr;
+    return get != nullptr && get(st, &green) == CUDA_SUCCESS && green != nullptr;
+}
+
+// The context's own stream of the same priority as the caller's; nullptr where there is none to be had, or none that the
+// caller's limits would hold for.
+cudaStream_t side_stream_of(fdd_ctx* ctx, cudaStream_t st) {
+    int priority = 0;
+    if (in_green_context(st) || cudaStreamGetPriority(st, &priority) != cudaSuccess) return nullptr;
+    for (const fdd_ctx::SideStream& s : ctx->side_streams)
+        if (s.priority == priority) return s.stream;
+    cudaStream_t made = nullptr;
+    if (cudaStreamCreateWithPriority(&made, cudaStreamNonBlocking, priority) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    ctx->side_streams.push_back({priority, made});
+    return made;
+}
+
 }  // namespace
 
 fdd_status fdd_decode_block(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, int n_layers,
@@ -104,10 +133,11 @@ fdd_status fdd_decode_block(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, 
     // One behind the other -> side by side, us: twelve steps of the smallest block 223 -> 157, three blocks of one rollout
     // 398 -> 260, of eight 737 -> 594, 36 layers of eight 1525 -> 1469, 32 rollouts on 16384 tokens 1879 -> 1824.
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    const bool beside = before_step == nullptr && forks <= kAttnMaxGatedForks && scale > 0.0f && cudaStreamIsCapturing(st, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone &&
+    bool beside = before_step == nullptr && forks <= kAttnMaxGatedForks && scale > 0.0f && cudaStreamIsCapturing(st, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone &&
                         attention_beside_unmasking(ctx, sets, n_sets, n_layers, n_inputs < max_steps ? n_inputs : max_steps, q, k_blk, v_blk, out, logits,
                                                    tokens, state, block_len, n_committed, n_left);
-    const cudaStream_t st_attn = beside ? ctx->side_stream : st;
+    const cudaStream_t side = beside ? side_stream_of(ctx, st) : nullptr, st_attn = side ? side : st;
+    beside = side != nullptr;
     auto cuda_ok = [&](cudaError_t e) {
         if (e != cudaSuccess) ctx->last_error = std::string("fdd_decode_block: ") + cudaGetErrorString(e);
         return e == cudaSuccess;

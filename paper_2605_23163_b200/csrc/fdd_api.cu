@@ -460,7 +460,6 @@ fdd_status fdd_create(const fdd_config* cfg, fdd_ctx** out) {
         if (e == cudaSuccess) e = cudaMemset(ctx->attn_unit_count, 0, sizeof(int) * 2 * static_cast<size_t>(ctx->attn_max_units));
     }
     if (e == cudaSuccess) e = cudaMalloc(&ctx->gate_slots, sizeof(int32_t) * kGateSlots * static_cast<size_t>(std::min(cfg->max_forks, kAttnMaxGatedForks)));
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&ctx->side_stream, cudaStreamNonBlocking);
     for (cudaEvent_t* ev : {&ctx->ev_gate[0], &ctx->ev_gate[1], &ctx->ev_end})
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     if (e != cudaSuccess) {
@@ -489,7 +488,7 @@ void fdd_destroy(fdd_ctx* ctx) {
     if (ctx->gate_slots) cudaFree(ctx->gate_slots);
     for (cudaEvent_t ev : {ctx->ev_gate[0], ctx->ev_gate[1], ctx->ev_end})
         if (ev) cudaEventDestroy(ev);
-    if (ctx->side_stream) cudaStreamDestroy(ctx->side_stream);
+    for (const fdd_ctx::SideStream& s : ctx->side_streams) cudaStreamDestroy(s.stream);
     delete static_cast<SeedChunk*>(ctx->seed_chunk);
     delete ctx;
 }

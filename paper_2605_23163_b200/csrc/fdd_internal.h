@@ -77,7 +77,8 @@ struct fdd_ctx {
     long long attn_merge_wait_limit = kMergeWaitDefault;   // SM clocks: wait for the pieces of a cut unit
     void* seed_chunk = nullptr;       // host staging of seeds on their way to the device as kernel arguments
     // fdd_decode_block runs the attention of its steps on a stream of its own, beside the unmasking (decode_loop.cu)
-    cudaStream_t side_stream = nullptr;
+    struct SideStream { int priority; cudaStream_t stream; };
+    std::vector<SideStream> side_streams;     // one for every priority that a caller's stream had
     cudaEvent_t ev_gate[2] = {nullptr, nullptr}, ev_end = nullptr;
     int32_t* gate_slots = nullptr;    // device [kGateSlots][rollouts a gate takes]: what every step left, for the attention of the next one
     int32_t* unmask_gate_out = nullptr;   // where fdd_unmask puts n_left a second time (nullptr: nowhere)

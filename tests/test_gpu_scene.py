@@ -551,3 +551,37 @@ def test_context_for_many_rollouts_and_layers():
             pu.assert_attention_close(out[l].float().cpu().numpy().astype(np.float64), ref.cpu().numpy())
     finally:
         fdd.fdd_destroy(ctx)
+
+
+def test_library_block_loop_on_streams_of_any_priority():
+    # The stream that the attention runs on has the priority of the caller's; several of them may be in use in turn.
+    hq, hkv, dim, vocab, n, d, prefix = 16, 2, 128, 512, 4, 16, 1000
+    ctx = fdd.fdd_create(hq, hkv, dim, vocab, 1, 0, d, n, fdd.FDD_LOGITS_BF16)
+    try:
+        gen = torch.Generator(device="cuda")
+        gen.manual_seed(8)
+        normal = lambda *shape: torch.randn(shape, generator=gen, device="cuda").to(torch.bfloat16)
+        pk, pv = normal(hkv, prefix, dim), normal(hkv, prefix, dim)
+        sk, sv = (torch.zeros((n, hkv, d, dim), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        forkset = fdd.fdd_fork(ctx, [pk], [pv], None, prefix, prefix, n, [1, 2, 3, 4], [sk], [sv], d)
+        q, k, v, logits = normal(n, d, hq, dim), normal(n, d, hkv, dim), normal(n, d, hkv, dim), normal(n * d, vocab)
+        ref = _attention64(q, k, v, pk, pv, dim ** -0.5).cpu().numpy()
+        torch.cuda.synchronize()
+        seen = []
+        for priority in (0, -1, -3, 0, -1):
+            stream = torch.cuda.Stream(priority=priority)
+            with torch.cuda.stream(stream):
+                out = torch.full_like(q, float("nan"))
+                tokens = torch.zeros(n * d, dtype=torch.int32, device="cuda")
+                state = torch.full((n * d,), MASKED, dtype=torch.uint8, device="cuda")
+                n_c, n_l = (torch.zeros(n, dtype=torch.int32, device="cuda") for _ in range(2))
+                steps, left = fdd.fdd_decode_block(ctx, [forkset], 1, d, [[q]], [[k]], [[v]], [[out]], [logits], tokens, state, [d], dim ** -0.5,
+                                                   0, 0.9, 0.0, 0, 0, n_c, n_l)
+                got = out.float().cpu().numpy().astype(np.float64)
+            assert left == 0
+            pu.assert_attention_close(got, ref)
+            seen.append((steps, tokens.cpu().tolist()))
+        assert all(x == seen[0] for x in seen)
+        fdd.fdd_poll_status(ctx)
+    finally:
+        fdd.fdd_destroy(ctx)
