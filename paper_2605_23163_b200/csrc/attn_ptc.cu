@@ -141,6 +141,8 @@ struct TcArgs {
     long long merge_wait_limit; // SM clocks a CTA waits for the other pieces of a cut unit before it gives up
 };
 
+static_assert(sizeof(TcArgs<kTcMaxSets>) <= 32764, "the arguments of an attention launch");
+
 struct TileInfo {
     int segment;   // 0 prefix, 1 suffix, 2 block
     int index;     // tile index inside the segment

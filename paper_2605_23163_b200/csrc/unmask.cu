@@ -359,7 +359,7 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* state,
                      const __grid_constant__ UnmaskSets sets, UnmaskPartial* __restrict__ partial,
                      int vocab, int tiles_per_item, float temperature,
                      uint32_t block_idx, uint32_t step, int select_state,
-                     const uint32_t* __restrict__ step_counter, int* __restrict__ status, uint32_t* shared_words) {
+                     const uint32_t* step_counter, int* __restrict__ status, uint32_t* shared_words) {
     // The launch may have been made resident before the kernel ahead of it on the stream was done (its
     // set-up then overlaps that kernel's tail); nothing is read before the wait.  The kernel behind
     // this one (the per-rollout step) may come in as soon as every CTA here has started.
@@ -388,7 +388,8 @@ unmask_stream_kernel(const T* __restrict__ logits, const uint8_t* state,
     }
     tc::grid_dependency_wait();
     tc::grid_launch_dependents();
-    if (step_counter != nullptr) step += *step_counter;    // the denoising step as counted on the device
+    // the denoising step as counted on the device (by the kernel ahead of this one: a plain load could be moved ahead of the wait)
+    if (step_counter != nullptr) step += load_shared_word(step_counter);
 
     // ---- set-up (the only CTA-wide part): which rows are selected.  Every warp then keeps the count of selected rows
     // before the words of each lane, which is all it takes to find the ri-th of them.
