@@ -143,9 +143,10 @@ fdd_status fdd_forkset_reset(fdd_ctx* ctx, fdd_forkset* set);
  *                  32-byte pieces).
  *   block_len      host int32 [n_sets]: d_s, 1 <= d_s <= cfg.max_block.
  *   scale          soft-max scale (1/sqrt(D) by convention), the same for every set of the call.
- * The tensor-core kernel is launched cooperatively (its CTAs wait, with a bound, for one another's
- * partial results): it needs as many free SMs as it has CTAs, and the launch fails with
- * FDD_ERR_CUDA where the device cannot give them (an MPS share of the SMs, for instance).
+ * Where work is cut between CTAs that wait, with a bound, for one another's partial results, the tensor-core kernel is
+ * launched cooperatively: it needs as many free SMs as it has CTAs, and the launch fails with
+ * FDD_ERR_CUDA where the device cannot give them (an MPS share of the SMs, for instance).  Calls over one set with few
+ * units of work are launched in thread-block clusters of 4 to 16 CTAs instead, which need one cluster's SMs at a time.
  * All sets of a call go into one launch (groups of 16 sets).  Rollouts with equal inputs agree
  * up to the rounding of the bf16 output, not bit for bit: where a unit of work is cut between
  * CTAs depends on its place in the call.
@@ -343,12 +344,13 @@ fdd_status fdd_average_rollouts_jmt(fdd_ctx* ctx, const float* traj, int n, int 
  *   before_step            NULL, or a function the library calls as before_step(user, t, stream)
  *                          before it issues step t: the place where a caller enqueues, on `stream`,
  *                          the model work that produces step t's q / k / v / logits
- * Without a callback the attention of the steps runs on a stream of the context's own, beside the unmasking (unless they
- * share memory that one of them writes); `stream` waits for it before the commits, and so does whatever
- * the caller enqueues on `stream` after the call.
+ * Without a callback the attention of the steps runs on a stream of the context's own, of the priority of `stream`, beside
+ * the unmasking (unless they share memory that one of them writes, or `stream` belongs to a green context); `stream` waits for it
+ * before the commits, and so does whatever the caller enqueues on `stream` after the call.  The attention of the step that
+ * is issued ahead is then not issued at all, and one event a step is recorded on `stream`.
  * The counts reach the host through pinned host memory that the unmasking step writes itself
- * (count and a per-step stamp in one 8-byte store), which the call polls: no copy and no event sits
- * between two steps on the stream.  The poll is bounded: it ends with FDD_ERR_CUDA if the stream
+ * (count and a per-step stamp in one 8-byte store), which the call polls: no copy sits between two steps on the
+ * stream, and with a callback no event either.  The poll is bounded: it ends with FDD_ERR_CUDA if the stream
  * reports an error or runs empty without the counts, and with FDD_ERR_DEVICE_TIMEOUT after 30 s.
  * The call returns when the counts of the last step have reached the host; the attention and the commits it issued
  * may still be running.
@@ -376,8 +378,9 @@ fdd_status fdd_decode_block(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, 
  * cudaMalloc may block on the whole device, take unbounded time or fail late, so fdd_create and
  * fdd_fork (which allocate scratch and seed storage) are not available to such callers.  This
  * call needs neither a context nor a fork set and performs no allocation of any kind: its scratch
- * is a fixed array inside the library image (FDD_UNMASK_STATIC_MAX_RECORDS records of 32 bytes =
- * 2 MiB, resident on every GPU that loads the library until the process exits).
+ * is two fixed arrays inside the library image (FDD_UNMASK_STATIC_MAX_RECORDS records of 32 bytes =
+ * 2 MiB, and 32 KiB of words that the warps of a call share, resident on every GPU that loads the library until the
+ * process exits).
  *
  * It computes exactly what fdd_unmask computes for one set (same kernels, same rule, same noise).
  *   logits        device [n_forks][block_len][vocab], fp32 or bf16 per logits_dtype
@@ -390,12 +393,12 @@ fdd_status fdd_decode_block(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, 
  * rejected with FDD_ERR_CAPACITY before any launch (e.g. vocab 151936 has 19 record slots per row,
  * so up to 3449 rows: 32 rollouts x 64 positions fit).
  * Set-up: the first call on each device (with that device current) asks the runtime for the
- * device address of the array (cudaGetSymbolAddress) and caches it; make that first call before
+ * device address of the arrays (cudaGetSymbolAddress) and caches it; make that first call before
  * any stream capture begins.  Later calls do no set-up.
- * Sharing: all calls on a device use the same array, which keeps whatever the previous call
- * left in it.  Nothing in it has to start at zero: every record that is read was written earlier
- * in the same call (the first record of a row says how many of its records are valid).  Two calls whose kernels can overlap on the GPU (different streams without
- * ordering) race on it; order them.  The host side is not thread-safe for the first call per device.
+ * Sharing: all calls on a device use the same arrays.  The records keep whatever the previous call left in them (every
+ * record that is read was written earlier in the same call; the first record of a row says how many are valid).  The
+ * shared words are zero between calls: they start so, and each call leaves them so.  Two calls whose kernels can overlap on the GPU
+ * (different streams without ordering) race on both, and may lose each other's work or candidates without an error; order them.  The host side is not thread-safe for the first call per device.
  */
 #define FDD_UNMASK_STATIC_MAX_RECORDS 65536
 fdd_status fdd_unmask_static(const void* logits, int logits_dtype, int n_forks, int block_len,
@@ -455,9 +458,10 @@ fdd_status fdd_pull_masked_rows(fdd_ctx* ctx, const void* host_logits, void* dev
  * fdd_set_merge_wait_limit -- how long a CTA of fdd_block_attn waits for the partial results of the
  * other CTAs that share a unit of work with it, in SM clocks (default 4e9, about two seconds).  When
  * the limit runs out the CTA records FDD_ERR_DEVICE_TIMEOUT in the device status word and returns
- * without writing its share of the output; the launch itself always ends.  fdd_poll_status then
+ * without writing its share of the output; the launch itself always ends.  The barrier of a cluster has no such limit (every
+ * CTA of a cluster reaches it), so a context with a limit other than the default makes no launches in clusters.  fdd_poll_status then
  * reports the error and puts the context's counters back in order, and the next call is valid.
- * Meant for deployments that want a tighter bound than the default, and for testing the error path
+ * Meant for deployments that want a tighter bound than the default, and for testing the error path.
  */
 fdd_status fdd_set_merge_wait_limit(fdd_ctx* ctx, long long sm_clocks);
 
