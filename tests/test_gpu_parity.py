@@ -551,6 +551,7 @@ def test_attention_units_cut_into_pieces_of_their_own(hq, hkv, dim, prefix, fork
     w = synth.Workload("units", hq, hkv, dim, 512, "bf16", "peaked", 0.9, 1.0, (sc,), seed=80 + prefix)
     ctx = harness.create_context(w)
     try:
+        fdd.fdd_set_merge_wait_limit(ctx, 3_999_999_999)     # (with the default limit few units go to clusters: the next test)
         scene = harness.GpuScene(ctx, w, 0)
         pk, pv = synth.make_prefix(w, 0)
         empty = ([np.zeros((0, hkv, dim), dtype=np.uint16)] * forks,) * 2
