@@ -1751,7 +1751,8 @@ const int* resident_clusters(int device) {
 // two: what takes least time by a fit to measured launches (nanoseconds: 16 / 2, 32 / 8, 4 / 1, 28 / 4 and 12 / 2 heads, prefix
 // 1000 to 12000, one to eight rollouts, launches one behind the other, within 10 %; two microseconds more for launches
 // that are not in clusters, which start later behind another kernel).  Clusters of other sizes than powers of two take 4 to
-// 10 us more than the fit.  Of two halves of the probabilities the query tiles' chains are serial: longer steps, and
+// 10 us more than the fit.  The fit is of launches with head dimension 128 on an otherwise idle chip; 64, and launches beside
+// the unmasking, go by the same.  Of two halves of the probabilities the query tiles' chains are serial: longer steps, and
 // four CTAs are never enough.
 bool unit_clusters(const SetParams& p, int ctas, const int* resident, int* size, int* unit) {
     if (p.tiles_total <= kWholeTiles) return false;
@@ -1837,8 +1838,9 @@ cudaError_t launch_group(fdd_ctx* ctx, const AttnProblem* probs, TcMapCache* con
     if (ctas > ctx->attn_max_ctas) ctas = ctx->attn_max_ctas;
     // Beside other kernels SMs are worth something: a CTA spends 13 us outside its tile steps, as much as seven of them
     // take, so it gets at least that many; half the chip a launch may have in any case, for the rollouts that are left
-    // late in a block.  (16 / 2 heads, prefix 4096, three blocks side by side with their unmasking: eight rollouts 677 ->
-    // 600 us, one rollout 323 -> 281; the launch by itself takes longer, 35 against 26 us.)
+    // late in a block.  (Before there were clusters, 16 / 2 heads, prefix 4096, three blocks side by side with their unmasking: eight
+    // rollouts 677 -> 600 us, one rollout 323 -> 281; the launch by itself takes longer, 35 against 26 us.  Those two go to clusters now, which
+    // are exempt: 541 -> 520 us and 264 -> 233 for the blocks without this limit on them.)
     const long long most_ctas = ctas;
     if (beside) ctas = std::min(ctas, std::max<long long>(ctx->attn_max_ctas / 2, beside_ctas));
     if (ctas < 1) ctas = 1;
