@@ -72,7 +72,7 @@ bool in_green_context(cudaStream_t st) {
 }
 
 // The context's own stream of the same priority as the caller's; nullptr where there is none to be had, or none that the
-// caller's limits would hold for.
+// caller's limits would hold for: the attention then goes behind the unmasking on the caller's stream.
 cudaStream_t side_stream_of(fdd_ctx* ctx, cudaStream_t st) {
     int priority = 0;
     if (in_green_context(st) || cudaStreamGetPriority(st, &priority) != cudaSuccess) return nullptr;
@@ -133,11 +133,10 @@ fdd_status fdd_decode_block(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, 
     // One behind the other -> side by side, us: twelve steps of the smallest block 223 -> 157, three blocks of one rollout
     // 398 -> 260, of eight 737 -> 594, 36 layers of eight 1525 -> 1469, 32 rollouts on 16384 tokens 1879 -> 1824.
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    bool beside = before_step == nullptr && forks <= kAttnMaxGatedForks && scale > 0.0f && cudaStreamIsCapturing(st, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone &&
+    const bool beside = before_step == nullptr && forks <= kAttnMaxGatedForks && scale > 0.0f && cudaStreamIsCapturing(st, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone &&
                         attention_beside_unmasking(ctx, sets, n_sets, n_layers, n_inputs < max_steps ? n_inputs : max_steps, q, k_blk, v_blk, out, logits,
                                                    tokens, state, block_len, n_committed, n_left);
-    const cudaStream_t side = beside ? side_stream_of(ctx, st) : nullptr, st_attn = side ? side : st;
-    beside = side != nullptr;
+    cudaStream_t st_attn = st;                          // (another one is looked for once the first unmasking is on its way)
     auto cuda_ok = [&](cudaError_t e) {
         if (e != cudaSuccess) ctx->last_error = std::string("fdd_decode_block: ") + cudaGetErrorString(e);
         return e == cudaSuccess;
@@ -186,6 +185,8 @@ fdd_status fdd_decode_block(fdd_ctx* ctx, fdd_forkset* const* sets, int n_sets, 
     // short, and the CTAs of the attention take whole SMs.
     auto enqueue_attention = [&](int t) -> fdd_status {
         if (!beside) return FDD_OK;
+        if (t == 0)
+            if (const cudaStream_t side = side_stream_of(ctx, st)) st_attn = side;
         return cuda_ok(cudaStreamWaitEvent(st_attn, ctx->ev_gate[t & 1], 0)) ? attend(t) : FDD_ERR_CUDA;
     };
 

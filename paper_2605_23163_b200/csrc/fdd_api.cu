@@ -460,6 +460,9 @@ fdd_status fdd_create(const fdd_config* cfg, fdd_ctx** out) {
         if (e == cudaSuccess) e = cudaMemset(ctx->attn_unit_count, 0, sizeof(int) * 2 * static_cast<size_t>(ctx->attn_max_units));
     }
     if (e == cudaSuccess) e = cudaMalloc(&ctx->gate_slots, sizeof(int32_t) * kGateSlots * static_cast<size_t>(std::min(cfg->max_forks, kAttnMaxGatedForks)));
+    cudaStream_t side = nullptr;                        // (those of other priorities than the usual one are made when they are met: decode_loop.cu)
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking);
+    if (e == cudaSuccess) ctx->side_streams.push_back({0, side});
     for (cudaEvent_t* ev : {&ctx->ev_gate[0], &ctx->ev_gate[1], &ctx->ev_end})
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     if (e != cudaSuccess) {
